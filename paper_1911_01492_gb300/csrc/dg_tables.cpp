@@ -10,6 +10,8 @@
 // lambda_a / (t - xi_a) * prod_b (t - xi_b) with lambda_a = 1 / prod_{b!=a}
 // (xi_a - xi_b); collocation derivative D[a][b] = (lambda_b / lambda_a) /
 // (xi_a - xi_b) for a != b and D[a][a] = -sum_{b!=a} D[a][b].
+// All of it in long double (at least 64 mantissa bits), rounded once at the
+// end: the tables agree to the last bit with those of the fixed-point operator.
 #include <cmath>
 #include <cstring>
 
@@ -17,8 +19,10 @@
 
 namespace {
 
+typedef long double ld;
+
 // P_j(t) and P_j'(t) for j = 0..n-1 at t in [-1,1]
-void legendre_all(int n, double t, double* P, double* dP) {
+void legendre_all(int n, ld t, ld* P, ld* dP) {
   P[0] = 1.0;
   dP[0] = 0.0;
   if (n > 1) {
@@ -26,21 +30,21 @@ void legendre_all(int n, double t, double* P, double* dP) {
     dP[1] = 1.0;
   }
   for (int j = 1; j + 1 < n; ++j) {
-    P[j + 1] = ((2.0 * j + 1.0) * t * P[j] - j * P[j - 1]) / (j + 1.0);
-    dP[j + 1] = dP[j - 1] + (2.0 * j + 1.0) * P[j];
+    P[j + 1] = ((2 * j + 1.0) * t * P[j] - j * P[j - 1]) / (j + 1.0);
+    dP[j + 1] = dP[j - 1] + (2 * j + 1.0) * P[j];
   }
 }
 
 // P_n(t) and P_n'(t)
-void legendre_n(int n, double t, double* Pn, double* dPn) {
-  double p0 = 1.0, p1 = t;
+void legendre_n(int n, ld t, ld* Pn, ld* dPn) {
+  ld p0 = 1.0, p1 = t;
   if (n == 0) {
     *Pn = 1.0;
     *dPn = 0.0;
     return;
   }
   for (int j = 1; j < n; ++j) {
-    double p2 = ((2.0 * j + 1.0) * t * p1 - j * p0) / (j + 1.0);
+    ld p2 = ((2 * j + 1.0) * t * p1 - j * p0) / (j + 1.0);
     p0 = p1;
     p1 = p2;
   }
@@ -48,18 +52,18 @@ void legendre_n(int n, double t, double* Pn, double* dPn) {
   *dPn = n * (t * p1 - p0) / (t * t - 1.0);  // (1 - t^2) P_n' = n (P_{n-1} - t P_n)
 }
 
-void gauss_01(int n, double* xi, double* w) {
-  const double pi = 3.14159265358979323846;
+void gauss_01(int n, ld* xi, ld* w) {
+  const ld pi = 3.14159265358979323846L;
   for (int i = 0; i < n; ++i) {
-    double t = std::cos(pi * (i + 0.75) / (n + 0.5));
+    ld t = std::cos(pi * (i + 0.75) / (n + 0.5));
     for (int it = 0; it < 100; ++it) {
-      double Pn, dPn;
+      ld Pn, dPn;
       legendre_n(n, t, &Pn, &dPn);
-      double dt = Pn / dPn;
+      ld dt = Pn / dPn;
       t -= dt;
-      if (std::fabs(dt) < 1e-17) break;
+      if (std::fabs(dt) < 1e-19L) break;
     }
-    double Pn, dPn;
+    ld Pn, dPn;
     legendre_n(n, t, &Pn, &dPn);
     // roots come out in decreasing t; store increasing on [0,1]
     xi[n - 1 - i] = 0.5 * (t + 1.0);
@@ -67,23 +71,23 @@ void gauss_01(int n, double* xi, double* w) {
   }
   // exact symmetry of the rule about 1/2
   for (int i = 0; i < n / 2; ++i) {
-    double s = 0.5 * ((1.0 - xi[n - 1 - i]) + xi[i]);
+    ld s = 0.5 * ((1.0 - xi[n - 1 - i]) + xi[i]);
     xi[i] = s;
     xi[n - 1 - i] = 1.0 - s;
-    double ww = 0.5 * (w[i] + w[n - 1 - i]);
+    ld ww = 0.5 * (w[i] + w[n - 1 - i]);
     w[i] = w[n - 1 - i] = ww;
   }
   if (n % 2 == 1) xi[n / 2] = 0.5;
 }
 
 // orthonormal L_i(s) = sqrt(2i+1) P_i(2s-1) and L_i'(s) = 2 sqrt(2i+1) P_i'(2s-1)
-void onb_all(int n, double s, double* L, double* dL) {
-  double P[DG_MAXN], dP[DG_MAXN];
-  legendre_all(n, 2.0 * s - 1.0, P, dP);
+void onb_all(int n, ld s, ld* L, ld* dL) {
+  ld P[DG_MAXN], dP[DG_MAXN];
+  legendre_all(n, 2 * s - 1.0, P, dP);
   for (int i = 0; i < n; ++i) {
-    double a = std::sqrt(2.0 * i + 1.0);
+    ld a = std::sqrt((ld)(2 * i + 1));
     L[i] = a * P[i];
-    dL[i] = 2.0 * a * dP[i];
+    dL[i] = 2 * a * dP[i];
   }
 }
 
@@ -112,62 +116,62 @@ void copy_round(const DGTab<S>& s, DGTab<D>* d) {
 
 void dg_build_tables(int n, double sigma, DGTab<double>* t, DGTab<float>* t32) {
   std::memset(t, 0, sizeof(*t));
-  double xi[DG_MAXN], w[DG_MAXN];
+  ld xi[DG_MAXN], w[DG_MAXN];
   gauss_01(n, xi, w);
   for (int a = 0; a < n; ++a) {
-    double L[DG_MAXN], dL[DG_MAXN];
+    ld L[DG_MAXN], dL[DG_MAXN];
     onb_all(n, xi[a], L, dL);
     for (int i = 0; i < n; ++i) {
-      t->B[a][i] = L[i];
-      t->Bd[a][i] = dL[i];
+      t->B[a][i] = (double)L[i];
+      t->Bd[a][i] = (double)dL[i];
     }
-    t->w[a] = w[a];
+    t->w[a] = (double)w[a];
   }
   {
-    double L0[DG_MAXN], dL0[DG_MAXN], L1[DG_MAXN], dL1[DG_MAXN];
+    ld L0[DG_MAXN], dL0[DG_MAXN], L1[DG_MAXN], dL1[DG_MAXN];
     onb_all(n, 0.0, L0, dL0);
     onb_all(n, 1.0, L1, dL1);
     for (int i = 0; i < n; ++i) {
-      t->a0[i] = L0[i];
-      t->a1[i] = L1[i];
-      t->d0[i] = dL0[i];
-      t->d1[i] = dL1[i];
+      t->a0[i] = (double)L0[i];
+      t->a1[i] = (double)L1[i];
+      t->d0[i] = (double)dL0[i];
+      t->d1[i] = (double)dL1[i];
     }
   }
   // barycentric weights of the Gauss points
-  double lam[DG_MAXN];
+  ld lam[DG_MAXN];
   for (int a = 0; a < n; ++a) {
-    double p = 1.0;
+    ld p = 1.0;
     for (int b = 0; b < n; ++b)
       if (b != a) p *= (xi[a] - xi[b]);
     lam[a] = 1.0 / p;
   }
   for (int a = 0; a < n; ++a) {
-    double s = 0.0;
+    ld s = 0.0;
     for (int b = 0; b < n; ++b) {
       if (b == a) continue;
-      double v = (lam[b] / lam[a]) / (xi[a] - xi[b]);
-      t->D[a][b] = v;
+      ld v = (lam[b] / lam[a]) / (xi[a] - xi[b]);
+      t->D[a][b] = (double)v;
       s += v;
     }
-    t->D[a][a] = -s;
+    t->D[a][a] = (double)-s;
   }
   // Lagrange values and derivatives at the ends s = 0, 1 (not nodes)
   for (int e = 0; e < 2; ++e) {
-    double s = (double)e;
+    ld s = (ld)e;
     for (int a = 0; a < n; ++a) {
-      double l = 1.0, dsum = 0.0;
+      ld l = 1.0, dsum = 0.0;
       for (int b = 0; b < n; ++b) {
         if (b == a) continue;
         l *= (s - xi[b]) / (xi[a] - xi[b]);
         dsum += 1.0 / (s - xi[b]);
       }
       if (e == 0) {
-        t->l0[a] = l;
-        t->dl0[a] = l * dsum;
+        t->l0[a] = (double)l;
+        t->dl0[a] = (double)(l * dsum);
       } else {
-        t->l1[a] = l;
-        t->dl1[a] = l * dsum;
+        t->l1[a] = (double)l;
+        t->dl1[a] = (double)(l * dsum);
       }
     }
   }
@@ -176,4 +180,11 @@ void dg_build_tables(int n, double sigma, DGTab<double>* t, DGTab<float>* t32) {
 }
 
 // Gauss-Legendre points and weights on [0,1] (the rule the tables use).
-void dg_gauss_points(int n, double* xi, double* w) { gauss_01(n, xi, w); }
+void dg_gauss_points(int n, double* xi, double* w) {
+  ld x[DG_MAXN], v[DG_MAXN];
+  gauss_01(n, x, v);
+  for (int a = 0; a < n; ++a) {
+    xi[a] = (double)x[a];
+    w[a] = (double)v[a];
+  }
+}
