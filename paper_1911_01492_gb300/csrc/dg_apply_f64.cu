@@ -1,18 +1,14 @@
-// FP64 instantiation of the two-pass operator application.
+// FP64 operator application by geometry and basis; the FP64 passes that remain
+// (traces for the curved geometries and the coefficient gradient).
 #include "dg_apply_impl.cuh"
 
 int dg_launch_apply_f64(const dg_mesh* m, const double* x, double* y, const int* skip,
                         cudaStream_t s) {
   // inside a solve in the scaled Gauss-point basis (DG_CG_NODAL): Q A Q^T
-  if (m != nullptr && m->nodal_op) return dg_launch_apply_nodal_f64(m, x, y, skip, s);
-  if (m != nullptr && m->multilinear) return dg_launch_apply_multilinear(m, x, y, skip, s);
-  if (m != nullptr && m->affine) return dg_launch_apply_affine(m, x, y, skip, s);
-  cudaError_t e = dgk::dispatch_n<double, dgk::ApplyF>(m->n, m, x, y, m->U64, m->X64, m->TR64,
-                                                       (const double*)m->kt64,
-                                                       (const double*)m->fw64, m->ncells, m->N,
-                                                       skip, &m->tab64, s);
-  if (e != cudaSuccess) return dg_cuda_fail(e, "apply (fp64) launch");
-  return DG_OK;
+  if (m->nodal_op) return dg_launch_fixed_apply(m, false, x, y, skip, s);
+  if (m->multilinear) return dg_launch_apply_multilinear(m, x, y, skip, s);
+  if (m->affine) return dg_launch_apply_affine(m, x, y, skip, s);
+  return dg_launch_fixed_apply(m, true, x, y, skip, s);
 }
 
 int dg_launch_trace_f64(const dg_mesh* m, const double* x, double* U, double* X, double* TR,
@@ -22,13 +18,17 @@ int dg_launch_trace_f64(const dg_mesh* m, const double* x, double* U, double* X,
   return DG_OK;
 }
 
-int dg_launch_pass_f64(const dg_mesh* m, int pass, const double* x, double* y, long long cbeg,
-                       long long cend, cudaStream_t s) {
-  cudaError_t e = dgk::dispatch_n<double, dgk::PassF>(m->n, m, pass, x, y, m->U64, m->X64,
-                                                      m->TR64, (const double*)m->kt64,
-                                                      (const double*)m->fw64, cbeg, cend, m->N,
-                                                      &m->tab64, s);
-  if (e != cudaSuccess) return dg_cuda_fail(e, "apply pass (fp64) launch");
+// Line operators of the batched solver in FP64, on the first batched solve
+// after the coefficient is set.
+int dg_ensure_lines64(dg_mesh* m, bool nodal, cudaStream_t s) {
+  bool& has = nodal ? m->has_nodal_lines : m->has_lines;
+  double*& lo = nodal ? m->lineopN64 : m->lineop64;
+  if (has) return DG_OK;
+  const size_t nlo = (size_t)3 * m->n * m->n * (size_t)(m->n * (m->n + 1) / 2) * (size_t)m->ncells;
+  if (lo == nullptr) DG_CUDA(cudaMalloc((void**)&lo, nlo * sizeof(double)));
+  cudaError_t e = dgk::dispatch_n<double, dgk::LineOpsF>(m->n, (const dg_mesh*)m, nodal, lo, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "line operators launch");
+  has = true;
   return DG_OK;
 }
 

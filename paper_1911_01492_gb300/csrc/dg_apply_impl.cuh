@@ -816,22 +816,6 @@ k_cell(const T* __restrict__ U, const T* __restrict__ Xm, const T* __restrict__ 
   cell_cells<N, T>(U, Xm, TR, kt, FW, y, c0, nblk, Nc, tab, reinterpret_cast<T*>(smem_raw));
 }
 
-// Pass 2 with the precomputed line operators (FP64 path of dg_apply).
-template <int N, typename T>
-__global__ void __launch_bounds__(Cfg<N>::THREADS)
-k_cell_lo(const T* __restrict__ U, const T* __restrict__ Xm, const T* __restrict__ TR,
-          const T* __restrict__ lineop, const T* __restrict__ FW, T* __restrict__ y,
-          long long cbeg, long long cend, int Nc, const int* __restrict__ skip,
-          const __grid_constant__ DGTab<T> tab) {
-  constexpr int C = Cfg<N>::CPB;
-  if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const long long c0 = cbeg + (long long)blockIdx.x * C;
-  const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
-  cell_cells<N, T, true>(U, Xm, TR, nullptr, FW, y, c0, nblk, Nc, tab,
-                         reinterpret_cast<T*>(smem_raw), lineop);
-}
-
 // Line operators from Kt = h w K and h gamma (one thread per cell, direction
 // and line):
 //   x-line (b, e):  M[i][j] = sum_a L_i'(xi_a) Kt(a, b, e) L_j'(xi_a)   (acts on x-modes)
@@ -956,12 +940,7 @@ cudaError_t launch_apply_n(const dg_mesh* m, const T* x, T* y, T* U, T* X, T* TR
   dg_timing_mark(m, 0, s);
   k_trace<N, T><<<blocks, Cfg<N>::THREADS, s1, s>>>(x, U, X, TR, 0, ncells, skip, tab);
   dg_timing_mark(m, 1, s);
-  if (sizeof(T) == 8 && m != nullptr && m->lineop64 != nullptr)
-    k_cell_lo<N, T><<<blocks, Cfg<N>::THREADS, s2, s>>>(U, X, TR, (const T*)m->lineop64, fw, y,
-                                                        0, ncells, Nc, skip, tab);
-  else
-    k_cell<N, T><<<blocks, Cfg<N>::THREADS, s2, s>>>(U, X, TR, kt, fw, y, 0, ncells, Nc, skip,
-                                                     tab);
+  k_cell<N, T><<<blocks, Cfg<N>::THREADS, s2, s>>>(U, X, TR, kt, fw, y, 0, ncells, Nc, skip, tab);
   dg_timing_mark(m, 2, s);
   return cudaGetLastError();
 }
@@ -979,9 +958,6 @@ cudaError_t launch_pass_n(const dg_mesh* m, int pass, const T* x, T* y, T* U, T*
   if (pass == 1)
     k_trace<N, T><<<blocks, Cfg<N>::THREADS, trace_smem<N, T>(), s>>>(x, U, X, TR, cbeg, cend,
                                                                        nullptr, tab);
-  else if (sizeof(T) == 8 && m->lineop64 != nullptr)
-    k_cell_lo<N, T><<<blocks, Cfg<N>::THREADS, cell_smem<N, T>(), s>>>(
-        U, X, TR, (const T*)m->lineop64, fw, y, cbeg, cend, Nc, nullptr, tab);
   else
     k_cell<N, T><<<blocks, Cfg<N>::THREADS, cell_smem<N, T>(), s>>>(U, X, TR, kt, fw, y, cbeg,
                                                                      cend, Nc, nullptr, tab);
@@ -1040,9 +1016,6 @@ struct PrepareF {
     cudaError_t e = cudaFuncSetAttribute(k_cell<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)cell_smem<N, T>());
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_cell_lo<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)cell_smem<N, T>());
-    if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_trace<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)trace_smem<N, T>());
     return e;
@@ -1064,11 +1037,14 @@ namespace dgk {
 template <int N>
 struct LineOpsF {
   template <typename T>
-  static cudaError_t run(const double* kt, const double* gh, double* lineop, long long ncells,
-                         int Nc, const DGTab<double>* tab, cudaStream_t s) {
-    const long long threads = ncells * 3 * N * N;
-    k_line_ops<N><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(kt, gh, lineop, ncells, Nc,
-                                                                    *tab, DGTabN<double>{});
+  static cudaError_t run(const dg_mesh* m, bool nodal, double* lineop, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((m->ncells * 3 * N * N + 255) / 256);
+    if (nodal)
+      k_line_ops<N, true><<<blocks, 256, 0, s>>>(m->kt64, m->gh64, lineop, m->ncells, m->N,
+                                                 m->tab64, m->tabN64);
+    else
+      k_line_ops<N, false><<<blocks, 256, 0, s>>>(m->kt64, m->gh64, lineop, m->ncells, m->N,
+                                                  m->tab64, m->tabN64);
     return cudaGetLastError();
   }
 };

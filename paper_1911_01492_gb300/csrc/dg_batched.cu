@@ -998,8 +998,6 @@ extern "C" int dg_cg_solve_batched_mode(const dg_mesh* const* meshes, int count,
       return dg_fail(DG_ERR_INVALID_ARG,
                      "dg_cg_solve_batched: sample %d has an affine or multilinear geometry (not "
                      "batched)", s);
-    if (m->lineop64 == nullptr)
-      return dg_fail(DG_ERR_INVALID_ARG, "dg_cg_solve_batched: sample %d has no line operators", s);
     for (int t = 0; t < s; ++t)
       if (meshes[t] == meshes[s])
         return dg_fail(DG_ERR_INVALID_ARG,
@@ -1007,6 +1005,9 @@ extern "C" int dg_cg_solve_batched_mode(const dg_mesh* const* meshes, int count,
                        s);
     maxn = m->n > maxn ? m->n : maxn;
   }
+  for (int s = 0; s < count; ++s)
+    if (int rc = dg_ensure_lines64(const_cast<dg_mesh*>(meshes[s]), nodal, (cudaStream_t)stream))
+      return rc;
   if (nodal) return solve_batched_nodal(meshes, count, b, x, rtol, maxit, maxn, mode, st, stream);
   if (maxn <= 5)
     return solve_batched<128, 5, false>(meshes, count, b, x, rtol, maxit, jacobi, mode, st,

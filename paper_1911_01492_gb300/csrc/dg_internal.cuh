@@ -45,6 +45,31 @@ void dg_build_tables(int n, double sigma, DGTab<double>* t64, DGTab<float>* t32)
 // the n Gauss-Legendre points and weights on [0,1] of those tables
 void dg_gauss_points(int n, double* xi, double* w);
 
+// Fixed-point tables of the FP64 operator (dg_fixed.cuh, dg_fixed_tables.cpp):
+// a constant in (-2, 2) times 2^60, as h 2^30 + l.
+struct FxPair {
+  int h, l;
+};
+#define DG_MAXH ((DG_MAXN + 1) / 2)  // mirror pairs of a line
+#define DG_MAXP (DG_MAXN * (DG_MAXN + 1) / 2)
+// Even and odd halves over the mirror pairs (a, n-1-a) of the end-value vectors.
+struct DGTabX {
+  FxPair q[DG_MAXN][DG_MAXN];           // sqrt(w_a) L_i(xi_a)
+  FxPair ve[DG_MAXH], vo[DG_MAXH];      // face value l               2^-cv
+  FxPair ae[DG_MAXH], ao[DG_MAXH];      // sigma l + d (d: half derivative) 2^-ca
+  FxPair le[DG_MAXH], lo[DG_MAXH];      // test value l               2^-cl
+  FxPair de[DG_MAXH], dn[DG_MAXH];      // test derivative -d         2^(cv-ca-cl)
+  int cg;    // ca + cl: exponent a face coefficient takes up
+  int bump;  // face contributions sit 2^bump below the common exponent
+};
+struct DGTabXSetup {
+  FxPair DD[DG_MAXN][DG_MAXP];  // h Dh[f][i] Dh[f][j]  2^-cB
+  FxPair F[2][DG_MAXP];         // own-side terms of the lower face: inside, boundary
+  int ch, cB;                   // h <= 2^ch; entries < 2^(cB + exponent of K)
+};
+// false if a constant leaves its range (degrees 1..8 are inside)
+bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s);
+
 // CG scalar state kept on the device (one per solve / per batched sample).
 struct DGCGState {
   double rho;       // <z, r> of the current residual (z = M^-1 r; = <r, r> without M)
@@ -100,6 +125,15 @@ struct dg_mesh {
   DGTab<double> tab64;
   DGTab<float> tab32;
 
+  // fixed-point FP64 operator (dg_fixed.cu): tables; per cell and line the
+  // operators of Q A Q^T [c][3][n(n+1)/2][n^2] and their exponent [c], per face
+  // the neighbour coefficient and its exponent [c][6], the exponent of the
+  // vector of the running application [c]
+  DGTabX tabX;
+  DGTabXSetup tabXS;
+  FxPair *lineopX, *gamX;
+  int *expM, *expG, *expU;
+
   // coefficient data (dg_set_coefficient)
   bool has_coef;
   double* kt64;     // h w_q K_{c,q}                  [c][q]
@@ -108,7 +142,7 @@ struct dg_mesh {
   float* gh32;
   double* dgam;     // d gamma_F / d log Kbar_c       [c][6]
   double* fw64;     // face-point weights W/2 and derivative weight  [c][6][2][n^2]
-  double* lineop64; // per-line volume operators (FP64)  [c][3][n^2][n(n+1)/2]
+  double* lineop64; // FP64 line operators of the batched solver [c][3][n^2][n(n+1)/2]
   float* fw32;
   // Jacobi preconditioner: 1 / diag(A), formed on the first preconditioned solve
   double* diag64;
@@ -128,7 +162,7 @@ struct dg_mesh {
   // the coefficient is set) and the solve's b and x in that basis
   DGTabN<double> tabN64;
   DGTabN<float> tabN32;
-  bool has_nodal, has_nodal_diag;
+  bool has_lines, has_nodal_lines, has_nodal_diag;
   bool nodal_op;      // set while a solve runs in that basis: the internal
                       // FP64 apply launcher then applies Q A Q^T
   double* lineopN64;  // [c][3][n^2][n(n+1)/2]
@@ -206,9 +240,16 @@ int dg_cuda_fail(cudaError_t e, const char* what);
   } while (0)
 
 // launchers (dg_apply_f64.cu / dg_apply_f32.cu)
-// one pass (1: traces, 2: cell terms) over the cells [cbeg, cend)
-int dg_launch_pass_f64(const dg_mesh* m, int pass, const double* x, double* y, long long cbeg,
-                       long long cend, cudaStream_t s);
+// the FP64 operator in fixed point (dg_fixed.cu), for vectors of Legendre
+// coefficients (modal) or scaled point values: its coefficient data, one pass
+// (1: traces, 2: cell terms) over the cells [cbeg, cend), both passes
+int dg_prepare_fixed(int n);
+int dg_setup_fixed(dg_mesh* m, const double* K, cudaStream_t s);
+int dg_launch_fixed_pass(const dg_mesh* m, bool modal, int pass, const double* x, double* y,
+                         long long cbeg, long long cend, const int* skip, cudaStream_t s);
+int dg_launch_fixed_apply(const dg_mesh* m, bool modal, const double* x, double* y,
+                          const int* skip, cudaStream_t s);
+// one pass of the FP32 operator over the cells [cbeg, cend)
 int dg_launch_pass_f32(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
                        long long cend, cudaStream_t s);
 int dg_launch_apply_f64(const dg_mesh* m, const double* x, double* y, const int* skip,
@@ -246,8 +287,8 @@ void dg_build_nodal_tables(const DGTab<double>& t, int n, DGTabN<double>* d, DGT
 int dg_ensure_nodal(dg_mesh* m, cudaStream_t s);
 int dg_ensure_nodal_diag(dg_mesh* m, cudaStream_t s);
 int dg_ensure_nodal32(dg_mesh* m, cudaStream_t s);  // h K in FP32 for the mixed CG
-int dg_launch_apply_nodal_f64(const dg_mesh* m, const double* x, double* y, const int* skip,
-                              cudaStream_t s);
+// FP64 line operators of the batched solver (nodal: of Q A Q^T), if needed
+int dg_ensure_lines64(dg_mesh* m, bool nodal, cudaStream_t s);
 int dg_launch_collocation(const dg_mesh* m, const double* in, double* out, bool to_nodal,
                           cudaStream_t s);
 

@@ -102,7 +102,7 @@ static cudaError_t dmalloc(P** p, size_t count) {
 }
 
 static void free_all(dg_mesh* m) {
-  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->fw64, m->fw32, m->lineop64, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->lineopN64, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen,
+  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->fw64, m->fw32, m->lineop64, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->lineopN64, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen,
                   m->U64,  m->X64,  m->TR64, m->U32,  m->X32,  m->TR32, m->U64b,
                   m->X64b, m->TR64b, m->hx_dev, m->hy_dev, m->r64, m->p64, m->q64,
                   m->t64,  m->s64, m->d32,  m->r32, m->p32, m->q32, m->partials, m->state,
@@ -150,6 +150,10 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   }
   dg_build_tables(m->n, m->sigma, &m->tab64, &m->tab32);
   dg_build_nodal_tables(m->tab64, m->n, &m->tabN64, &m->tabN32);
+  if (!dg_build_fixed_tables(m->n, m->h, &m->tabX, &m->tabXS)) {
+    free(m);
+    return dg_fail(DG_ERR_INVALID_ARG, "dg_create_mesh: fixed-point tables out of range");
+  }
   cudaError_t e = cudaGetDevice(&m->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, m->device);
   const size_t nd = (size_t)m->ndofs, nc = (size_t)m->ncells, ntr = (size_t)(12 * n2) * nc;
@@ -161,7 +165,11 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->fw64, ntr);
   if (e == cudaSuccess) e = dmalloc(&m->fw32, ntr);
   if (e == cudaSuccess)
-    e = dmalloc(&m->lineop64, (size_t)3 * n2 * (size_t)(m->n * (m->n + 1) / 2) * nc);
+    e = dmalloc(&m->lineopX, (size_t)3 * n2 * (size_t)(m->n * (m->n + 1) / 2) * nc);
+  if (e == cudaSuccess) e = dmalloc(&m->gamX, 6 * nc);
+  if (e == cudaSuccess) e = dmalloc(&m->expM, nc);
+  if (e == cudaSuccess) e = dmalloc(&m->expG, 6 * nc);
+  if (e == cudaSuccess) e = dmalloc(&m->expU, nc);
   if (e == cudaSuccess) e = dmalloc(&m->kbar, nc);
   if (e == cudaSuccess) e = dmalloc(&m->dflag, 1);
   if (e == cudaSuccess) e = dmalloc(&m->U64, nd);
@@ -176,7 +184,8 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
     free(m);
     return rc;
   }
-  int rc = dg_prepare_apply_f64(m->n);
+  int rc = dg_prepare_fixed(m->n);
+  if (rc == DG_OK) rc = dg_prepare_apply_f64(m->n);
   if (rc == DG_OK) rc = dg_prepare_apply_f32(m->n);
   if (rc == DG_OK) rc = dg_prepare_affine(m->n);
   if (rc == DG_OK) rc = dg_prepare_grad(m->n);
@@ -222,7 +231,8 @@ extern "C" int dg_set_boundary(dg_mesh* m, int dirichlet_mask) {
   m->has_diag = false;
   m->has_block = false;
   m->has_kron = false;
-  m->has_nodal = false;
+  m->has_lines = false;
+  m->has_nodal_lines = false;
   m->has_nodal_diag = false;
   m->has_nodal32 = false;
   m->has_kron_nodal = false;
@@ -281,7 +291,8 @@ extern "C" int dg_set_coefficient(dg_mesh* m, const double* K, void* stream) {
   m->has_diag = false;
   m->has_block = false;
   m->has_kron = false;
-  m->has_nodal = false;
+  m->has_lines = false;
+  m->has_nodal_lines = false;
   m->has_nodal_diag = false;
   m->has_nodal32 = false;
   m->has_kron_nodal = false;
@@ -300,11 +311,8 @@ extern "C" int dg_set_coefficient(dg_mesh* m, const double* K, void* stream) {
     dgk::k_face_weights<double><<<blocks, 256, 0, s>>>(m->gh64, m->fw64, m->N, m->n, m->tab64);
     dgk::k_face_weights<float><<<blocks, 256, 0, s>>>(m->gh64, m->fw32, m->N, m->n, m->tab64);
     DG_CUDA(cudaGetLastError());
-    cudaError_t e = dgk::dispatch_n<double, dgk::LineOpsF>(m->n, (const double*)m->kt64,
-                                                           (const double*)m->gh64, m->lineop64,
-                                                           m->ncells, m->N,
-                                                           (const DGTab<double>*)&m->tab64, s);
-    if (e != cudaSuccess) return dg_cuda_fail(e, "dg_set_coefficient: line operators");
+    if (!m->affine && !m->multilinear)
+      if (int rc = dg_setup_fixed(m, K, s)) return rc;
   }
   int flag = 0;
   DG_CUDA(cudaMemcpyAsync(&flag, m->dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -407,8 +415,8 @@ extern "C" int dg_apply_host(const dg_mesh* mc, const void* x_host, void* y_host
   };
   auto pass = [&](int p, int sl, cudaStream_t st) {
     return prec == DG_FP64
-               ? dg_launch_pass_f64(m, p, (const double*)xd, (double*)yd, cells(sl),
-                                    cells(sl + 1), st)
+               ? dg_launch_fixed_pass(m, true, p, (const double*)xd, (double*)yd, cells(sl),
+                                      cells(sl + 1), nullptr, st)
                : dg_launch_pass_f32(m, p, (const float*)xd, (float*)yd, cells(sl),
                                     cells(sl + 1), st);
   };

@@ -111,34 +111,6 @@ k_collocation(const double* __restrict__ in, double* __restrict__ out, long long
   }
 }
 
-// The two passes (dg_nodal_impl.cuh) as stand-alone kernels over blocks of CPB
-// cells.
-template <int N, typename T>
-__global__ void __launch_bounds__(Cfg<N>::THREADS)
-k_trace_nd(const T* __restrict__ x, T* __restrict__ TR, long long ncells, const int* skip,
-           const __grid_constant__ DGTabN<T> tn) {
-  constexpr int C = Cfg<N>::CPB;
-  if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const long long c0 = (long long)blockIdx.x * C;
-  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
-  trace_cells_nd<N, T>(x, TR, c0, nblk, tn, reinterpret_cast<T*>(smem_raw));
-}
-
-template <int N>
-__global__ void __launch_bounds__(Cfg<N>::THREADS)
-k_cell_nd(const double* __restrict__ x, const double* __restrict__ TR,
-          const double* __restrict__ lineop, const double* __restrict__ gh,
-          double* __restrict__ y, long long ncells, int Nc, const int* skip,
-          const __grid_constant__ DGTabN<double> tn) {
-  constexpr int C = Cfg<N>::CPB;
-  if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const long long c0 = (long long)blockIdx.x * C;
-  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
-  cell_cells_nd<N>(x, TR, lineop, gh, y, c0, nblk, Nc, tn, reinterpret_cast<double*>(smem_raw));
-}
-
 // 1 / diag(Q A Q^T): at point (a, b, e) the sum of the diagonal entries of the
 // x-, y- and z-line operators through it (the neighbour terms couple other
 // cells only).  One thread per DOF.
@@ -174,26 +146,11 @@ __global__ void k_hk32(const double* __restrict__ kt, float* __restrict__ hk, lo
 template <int N>
 struct NodalF {
   template <typename T>
-  static cudaError_t apply(const dg_mesh* m, const double* x, double* y, const int* skip,
-                           cudaStream_t s) {
-    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
-    const size_t s1 = sizeof(double) * Cfg<N>::CPB * N * N * N;
-    dg_timing_mark(m, 0, s);
-    k_trace_nd<N, double><<<blocks, Cfg<N>::THREADS, s1, s>>>(x, m->TR64, m->ncells, skip,
-                                                             m->tabN64);
-    dg_timing_mark(m, 1, s);
-    k_cell_nd<N><<<blocks, Cfg<N>::THREADS, 2 * s1, s>>>(x, m->TR64, m->lineopN64, m->gh64, y,
-                                                        m->ncells, m->N, skip, m->tabN64);
-    dg_timing_mark(m, 2, s);
-    return cudaGetLastError();
-  }
-  template <typename T>
   static cudaError_t run(int what, const dg_mesh* m, const double* x, double* y,
-                         const int* skip, cudaStream_t s) {
+                         cudaStream_t s) {
     const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
     const size_t s1 = sizeof(double) * Cfg<N>::CPB * N * N * N;
     switch (what) {
-      case 0: return apply<T>(m, x, y, skip, s);
       case 1:
         k_collocation<N, true><<<blocks, Cfg<N>::THREADS, s1, s>>>(x, y, m->ncells, m->tab64,
                                                                    m->tabN64);
@@ -202,13 +159,7 @@ struct NodalF {
         k_collocation<N, false><<<blocks, Cfg<N>::THREADS, s1, s>>>(x, y, m->ncells, m->tab64,
                                                                     m->tabN64);
         return cudaGetLastError();
-      case 3: {
-        const long long threads = m->ncells * 3 * N * N;
-        k_line_ops<N, true><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-            m->kt64, m->gh64, m->lineopN64, m->ncells, m->N, m->tab64, m->tabN64);
-        return cudaGetLastError();
-      }
-      case 4:
+      case 3:
         k_diag_nd<N><<<(unsigned)((m->ndofs + 255) / 256), 256, 0, s>>>(
             m->lineopN64, m->dinvN64, m->dinvN32, m->ndofs);
         return cudaGetLastError();
@@ -249,18 +200,18 @@ void dg_build_nodal_tables(const DGTab<double>& t, int n, DGTabN<double>* d, DGT
 }
 
 namespace {
-int run_nodal(int what, const dg_mesh* m, const double* x, double* y, const int* skip,
-              cudaStream_t s, const char* who) {
+int run_nodal(int what, const dg_mesh* m, const double* x, double* y, cudaStream_t s,
+              const char* who) {
   cudaError_t e = cudaErrorInvalidValue;
   switch (m->n) {
-    case 2: e = dgk::NodalF<2>::run<double>(what, m, x, y, skip, s); break;
-    case 3: e = dgk::NodalF<3>::run<double>(what, m, x, y, skip, s); break;
-    case 4: e = dgk::NodalF<4>::run<double>(what, m, x, y, skip, s); break;
-    case 5: e = dgk::NodalF<5>::run<double>(what, m, x, y, skip, s); break;
-    case 6: e = dgk::NodalF<6>::run<double>(what, m, x, y, skip, s); break;
-    case 7: e = dgk::NodalF<7>::run<double>(what, m, x, y, skip, s); break;
-    case 8: e = dgk::NodalF<8>::run<double>(what, m, x, y, skip, s); break;
-    case 9: e = dgk::NodalF<9>::run<double>(what, m, x, y, skip, s); break;
+    case 2: e = dgk::NodalF<2>::run<double>(what, m, x, y, s); break;
+    case 3: e = dgk::NodalF<3>::run<double>(what, m, x, y, s); break;
+    case 4: e = dgk::NodalF<4>::run<double>(what, m, x, y, s); break;
+    case 5: e = dgk::NodalF<5>::run<double>(what, m, x, y, s); break;
+    case 6: e = dgk::NodalF<6>::run<double>(what, m, x, y, s); break;
+    case 7: e = dgk::NodalF<7>::run<double>(what, m, x, y, s); break;
+    case 8: e = dgk::NodalF<8>::run<double>(what, m, x, y, s); break;
+    case 9: e = dgk::NodalF<9>::run<double>(what, m, x, y, s); break;
     default: break;
   }
   if (e != cudaSuccess) return dg_cuda_fail(e, who);
@@ -269,26 +220,22 @@ int run_nodal(int what, const dg_mesh* m, const double* x, double* y, const int*
 }  // namespace
 
 int dg_ensure_nodal(dg_mesh* m, cudaStream_t s) {
-  if (m->has_nodal) return DG_OK;
+  (void)s;
   if (int rc = dg_require_cube(m, "the scaled Gauss-point basis")) return rc;
   const size_t nd = (size_t)m->ndofs;
-  const size_t nlo = (size_t)3 * m->n * m->n * (size_t)(m->n * (m->n + 1) / 2) * (size_t)m->ncells;
-  if (m->lineopN64 == nullptr) DG_CUDA(cudaMalloc((void**)&m->lineopN64, nlo * sizeof(double)));
   if (m->bN64 == nullptr) DG_CUDA(cudaMalloc((void**)&m->bN64, nd * sizeof(double)));
   if (m->xN64 == nullptr) DG_CUDA(cudaMalloc((void**)&m->xN64, nd * sizeof(double)));
-  int rc = run_nodal(3, m, nullptr, nullptr, nullptr, s, "nodal line operators");
-  if (rc) return rc;
-  m->has_nodal = true;
   return DG_OK;
 }
 
 int dg_ensure_nodal_diag(dg_mesh* m, cudaStream_t s) {
   int rc = dg_ensure_nodal(m, s);
   if (rc || m->has_nodal_diag) return rc;
+  if ((rc = dg_ensure_lines64(m, true, s))) return rc;
   const size_t nd = (size_t)m->ndofs;
   if (m->dinvN64 == nullptr) DG_CUDA(cudaMalloc((void**)&m->dinvN64, nd * sizeof(double)));
   if (m->dinvN32 == nullptr) DG_CUDA(cudaMalloc((void**)&m->dinvN32, nd * sizeof(float)));
-  rc = run_nodal(4, m, nullptr, nullptr, nullptr, s, "nodal Jacobi diagonal");
+  rc = run_nodal(3, m, nullptr, nullptr, s, "nodal Jacobi diagonal");
   if (rc) return rc;
   m->has_nodal_diag = true;
   return DG_OK;
@@ -305,14 +252,9 @@ int dg_ensure_nodal32(dg_mesh* m, cudaStream_t s) {
   return DG_OK;
 }
 
-int dg_launch_apply_nodal_f64(const dg_mesh* m, const double* x, double* y, const int* skip,
-                              cudaStream_t s) {
-  return run_nodal(0, m, x, y, skip, s, "apply in the point basis (fp64) launch");
-}
-
 int dg_launch_collocation(const dg_mesh* m, const double* in, double* out, bool to_nodal,
                           cudaStream_t s) {
-  return run_nodal(to_nodal ? 1 : 2, m, in, out, nullptr, s, "basis transform launch");
+  return run_nodal(to_nodal ? 1 : 2, m, in, out, s, "basis transform launch");
 }
 
 static int check_nodal_args(const dg_mesh* m, const void* a, const void* b, const char* who) {
@@ -335,8 +277,5 @@ extern "C" int dg_to_modal(const dg_mesh* m, const double* xhat, double* x, void
 extern "C" int dg_apply_nodal(const dg_mesh* mc, const double* xhat, double* yhat, void* stream) {
   if (int rc = check_nodal_args(mc, xhat, yhat, "dg_apply_nodal")) return rc;
   if (!mc->has_coef) return dg_fail(DG_ERR_INVALID_ARG, "dg_apply_nodal: coefficient not set");
-  dg_mesh* m = const_cast<dg_mesh*>(mc);
-  cudaStream_t s = (cudaStream_t)stream;
-  if (int rc = dg_ensure_nodal(m, s)) return rc;
-  return dg_launch_apply_nodal_f64(m, xhat, yhat, nullptr, s);
+  return dg_launch_fixed_apply(mc, false, xhat, yhat, nullptr, (cudaStream_t)stream);
 }
