@@ -45,6 +45,15 @@ struct FxPad {
   static constexpr int SY = N + (N % 2 == 0 ? 1 : 0), SZ = N * SY, SC = N * SZ;
 };
 
+// Shared memory of the two passes in a block of BT threads.
+template <int N, int BT>
+struct FxSmem {
+  static constexpr int C = Cfg<N>::CPB;
+  static constexpr int NS = (BT + N * N - 1) / (N * N);  // n^2 thread groups of the block
+  static constexpr size_t trace = 8 * C * FxPad<N>::SC + 4 * 2 * NS;
+  static constexpr size_t cell = 8 * 2 * C * FxPad<N>::SC + 8 * 6 * C + 4 * (7 * C + NS);
+};
+
 struct FxVal { int h, l; };  // a value v = h 2^30 + l
 
 __device__ __forceinline__ FxVal fx_split(long long v) {
@@ -125,15 +134,15 @@ __device__ __forceinline__ unsigned fx_mag_hi(long long v) {
 __device__ __forceinline__ int fx_bits(unsigned mag_hi) { return 64 - __clz((int)mag_hi); }
 
 // Largest v over the threads of the calling thread's cell.  Cells that lie
-// inside one warp need no barrier; otherwise slots[CPB] (zeroed before an
+// inside one warp need no barrier; otherwise slots (zeroed before an
 // earlier barrier) collects the warps' maxima.  Every thread of the block calls it.
-template <int N>
+template <int N, int BT>
 __device__ __forceinline__ unsigned fx_cell_max(unsigned v, int lc, unsigned* slots) {
-  constexpr int N2 = N * N, T = Cfg<N>::THREADS;
+  constexpr int N2 = N * N;
   const int lane = threadIdx.x & 31, base = (int)threadIdx.x - lane;
   const int lo = lc * N2 > base ? lc * N2 - base : 0;
   int hi = (lc + 1) * N2 - base;
-  const int lanes = T - base < 32 ? T - base : 32;
+  const int lanes = BT - base < 32 ? BT - base : 32;
   if (hi > lanes) hi = lanes;
   const unsigned mask = (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
   v = __reduce_max_sync(mask, v);
@@ -192,6 +201,363 @@ __device__ __forceinline__ void fx_bwd(const DGTabX& t, const long long (&r)[N],
       for (int a = 0; a < H; ++a) fx_mac(A, t.q[a][i], o[a]);
     }
     x[i] = fx_value(A);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The two passes (dg_fixed.cu), as functions of a block over a group of cells.
+// ---------------------------------------------------------------------------
+template <int N>
+__device__ __forceinline__ void fx_store_traces(const DGTabX& t, const long long (&u)[N],
+                                                long long* __restrict__ tr, int dir, int pt) {
+  constexpr int N2 = N * N, H = N / 2;
+  FxAcc ve = fx_zero(), vo = fx_zero(), ae = fx_zero(), ao = fx_zero();
+#pragma unroll
+  for (int a = 0; a < H; ++a) {
+    const FxVal e = fx_split(u[a] + u[N - 1 - a]), o = fx_split(u[a] - u[N - 1 - a]);
+    fx_mac(ve, t.ve[a], e);
+    fx_mac(ae, t.ae[a], e);
+    fx_mac(vo, t.vo[a], o);
+    fx_mac(ao, t.ao[a], o);
+  }
+  if (N % 2 == 1) {
+    const FxVal e = fx_split(u[H]);
+    fx_mac(ve, t.ve[H], e);
+    fx_mac(ae, t.ae[H], e);
+  }
+  const long long v = fx_value(ve), w = fx_value(vo), a = fx_value(ae), b = fx_value(ao);
+  tr[(4 * dir + 0) * N2 + pt] = v + w;  // lower face
+  tr[(4 * dir + 1) * N2 + pt] = a + b;
+  tr[(4 * dir + 2) * N2 + pt] = v - w;  // upper face
+  tr[(4 * dir + 3) * N2 + pt] = b - a;
+}
+
+// Pass 1 over the cells c0 .. c0+nblk-1 (nblk <= CPB) by the calling block of
+// BT threads (at least CPB n^2; the others only take part in the barriers).
+// smem: FxSmem<N, BT>::trace bytes.  Every thread of the block calls it; a
+// barrier must follow before smem is used again.
+template <int N, bool MODAL, int BT>
+__device__ __forceinline__ void fx_trace_cells(const double* __restrict__ x,
+                                               long long* __restrict__ U,
+                                               long long* __restrict__ TR,
+                                               int* __restrict__ expU, long long c0, int nblk,
+                                               const DGTabX& tab, long long* smem) {
+  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
+  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC;
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
+  const bool active = lc < nblk;
+  const long long c = c0 + lc;
+  const bool live = BT <= Cfg<N>::THREADS || lc < C;
+  long long* sc = smem + (live ? lc : 0) * SC;
+  unsigned* slots = reinterpret_cast<unsigned*>(smem + C * SC);
+  constexpr int NS = FxSmem<N, BT>::NS;
+  if (32 % N2 != 0) {
+    if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
+    __syncthreads();
+  }
+  double xv[N];
+  unsigned big = 0;
+#pragma unroll
+  for (int l = 0; l < N; ++l) {
+    xv[l] = active ? x[c * N3 + l * N2 + q * N + p] : 0.0;
+    const unsigned m = fx_abs_hi(xv[l]);
+    big = m > big ? m : big;
+  }
+  const int E = fx_exponent(fx_cell_max<N, BT>(big, lc, slots));
+  long long v[N], u[N];
+  int eu;  // u[] 2^eu
+  if (MODAL) {
+    constexpr int S0 = FxScale<N>::S0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], S0 - E, E);
+    // along z: thread owns (i = p, j = q)
+    fx_fwd<N>(tab, v, u);
+#pragma unroll
+    for (int e = 0; e < N; ++e)
+      if (live) sc[e * SZ + q * SY + p] = u[e];
+    __syncthreads();
+    // along y: (i = p, e = q)
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = sc[q * SZ + j * SY + p];
+    fx_fwd<N>(tab, v, u);
+#pragma unroll
+    for (int b = 0; b < N; ++b)
+      if (live) sc[q * SZ + b * SY + p] = u[b];
+    __syncthreads();
+    // along x: (b = p, e = q)
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = sc[q * SZ + p * SY + i];
+    fx_fwd<N>(tab, v, u);
+    // the largest point value to [2^59, 2^60)
+    big = 0;
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      const unsigned m = fx_mag_hi(u[a]);
+      big = m > big ? m : big;
+    }
+    const int up = 60 - fx_bits(fx_cell_max<N, BT>(big, lc, slots + NS));
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      u[a] = fx_shift(u[a], up);
+      if (live) sc[q * SZ + p * SY + a] = u[a];
+    }
+    eu = E - S0 - up;
+    if (active) fx_store_traces<N>(tab, u, TR + c * (12 * N2), 0, pt);
+  } else {
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+      u[l] = fx_from_double(xv[l], 60 - E, E);
+      if (live) sc[l * SZ + q * SY + p] = u[l];
+    }
+    eu = E - 60;
+  }
+  if (E == FX_NAN) eu = FX_NAN;
+  if (active && pt == 0) expU[c] = eu;
+  __syncthreads();
+  if (!active) return;  // no barrier follows
+  long long* tr = TR + c * (12 * N2);
+  if (MODAL) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      u[e] = sc[e * SZ + q * SY + p];
+      U[c * N3 + e * N2 + q * N + p] = u[e];
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < N; ++a) v[a] = sc[q * SZ + p * SY + a];
+    fx_store_traces<N>(tab, v, tr, 0, pt);
+  }
+  fx_store_traces<N>(tab, u, tr, 2, pt);
+#pragma unroll
+  for (int b = 0; b < N; ++b) v[b] = sc[q * SZ + b * SY + p];
+  fx_store_traces<N>(tab, v, tr, 1, pt);
+}
+
+__device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// Pass 2 over the cells c0 .. c0+nblk-1, called like pass 1; smem:
+// FxSmem<N, BT>::cell bytes.  xU: MODAL: the point values of pass 1 (integers);
+// otherwise the vector itself.
+template <int N, bool MODAL, int BT>
+__device__ __forceinline__ void fx_cell_cells(
+    const void* __restrict__ xU, const long long* __restrict__ TR, const int* __restrict__ expU,
+    const FxPair* __restrict__ lineop, const FxPair* __restrict__ gam,
+    const int* __restrict__ expM, const int* __restrict__ expG, double* __restrict__ y,
+    long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
+  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
+  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC;
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
+  const bool active = lc < nblk;
+  const bool live = BT <= Cfg<N>::THREADS || lc < C;
+  const long long c = c0 + (active ? lc : 0);
+  long long* su = smem + (live ? lc : 0) * SC;
+  long long* sr = su + C * SC;
+  FxPair(*sg)[6] = reinterpret_cast<FxPair(*)[6]>(smem + 2 * C * SC);  // face coefficients
+  int(*sexp)[7] = reinterpret_cast<int(*)[7]>(sg + C);  // exponents: six faces, own terms
+  unsigned* slots = reinterpret_cast<unsigned*>(sexp + C);
+  // the block's operators to L2, while exponents and vectors arrive (odd sizes
+  // would leave the 16-byte grid)
+  if (NP * N2 % 2 == 0 && threadIdx.x == 0)
+    fx_prefetch_l2(lineop + c0 * (3 * NP * N2), nblk * (3 * NP * N2) * 8);
+  // cell coordinates: 32-bit divisions (n_cells <= 1024)
+  const unsigned nu = (unsigned)Nc;
+  const long long stride[3] = {1, Nc, (long long)Nc * Nc};
+  // exponents of the seven contributions to a cell
+  for (int i = threadIdx.x; i < nblk * 7; i += BT) {
+    const int l2 = i / 7, f = i - l2 * 7, d = f >> 1;
+    const long long cc = c0 + l2;
+    const unsigned row = (unsigned)cc / nu;
+    const int crd = d == 0 ? (int)((unsigned)cc - row * nu) : d == 1 ? (int)(row % nu) : (int)(row / nu);
+    int e;
+    if (f == 6) {
+      e = expU[cc] + expM[cc];
+    } else {
+      const long long st = f & 1 ? stride[d] : -stride[d];
+      e = (f & 1 ? crd < Nc - 1 : crd > 0) ? expU[cc + st] + expG[cc * 6 + f] : -4 * FX_NAN;
+    }
+    sexp[l2][f] = e;
+    if (f < 6) sg[l2][f] = gam[cc * 6 + f];
+  }
+  if (MODAL && 32 % N2 != 0 && threadIdx.x < FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
+  long long u[N], r[N];
+  // z-lines (a = p, b = q)
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    const long long at = c * N3 + e * N2 + q * N + p;
+    u[e] = MODAL ? static_cast<const long long*>(xU)[at]
+                 : __double_as_longlong(static_cast<const double*>(xU)[at]);
+  }
+  // their operators too, where the registers allow it (measured at 64^3 Q3:
+  // 336 against 340 us; 40^3 Q4: 172 against 178 us; from n = 6 on it is slower)
+  constexpr bool PRE = N == 4 || N == 5;
+  FxPair Mz[PRE ? NP : 1];
+  if constexpr (PRE) {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) Mz[k] = lineop[((c * 3 + 2) * NP + k) * N2 + pt];
+  }
+  __syncthreads();
+  const int eown = sexp[active ? lc : 0][6];
+  int eout = eown;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) eout = max(eout, sexp[active ? lc : 0][f] + tab.bump);
+  const bool bad = eout >= FX_NAN / 2;
+  for (int f = pt; f < 6; f += N2) {
+    if (!active) break;
+    const int down = min(eout - sexp[lc][f], 63);
+    const FxPair g = sg[lc][f];
+    sg[lc][f] = sexp[lc][f] == -4 * FX_NAN
+                    ? FxPair{0, 0}
+                    : fx_pair((((long long)g.h << 30) + g.l) >> down);
+  }
+  {
+    const int down = min(eout - eown, 63);
+    if (!MODAL) {
+      const int E = (active ? expU[c] : 0) + 60;
+#pragma unroll
+      for (int e = 0; e < N; ++e) u[e] = fx_from_double(__longlong_as_double(u[e]), 60 - E, E);
+    }
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      u[e] >>= down;
+      if (live) su[e * SZ + q * SY + p] = u[e];
+    }
+  }
+  __syncthreads();
+  const unsigned row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  // r (= or +=) the line's terms: |r| < 2^62.3 in the end
+  auto line = [&](int dir, bool first) {
+    const FxPair* Mp = lineop + ((c * 3 + dir) * NP) * N2 + pt;
+    FxPair Mv[PRE ? NP : 1];
+    if constexpr (PRE) {
+#pragma unroll
+      for (int k = 0; k < NP; ++k) Mv[k] = dir == 2 ? Mz[k] : Mp[k * N2];
+    }
+    // absent neighbours: any value times a zero coefficient
+    const long long* t0 =
+        TR + (crd[dir] > 0 ? c - stride[dir] : c) * (12 * N2) + (4 * dir + 2) * N2 + pt;
+    const long long* t1 =
+        TR + (crd[dir] < Nc - 1 ? c + stride[dir] : c) * (12 * N2) + (4 * dir) * N2 + pt;
+    const FxVal v0 = fx_split(t0[0]), a0 = fx_split(t0[N2]);
+    const FxVal v1 = fx_split(t1[0]), a1 = fx_split(t1[N2]);
+    FxVal us[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) us[e] = fx_split(u[e]);
+    FxAcc R[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) R[e] = fx_zero();
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+#pragma unroll
+      for (int f = e; f < N; ++f) {
+        const FxPair m = PRE ? Mv[PRE ? packed<N>(e, f) : 0] : Mp[packed<N>(e, f) * N2];
+        fx_mac(R[e], m, us[f]);
+        if (f != e) fx_mac(R[f], m, us[e]);
+      }
+    }
+    const FxPair g0 = sg[active ? lc : 0][2 * dir], g1 = sg[active ? lc : 0][2 * dir + 1];
+    FxAcc A0 = fx_zero(), B0 = fx_zero(), A1 = fx_zero(), B1 = fx_zero();
+    fx_mac(A0, g0, a0);
+    fx_mac(B0, g0, v0);
+    fx_mac(A1, g1, a1);
+    fx_mac(B1, g1, v1);
+    const long long al0 = fx_value(A0), be0 = fx_value(B0), al1 = fx_value(A1),
+                    be1 = fx_value(B1);
+    const FxVal ad = fx_split(al0 - al1), as = fx_split(al0 + al1);
+    const FxVal bs = fx_split(be0 + be1), bd = fx_split(be0 - be1);
+#pragma unroll
+    for (int a = 0; a < (N + 1) / 2; ++a) {
+      FxAcc Pe = fx_zero();
+      fx_mac(Pe, tab.le[a], ad);
+      fx_mac(Pe, tab.de[a], bs);
+      const long long pe = fx_value(Pe);
+      if (a == N - 1 - a) {
+        r[a] = first ? pe : r[a] + pe;
+      } else {
+        FxAcc Po = fx_zero();
+        fx_mac(Po, tab.lo[a], as);
+        fx_mac(Po, tab.dn[a], bd);
+        const long long po = fx_value(Po);
+        r[a] = first ? pe + po : r[a] + (pe + po);
+        r[N - 1 - a] = first ? pe - po : r[N - 1 - a] + (pe - po);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < N; ++e) r[e] += fx_value(R[e]);
+  };
+  line(2, true);
+#pragma unroll
+  for (int e = 0; e < N; ++e)
+    if (live) sr[e * SZ + q * SY + p] = r[e];
+  __syncthreads();
+  // y-lines (a = p, e = q)
+#pragma unroll
+  for (int b = 0; b < N; ++b) {
+    u[b] = su[q * SZ + b * SY + p];
+    r[b] = sr[q * SZ + b * SY + p];
+  }
+  line(1, false);
+#pragma unroll
+  for (int b = 0; b < N; ++b)
+    if (live) sr[q * SZ + b * SY + p] = r[b];
+  __syncthreads();
+  // x-lines (b = p, e = q): the sum of all three directions
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    u[a] = su[q * SZ + p * SY + a];
+    r[a] = sr[q * SZ + p * SY + a];
+  }
+  line(0, false);
+  const double qnan = __longlong_as_double(0x7ff8000000000000ll);
+  if (!MODAL) {
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+      if (live)
+        sr[q * SZ + p * SY + a] =
+            __double_as_longlong(bad ? qnan : fx_to_double(r[a], eout - 1));
+    __syncthreads();
+    if (active) {  // written from the z-lines: consecutive lanes, consecutive words
+#pragma unroll
+      for (int e = 0; e < N; ++e)
+        y[c * N3 + e * N2 + q * N + p] = __longlong_as_double(sr[e * SZ + q * SY + p]);
+    }
+    return;
+  }
+  // the sum to a cell 2-norm of at most 2^60, then Q^T
+  unsigned big = 0;
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    const unsigned m = fx_mag_hi(r[a]);
+    big = m > big ? m : big;
+  }
+  const int up = FxScale<N>::S0 - fx_bits(fx_cell_max<N, BT>(big, lc, slots));
+#pragma unroll
+  for (int a = 0; a < N; ++a) r[a] = fx_shift(r[a], up);
+  fx_bwd<N>(tab, r, u);
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (live) su[q * SZ + p * SY + i] = u[i];
+  __syncthreads();
+  // y: (i = p, e = q)
+#pragma unroll
+  for (int b = 0; b < N; ++b) r[b] = su[q * SZ + b * SY + p];
+  fx_bwd<N>(tab, r, u);
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (live) su[q * SZ + j * SY + p] = u[j];
+  __syncthreads();
+  // z: (i = p, j = q)
+#pragma unroll
+  for (int e = 0; e < N; ++e) r[e] = su[e * SZ + q * SY + p];
+  fx_bwd<N>(tab, r, u);
+  if (active) {
+#pragma unroll
+    for (int l = 0; l < N; ++l)
+      y[c * N3 + l * N2 + q * N + p] = bad ? qnan : fx_to_double(u[l], eout - 1 - up);
   }
 }
 
