@@ -18,20 +18,6 @@ int dg_launch_trace_f64(const dg_mesh* m, const double* x, double* U, double* X,
   return DG_OK;
 }
 
-// Line operators of the batched solver in FP64, on the first batched solve
-// after the coefficient is set.
-int dg_ensure_lines64(dg_mesh* m, bool nodal, cudaStream_t s) {
-  bool& has = nodal ? m->has_nodal_lines : m->has_lines;
-  double*& lo = nodal ? m->lineopN64 : m->lineop64;
-  if (has) return DG_OK;
-  const size_t nlo = (size_t)3 * m->n * m->n * (size_t)(m->n * (m->n + 1) / 2) * (size_t)m->ncells;
-  if (lo == nullptr) DG_CUDA(cudaMalloc((void**)&lo, nlo * sizeof(double)));
-  cudaError_t e = dgk::dispatch_n<double, dgk::LineOpsF>(m->n, (const dg_mesh*)m, nodal, lo, s);
-  if (e != cudaSuccess) return dg_cuda_fail(e, "line operators launch");
-  has = true;
-  return DG_OK;
-}
-
 int dg_prepare_apply_f64(int n) {
   cudaError_t e = dgk::dispatch_n<double, dgk::PrepareF>(n);
   if (e != cudaSuccess) return dg_cuda_fail(e, "apply (fp64) kernel attributes");

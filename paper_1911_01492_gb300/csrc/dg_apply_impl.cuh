@@ -278,44 +278,6 @@ struct FaceGlobal {
   }
 };
 
-// FaceNbr: only the neighbour part of an interior face's flux; the own-side
-// part (and the whole boundary form) is inside the line operators.  With the
-// neighbour trace (un, gn) and W/2 = Wh (equal to the derivative weight
-// inside), the upper face gives cv = -Wh (2 sigma un + gn), cdm = -Wh un and
-// the lower face cv = Wh (gn - 2 sigma un), cdm = Wh un: three operations
-// and three loads per face point instead of five and six.
-template <typename T>
-struct FaceNbr {
-  const T* TR;
-  const T* FW;
-  static constexpr bool OWN_IN_THREAD = false;  // own terms are in the line operators
-  struct Pre {};
-  template <int N>
-  __device__ __forceinline__ void prefetch(Pre&, long long, int, const bool (&)[6],
-                                           const long long (&)[6]) const {}
-  template <int N, bool UPPER>
-  __device__ __forceinline__ void get(const Pre&, long long c, int lc, int f, bool in,
-                                      long long cn, int fn, int pt, T, T, T& cv,
-                                      T& cdm) const {
-    constexpr int N2 = N * N;
-    constexpr T S2 = T(4 * N * N);
-    (void)lc;
-    cv = T(0);
-    cdm = T(0);
-    if (!in) return;
-    T un, gn;
-    load_trace<N>(TR, cn, fn, pt, un, gn);
-    const T wh = FW[c * (12 * N2) + (2 * f) * N2 + pt];
-    if (UPPER) {
-      cv = -wh * fma(S2, un, gn);
-      cdm = -wh * un;
-    } else {
-      cv = wh * fma(-S2, un, gn);
-      cdm = wh * un;
-    }
-  }
-};
-
 // FaceLocal: own traces formed by the calling line-thread from its own line's
 // values (passed in as uo, go), neighbour traces from the pass-1 buffer,
 // weights from h*gamma per face (W/2 = h gamma w_s w_t / 2; the derivative
@@ -555,16 +517,11 @@ __host__ __device__ constexpr int packed(int i, int j) {
   return i <= j ? i * N - i * (i - 1) / 2 + (j - i) : j * N - j * (j - 1) / 2 + (i - j);
 }
 
-// LINEOP = true: the volume term of a line and the own-side terms of its two
-// face points are one precomputed symmetric operator per line (lineop:
-// [c][x,y,z][line][packed n(n+1)/2], see k_line_ops) instead of
-// D^T diag(Kt) D (y, z) and L'^T diag(Kt) L' (x); the face policy then adds
-// only the neighbour part of interior faces (FaceNbr).
-template <int N, typename T, typename FS, bool LINEOP = false>
+template <int N, typename T, typename FS>
 __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long long c0,
                                           int nblk, int Nc, const DGTab<T>& tab, T* su, T* sx,
-                                          T* sr, T* sk, const T* __restrict__ lineop = nullptr) {
-  constexpr int N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
+                                          T* sr, T* sk) {
+  constexpr int N2 = N * N, N3 = N * N * N;
 
   const int lc = threadIdx.x / N2;
   const int t2 = threadIdx.x - lc * N2;
@@ -609,21 +566,7 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       T u[N], r[N];
 #pragma unroll
       for (int e = 0; e < N; ++e) u[e] = su[o + base + e * step];
-      if (LINEOP) {
-        // dir 0 = z-lines (operator slot 2), dir 1 = y-lines (slot 1)
-        const T* Mp = lineop + ((c * 3 + (2 - dir)) * N2 + pt) * NP;
-        T Mv[NP];
-#pragma unroll
-        for (int t = 0; t < NP; ++t) Mv[t] = Mp[t];
-#pragma unroll
-        for (int e = 0; e < N; ++e) {
-          T acc = (dir == 0) ? Mv[packed<N>(e, 0)] * u[0]
-                             : fma(Mv[packed<N>(e, 0)], u[0], sr[o + base + e * step]);
-#pragma unroll
-          for (int f = 1; f < N; ++f) acc = fma(Mv[packed<N>(e, f)], u[f], acc);
-          r[e] = acc;
-        }
-      } else {
+      {
         T kg[N];
 #pragma unroll
         for (int e = 0; e < N; ++e) {
@@ -685,18 +628,7 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       X[i] = sx[o + base + i];
       rr[i] = sr[o + base + i];
     }
-    if (LINEOP) {
-      b_bwd<N>(tab, rr, R);
-      const T* Mp = lineop + ((c * 3 + 0) * N2 + pt) * NP;
-      T Mv[NP];
-#pragma unroll
-      for (int t = 0; t < NP; ++t) Mv[t] = Mp[t];
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) R[i] = fma(Mv[packed<N>(i, j)], X[j], R[i]);
-      }
-    } else {
+    {
       T g[N], kg[N];
       bd_fwd<N>(tab, X, g);
 #pragma unroll
@@ -769,13 +701,12 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
 
 // Pass 2 over the cells c0 .. c0+nblk-1 (nblk <= CPB) by the calling block;
 // smem: 4 CPB n^3 values of shared memory.
-// LINEOP: the volume term uses the precomputed line operators (kt unused).
-template <int N, typename T, bool LINEOP = false>
+template <int N, typename T>
 __device__ __forceinline__ void cell_cells(const T* __restrict__ U, const T* __restrict__ Xm,
                                            const T* __restrict__ TR, const T* __restrict__ kt,
                                            const T* __restrict__ FW, T* __restrict__ y,
                                            long long c0, int nblk, int Nc, const DGTab<T>& tab,
-                                           T* smem, const T* __restrict__ lineop = nullptr) {
+                                           T* smem) {
   constexpr int N3 = N * N * N, C = Cfg<N>::CPB;
   T* su = smem;
   T* sx = su + C * N3;
@@ -788,18 +719,12 @@ __device__ __forceinline__ void cell_cells(const T* __restrict__ U, const T* __r
     for (int t = threadIdx.x; t < nblk * N3; t += blockDim.x) {
       su[t] = ub[t];
       sx[t] = xb[t];
-      if (!LINEOP) sk[t] = kb[t];
+      sk[t] = kb[t];
     }
   }
   __syncthreads();
-  if constexpr (LINEOP) {
-    // the line operators hold the volume term and the own-side face terms
-    const FaceNbr<T> fs{TR, FW};
-    cell_core<N, T, FaceNbr<T>, true>(fs, y, c0, nblk, Nc, tab, su, sx, sr, sk, lineop);
-  } else {
-    const FaceGlobal<T> fs{TR, FW};
-    cell_core<N, T, FaceGlobal<T>, false>(fs, y, c0, nblk, Nc, tab, su, sx, sr, sk, lineop);
-  }
+  const FaceGlobal<T> fs{TR, FW};
+  cell_core<N, T, FaceGlobal<T>>(fs, y, c0, nblk, Nc, tab, su, sx, sr, sk);
 }
 
 template <int N, typename T>
@@ -814,93 +739,6 @@ k_cell(const T* __restrict__ U, const T* __restrict__ Xm, const T* __restrict__ 
   const long long c0 = cbeg + (long long)blockIdx.x * C;
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
   cell_cells<N, T>(U, Xm, TR, kt, FW, y, c0, nblk, Nc, tab, reinterpret_cast<T*>(smem_raw));
-}
-
-// Line operators from Kt = h w K and h gamma (one thread per cell, direction
-// and line):
-//   x-line (b, e):  M[i][j] = sum_a L_i'(xi_a) Kt(a, b, e) L_j'(xi_a)   (acts on x-modes)
-//   y-line (a, e):  M[i][j] = sum_f D[f][i] Kt(a, f, e) D[f][j]         (acts on nodal values)
-//   z-line (a, b):  M[i][j] = sum_f D[f][i] Kt(a, b, f) D[f][j]
-// plus the own-side part of the flux at the line's two face points, so that
-// pass 2 only adds the neighbour part of interior faces (FaceNbr).
-// Stored as lineop[((c*3 + dir)*n^2 + line)*n(n+1)/2 + packed(i, j)].
-// NODAL: the line operators of Q A Q^T in the scaled Gauss-point basis
-// (dg_nodal.cu): x-lines in the collocation form like y and z, every entry
-// (i, j) of the line (s, t) multiplied by isw_i isw_j / (w_s w_t), which
-// removes the tangential weights of Kt and of the face weight.
-template <int N, bool NODAL = false>
-__global__ void k_line_ops(const double* __restrict__ kt, const double* __restrict__ gh,
-                           double* __restrict__ lineop, long long ncells, int Nc,
-                           const __grid_constant__ DGTab<double> tab,
-                           const __grid_constant__ DGTabN<double> tn) {
-  constexpr int N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncells * 3 * N2) return;
-  const long long c = t / (3 * N2);
-  const int dir = (int)((t / N2) % 3);
-  const int line = (int)(t % N2);
-  const int p = line % N, q = line / N;
-  double k[N];
-#pragma unroll
-  for (int f = 0; f < N; ++f) {
-    // point index a + N(b + N e) along the line
-    const int qi = dir == 0 ? f + N * (p + N * q)      // x-line (b = p, e = q)
-                 : dir == 1 ? p + N * (f + N * q)      // y-line (a = p, e = q)
-                            : p + N * (q + N * f);     // z-line (a = p, b = q)
-    k[f] = kt[c * N3 + qi];
-  }
-  double* M = lineop + (t)*NP;
-  // volume: M[i][j] = sum_f g_i(f) k_f g_j(f), with gk[i][f] = g_i(f) k_f formed once
-  double gk[N][N];
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-#pragma unroll
-    for (int f = 0; f < N; ++f)
-      gk[i][f] = (dir == 0 && !NODAL ? tab.Bd[f][i] : tab.D[f][i]) * k[f];
-  }
-  // Own-side face terms of the line's two faces (both trial and test function
-  // on this cell's side).  At the face point of this line, with v the test
-  // values and d the test derivatives (d/dxi) at the face (modal a, L' on
-  // x-lines; Lagrange l, l' on y- and z-lines), the flux adds
-  //   Wh (2 sigma v v^T -+ c (v d^T + d v^T)),  Wh = h gamma_F w_s w_t / 2,
-  // "-" on the upper face, "+" on the lower one, c = 1 inside and 2 on the
-  // boundary (where the whole one-sided form is own-side).  Entry (i, j) of
-  // each face term is v_i P_j + d_i Q_j with P = Wh (2 sigma v -+ c d) and
-  // Q = -+ Wh c v.
-  const long long crd = dir == 0 ? c % Nc : dir == 1 ? (c / Nc) % Nc : c / ((long long)Nc * Nc);
-  const double w2 = tab.w[p] * tab.w[q];
-  const double whl = 0.5 * gh[c * 6 + 2 * dir] * w2, whu = 0.5 * gh[c * 6 + 2 * dir + 1] * w2;
-  const double cl = (crd > 0 ? 1.0 : 2.0) * whl, cu = (crd < Nc - 1 ? 1.0 : 2.0) * whu;
-  constexpr double S2 = 4.0 * N * N;  // 2 sigma, sigma = 2 (k+1)^2
-  double v0[N], d0[N], v1[N], d1[N], P0[N], Q0[N], P1[N], Q1[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    const bool modal = dir == 0 && !NODAL;
-    v0[j] = modal ? tab.a0[j] : tab.l0[j];
-    d0[j] = modal ? tab.d0[j] : tab.dl0[j];
-    v1[j] = modal ? tab.a1[j] : tab.l1[j];
-    d1[j] = modal ? tab.d1[j] : tab.dl1[j];
-    P0[j] = fma(whl * S2, v0[j], cl * d0[j]);
-    Q0[j] = cl * v0[j];
-    P1[j] = fma(whu * S2, v1[j], -cu * d1[j]);
-    Q1[j] = -cu * v1[j];
-  }
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-#pragma unroll
-    for (int j = i; j < N; ++j) {
-      double acc = 0.0;
-#pragma unroll
-      for (int f = 0; f < N; ++f)
-        acc = fma(gk[i][f], dir == 0 && !NODAL ? tab.Bd[f][j] : tab.D[f][j], acc);
-      acc = fma(v0[i], P0[j], acc);
-      acc = fma(d0[i], Q0[j], acc);
-      acc = fma(v1[i], P1[j], acc);
-      acc = fma(d1[i], Q1[j], acc);
-      if (NODAL) acc *= (tn.isw[i] * tn.isw[j]) / w2;
-      M[packed<N>(i, j)] = acc;
-    }
-  }
 }
 
 template <int N, typename T>
@@ -1031,21 +869,4 @@ struct TraceF {
   }
 };
 
-}  // namespace dgk
-
-namespace dgk {
-template <int N>
-struct LineOpsF {
-  template <typename T>
-  static cudaError_t run(const dg_mesh* m, bool nodal, double* lineop, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((m->ncells * 3 * N * N + 255) / 256);
-    if (nodal)
-      k_line_ops<N, true><<<blocks, 256, 0, s>>>(m->kt64, m->gh64, lineop, m->ncells, m->N,
-                                                 m->tab64, m->tabN64);
-    else
-      k_line_ops<N, false><<<blocks, 256, 0, s>>>(m->kt64, m->gh64, lineop, m->ncells, m->N,
-                                                  m->tab64, m->tabN64);
-    return cudaGetLastError();
-  }
-};
 }  // namespace dgk

@@ -49,7 +49,7 @@
 #include <string>
 #include <vector>
 
-#include "dg_nodal_impl.cuh"
+#include "dg_fixed.cuh"
 
 namespace {
 
@@ -58,18 +58,17 @@ constexpr int TILES[3] = {1, 2, 4};   // cell groups per work unit (tuned)
 constexpr double LAUNCH_SECONDS = 2.0;   // work per production launch (estimate)
 constexpr double EST_DOF_RATE = 7.0e9;   // DOF-iterations per second for that estimate
 
-__constant__ DGTab<double> c_btab[DG_MAXN - 1];  // tables for n = 2..9
-__constant__ DGTabN<double> c_btabN[DG_MAXN - 1];  // scaled Gauss-point basis, n = 2..9
+__constant__ DGTabX c_btab[DG_MAXN - 1];  // fixed-point tables for n = 2..9
 
 struct SampleDev {
   const double* b;
   double* x;
   double *r, *u, *w, *p, *s;  // u == r when M = I
-  double *U, *X, *TR;
-  const double* kt;      // h w K (not read: the line operators hold the volume term)
-  const double* fw;
-  const double* lineop;  // line operators of A, or of Q A Q^T in the scaled Gauss-point basis
-  const double* gh;      // h gamma per face side (the point basis's face weights)
+  // fixed-point operator (dg_fixed.cuh)
+  long long *U, *TR;
+  int* expU;
+  const FxPair *lineop, *gam;
+  const int *expM, *expG;
   const double* dinv;  // 1 / diag(A) for M = diag(A); nullptr for M = I
   long long ncells;
   int Nc;          // cells per direction
@@ -143,62 +142,56 @@ __host__ __device__ constexpr int group_cells(int n) {
        : n == 8 ? dgk::Cfg<8>::CPB : dgk::Cfg<9>::CPB;
 }
 
-// ND: the samples' vectors are in the scaled Gauss-point basis (DG_CG_NODAL)
-// and the passes are the transform-free ones of dg_nodal_impl.cuh.
-template <int N, bool ND>
+// ND: the samples' vectors are in the scaled Gauss-point basis (DG_CG_NODAL).
+template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass1(const SampleDev& S, long long c0, int nblk,
-                                            double* smem) {
-  if constexpr (ND)
-    dgk::trace_cells_nd<N, double>(S.u, S.TR, c0, nblk, c_btabN[N - 2], smem);
-  else
-    dgk::trace_cells<N, double>(S.u, S.U, S.X, S.TR, c0, nblk, c_btab[N - 2], smem);
+                                            long long* smem) {
+  dgk::fx_trace_cells<N, !ND, BT>(S.u, S.U, S.TR, S.expU, c0, nblk, c_btab[N - 2], smem);
 }
-template <int N, bool ND>
+template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass2(const SampleDev& S, long long c0, int nblk,
-                                            double* smem) {
-  if constexpr (ND)
-    dgk::cell_cells_nd<N>(S.u, S.TR, S.lineop, S.gh, S.w, c0, nblk, S.Nc, c_btabN[N - 2], smem);
-  else
-    dgk::cell_cells<N, double, true>(S.U, S.X, S.TR, S.kt, S.fw, S.w, c0, nblk, S.Nc,
-                                     c_btab[N - 2], smem, S.lineop);
+                                            long long* smem) {
+  dgk::fx_cell_cells<N, !ND, BT>(ND ? (const void*)S.u : (const void*)S.U, S.TR, S.expU,
+                                 S.lineop, S.gam, S.expM, S.expG, S.w, c0, nblk, S.Nc,
+                                 c_btab[N - 2], smem);
 }
 
-template <int MAXN, bool ND>
+template <int MAXN, bool ND, int BT>
 __device__ __forceinline__ void pass1_dispatch(const SampleDev& sd, long long c, int nblk,
-                                               double* smem) {
+                                               long long* smem) {
   switch (sd.n) {
-    case 2: group_pass1<2, ND>(sd, c, nblk, smem); break;
-    case 3: group_pass1<3, ND>(sd, c, nblk, smem); break;
-    case 4: group_pass1<4, ND>(sd, c, nblk, smem); break;
-    case 5: group_pass1<5, ND>(sd, c, nblk, smem); break;
+    case 2: group_pass1<2, ND, BT>(sd, c, nblk, smem); break;
+    case 3: group_pass1<3, ND, BT>(sd, c, nblk, smem); break;
+    case 4: group_pass1<4, ND, BT>(sd, c, nblk, smem); break;
+    case 5: group_pass1<5, ND, BT>(sd, c, nblk, smem); break;
     default:
       if constexpr (MAXN > 5) {
         switch (sd.n) {
-          case 6: group_pass1<6, ND>(sd, c, nblk, smem); break;
-          case 7: group_pass1<7, ND>(sd, c, nblk, smem); break;
-          case 8: group_pass1<8, ND>(sd, c, nblk, smem); break;
-          default: group_pass1<9, ND>(sd, c, nblk, smem); break;
+          case 6: group_pass1<6, ND, BT>(sd, c, nblk, smem); break;
+          case 7: group_pass1<7, ND, BT>(sd, c, nblk, smem); break;
+          case 8: group_pass1<8, ND, BT>(sd, c, nblk, smem); break;
+          default: group_pass1<9, ND, BT>(sd, c, nblk, smem); break;
         }
       }
       break;
   }
 }
 
-template <int MAXN, bool ND>
+template <int MAXN, bool ND, int BT>
 __device__ __forceinline__ void pass2_dispatch(const SampleDev& sd, long long c, int nblk,
-                                               double* smem) {
+                                               long long* smem) {
   switch (sd.n) {
-    case 2: group_pass2<2, ND>(sd, c, nblk, smem); break;
-    case 3: group_pass2<3, ND>(sd, c, nblk, smem); break;
-    case 4: group_pass2<4, ND>(sd, c, nblk, smem); break;
-    case 5: group_pass2<5, ND>(sd, c, nblk, smem); break;
+    case 2: group_pass2<2, ND, BT>(sd, c, nblk, smem); break;
+    case 3: group_pass2<3, ND, BT>(sd, c, nblk, smem); break;
+    case 4: group_pass2<4, ND, BT>(sd, c, nblk, smem); break;
+    case 5: group_pass2<5, ND, BT>(sd, c, nblk, smem); break;
     default:
       if constexpr (MAXN > 5) {
         switch (sd.n) {
-          case 6: group_pass2<6, ND>(sd, c, nblk, smem); break;
-          case 7: group_pass2<7, ND>(sd, c, nblk, smem); break;
-          case 8: group_pass2<8, ND>(sd, c, nblk, smem); break;
-          default: group_pass2<9, ND>(sd, c, nblk, smem); break;
+          case 6: group_pass2<6, ND, BT>(sd, c, nblk, smem); break;
+          case 7: group_pass2<7, ND, BT>(sd, c, nblk, smem); break;
+          case 8: group_pass2<8, ND, BT>(sd, c, nblk, smem); break;
+          default: group_pass2<9, ND, BT>(sd, c, nblk, smem); break;
         }
       }
       break;
@@ -213,7 +206,7 @@ kb_persistent(const SampleDev* __restrict__ S, const int2* __restrict__ units, i
               BState* st, double* part, unsigned* tickets, BCtl* ctl, int iters, long long limit,
               int stall_test) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* smem = reinterpret_cast<double*>(smem_raw);
+  long long* smem = reinterpret_cast<long long*>(smem_raw);
   __shared__ double sred[BT / 32];
   __shared__ bool is_last;
   const unsigned nb = gridDim.x;
@@ -255,7 +248,7 @@ kb_persistent(const SampleDev* __restrict__ S, const int2* __restrict__ units, i
       __syncthreads();
       for (long long c = c0; c < c1; c += cpb) {
         const int nblk = (int)((c1 - c) < cpb ? (c1 - c) : cpb);
-        pass1_dispatch<MAXN, ND>(sd, c, nblk, smem);
+        pass1_dispatch<MAXN, ND, BT>(sd, c, nblk, smem);
         __syncthreads();
       }
     }
@@ -271,7 +264,7 @@ kb_persistent(const SampleDev* __restrict__ S, const int2* __restrict__ units, i
                                                                     : sd.ncells;
       for (long long c = c0; c < c1; c += cpb) {
         const int nblk = (int)((c1 - c) < cpb ? (c1 - c) : cpb);
-        pass2_dispatch<MAXN, ND>(sd, c, nblk, smem);
+        pass2_dispatch<MAXN, ND, BT>(sd, c, nblk, smem);
         __syncthreads();
       }
       const long long n3 = (long long)sd.n * sd.n * sd.n;
@@ -441,13 +434,16 @@ kb_init_scalars(const double* __restrict__ r, const double* __restrict__ u,
   }
 }
 
-// ||b - q||^2 and ||b||^2 into out[0..1] (single block, fixed order).
+// ||b - q||^2 and ||b||^2 into out[0..1]: the blocks' partials added by the
+// last block in a fixed order.
 __global__ void __launch_bounds__(256)
 kb_residual(const double* __restrict__ b, const double* __restrict__ q, long long n,
-            double* out) {
+            double* partials, unsigned* ticket, double* out) {
   __shared__ double sred[8];
+  __shared__ bool last;
   double rr = 0.0, bb = 0.0;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
     const double ri = b[i] - q[i];
     rr = fma(ri, ri, rr);
     bb = fma(b[i], b[i], bb);
@@ -455,39 +451,38 @@ kb_residual(const double* __restrict__ b, const double* __restrict__ q, long lon
   rr = block_sum<256>(rr, sred);
   bb = block_sum<256>(bb, sred);
   if (threadIdx.x == 0) {
+    partials[2 * blockIdx.x] = rr;
+    partials[2 * blockIdx.x + 1] = bb;
+    __threadfence();
+    last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  rr = bb = 0.0;
+  for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
+    rr += __ldcg(partials + 2 * i);
+    bb += __ldcg(partials + 2 * i + 1);
+  }
+  rr = block_sum<256>(rr, sred);
+  bb = block_sum<256>(bb, sred);
+  if (threadIdx.x == 0) {
     out[0] = rr;
     out[1] = bb;
+    *ticket = 0u;
   }
 }
 
-template <int MAXN, bool ND>
-size_t persistent_smem() {
-  if constexpr (ND) {  // the point basis's passes need half the shared memory
-    size_t m = 0;
-    m = std::max(m, dgk::cell_smem_nd<2>());
-    m = std::max(m, dgk::cell_smem_nd<3>());
-    m = std::max(m, dgk::cell_smem_nd<4>());
-    m = std::max(m, dgk::cell_smem_nd<5>());
-    if (MAXN > 5) {
-      m = std::max(m, dgk::cell_smem_nd<6>());
-      m = std::max(m, dgk::cell_smem_nd<7>());
-      m = std::max(m, dgk::cell_smem_nd<8>());
-      m = std::max(m, dgk::cell_smem_nd<9>());
-    }
+template <int N, int MAXN, int BT>
+constexpr size_t persistent_smem() {  // the larger of the two passes, over all n <= MAXN
+  constexpr size_t a = dgk::FxSmem<N, BT>::trace, b = dgk::FxSmem<N, BT>::cell;
+  constexpr size_t m = a > b ? a : b;
+  if constexpr (N == MAXN) {
     return m;
+  } else {
+    constexpr size_t o = persistent_smem<N + 1, MAXN, BT>();
+    return m > o ? m : o;
   }
-  size_t m = 0;
-  m = std::max(m, dgk::cell_smem<2, double>());
-  m = std::max(m, dgk::cell_smem<3, double>());
-  m = std::max(m, dgk::cell_smem<4, double>());
-  m = std::max(m, dgk::cell_smem<5, double>());
-  if (MAXN > 5) {
-    m = std::max(m, dgk::cell_smem<6, double>());
-    m = std::max(m, dgk::cell_smem<7, double>());
-    m = std::max(m, dgk::cell_smem<8, double>());
-    m = std::max(m, dgk::cell_smem<9, double>());
-  }
-  return m;
 }
 
 double now_s() {
@@ -562,7 +557,7 @@ int launch_persistent(Batch& B, int count, int tsel, int blocks, int iters, long
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(BT);
-  cfg.dynamicSmemBytes = persistent_smem<MAXN, ND>();
+  cfg.dynamicSmemBytes = persistent_smem<2, MAXN, BT>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -618,13 +613,13 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
     d.w = m->q64;
     d.s = m->s64;
     d.u = m->r64;  // M = I: u is r itself
-    d.U = m->U64;
-    d.X = m->X64;
-    d.TR = m->TR64;
-    d.kt = m->kt64;
-    d.fw = m->fw64;
-    d.lineop = ND ? m->lineopN64 : m->lineop64;
-    d.gh = m->gh64;
+    d.U = reinterpret_cast<long long*>(m->U64);
+    d.TR = reinterpret_cast<long long*>(m->TR64);
+    d.expU = m->expU;
+    d.lineop = m->lineopX;
+    d.gam = m->gamX;
+    d.expM = m->expM;
+    d.expG = m->expG;
     d.dinv = nullptr;
     if (jacobi) {
       rc = dg_ensure_diagonal(m, m->solve_stream);
@@ -662,7 +657,8 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
   DG_CUDA(cudaMalloc(&B.d_part, sizeof(double) * 3 * B.nunits[0]));
   DG_CUDA(cudaMalloc(&B.d_tickets, sizeof(unsigned) * count));
   DG_CUDA(cudaMalloc(&B.d_ctl, sizeof(BCtl)));
-  DG_CUDA(cudaMalloc(&B.d_aux, sizeof(double) * 2 * 1024));
+  // init partials, then one residual pair per sample
+  DG_CUDA(cudaMalloc(&B.d_aux, sizeof(double) * 2 * (1024 + (size_t)count)));
   DG_CUDA(cudaMalloc(&B.d_ticket, sizeof(unsigned)));
   DG_CUDA(cudaMallocHost(&B.h_ctl, sizeof(BCtl)));
   *B.h_ctl = BCtl{};
@@ -673,19 +669,15 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
                             cudaMemcpyHostToDevice, s));
   DG_CUDA(cudaMemsetAsync(B.d_ticket, 0, sizeof(unsigned), s));
   DG_CUDA(cudaMemsetAsync(B.d_tickets, 0, sizeof(unsigned) * count, s));
-  {
-    DGTab<double> t64[DG_MAXN - 1];
-    DGTab<float> t32;
-    for (int n = 2; n <= DG_MAXN; ++n) dg_build_tables(n, 2.0 * n * n, &t64[n - 2], &t32);
-    DG_CUDA(cudaMemcpyToSymbolAsync(c_btab, t64, sizeof(t64), 0, cudaMemcpyHostToDevice, s));
-    if (ND) {
-      DGTabN<double> tn64[DG_MAXN - 1];
-      DGTabN<float> tn32;
-      for (int n = 2; n <= DG_MAXN; ++n) dg_build_nodal_tables(t64[n - 2], n, &tn64[n - 2], &tn32);
-      DG_CUDA(cudaMemcpyToSymbolAsync(c_btabN, tn64, sizeof(tn64), 0, cudaMemcpyHostToDevice, s));
-    }
+  bool have[DG_MAXN + 1] = {};
+  for (const dg_mesh* m : B.meshes) {  // the tables of each n in the batch
+    if (have[m->n]) continue;
+    have[m->n] = true;
+    DG_CUDA(cudaMemcpyToSymbolAsync(c_btab, &m->tabX, sizeof(DGTabX),
+                                    sizeof(DGTabX) * (size_t)(m->n - 2), cudaMemcpyHostToDevice,
+                                    s));
   }
-  const size_t smem = persistent_smem<MAXN, ND>();
+  const size_t smem = persistent_smem<2, MAXN, BT>();
   DG_CUDA(cudaFuncSetAttribute(kb_persistent<BT, MAXN, ND>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int max_bpsm = 0;
@@ -855,16 +847,24 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
                             cudaMemcpyDeviceToHost, s));
     DG_CUDA(cudaStreamSynchronize(s));
     bool any_restart = false;
+    std::vector<double> outs(2 * (size_t)count);
+    double* d_out = B.d_aux + 2 * 1024;
+    for (int i = 0; i < count; ++i) {
+      if (round > 0 && status[i] != DG_ERR_NOT_CONVERGED) continue;
+      dg_mesh* m = B.meshes[i];
+      rc = dg_launch_apply_f64(m, x[i], m->q64, nullptr, s);
+      if (rc) return rc;
+      kb_residual<<<256, 256, 0, s>>>(b[i], m->q64, m->ndofs, B.d_aux, B.d_ticket, d_out + 2 * i);
+      DG_CUDA(cudaGetLastError());
+    }
+    DG_CUDA(cudaMemcpyAsync(outs.data(), d_out, sizeof(double) * outs.size(),
+                            cudaMemcpyDeviceToHost, s));
+    DG_CUDA(cudaStreamSynchronize(s));
     for (int i = 0; i < count; ++i) {
       if (round > 0 && status[i] != DG_ERR_NOT_CONVERGED) continue;
       dg_mesh* m = B.meshes[i];
       iters_total[i] = hst[i].iters;
-      rc = dg_launch_apply_f64(m, x[i], m->q64, nullptr, s);
-      if (rc) return rc;
-      kb_residual<<<1, 256, 0, s>>>(b[i], m->q64, m->ndofs, B.d_aux);
-      double out[2];
-      DG_CUDA(cudaMemcpyAsync(out, B.d_aux, sizeof(out), cudaMemcpyDeviceToHost, s));
-      DG_CUDA(cudaStreamSynchronize(s));
+      const double* out = &outs[2 * (size_t)i];
       rel[i] = out[1] > 0 ? std::sqrt(out[0] / out[1]) : 0.0;
       if (out[1] == 0.0 && !hst[i].breakdown)  // A x = 0 has the solution x = 0
         DG_CUDA(cudaMemsetAsync(x[i], 0, sizeof(double) * (size_t)m->ndofs, s));
@@ -943,7 +943,8 @@ int solve_batched_nodal(const dg_mesh* const* meshes, int count, const double* c
     if (r2) return r2;
     r2 = dg_launch_apply_f64(m, x[i], m->q64, nullptr, us);
     if (r2) return r2;
-    kb_residual<<<1, 256, 0, us>>>(b[i], m->q64, m->ndofs, m->partials);
+    kb_residual<<<256, 256, 0, us>>>(b[i], m->q64, m->ndofs, m->partials + 2, &m->state->ticket,
+                                     m->partials);
     double out[2];
     DG_CUDA(cudaMemcpyAsync(out, m->partials, sizeof(out), cudaMemcpyDeviceToHost, us));
     DG_CUDA(cudaStreamSynchronize(us));
@@ -1005,9 +1006,6 @@ extern "C" int dg_cg_solve_batched_mode(const dg_mesh* const* meshes, int count,
                        s);
     maxn = m->n > maxn ? m->n : maxn;
   }
-  for (int s = 0; s < count; ++s)
-    if (int rc = dg_ensure_lines64(const_cast<dg_mesh*>(meshes[s]), nodal, (cudaStream_t)stream))
-      return rc;
   if (nodal) return solve_batched_nodal(meshes, count, b, x, rtol, maxit, maxn, mode, st, stream);
   if (maxn <= 5)
     return solve_batched<128, 5, false>(meshes, count, b, x, rtol, maxit, jacobi, mode, st,

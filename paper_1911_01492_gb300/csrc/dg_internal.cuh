@@ -142,7 +142,6 @@ struct dg_mesh {
   float* gh32;
   double* dgam;     // d gamma_F / d log Kbar_c       [c][6]
   double* fw64;     // face-point weights W/2 and derivative weight  [c][6][2][n^2]
-  double* lineop64; // FP64 line operators of the batched solver [c][3][n^2][n(n+1)/2]
   float* fw32;
   // Jacobi preconditioner: 1 / diag(A), formed on the first preconditioned solve
   double* diag64;
@@ -162,10 +161,9 @@ struct dg_mesh {
   // the coefficient is set) and the solve's b and x in that basis
   DGTabN<double> tabN64;
   DGTabN<float> tabN32;
-  bool has_lines, has_nodal_lines, has_nodal_diag;
+  bool has_nodal_diag;
   bool nodal_op;      // set while a solve runs in that basis: the internal
                       // FP64 apply launcher then applies Q A Q^T
-  double* lineopN64;  // [c][3][n^2][n(n+1)/2]
   double* dinvN64;
   float* dinvN32;
   double *bN64, *xN64;
@@ -287,8 +285,6 @@ void dg_build_nodal_tables(const DGTab<double>& t, int n, DGTabN<double>* d, DGT
 int dg_ensure_nodal(dg_mesh* m, cudaStream_t s);
 int dg_ensure_nodal_diag(dg_mesh* m, cudaStream_t s);
 int dg_ensure_nodal32(dg_mesh* m, cudaStream_t s);  // h K in FP32 for the mixed CG
-// FP64 line operators of the batched solver (nodal: of Q A Q^T), if needed
-int dg_ensure_lines64(dg_mesh* m, bool nodal, cudaStream_t s);
 int dg_launch_collocation(const dg_mesh* m, const double* in, double* out, bool to_nodal,
                           cudaStream_t s);
 

@@ -24,7 +24,7 @@
 // h gamma w_s w_t / 2 of a face point loses its tangential weights against
 // the two isw factors of the traces, so every point of a face has the weight
 // h gamma / 2 and no per-point face-weight array is read.
-#include "dg_nodal_impl.cuh"
+#include "dg_apply_impl.cuh"
 
 namespace dgk {
 
@@ -113,21 +113,27 @@ k_collocation(const double* __restrict__ in, double* __restrict__ out, long long
 
 // 1 / diag(Q A Q^T): at point (a, b, e) the sum of the diagonal entries of the
 // x-, y- and z-line operators through it (the neighbour terms couple other
-// cells only).  One thread per DOF.
+// cells only).  The operators are integers with one exponent per cell
+// (dg_fixed.cu): the sum is one too.  One thread per DOF.
 template <int N>
-__global__ void k_diag_nd(const double* __restrict__ lineop, double* __restrict__ dinv64,
-                          float* __restrict__ dinv32, long long ndofs) {
+__global__ void k_diag_nd(const FxPair* __restrict__ lineop, const int* __restrict__ expM,
+                          double* __restrict__ dinv64, float* __restrict__ dinv32,
+                          long long ndofs) {
   constexpr int N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ndofs) return;
   const long long c = t / N3;
   const int qi = (int)(t - c * N3);
   const int a = qi % N, b = (qi / N) % N, e = qi / N2;
-  const double* L = lineop + c * 3 * N2 * NP;
-  const double d = L[(0 * N2 + b + N * e) * NP + packed<N>(a, a)] +
-                   L[(1 * N2 + a + N * e) * NP + packed<N>(b, b)] +
-                   L[(2 * N2 + a + N * b) * NP + packed<N>(e, e)];
-  const double di = 1.0 / d;
+  const FxPair* L = lineop + c * 3 * NP * N2;
+  auto entry = [L](int dir, int line, int k) {
+    const FxPair v = L[(dir * NP + k) * N2 + line];
+    return ((long long)v.h << 30) + v.l;
+  };
+  const long long sum = entry(0, b + N * e, packed<N>(a, a)) +
+                        entry(1, a + N * e, packed<N>(b, b)) +
+                        entry(2, a + N * b, packed<N>(e, e));
+  const double di = 1.0 / scalbn((double)sum, expM[c] - 61);
   dinv64[t] = di;
   dinv32[t] = (float)di;
 }
@@ -161,7 +167,7 @@ struct NodalF {
         return cudaGetLastError();
       case 3:
         k_diag_nd<N><<<(unsigned)((m->ndofs + 255) / 256), 256, 0, s>>>(
-            m->lineopN64, m->dinvN64, m->dinvN32, m->ndofs);
+            m->lineopX, m->expM, m->dinvN64, m->dinvN32, m->ndofs);
         return cudaGetLastError();
       default: return cudaErrorInvalidValue;
     }
@@ -231,7 +237,6 @@ int dg_ensure_nodal(dg_mesh* m, cudaStream_t s) {
 int dg_ensure_nodal_diag(dg_mesh* m, cudaStream_t s) {
   int rc = dg_ensure_nodal(m, s);
   if (rc || m->has_nodal_diag) return rc;
-  if ((rc = dg_ensure_lines64(m, true, s))) return rc;
   const size_t nd = (size_t)m->ndofs;
   if (m->dinvN64 == nullptr) DG_CUDA(cudaMalloc((void**)&m->dinvN64, nd * sizeof(double)));
   if (m->dinvN32 == nullptr) DG_CUDA(cudaMalloc((void**)&m->dinvN32, nd * sizeof(float)));
