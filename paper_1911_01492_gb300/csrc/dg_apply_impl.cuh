@@ -40,23 +40,31 @@
 namespace dgk {
 
 // Sum of partials[0 .. count) in the last block of a grid reduction, by all
-// NT threads of the block in a fixed order: each thread keeps four
+// NT threads of the block in a fixed order: each thread keeps sixteen
 // independent chains of L2 loads (ld.global.cg: the other blocks' partials,
-// published before their ticket increment), then warp 0 adds the threads'
-// sums with a fixed tree.  Valid in warp 0; every thread of the block calls it.
+// published before their ticket increment) - one SM reads them alone, so with
+// four chains 22,000 partials took 35 dependent round trips - then warp 0
+// adds the threads' sums with a fixed tree.  Valid in warp 0; every thread of
+// the block calls it.
 template <int NT>
 __device__ __forceinline__ double last_block_total(const double* __restrict__ partials,
                                                    int count, double* scratch) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int b = threadIdx.x;
-  for (; b + 3 * NT < count; b += 4 * NT) {
-    a0 += __ldcg(partials + b);
-    a1 += __ldcg(partials + b + NT);
-    a2 += __ldcg(partials + b + 2 * NT);
-    a3 += __ldcg(partials + b + 3 * NT);
+  constexpr int CH = 16;
+  double a[CH];
+#pragma unroll
+  for (int k = 0; k < CH; ++k) a[k] = 0.0;
+  for (int b = threadIdx.x; b < count; b += CH * NT) {
+    double v[CH];
+#pragma unroll
+    for (int k = 0; k < CH; ++k) v[k] = b + k * NT < count ? __ldcg(partials + b + k * NT) : 0.0;
+#pragma unroll
+    for (int k = 0; k < CH; ++k) a[k] += v[k];
   }
-  for (; b < count; b += NT) a0 += __ldcg(partials + b);
-  scratch[threadIdx.x] = (a0 + a1) + (a2 + a3);
+#pragma unroll
+  for (int w = CH / 2; w > 0; w /= 2)
+#pragma unroll
+    for (int k = 0; k < w; ++k) a[k] += a[k + w];
+  scratch[threadIdx.x] = a[0];
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x < 32) {

@@ -146,13 +146,13 @@ __host__ __device__ constexpr int group_cells(int n) {
 template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass1(const SampleDev& S, long long c0, int nblk,
                                             long long* smem) {
-  dgk::fx_trace_cells<N, !ND, BT>(S.u, S.U, S.TR, S.expU, c0, nblk, c_btab[N - 2], smem);
+  dgk::fx_trace_cells<N, !ND, BT>(dgk::FxLoad{S.u}, S.U, S.TR, S.expU, c0, nblk, c_btab[N - 2], smem);
 }
 template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass2(const SampleDev& S, long long c0, int nblk,
                                             long long* smem) {
   dgk::fx_cell_cells<N, !ND, BT>(ND ? (const void*)S.u : (const void*)S.U, S.TR, S.expU,
-                                 S.lineop, S.gam, S.expM, S.expG, S.w, c0, nblk, S.Nc,
+                                 S.lineop, S.gam, S.expM, S.expG, dgk::FxStore{S.w}, c0, nblk, S.Nc,
                                  c_btab[N - 2], smem);
 }
 

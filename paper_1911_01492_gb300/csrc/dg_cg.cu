@@ -540,10 +540,17 @@ bool aligned16(const void* ptr) { return ((uintptr_t)ptr & 15u) == 0; }
 // One iteration of plain CG on FP64 or FP32 vectors.  With f0 <= f1 the
 // operator is restricted to the DOFs [f0, f1): q = A p is set to zero outside
 // them (p, r and x then stay zero there too).
+//
+// FP64 on a cube mesh: the direction update opens the iteration, inside pass 1
+// (beta = 0 in the first one), and <p, q> and alpha come with pass 2.  Elsewhere
+// the update of p closes it.
 template <typename T>
 int launch_iteration(dg_mesh* m, T* x, T* r, T* p, T* q, const T* dinv, cudaStream_t s,
                      long long f0 = -1, long long f1 = -1) {
-  int rc = (sizeof(T) == 8)
+  const bool fused = sizeof(T) == 8 && !m->affine && !m->multilinear;
+  int rc = fused ? dg_launch_fixed_cg(m, (const double*)r, (const double*)dinv, (double*)p,
+                                      (double*)q, s)
+           : sizeof(T) == 8
                ? dg_launch_apply_f64(m, (const double*)p, (double*)q, &m->state->done, s)
                : dg_launch_apply_f32(m, (const float*)p, (float*)q, &m->state->done, s);
   if (rc) return rc;
@@ -553,56 +560,55 @@ int launch_iteration(dg_mesh* m, T* x, T* r, T* p, T* q, const T* dinv, cudaStre
   // 16-byte vector kernels when every operand allows it (x is the caller's)
   const bool vec = aligned16(x) && aligned16(r) && aligned16(p) && aligned16(q) &&
                    aligned16(dinv);
-  if (vec)
-    k_dot_pq<T, true><<<RED_LAUNCH>>>(p, q, n, m->partials, m->state);
-  else
-    k_dot_pq<T, false><<<RED_LAUNCH>>>(p, q, n, m->partials, m->state);
-  if (dinv && vec) {
-    k_update_xr<T, false, true, true><<<RED_LAUNCH>>>(x, r, p, q, dinv, n, m->partials,
-                                                      m->state);
-    k_update_p<T, true, true><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
-  } else if (dinv) {
+  if (!fused) {
+    if (vec)
+      k_dot_pq<T, true><<<RED_LAUNCH>>>(p, q, n, m->partials, m->state);
+    else
+      k_dot_pq<T, false><<<RED_LAUNCH>>>(p, q, n, m->partials, m->state);
+  }
+  if (dinv && vec)
+    k_update_xr<T, false, true, true><<<RED_LAUNCH>>>(x, r, p, q, dinv, n, m->partials, m->state);
+  else if (dinv)
     k_update_xr<T, false, true, false><<<RED_LAUNCH>>>(x, r, p, q, dinv, n, m->partials,
                                                        m->state);
-    k_update_p<T, true, false><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
-  } else if (vec) {
+  else if (vec)
     k_update_xr<T, false, false, true><<<RED_LAUNCH>>>(x, r, p, q, dinv, n, m->partials,
                                                        m->state);
-    k_update_p<T, false, true><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
-  } else {
+  else
     k_update_xr<T, false, false, false><<<RED_LAUNCH>>>(x, r, p, q, dinv, n, m->partials,
                                                         m->state);
-    k_update_p<T, false, false><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
+  if (!fused) {
+    if (dinv && vec)
+      k_update_p<T, true, true><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
+    else if (dinv)
+      k_update_p<T, true, false><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
+    else if (vec)
+      k_update_p<T, false, true><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
+    else
+      k_update_p<T, false, false><<<RED_LAUNCH>>>(p, r, dinv, n, m->state);
   }
   DG_CUDA(cudaGetLastError());
   return DG_OK;
 }
 
-// One iteration of FP64 PCG with the cell-block Jacobi preconditioner:
-// q = A p, alpha, x and r updates with <r, r>, z = M^-1 r with <z, r> (rho,
-// beta), p = z + beta p.
-int launch_iteration_block(dg_mesh* m, double* x, cudaStream_t s) {
-  int rc = dg_launch_apply_f64(m, m->p64, m->q64, &m->state->done, s);
+// One iteration of FP64 PCG with cell blocks (exact or Kronecker): p = z + beta p,
+// q = A p, alpha (dg_launch_fixed_cg), x and r updates with <r, r>, z = M^-1 r in
+// t64 with <z, r> (rho, beta).
+int launch_iteration_blocks(dg_mesh* m, double* x, bool kron, cudaStream_t s) {
+  int rc = dg_launch_fixed_cg(m, m->t64, nullptr, m->p64, m->q64, s);
   if (rc) return rc;
   const long long n = m->ndofs;
-  const bool vec = aligned16(x);
-  if (vec) {
-    k_dot_pq<double, true><<<RED_LAUNCH>>>(m->p64, m->q64, n, m->partials, m->state);
+  if (aligned16(x))
     k_update_xr<double, false, false, true, true><<<RED_LAUNCH>>>(x, m->r64, m->p64, m->q64,
                                                                   nullptr, n, m->partials,
                                                                   m->state);
-  } else {
-    k_dot_pq<double, false><<<RED_LAUNCH>>>(m->p64, m->q64, n, m->partials, m->state);
+  else
     k_update_xr<double, false, false, false, true><<<RED_LAUNCH>>>(x, m->r64, m->p64, m->q64,
                                                                    nullptr, n, m->partials,
                                                                    m->state);
-  }
   DG_CUDA(cudaGetLastError());
-  rc = dg_launch_block_apply(m, m->r64, m->t64, nullptr, false, s);
-  if (rc) return rc;
-  k_update_p<double, false, true><<<RED_LAUNCH>>>(m->p64, m->t64, nullptr, n, m->state);
-  DG_CUDA(cudaGetLastError());
-  return DG_OK;
+  return kron ? dg_launch_kron_apply(m, m->r64, m->t64, nullptr, DG_KRON_FP64, s)
+              : dg_launch_block_apply(m, m->r64, m->t64, nullptr, false, s);
 }
 
 // One FP32 iteration of the mixed CG: direction update, operator and <p, q>
@@ -629,31 +635,6 @@ int launch_iteration_mixed(dg_mesh* m, const float* dinv, cudaStream_t s, bool k
   else
     k_update_xr<float, true, false, true><<<RED_LAUNCH>>>(m->d32, m->r32, m->p32, m->q32, dinv,
                                                           n, m->partials, m->state);
-  DG_CUDA(cudaGetLastError());
-  return DG_OK;
-}
-
-// One FP64 PCG iteration with the Kronecker cell blocks: q = A p, alpha, x and
-// r updates with <r, r>, z = M^-1 r with <z, r> (rho, beta), p = z + beta p.
-int launch_iteration_kron(dg_mesh* m, double* x, cudaStream_t s) {
-  int rc = dg_launch_apply_f64(m, m->p64, m->q64, &m->state->done, s);
-  if (rc) return rc;
-  const long long n = m->ndofs;
-  if (aligned16(x)) {
-    k_dot_pq<double, true><<<RED_LAUNCH>>>(m->p64, m->q64, n, m->partials, m->state);
-    k_update_xr<double, false, false, true, true><<<RED_LAUNCH>>>(x, m->r64, m->p64, m->q64,
-                                                                  nullptr, n, m->partials,
-                                                                  m->state);
-  } else {
-    k_dot_pq<double, false><<<RED_LAUNCH>>>(m->p64, m->q64, n, m->partials, m->state);
-    k_update_xr<double, false, false, false, true><<<RED_LAUNCH>>>(x, m->r64, m->p64, m->q64,
-                                                                   nullptr, n, m->partials,
-                                                                   m->state);
-  }
-  DG_CUDA(cudaGetLastError());
-  rc = dg_launch_kron_apply(m, m->r64, m->t64, nullptr, DG_KRON_FP64, s);
-  if (rc) return rc;
-  k_update_p<double, false, true><<<RED_LAUNCH>>>(m->p64, m->t64, nullptr, n, m->state);
   DG_CUDA(cudaGetLastError());
   return DG_OK;
 }
@@ -769,9 +750,8 @@ int cg_fp64(dg_mesh* m, const double* b, double* x, double rtol, int maxit, dg_c
       if (rc) return rc;
     }
     rc = run_graph(m, s, chunk_for(m), [&] {
-      return block ? launch_iteration_block(m, x, s)
-             : kron ? launch_iteration_kron(m, x, s)
-                    : launch_iteration<double>(m, x, m->r64, m->p64, m->q64, dinv, s);
+      return block || kron ? launch_iteration_blocks(m, x, kron, s)
+                           : launch_iteration<double>(m, x, m->r64, m->p64, m->q64, dinv, s);
     });
     if (rc) return rc;
     const DGCGState hs = *m->state_host;

@@ -26,14 +26,16 @@
 
 namespace dgk {
 
-template <int N, bool MODAL>
+// XL: FxLoad, or FxDirection inside a CG iteration (then x.begin() reads beta)
+template <int N, bool MODAL, typename XL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
-k_trace_fx(const double* __restrict__ x, long long* __restrict__ U, long long* __restrict__ TR,
+k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
            int* __restrict__ expU, long long cbeg, long long cend, const int* __restrict__ skip,
            const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   if (skip != nullptr && *skip) return;
   __shared__ long long smem[(FxSmem<N, T>::trace + 7) / 8];
+  x.begin();
   const long long c0 = cbeg + (long long)blockIdx.x * C;
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
   fx_trace_cells<N, MODAL, T>(x, U, TR, expU, c0, nblk, tab, smem);
@@ -61,8 +63,85 @@ k_cell_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long c0 = cbeg + (long long)blockIdx.x * C;
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
-  fx_cell_cells<N, MODAL, T>(xU, TR, expU, lineop, gam, expM, expG, y, c0, nblk, Nc, tab,
-                             reinterpret_cast<long long*>(smem_raw));
+  fx_cell_cells<N, MODAL, T>(xU, TR, expU, lineop, gam, expM, expG, FxStore{y}, c0, nblk, Nc,
+                             tab, reinterpret_cast<long long*>(smem_raw));
+}
+
+// Inside a CG iteration (Section 2.4) the passes take the vector work along.
+// With FP64 passes that was slower than separate kernels (they shared the FP64
+// pipe); the fixed-point passes leave that pipe idle, and the two vector kernels,
+// their traffic (40 B per DOF) and their launches go.  32^3 Q3 with Jacobi:
+// 236 -> 213 ms per solve (with the shorter pass 2).
+// Pass 1 of p = z + beta p, z = r, dinv r (PC) or M^-1 r already formed.
+template <bool PC>
+struct FxDirection {
+  double* p;
+  const double *z, *dinv;
+  const DGCGState* st;
+  double beta;
+  __device__ __forceinline__ void begin() { beta = st->beta; }
+  __device__ __forceinline__ double operator()(long long i) const {
+    const double v = fma(beta, p[i], PC ? dinv[i] * z[i] : z[i]);
+    p[i] = v;
+    return v;
+  }
+};
+
+// Pass 2 with <p, q> and alpha = rho / <p, q>: one partial per block, added by
+// the last block in a fixed order.
+template <int N, bool MODAL>
+__global__ void __launch_bounds__(Cfg<N>::THREADS, FxCellBlocks<N>::value)
+k_cell_dot_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
+              const int* __restrict__ expU, const FxPair* __restrict__ lineop,
+              const FxPair* __restrict__ gam, const int* __restrict__ expM,
+              const int* __restrict__ expG, const double* __restrict__ p, double* __restrict__ q,
+              long long ncells, int Nc, double* __restrict__ partials, DGCGState* st,
+              const __grid_constant__ DGTabX tab) {
+  constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
+  if (st->done) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ bool is_last;
+  const long long c0 = (long long)blockIdx.x * C;
+  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
+  double acc = 0.0;
+  fx_cell_cells<N, MODAL, T>(
+      xU, TR, expU, lineop, gam, expM, expG,
+      [&](long long i, double v) {
+        q[i] = v;
+        acc = fma(p[i], v, acc);
+      },
+      c0, nblk, Nc, tab, reinterpret_cast<long long*>(smem_raw));
+  __syncthreads();
+  double* rd = reinterpret_cast<double*>(smem_raw);
+  static_assert(FxSmem<N, T>::cell >= sizeof(double) * T, "reduction scratch");
+  rd[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = 0.0;
+    for (int i = threadIdx.x; i < T; i += 32) t += rd[i];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (threadIdx.x == 0) {
+      partials[blockIdx.x] = t;
+      __threadfence();
+      is_last = (atomicAdd(&st->ticket, 1u) == gridDim.x - 1);
+    }
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const double tot = last_block_total<T>(partials, (int)gridDim.x, rd);
+  if (threadIdx.x == 0) {
+    st->pq = tot;
+    if (!(tot > 0.0) || !isfinite(tot)) {
+      st->breakdown = 1;
+      st->done = 1;
+      st->ru_skip = 1;
+    } else {
+      st->alpha = st->rho / tot;
+    }
+    st->ticket = 0u;
+  }
 }
 
 // Line operators, face coefficients and their exponents from K and h gamma: one
@@ -189,8 +268,8 @@ struct FixedF {
     long long* U = reinterpret_cast<long long*>(m->U64);
     long long* TR = reinterpret_cast<long long*>(m->TR64);
     if (pass == 1)
-      k_trace_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, 0, s>>>(x, U, TR, m->expU, cbeg, cend, skip,
-                                                             m->tabX);
+      k_trace_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, 0, s>>>(FxLoad{x}, U, TR, m->expU, cbeg,
+                                                             cend, skip, m->tabX);
     else
       k_cell_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, SMEM, s>>>(
           MODAL ? (const void*)U : (const void*)x, TR, m->expU, m->lineopX, m->gamX, m->expM,
@@ -205,6 +284,32 @@ struct FixedF {
   }
 };
 
+// q = A p with p = z + beta p and alpha, on the mesh's solver state.
+template <int N>
+struct FixedCgF {
+  template <bool MODAL, bool PC>
+  static cudaError_t go(const dg_mesh* m, const double* z, const double* dinv, double* p,
+                        double* q, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
+    long long* U = reinterpret_cast<long long*>(m->U64);
+    long long* TR = reinterpret_cast<long long*>(m->TR64);
+    k_trace_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, 0, s>>>(
+        FxDirection<PC>{p, z, dinv, m->state, 0.0}, U, TR, m->expU, 0, m->ncells,
+        &m->state->done, m->tabX);
+    k_cell_dot_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, FixedF<N>::SMEM, s>>>(
+        MODAL ? (const void*)U : (const void*)p, TR, m->expU, m->lineopX, m->gamX, m->expM,
+        m->expG, p, q, m->ncells, m->N, m->partials_cells, m->state, m->tabX);
+    return cudaGetLastError();
+  }
+  template <typename T>
+  static cudaError_t run(const dg_mesh* m, const double* z, const double* dinv, double* p,
+                         double* q, cudaStream_t s) {
+    if (m->nodal_op)
+      return dinv ? go<false, true>(m, z, dinv, p, q, s) : go<false, false>(m, z, dinv, p, q, s);
+    return dinv ? go<true, true>(m, z, dinv, p, q, s) : go<true, false>(m, z, dinv, p, q, s);
+  }
+};
+
 template <int N>
 struct FixedPrepF {
   template <typename T>
@@ -215,6 +320,12 @@ struct FixedPrepF {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_cell_fx<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)FixedF<N>::SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_cell_dot_fx<N, true>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FixedF<N>::SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_cell_dot_fx<N, false>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FixedF<N>::SMEM);
     return e;
   }
 };
@@ -262,5 +373,12 @@ int dg_launch_fixed_apply(const dg_mesh* m, bool modal, const double* x, double*
   rc = dg_launch_fixed_pass(m, modal, 2, x, y, 0, m->ncells, skip, s);
   if (rc) return rc;
   dg_timing_mark(m, 2, s);
+  return DG_OK;
+}
+
+int dg_launch_fixed_cg(const dg_mesh* m, const double* z, const double* dinv, double* p,
+                       double* q, cudaStream_t s) {
+  cudaError_t e = dgk::dispatch_n<double, dgk::FixedCgF>(m->n, m, z, dinv, p, q, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "CG operator (fp64) launch");
   return DG_OK;
 }

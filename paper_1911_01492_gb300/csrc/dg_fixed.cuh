@@ -117,13 +117,15 @@ __device__ __forceinline__ long long fx_from_double(double x, int k, int E) {
   return e > (k < 0 ? -k : 0) ? __double2ll_rn(s) : 0;
 }
 
-// v 2^k
-__device__ __forceinline__ double fx_to_double(long long v, int k) {
-  const double d = (double)v;
+// d 2^k, v 2^k
+__device__ __forceinline__ double fx_scale(double d, int k) {
   if (k > 900 || k < -900) return scalbn(d, k);
-  return v != 0 ? __hiloint2double(__double2hiint(d) + (int)((unsigned)k << 20),
-                                   __double2loint(d))
-                : 0.0;
+  return d != 0.0 ? __hiloint2double(__double2hiint(d) + (int)((unsigned)k << 20),
+                                     __double2loint(d))
+                  : 0.0;
+}
+__device__ __forceinline__ double fx_to_double(long long v, int k) {
+  return fx_scale((double)v, k);
 }
 
 // magnitude's high word, for fx_bits of a maximum
@@ -232,13 +234,24 @@ __device__ __forceinline__ void fx_store_traces(const DGTabX& t, const long long
   tr[(4 * dir + 3) * N2 + pt] = b - a;
 }
 
+// Where pass 1 takes the vector from and pass 2 puts the result: functions of
+// the DOF index, called once per DOF by the thread that owns it there.
+struct FxLoad {
+  const double* x;
+  __device__ __forceinline__ void begin() const {}
+  __device__ __forceinline__ double operator()(long long i) const { return x[i]; }
+};
+struct FxStore {
+  double* y;
+  __device__ __forceinline__ void operator()(long long i, double v) const { y[i] = v; }
+};
+
 // Pass 1 over the cells c0 .. c0+nblk-1 (nblk <= CPB) by the calling block of
 // BT threads (at least CPB n^2; the others only take part in the barriers).
 // smem: FxSmem<N, BT>::trace bytes.  Every thread of the block calls it; a
 // barrier must follow before smem is used again.
-template <int N, bool MODAL, int BT>
-__device__ __forceinline__ void fx_trace_cells(const double* __restrict__ x,
-                                               long long* __restrict__ U,
+template <int N, bool MODAL, int BT, typename XL>
+__device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restrict__ U,
                                                long long* __restrict__ TR,
                                                int* __restrict__ expU, long long c0, int nblk,
                                                const DGTabX& tab, long long* smem) {
@@ -260,7 +273,7 @@ __device__ __forceinline__ void fx_trace_cells(const double* __restrict__ x,
   unsigned big = 0;
 #pragma unroll
   for (int l = 0; l < N; ++l) {
-    xv[l] = active ? x[c * N3 + l * N2 + q * N + p] : 0.0;
+    xv[l] = active ? x(c * N3 + l * N2 + q * N + p) : 0.0;
     const unsigned m = fx_abs_hi(xv[l]);
     big = m > big ? m : big;
   }
@@ -341,12 +354,11 @@ __device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
 // Pass 2 over the cells c0 .. c0+nblk-1, called like pass 1; smem:
 // FxSmem<N, BT>::cell bytes.  xU: MODAL: the point values of pass 1 (integers);
 // otherwise the vector itself.
-template <int N, bool MODAL, int BT>
+template <int N, bool MODAL, int BT, typename YS>
 __device__ __forceinline__ void fx_cell_cells(
     const void* __restrict__ xU, const long long* __restrict__ TR, const int* __restrict__ expU,
     const FxPair* __restrict__ lineop, const FxPair* __restrict__ gam,
-    const int* __restrict__ expM, const int* __restrict__ expG, double* __restrict__ y,
-    long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
+    const int* __restrict__ expM, const int* __restrict__ expG, YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
   constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC;
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -523,7 +535,7 @@ __device__ __forceinline__ void fx_cell_cells(
     if (active) {  // written from the z-lines: consecutive lanes, consecutive words
 #pragma unroll
       for (int e = 0; e < N; ++e)
-        y[c * N3 + e * N2 + q * N + p] = __longlong_as_double(sr[e * SZ + q * SY + p]);
+        y(c * N3 + e * N2 + q * N + p, __longlong_as_double(sr[e * SZ + q * SY + p]));
     }
     return;
   }
@@ -557,7 +569,7 @@ __device__ __forceinline__ void fx_cell_cells(
   if (active) {
 #pragma unroll
     for (int l = 0; l < N; ++l)
-      y[c * N3 + l * N2 + q * N + p] = bad ? qnan : fx_to_double(u[l], eout - 1 - up);
+      y(c * N3 + l * N2 + q * N + p, bad ? qnan : fx_to_double(u[l], eout - 1 - up));
   }
 }
 

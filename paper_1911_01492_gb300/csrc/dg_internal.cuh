@@ -156,6 +156,11 @@ struct dg_mesh {
   double* kron64;
   float* kron32;
   bool has_kron;
+  // the same for the FP64 application in fixed point: eigenbases [c][3][n][n] in
+  // the Legendre and in the point basis, reciprocal eigenvalue sums [c][n^3]
+  FxPair *kronX, *kronNX;
+  double* kronW;
+  bool has_kron_x, has_kron_nx;
   // scaled Gauss-point basis (DG_CG_NODAL, dg_nodal.cu): its 1D tables, the
   // line operators and Jacobi diagonal of Q A Q^T (formed on first use after
   // the coefficient is set) and the solve's b and x in that basis
@@ -247,6 +252,9 @@ int dg_launch_fixed_pass(const dg_mesh* m, bool modal, int pass, const double* x
                          long long cbeg, long long cend, const int* skip, cudaStream_t s);
 int dg_launch_fixed_apply(const dg_mesh* m, bool modal, const double* x, double* y,
                           const int* skip, cudaStream_t s);
+// inside a CG iteration: p = z + beta p (z = dinv z with dinv), q = A p, alpha
+int dg_launch_fixed_cg(const dg_mesh* m, const double* z, const double* dinv, double* p,
+                       double* q, cudaStream_t s);
 // one pass of the FP32 operator over the cells [cbeg, cend)
 int dg_launch_pass_f32(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
                        long long cend, cudaStream_t s);
