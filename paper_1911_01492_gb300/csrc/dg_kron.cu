@@ -16,12 +16,12 @@
 //   eigen-decomposition by cyclic Jacobi rotations; stores Q_d and lambda_d in
 //   FP64 and FP32 ([c][ Q_x Q_y Q_z (row-major [i][j], column j the j-th
 //   eigenvector) | l_x l_y l_z ]).
-// k_kron_apply: z = M^-1 r for a group of cells per block (one thread per
+// k_kron_apply (FP32): z = M^-1 r for a group of cells per block (one thread per
 //   plane of lines, the 1D factor in registers, in place in shared memory),
 //   <z, r> formed in the scaling phase and reduced by the last block.
-#include "dg_internal.cuh"
-
-#include "dg_apply_impl.cuh"
+// k_kron_apply_fx (FP64): the same with the contractions in block fixed point
+//   (dg_fixed.cuh), one thread per line.
+#include "dg_fixed.cuh"
 
 namespace dgk {
 namespace {
@@ -243,10 +243,7 @@ __device__ __forceinline__ T kron_solve_cells(T* sw, const T* sq, int nblk) {
         T a = q[0][k] * v[0];
 #pragma unroll
         for (int l = 1; l < N; ++l) a = fma(q[l][k], v[l], a);
-        if constexpr (sizeof(T) == 4)
-          u[k] = a * __fdividef(1.0f, lxy + lam[2 * N + k]);
-        else
-          u[k] = a / (lxy + lam[2 * N + k]);
+        u[k] = a * __fdividef(1.0f, lxy + lam[2 * N + k]);
         acc = fma(a, u[k], acc);
       }
 #pragma unroll
@@ -317,6 +314,157 @@ k_kron_apply(const T* __restrict__ KD, const T* __restrict__ r, T* __restrict__ 
   kron_finish<NT, MODE>(part, partials, st, rd);
 }
 
+// z = M^-1 r in FP64 vectors, contractions in block fixed point: in FP64 the
+// 6n multiply-adds and the division per DOF kept the FP64 pipe busy for
+// 6n + 12 instructions (0.94 ms at 48^3 Q4); here they are 6n integer
+// products of 12 issue cycles each and the divisions are done once,
+// in k_kron_fix.  KX: the 1D factors [c][x,y,z][i][j] 2^60; winv: 1 / (lx + ly
+// + lz) [c][i][j + n l].  The transformed residual t is scaled to w t with the
+// largest magnitude of the cell again below 2^S0, whatever the spread of the
+// eigenvalues; <z, r> = sum w t^2 accumulates in 64-bit integers per thread.
+template <int N, int MODE>
+__global__ void __launch_bounds__(Cfg<N>::THREADS)
+k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
+                const double* __restrict__ r, double* __restrict__ z, double* __restrict__ p,
+                long long ncells, double* __restrict__ partials, DGCGState* st) {
+  constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
+  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC, S0 = FxScale<N>::S0;
+  if (MODE != 1 && st->done) return;
+  __shared__ long long s[C * SC];
+  __shared__ FxPair sq[C * 3 * N2];
+  __shared__ double rd[T];
+  __shared__ unsigned slots[2][FxSmem<N, T>::NS];
+  const long long c0 = (long long)blockIdx.x * C;
+  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int pp = pt % N, qq = pt / N;
+  const bool active = lc < nblk;
+  const long long c = c0 + (active ? lc : 0);
+  long long* sc = s + lc * SC;
+  const FxPair* Q = sq + lc * 3 * N2;
+  double rv[N], w[N];
+#pragma unroll
+  for (int l = 0; l < N; ++l) rv[l] = active ? r[c * N3 + l * N2 + pt] : 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) w[i] = winv[c * N3 + i * N2 + pt];
+  for (int i = threadIdx.x; i < nblk * 3 * N2; i += T) sq[i] = KX[c0 * 3 * N2 + i];
+  if (threadIdx.x < FxSmem<N, T>::NS) slots[0][threadIdx.x] = slots[1][threadIdx.x] = 0;
+  unsigned big = 0;
+#pragma unroll
+  for (int l = 0; l < N; ++l) big = max(big, fx_abs_hi(rv[l]));
+  __syncthreads();
+  const int E = fx_exponent(fx_cell_max<N, T>(big, lc, slots[0]));
+  long long v[N], u[N];
+#pragma unroll
+  for (int l = 0; l < N; ++l) v[l] = fx_from_double(rv[l], S0 - E, E);
+  // u[k] = sum_i Q[i][k] v[i] (tr) or sum_i Q[k][i] v[i]
+  auto line = [&](int d, bool tr) {
+    FxVal e[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) e[i] = fx_split(v[i]);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      FxAcc A = fx_zero();
+#pragma unroll
+      for (int i = 0; i < N; ++i) fx_mac(A, Q[d * N2 + (tr ? i * N + k : k * N + i)], e[i]);
+      u[k] = fx_value(A);
+    }
+  };
+  auto put = [&](int at, int step) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) sc[at + i * step] = u[i];
+    __syncthreads();
+  };
+  auto get = [&](int at, int step) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = sc[at + i * step];
+  };
+  const int zl = qq * SY + pp, yl = qq * SZ + pp, xl = qq * SZ + pp * SY;
+  line(2, true);  // z-lines
+  put(zl, SZ);
+  get(yl, SY);
+  line(1, true);
+  put(yl, SY);
+  get(xl, 1);
+  line(0, true);
+  // w t: mantissa of w in [2^59, 2^60), its exponent with the magnitude of t
+  unsigned top = 0;
+  int ew[N];
+  FxVal m[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const long long b = __double_as_longlong(w[i]);
+    ew[i] = (int)(b >> 52) - 1022;
+    m[i] = fx_split(((b & 0xfffffffffffffll) | 0x10000000000000ll) << 7);
+    // biased to stay positive
+    top = max(top, (unsigned)(fx_bits(fx_mag_hi(u[i])) + ew[i] + 4096));
+  }
+  const int B = (int)fx_cell_max<N, T>(top, lc, slots[1]) - 4096;
+  FxAcc dot = {0, 0};
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    FxAcc A = fx_zero();
+    const FxPair t = fx_pair(u[i]);
+    fx_mac(A, t, m[i]);
+    const int sh = ew[i] + S0 - B;
+    v[i] = fx_shift(fx_value(A), sh < -63 ? -63 : sh);
+    fx_mac(dot, t, fx_split(v[i]));
+  }
+  // v stands for v 2^(E - S0 + B - S0); <z, r> sums t v
+  const bool bad = E >= FX_NAN;
+  const double qnan = __longlong_as_double(0x7ff8000000000000ll);
+  const int ez = E - 2 * S0 + B;
+  const double acc = !active ? 0.0
+                     : bad   ? qnan
+                             : fx_scale(fma((double)dot.m, 0x1p-30, (double)dot.h),
+                                        ez + E - S0 + 60);
+  line(0, false);
+  put(xl, 1);
+  get(yl, SY);
+  line(1, false);
+  put(yl, SY);
+  get(zl, SZ);
+  line(2, false);
+  if (active) {
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+      const double zv = bad ? qnan : fx_to_double(u[l], ez);
+      z[c * N3 + l * N2 + pt] = zv;
+      if (MODE == 1) p[c * N3 + l * N2 + pt] = zv;
+    }
+  }
+  const double part = block_total<T>(acc, rd);
+  kron_finish<T, MODE>(part, partials, st, rd);
+}
+
+// Factors of the FP64 application from the FP64 ones: the eigenbases as
+// fixed-point pairs, one reciprocal per DOF.  One thread per DOF.
+template <int N>
+__global__ void k_kron_fix(const double* __restrict__ K64, FxPair* __restrict__ KX,
+                           double* __restrict__ winv, long long ncells) {
+  constexpr int N2 = N * N, N3 = N * N * N, KS = 3 * N2 + 3 * N;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= ncells * N3) return;
+  const long long c = t / N3;
+  const int k = (int)(t - c * N3);
+  const double* L = K64 + c * KS + 3 * N2;
+  const int i = k / N2, j = k % N, l = (k / N) % N;
+  winv[t] = 1.0 / (L[i] + L[N + j] + L[2 * N + l]);
+  for (int e = k; e < 3 * N2; e += N3)
+    KX[c * 3 * N2 + e] = fx_pair(__double2ll_rn(K64[c * KS + e] * 0x1p60));
+}
+
+template <int N>
+struct KronFixF {
+  template <typename T>
+  static cudaError_t run(const double* K64, FxPair* KX, double* winv, long long ncells,
+                         cudaStream_t s) {
+    const long long n = ncells * N * N * N;
+    k_kron_fix<N><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(K64, KX, winv, ncells);
+    return cudaGetLastError();
+  }
+};
+
 // The factors in the scaled Gauss-point basis: per cell and direction
 // Qhat = q Q with q[a][i] = sqrt(w_a) L_i(xi_a) (orthogonal), the eigenvalues
 // unchanged: Q M Q^T is again a Kronecker sum with these eigenbases.  One
@@ -376,23 +524,22 @@ struct KronApplyF {
   template <typename T>
   static cudaError_t run(const dg_mesh* m, const void* r, void* z, void* p, int mode,
                          cudaStream_t s) {
-    using K64 = KronCfg<N, double>;
     using K32 = KronCfg<N, float>;
     // inside a solve in the scaled Gauss-point basis: the rotated factors
-    const double* f64 = m->nodal_op ? m->kronN64 : m->kron64;
+    const FxPair* fx = m->nodal_op ? m->kronNX : m->kronX;
     const float* f32 = m->nodal_op ? m->kronN32 : m->kron32;
-    const unsigned b64 = (unsigned)((m->ncells + K64::C - 1) / K64::C);
+    const unsigned bx = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
     const unsigned b32 = (unsigned)((m->ncells + K32::C - 1) / K32::C);
     switch (mode) {
       case DG_KRON_FP64:
-        k_kron_apply<N, double, 0><<<b64, K64::THREADS, 0, s>>>(
-            f64, (const double*)r, (double*)z, nullptr, m->ncells, m->partials_cells,
+        k_kron_apply_fx<N, 0><<<bx, Cfg<N>::THREADS, 0, s>>>(
+            fx, m->kronW, (const double*)r, (double*)z, nullptr, m->ncells, m->partials_cells,
             m->state);
         break;
       case DG_KRON_FP64_INIT:
-        k_kron_apply<N, double, 1><<<b64, K64::THREADS, 0, s>>>(
-            f64, (const double*)r, (double*)z, (double*)p, m->ncells, m->partials_cells,
-            m->state);
+        k_kron_apply_fx<N, 1><<<bx, Cfg<N>::THREADS, 0, s>>>(
+            fx, m->kronW, (const double*)r, (double*)z, (double*)p, m->ncells,
+            m->partials_cells, m->state);
         break;
       default:
         k_kron_apply<N, float, 2><<<b32, K32::THREADS, 0, s>>>(
@@ -445,8 +592,26 @@ int dg_ensure_kron_nodal(dg_mesh* m, cudaStream_t s) {
   return DG_OK;
 }
 
+// The fixed-point factors of the FP64 application in the current basis.
+static int ensure_kron_fx(dg_mesh* m, cudaStream_t s) {
+  bool& has = m->nodal_op ? m->has_kron_nx : m->has_kron_x;
+  FxPair*& X = m->nodal_op ? m->kronNX : m->kronX;
+  if (has) return DG_OK;
+  const size_t nq = (size_t)(3 * m->n * m->n) * (size_t)m->ncells;
+  if (X == nullptr) DG_CUDA(cudaMalloc((void**)&X, sizeof(FxPair) * nq));
+  if (m->kronW == nullptr)
+    DG_CUDA(cudaMalloc((void**)&m->kronW, sizeof(double) * (size_t)m->ndofs));
+  cudaError_t e = dgk::dispatch_n<double, dgk::KronFixF>(
+      m->n, (const double*)(m->nodal_op ? m->kronN64 : m->kron64), X, m->kronW, m->ncells, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "Kronecker cell blocks: fixed-point factors");
+  has = true;
+  return DG_OK;
+}
+
 int dg_launch_kron_apply(const dg_mesh* m, const void* r, void* z, void* p, int mode,
                          cudaStream_t s) {
+  if (mode == DG_KRON_FP64_INIT)  // runs before the iterations are captured
+    if (int rc = ensure_kron_fx(const_cast<dg_mesh*>(m), s)) return rc;
   cudaError_t e = dgk::dispatch_n<double, dgk::KronApplyF>(m->n, m, r, z, p, mode, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "Kronecker cell blocks: apply");
   return DG_OK;
