@@ -68,7 +68,6 @@ struct AccF {
   }
   __device__ double block_total();
 };
-__device__ __forceinline__ void merge(AccD& a, const AccD& b) { a.s += b.s; }
 __device__ __forceinline__ void merge(AccF& a, const AccF& b) {
   float s, t;
   two_sum(a.hi, b.hi, s, t);
@@ -92,11 +91,17 @@ __device__ __forceinline__ void grid_stride4(long long n, F&& f) {
   for (; i < n; i += S) f(i, 0);
 }
 
+// Accumulators per thread: four in FP32 (dependency chains), one in FP64, where
+// the pipe's rate leaves no latency to hide and every merge costs a slot.
+template <typename A> struct Lanes { static constexpr int value = 4; };
+template <> struct Lanes<AccD> { static constexpr int value = 1; };
 template <typename A>
 __device__ __forceinline__ A merge4(A (&a)[4]) {
-  merge(a[0], a[1]);
-  merge(a[2], a[3]);
-  merge(a[0], a[2]);
+  if constexpr (Lanes<A>::value == 4) {
+    merge(a[0], a[1]);
+    merge(a[2], a[3]);
+    merge(a[0], a[2]);
+  }
   return a[0];
 }
 
@@ -104,15 +109,21 @@ template <typename T> struct AccOf;
 template <> struct AccOf<double> { using type = AccD; };
 template <> struct AccOf<float> { using type = AccF; };
 
+// The threads' sums go through shared memory to one warp, eight each, then a
+// shuffle tree: 13 FP64 instructions per block.  Shuffle trees in all eight
+// warps were 45, which the FP64 pipe (one per 64 cycles) makes 6 us of a
+// kernel with eight blocks per SM.
 __device__ double AccD::block_total() {
-  __shared__ double sw[DG_RED_THREADS / 32];
-  double v = warp_sum(s);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __shared__ double sw[DG_RED_THREADS];
   __syncthreads();
-  if (l == 0) sw[w] = v;
+  sw[threadIdx.x] = s;
   __syncthreads();
   double r = 0.0;
-  if (threadIdx.x < 32) r = warp_sum((l < DG_RED_THREADS / 32) ? sw[l] : 0.0);
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int i = 0; i < DG_RED_THREADS / 32; ++i) r += sw[threadIdx.x + 32 * i];
+    r = warp_sum(r);
+  }
   return r;
 }
 
@@ -194,6 +205,7 @@ k_init(const T* __restrict__ b, const T* __restrict__ q, T* __restrict__ r, T* _
     T zi = ri;
     if constexpr (PC) zi = dinv[i] * ri;
     p[i] = zi;
+    j &= Lanes<A>::value - 1;
     ar[j].add_prod(ri, ri);
     ab[j].add_prod(b[i], b[i]);
     az[j].add_prod(zi, ri);
@@ -259,7 +271,7 @@ k_dot_pq(const T* __restrict__ p, const T* __restrict__ q, long long n, double* 
       for (int u = 0; u < 2; ++u) {
         if (u == 1 && !two) break;
 #pragma unroll
-        for (int c = 0; c < W; ++c) a4[(u * W + c) & 3].add_prod(ps[u][c], qs[u][c]);
+        for (int c = 0; c < W; ++c) a4[(u * W + c) & (Lanes<A>::value - 1)].add_prod(ps[u][c], qs[u][c]);
       }
     }
     tail = nv * W;
@@ -336,7 +348,7 @@ k_update_xr(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
         if (u == 1 && !two) break;
 #pragma unroll
         for (int c = 0; c < W; ++c) {
-          const int j = (u * W + c) & 3;
+          const int j = (u * W + c) & (Lanes<A>::value - 1);
           xs[u][c] = fma(a, ps[u][c], xs[u][c]);
           rs[u][c] = fma(-a, qs[u][c], rs[u][c]);
           a4[j].add_prod(rs[u][c], rs[u][c]);
@@ -466,8 +478,8 @@ k_refine_r(const double* __restrict__ b, const double* __restrict__ q, double* _
     const double ri = b[i] - q[i];
     r[i] = ri;
     r32[i] = (float)ri;
-    a4[j].add_prod(ri, ri);
-    if constexpr (PC) z4[j].add_prod(dinv[i] * ri, ri);
+    a4[0].add_prod(ri, ri);
+    if constexpr (PC) z4[0].add_prod(dinv[i] * ri, ri);
   });
   constexpr int K = PC ? 2 : 1;
   AccD acc[K];
@@ -502,8 +514,8 @@ k_residual(const double* __restrict__ b, const double* __restrict__ q, double* _
   grid_stride4(n, [&](long long i, int j) {
     const double ri = b[i] - q[i];
     r[i] = ri;
-    ar[j].add_prod(ri, ri);
-    ab[j].add_prod(b[i], b[i]);
+    ar[0].add_prod(ri, ri);
+    ab[0].add_prod(b[i], b[i]);
   });
   AccD acc[2] = {merge4(ar), merge4(ab)};
   double tot[2];
