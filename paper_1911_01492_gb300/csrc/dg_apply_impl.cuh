@@ -83,6 +83,13 @@ struct Cfg {
   static constexpr int THREADS = CPB * N * N;
 };
 
+// Shared-memory strides of a cell's n x n x n values: with an odd row length the
+// x- and y-lines of the lanes of a warp start on different banks.
+template <int N>
+struct LinePad {
+  static constexpr int SY = N + (N % 2 == 0 ? 1 : 0), SZ = N * SY, SC = N * SZ;
+};
+
 // ---------------------------------------------------------------------------
 // 1D line contractions with the parity split (H = N/2 mirror pairs a, N-1-a;
 // for odd N the middle point m = N/2 sits at xi = 1/2).
@@ -374,7 +381,8 @@ struct ZFromGlobal {
 // (x-mode p, y-mode q of cell lc); a kernel that produces those values itself
 // (a direction update, a load from global memory) passes its own loader and
 // needs no barrier between producing them and the first contraction.
-template <int N, typename T, int MODE, typename ZL = ZFromShared>
+// SY, SZ: shared-memory strides of s along y and z (see LinePad).
+template <int N, typename T, int MODE, typename ZL = ZFromShared, int SY = N, int SZ = N * N>
 __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm,
                                            T* __restrict__ TR, long long c0, int nblk,
                                            const DGTab<T>& tab, T* s, T* sx,
@@ -385,7 +393,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
   const int t2 = threadIdx.x - lc * N2;
   const int p = t2 % N, q = t2 / N;
   const bool active = lc < nblk;
-  T* sc = s + lc * N3;
+  T* sc = s + lc * (N * SZ);
   const long long c = c0 + lc;
 
   // along z: thread owns (i = p, j = q)
@@ -394,17 +402,17 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
     zload.template operator()<N, T>(sc, lc, p, q, v);
     b_fwd<N>(tab, v, u);
 #pragma unroll
-    for (int e = 0; e < N; ++e) sc[e * N2 + q * N + p] = u[e];
+    for (int e = 0; e < N; ++e) sc[e * SZ + q * SY + p] = u[e];
   }
   __syncthreads();
   // along y: thread owns (i = p, e = q)
   if (active) {
     T v[N], u[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = sc[q * N2 + j * N + p];
+    for (int j = 0; j < N; ++j) v[j] = sc[q * SZ + j * SY + p];
     b_fwd<N>(tab, v, u);
 #pragma unroll
-    for (int b = 0; b < N; ++b) sc[q * N2 + b * N + p] = u[b];
+    for (int b = 0; b < N; ++b) sc[q * SZ + b * SY + p] = u[b];
   }
   __syncthreads();
   // along x: thread owns (b = p, e = q); X is modal in x, nodal in y and z
@@ -412,7 +420,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
   if (active) {
     T X[N], u[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) X[i] = sc[q * N2 + p * N + i];
+    for (int i = 0; i < N; ++i) X[i] = sc[q * SZ + p * SY + i];
     if (MODE != 2) {
       T* xm = (MODE == 0) ? Xm + c * N3 + q * N2 + p * N : sx + lc * N3 + q * N2 + p * N;
 #pragma unroll
@@ -444,7 +452,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
     b_fwd<N>(tab, X, u);
 #pragma unroll
     for (int a = 0; a < N; ++a) {
-      sc[q * N2 + p * N + a] = u[a];
+      sc[q * SZ + p * SY + a] = u[a];
       if (MODE == 0) U[c * N3 + q * N2 + p * N + a] = u[a];
     }
   }
@@ -457,10 +465,10 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
       T u[N];
       if (dir == 0) {
 #pragma unroll
-        for (int b = 0; b < N; ++b) u[b] = sc[q * N2 + b * N + p];
+        for (int b = 0; b < N; ++b) u[b] = sc[q * SZ + b * SY + p];
       } else {
 #pragma unroll
-        for (int e = 0; e < N; ++e) u[e] = sc[e * N2 + q * N + p];
+        for (int e = 0; e < N; ++e) u[e] = sc[e * SZ + q * SY + p];
       }
       T vm = tab.l0[0] * u[0], vp = tab.l1[0] * u[0];
       T gm = tab.dl0[0] * u[0], gp = tab.dl1[0] * u[0];
@@ -776,40 +784,6 @@ __global__ void k_face_weights(const double* __restrict__ gh, T* __restrict__ FW
 }
 
 
-// Launch both passes for one precision.  U, X, TR: workspaces of the mesh.
-template <int N, typename T>
-cudaError_t launch_apply_n(const dg_mesh* m, const T* x, T* y, T* U, T* X, T* TR, const T* kt,
-                           const T* fw, long long ncells, int Nc, const int* skip,
-                           const DGTab<T>& tab, cudaStream_t s) {
-  const unsigned blocks = (unsigned)((ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
-  const size_t s1 = trace_smem<N, T>(), s2 = cell_smem<N, T>();
-  dg_timing_mark(m, 0, s);
-  k_trace<N, T><<<blocks, Cfg<N>::THREADS, s1, s>>>(x, U, X, TR, 0, ncells, skip, tab);
-  dg_timing_mark(m, 1, s);
-  k_cell<N, T><<<blocks, Cfg<N>::THREADS, s2, s>>>(U, X, TR, kt, fw, y, 0, ncells, Nc, skip, tab);
-  dg_timing_mark(m, 2, s);
-  return cudaGetLastError();
-}
-
-// One pass over the cells [cbeg, cend) (pipelined host-buffer apply).
-// Pass 1 reads x and writes U, X, TR of those cells only; pass 2 reads the
-// traces of their face neighbours, so it may run on a range only after pass 1
-// has run on every neighbour of the range.
-template <int N, typename T>
-cudaError_t launch_pass_n(const dg_mesh* m, int pass, const T* x, T* y, T* U, T* X, T* TR,
-                          const T* kt, const T* fw, long long cbeg, long long cend, int Nc,
-                          const DGTab<T>& tab, cudaStream_t s) {
-  if (cend <= cbeg) return cudaSuccess;
-  const unsigned blocks = (unsigned)((cend - cbeg + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
-  if (pass == 1)
-    k_trace<N, T><<<blocks, Cfg<N>::THREADS, trace_smem<N, T>(), s>>>(x, U, X, TR, cbeg, cend,
-                                                                       nullptr, tab);
-  else
-    k_cell<N, T><<<blocks, Cfg<N>::THREADS, cell_smem<N, T>(), s>>>(U, X, TR, kt, fw, y, cbeg,
-                                                                     cend, Nc, nullptr, tab);
-  return cudaGetLastError();
-}
-
 template <int N, typename T>
 cudaError_t launch_trace_n(const T* x, T* U, T* X, T* TR, long long ncells, const DGTab<T>& tab,
                            cudaStream_t s) {
@@ -833,26 +807,6 @@ cudaError_t dispatch_n(int n, Args... args) {
     default: return cudaErrorInvalidValue;
   }
 }
-
-template <int N>
-struct ApplyF {
-  template <typename T>
-  static cudaError_t run(const dg_mesh* m, const T* x, T* y, T* U, T* X, T* TR, const T* kt,
-                         const T* fw, long long ncells, int Nc, const int* skip,
-                         const DGTab<T>* tab, cudaStream_t s) {
-    return launch_apply_n<N, T>(m, x, y, U, X, TR, kt, fw, ncells, Nc, skip, *tab, s);
-  }
-};
-
-template <int N>
-struct PassF {
-  template <typename T>
-  static cudaError_t run(const dg_mesh* m, int pass, const T* x, T* y, T* U, T* X, T* TR,
-                         const T* kt, const T* fw, long long cbeg, long long cend, int Nc,
-                         const DGTab<T>* tab, cudaStream_t s) {
-    return launch_pass_n<N, T>(m, pass, x, y, U, X, TR, kt, fw, cbeg, cend, Nc, *tab, s);
-  }
-};
 
 // Opt in to the dynamic shared memory the kernels use (above 48 KB for large n).
 template <int N>

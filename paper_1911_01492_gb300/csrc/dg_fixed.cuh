@@ -38,20 +38,13 @@ struct FxScale {
   static constexpr int S0 = N == 2 ? 58 : N == 3 ? 57 : N == 4 ? 57 : N <= 6 ? 56 : 55;
 };
 
-// shared-memory strides of a cell's n x n x n values (8-byte words): odd row
-// strides keep the x- and y-line accesses of 16 lanes on different banks
-template <int N>
-struct FxPad {
-  static constexpr int SY = N + (N % 2 == 0 ? 1 : 0), SZ = N * SY, SC = N * SZ;
-};
-
 // Shared memory of the two passes in a block of BT threads.
 template <int N, int BT>
 struct FxSmem {
   static constexpr int C = Cfg<N>::CPB;
   static constexpr int NS = (BT + N * N - 1) / (N * N);  // n^2 thread groups of the block
-  static constexpr size_t trace = 8 * C * FxPad<N>::SC + 4 * 2 * NS;
-  static constexpr size_t cell = 8 * 2 * C * FxPad<N>::SC + 8 * 6 * C + 4 * (7 * C + NS);
+  static constexpr size_t trace = 8 * C * LinePad<N>::SC + 4 * 2 * NS;
+  static constexpr size_t cell = 8 * 2 * C * LinePad<N>::SC + 8 * 6 * C + 4 * (7 * C + NS);
 };
 
 struct FxVal { int h, l; };  // a value v = h 2^30 + l
@@ -256,7 +249,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
                                                int* __restrict__ expU, long long c0, int nblk,
                                                const DGTabX& tab, long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
-  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
   const int p = pt % N, q = pt / N;
   const bool active = lc < nblk;
@@ -360,7 +353,7 @@ __device__ __forceinline__ void fx_cell_cells(
     const FxPair* __restrict__ lineop, const FxPair* __restrict__ gam,
     const int* __restrict__ expM, const int* __restrict__ expG, YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
-  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
   const int p = pt % N, q = pt / N;
   const bool active = lc < nblk;

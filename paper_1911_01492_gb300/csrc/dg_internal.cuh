@@ -141,8 +141,6 @@ struct dg_mesh {
   double* gh64;     // h gamma_F per face side        [c][6] (x-, x+, y-, y+, z-, z+)
   float* gh32;
   double* dgam;     // d gamma_F / d log Kbar_c       [c][6]
-  double* fw64;     // face-point weights W/2 and derivative weight  [c][6][2][n^2]
-  float* fw32;
   // Jacobi preconditioner: 1 / diag(A), formed on the first preconditioned solve
   double* diag64;
   double* dinv64;
@@ -184,7 +182,7 @@ struct dg_mesh {
 
   // apply workspaces: nodal values, x-modal/yz-nodal values, face traces
   double *U64, *X64, *TR64;
-  float *U32, *X32, *TR32;
+  float* TR32;
   // second set for the coefficient gradient (traces of v), lazily allocated
   double *U64b, *X64b, *TR64b;
   // host staging for dg_apply_host: device copies of x and y, copy-in,
@@ -242,7 +240,7 @@ int dg_cuda_fail(cudaError_t e, const char* what);
     if (e__ != cudaSuccess) return dg_cuda_fail(e__, #call); \
   } while (0)
 
-// launchers (dg_apply_f64.cu / dg_apply_f32.cu)
+// launchers (dg_apply_f64.cu, dg_mixed32.cu)
 // the FP64 operator in fixed point (dg_fixed.cu), for vectors of Legendre
 // coefficients (modal) or scaled point values: its coefficient data, one pass
 // (1: traces, 2: cell terms) over the cells [cbeg, cend), both passes
@@ -257,7 +255,7 @@ int dg_launch_fixed_cg(const dg_mesh* m, const double* z, const double* dinv, do
                        double* q, cudaStream_t s);
 // one pass of the FP32 operator over the cells [cbeg, cend)
 int dg_launch_pass_f32(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
-                       long long cend, cudaStream_t s);
+                       long long cend, const int* skip, cudaStream_t s);
 int dg_launch_apply_f64(const dg_mesh* m, const double* x, double* y, const int* skip,
                         cudaStream_t s);
 int dg_launch_apply_f32(const dg_mesh* m, const float* x, float* y, const int* skip,

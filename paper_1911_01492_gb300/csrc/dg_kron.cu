@@ -328,7 +328,7 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
                 const double* __restrict__ r, double* __restrict__ z, double* __restrict__ p,
                 long long ncells, double* __restrict__ partials, DGCGState* st) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
-  constexpr int SY = FxPad<N>::SY, SZ = FxPad<N>::SZ, SC = FxPad<N>::SC, S0 = FxScale<N>::S0;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC, S0 = FxScale<N>::S0;
   if (MODE != 1 && st->done) return;
   __shared__ long long s[C * SC];
   __shared__ FxPair sq[C * 3 * N2];

@@ -102,8 +102,8 @@ static cudaError_t dmalloc(P** p, size_t count) {
 }
 
 static void free_all(dg_mesh* m) {
-  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->fw64, m->fw32, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen,
-                  m->U64,  m->X64,  m->TR64, m->U32,  m->X32,  m->TR32, m->U64b,
+  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen,
+                  m->U64,  m->X64,  m->TR64, m->TR32, m->U64b,
                   m->X64b, m->TR64b, m->hx_dev, m->hy_dev, m->r64, m->p64, m->q64,
                   m->t64,  m->s64, m->d32,  m->r32, m->p32, m->q32, m->partials, m->state,
                   m->partials_cells};
@@ -162,8 +162,6 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->gh64, 6 * nc);
   if (e == cudaSuccess) e = dmalloc(&m->gh32, 6 * nc);
   if (e == cudaSuccess) e = dmalloc(&m->dgam, 6 * nc);
-  if (e == cudaSuccess) e = dmalloc(&m->fw64, ntr);
-  if (e == cudaSuccess) e = dmalloc(&m->fw32, ntr);
   if (e == cudaSuccess)
     e = dmalloc(&m->lineopX, (size_t)3 * n2 * (size_t)(m->n * (m->n + 1) / 2) * nc);
   if (e == cudaSuccess) e = dmalloc(&m->gamX, 6 * nc);
@@ -175,8 +173,6 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->U64, nd);
   if (e == cudaSuccess) e = dmalloc(&m->X64, nd);
   if (e == cudaSuccess) e = dmalloc(&m->TR64, ntr);
-  if (e == cudaSuccess) e = dmalloc(&m->U32, nd);
-  if (e == cudaSuccess) e = dmalloc(&m->X32, nd);
   if (e == cudaSuccess) e = dmalloc(&m->TR32, ntr);
   if (e != cudaSuccess) {
     int rc = dg_cuda_fail(e, "dg_create_mesh: device allocation");
@@ -306,8 +302,6 @@ extern "C" int dg_set_coefficient(dg_mesh* m, const double* K, void* stream) {
     const unsigned blocks = (unsigned)((m->ncells + 255) / 256);
     k_coef_faces<<<blocks, 256, 0, s>>>(m->kbar, m->gh64, m->gh32, m->dgam, m->N, m->h,
                                         m->dirichlet_mask);
-    dgk::k_face_weights<double><<<blocks, 256, 0, s>>>(m->gh64, m->fw64, m->N, m->n, m->tab64);
-    dgk::k_face_weights<float><<<blocks, 256, 0, s>>>(m->gh64, m->fw32, m->N, m->n, m->tab64);
     DG_CUDA(cudaGetLastError());
     if (!m->affine && !m->multilinear)
       if (int rc = dg_setup_fixed(m, K, s)) return rc;
@@ -416,7 +410,7 @@ extern "C" int dg_apply_host(const dg_mesh* mc, const void* x_host, void* y_host
                ? dg_launch_fixed_pass(m, true, p, (const double*)xd, (double*)yd, cells(sl),
                                       cells(sl + 1), nullptr, st)
                : dg_launch_pass_f32(m, p, (const float*)xd, (float*)yd, cells(sl),
-                                    cells(sl + 1), st);
+                                    cells(sl + 1), nullptr, st);
   };
   for (int sl = 0; sl < nslab; ++sl) {
     size_t off, bytes;

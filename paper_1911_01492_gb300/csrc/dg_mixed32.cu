@@ -320,32 +320,37 @@ k_dir32_bulk(const float* __restrict__ r, float* __restrict__ p, float* __restri
 // direction kernel, and <p, q> folded into the epilogue, where each z-line
 // thread still holds its z-line of p and of q in registers.  Registers are
 // capped at 64 for n <= 5 (eight blocks per SM).
+// DOT = false: the operator alone (dg_apply in FP32) on the cells [cbeg,
+// ncells), with traces from k_trace32; no solver state (skip: see k_trace32).
 // ---------------------------------------------------------------------------
-template <int N>
+template <int N, bool DOT>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, N <= 5 ? 8 : 1)
 k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
            const float* __restrict__ kt, const float* __restrict__ gh, float* __restrict__ qg,
-           long long ncells, int Nc, double* __restrict__ partials, DGCGState* st,
+           long long cbeg, long long ncells, int Nc, const int* __restrict__ skip,
+           double* __restrict__ partials, DGCGState* st,
            const __grid_constant__ DGTab<float> tab) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NT = Cfg<N>::THREADS;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   constexpr float S2 = 4.0f * N * N;  // 2 sigma, sigma = 2 (k+1)^2
   // nothing to do once done, at the cap, or with an FP64 refinement pending
-  if (st->done || st->iters >= st->maxit || st->ru_skip == 0) return;
+  if (DOT && (st->done || st->iters >= st->maxit || st->ru_skip == 0)) return;
+  if (!DOT && skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   F2* su = reinterpret_cast<F2*>(smem_raw);
-  F2* sx = su + C * N3;
-  F2* sr = sx + C * N3;
-  F2* sk = sr + C * N3;
-  __shared__ float rh[NT], rl[NT];
+  F2* sx = su + C * SC;
+  F2* sr = sx + C * SC;
+  F2* sk = sr + C * SC;
+  __shared__ float rh[DOT ? NT : 1], rl[DOT ? NT : 1];
   __shared__ bool is_last;
   __shared__ int sbase[3];
-  const long long c0 = (long long)blockIdx.x * (2 * C);
+  const long long c0 = cbeg + (long long)blockIdx.x * (2 * C);
   const int lc = threadIdx.x / N2;
   const int t2 = threadIdx.x - lc * N2;
   const int p = t2 % N, q = t2 / N;
   const long long ca = c0 + 2 * lc, cb = ca + 1;
   const bool va = ca < ncells, vb = cb < ncells;
-  const int o = lc * N3;
+  const int o = lc * SC;
   if (threadIdx.x == 0) {
     const unsigned cu = (unsigned)c0, n = (unsigned)Nc;
     sbase[0] = (int)(cu % n);
@@ -374,30 +379,33 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
     }
     b_fwd<N>(tab, preg, u);
 #pragma unroll
-    for (int e = 0; e < N; ++e) su[o + e * N2 + q * N + p] = u[e];
+    for (int e = 0; e < N; ++e) su[o + e * SZ + q * SY + p] = u[e];
   }
   __syncthreads();
   {  // y-lines: (i = p, e = q)
     F2 v[N], u[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = su[o + q * N2 + j * N + p];
+    for (int j = 0; j < N; ++j) v[j] = su[o + q * SZ + j * SY + p];
     b_fwd<N>(tab, v, u);
 #pragma unroll
-    for (int b = 0; b < N; ++b) su[o + q * N2 + b * N + p] = u[b];
+    for (int b = 0; b < N; ++b) su[o + q * SZ + b * SY + p] = u[b];
   }
   __syncthreads();
   {  // x-lines: (b = p, e = q); X (x-modal) kept in sx, nodal values in su
     F2 X[N], u[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) X[i] = su[o + q * N2 + p * N + i];
+    for (int i = 0; i < N; ++i) X[i] = su[o + q * SZ + p * SY + i];
 #pragma unroll
-    for (int i = 0; i < N; ++i) sx[o + q * N2 + p * N + i] = X[i];
+    for (int i = 0; i < N; ++i) sx[o + q * SZ + p * SY + i] = X[i];
     b_fwd<N>(tab, X, u);
 #pragma unroll
-    for (int a = 0; a < N; ++a) su[o + q * N2 + p * N + a] = u[a];
+    for (int a = 0; a < N; ++a) su[o + q * SZ + p * SY + a] = u[a];
   }
 #pragma unroll
-  for (int k = 0; k < N; ++k) sk[threadIdx.x + k * NT] = kreg[k];
+  for (int k = 0; k < N; ++k) {
+    const int t = threadIdx.x + k * NT;  // cell, then e, b, a
+    sk[t / N3 * SC + t % N3 / N2 * SZ + t % N2 / N * SY + t % N] = kreg[k];
+  }
   // cell coordinates of both lanes; interior flags as bits (face f: bit f for
   // lane a, bit 8 + f for lane b)
   int cxa = sbase[0] + 2 * lc, cya = sbase[1], cza = sbase[2];
@@ -453,8 +461,8 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   // neighbour face terms
 #pragma unroll
   for (int dir = 0; dir < 2; ++dir) {
-    const int base = (dir == 0) ? (q * N + p) : (q * N2 + p);
-    const int step = (dir == 0) ? N2 : N;
+    const int base = (dir == 0) ? (q * SY + p) : (q * SZ + p);
+    const int step = (dir == 0) ? SZ : SY;
     F2 u[N], r[N], kg[N];
 #pragma unroll
     for (int e = 0; e < N; ++e) u[e] = su[o + base + e * step];
@@ -505,7 +513,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
     __syncthreads();
   }
   {  // x-lines: (b = p, e = q); result x-modal, yz-nodal
-    const int base = q * N2 + p * N;
+    const int base = q * SZ + p * SY;
     F2 X[N], rr[N], R[N], g[N], kg[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -555,10 +563,10 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   {  // back along y: (i = p, e = q)
     F2 v[N], R[N];
 #pragma unroll
-    for (int b = 0; b < N; ++b) v[b] = sx[o + q * N2 + b * N + p];
+    for (int b = 0; b < N; ++b) v[b] = sx[o + q * SZ + b * SY + p];
     b_bwd<N>(tab, v, R);
 #pragma unroll
-    for (int j = 0; j < N; ++j) sx[o + q * N2 + j * N + p] = R[j];
+    for (int j = 0; j < N; ++j) sx[o + q * SZ + j * SY + p] = R[j];
   }
   __syncthreads();
   // back along z: (i = p, j = q), the thread's z-line of q: store it and fold
@@ -567,13 +575,14 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   {
     F2 v[N], R[N];
 #pragma unroll
-    for (int e = 0; e < N; ++e) v[e] = sx[o + e * N2 + q * N + p];
+    for (int e = 0; e < N; ++e) v[e] = sx[o + e * SZ + q * SY + p];
     b_bwd<N>(tab, v, R);
 #pragma unroll
     for (int l = 0; l < N; ++l) {
       const int idx = l * N2 + q * N + p;
       if (va) qg[ca * N3 + idx] = R[l].v.x;
       if (vb) qg[cb * N3 + idx] = R[l].v.y;
+      if constexpr (!DOT) continue;
       const F2 pr = preg[l] * R[l];
       const F2 er = fma(preg[l], R[l], -pr);  // preg R = pr + er exactly
       const F2 s1 = hi + pr;
@@ -583,6 +592,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
       lo = lo + (t1 + er);
     }
   }
+  if constexpr (!DOT) return;
   {  // combine the lanes
     float s1, t1;
     two_sum_f(hi.v.x, hi.v.y, s1, t1);
@@ -920,9 +930,9 @@ struct Mixed32F {
       k_dir32_bulk<N, false><<<gb, Dir32Bulk<N, false>::THREADS, Dir32Bulk<N, false>::SMEM, s>>>(
           rin, m->p32, m->TR32, dinv, m->ncells, m->state, limit, stall_now ? 1 : 0,
           m->tab32, m->tabN32);
-    k_cell32x2<N><<<blocks2, Cfg<N>::THREADS, sizeof(F2) * 4 * C * N3, s>>>(
-        m->p32, m->TR32, m->kt32, m->gh32, m->q32, m->ncells, m->N, m->partials_cells,
-        m->state, m->tab32);
+    k_cell32x2<N, true><<<blocks2, Cfg<N>::THREADS, sizeof(F2) * 4 * C * LinePad<N>::SC, s>>>(
+        m->p32, m->TR32, m->kt32, m->gh32, m->q32, 0, m->ncells, m->N, nullptr,
+        m->partials_cells, m->state, m->tab32);
     return cudaGetLastError();
   }
 };
@@ -935,9 +945,9 @@ struct PrepareMixed32F {
   static cudaError_t run(dg_mesh* m) {
     const long long ngroups = (m->ncells + Dir32Bulk<N, false>::G - 1) / Dir32Bulk<N, false>::G;
     {
-      cudaError_t e = cudaFuncSetAttribute(k_cell32x2<N>,
+      cudaError_t e = cudaFuncSetAttribute(k_cell32x2<N, true>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(sizeof(F2) * 4 * Cfg<N>::CPB * N * N * N));
+                                           (int)(sizeof(F2) * 4 * Cfg<N>::CPB * LinePad<N>::SC));
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_cell32x2_nd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(sizeof(F2) * 3 * Cfg<N>::CPB * N * N * N));
@@ -965,7 +975,83 @@ struct PrepareMixed32F {
   }
 };
 
+// ---------------------------------------------------------------------------
+// dg_apply in FP32.  Pass 1 writes the face traces only; pass 2 (k_cell32x2)
+// transforms x again in shared memory, which costs less than the nodal and
+// x-modal workspaces' 16 bytes per DOF of traffic, two cells per instruction.
+// 64^3 Q3: 220 us with the generic passes, 129 us now; 48^3 Q4 183 and 115 us.
+// ---------------------------------------------------------------------------
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::THREADS)
+k_trace32(const float* __restrict__ x, float* __restrict__ TR, long long cbeg, long long cend,
+          const int* __restrict__ skip, const __grid_constant__ DGTab<float> tab) {
+  constexpr int C = Cfg<N>::CPB, N3 = N * N * N;
+  if (skip != nullptr && *skip) return;
+  using LP = LinePad<N>;
+  __shared__ float s[C * LP::SC];
+  const long long c0 = cbeg + (long long)blockIdx.x * C;
+  const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
+  const ZFromGlobal<float> zl{x + c0 * N3};
+  trace_core<N, float, 2, ZFromGlobal<float>, LP::SY, LP::SZ>(nullptr, nullptr, TR, c0, nblk, tab,
+                                                              s, nullptr, zl);
+}
+
+// pass 1 or 2 of the FP32 operator over the cells [cbeg, cend)
+template <int N>
+struct Pass32F {
+  template <typename T>
+  static cudaError_t run(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
+                         long long cend, const int* skip, cudaStream_t s) {
+    constexpr int C = Cfg<N>::CPB, N3 = N * N * N;
+    if (cend <= cbeg) return cudaSuccess;
+    if (pass == 1)
+      k_trace32<N><<<(unsigned)((cend - cbeg + C - 1) / C), Cfg<N>::THREADS, 0, s>>>(
+          x, m->TR32, cbeg, cend, skip, m->tab32);
+    else
+      k_cell32x2<N, false><<<(unsigned)((cend - cbeg + 2 * C - 1) / (2 * C)), Cfg<N>::THREADS,
+                             sizeof(F2) * 4 * C * LinePad<N>::SC, s>>>(x, m->TR32, m->kt32, m->gh32, y, cbeg,
+                                                          cend, m->N, skip, nullptr, nullptr,
+                                                          m->tab32);
+    return cudaGetLastError();
+  }
+};
+
+template <int N>
+struct Prepare32F {
+  template <typename T>
+  static cudaError_t run() {
+    return cudaFuncSetAttribute(k_cell32x2<N, false>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(F2) * 4 * Cfg<N>::CPB * LinePad<N>::SC));
+  }
+};
+
 }  // namespace dgk
+
+int dg_prepare_apply_f32(int n) {
+  cudaError_t e = dgk::dispatch_n<float, dgk::Prepare32F>(n);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "apply (fp32) kernel attributes");
+  return DG_OK;
+}
+
+int dg_launch_pass_f32(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
+                       long long cend, const int* skip, cudaStream_t s) {
+  cudaError_t e = dgk::dispatch_n<float, dgk::Pass32F>(m->n, m, pass, x, y, cbeg, cend, skip, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "apply (fp32) launch");
+  return DG_OK;
+}
+
+int dg_launch_apply_f32(const dg_mesh* m, const float* x, float* y, const int* skip,
+                        cudaStream_t s) {
+  dg_timing_mark(m, 0, s);
+  int rc = dg_launch_pass_f32(m, 1, x, y, 0, m->ncells, skip, s);
+  if (rc) return rc;
+  dg_timing_mark(m, 1, s);
+  rc = dg_launch_pass_f32(m, 2, x, y, 0, m->ncells, skip, s);
+  if (rc) return rc;
+  dg_timing_mark(m, 2, s);
+  return DG_OK;
+}
 
 int dg_prepare_mixed32(dg_mesh* m) {
   cudaError_t e = dgk::dispatch_n<float, dgk::PrepareMixed32F>(m->n, m);
