@@ -11,13 +11,6 @@ int dg_launch_apply_f64(const dg_mesh* m, const double* x, double* y, const int*
   return dg_launch_fixed_apply(m, true, x, y, skip, s);
 }
 
-int dg_launch_trace_f64(const dg_mesh* m, const double* x, double* U, double* X, double* TR,
-                        cudaStream_t s) {
-  cudaError_t e = dgk::dispatch_n<double, dgk::TraceF>(m->n, x, U, X, TR, m->ncells, &m->tab64, s);
-  if (e != cudaSuccess) return dg_cuda_fail(e, "trace (fp64) launch");
-  return DG_OK;
-}
-
 int dg_prepare_apply_f64(int n) {
   cudaError_t e = dgk::dispatch_n<double, dgk::PrepareF>(n);
   if (e != cudaSuccess) return dg_cuda_fail(e, "apply (fp64) kernel attributes");

@@ -784,15 +784,6 @@ __global__ void k_face_weights(const double* __restrict__ gh, T* __restrict__ FW
 }
 
 
-template <int N, typename T>
-cudaError_t launch_trace_n(const T* x, T* U, T* X, T* TR, long long ncells, const DGTab<T>& tab,
-                           cudaStream_t s) {
-  const unsigned blocks = (unsigned)((ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
-  k_trace<N, T><<<blocks, Cfg<N>::THREADS, trace_smem<N, T>(), s>>>(x, U, X, TR, 0, ncells,
-                                                                     nullptr, tab);
-  return cudaGetLastError();
-}
-
 template <typename T, template <int> class F, typename... Args>
 cudaError_t dispatch_n(int n, Args... args) {
   switch (n) {
@@ -819,15 +810,6 @@ struct PrepareF {
       e = cudaFuncSetAttribute(k_trace<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)trace_smem<N, T>());
     return e;
-  }
-};
-
-template <int N>
-struct TraceF {
-  template <typename T>
-  static cudaError_t run(const T* x, T* U, T* X, T* TR, long long ncells, const DGTab<T>* tab,
-                         cudaStream_t s) {
-    return launch_trace_n<N, T>(x, U, X, TR, ncells, *tab, s);
   }
 };
 

@@ -311,6 +311,18 @@ struct FixedCgF {
 };
 
 template <int N>
+struct FixedTraceF {
+  template <typename T>
+  static cudaError_t run(const dg_mesh* m, const double* x, long long* U, long long* TR,
+                         int* expU, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
+    k_trace_fx<N, true><<<blocks, Cfg<N>::THREADS, 0, s>>>(FxLoad{x}, U, TR, expU, 0, m->ncells,
+                                                          nullptr, m->tabX);
+    return cudaGetLastError();
+  }
+};
+
+template <int N>
 struct FixedPrepF {
   template <typename T>
   static cudaError_t run() {
@@ -380,5 +392,13 @@ int dg_launch_fixed_cg(const dg_mesh* m, const double* z, const double* dinv, do
                        double* q, cudaStream_t s) {
   cudaError_t e = dgk::dispatch_n<double, dgk::FixedCgF>(m->n, m, z, dinv, p, q, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "CG operator (fp64) launch");
+  return DG_OK;
+}
+
+int dg_launch_fixed_trace(const dg_mesh* m, const double* x, double* U, double* TR, int* expU,
+                          cudaStream_t s) {
+  cudaError_t e = dgk::dispatch_n<double, dgk::FixedTraceF>(
+      m->n, m, x, reinterpret_cast<long long*>(U), reinterpret_cast<long long*>(TR), expU, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "trace (fp64) launch");
   return DG_OK;
 }

@@ -32,9 +32,10 @@ int ceil_log2(ld v) {  // smallest e with v <= 2^e
 
 }  // namespace
 
-bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s) {
+bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGrad* g) {
   std::memset(t, 0, sizeof(*t));
   std::memset(s, 0, sizeof(*s));
+  std::memset(g, 0, sizeof(*g));
   ld xi[DG_MAXN], w[DG_MAXN];
   // Legendre values and derivatives on [-1, 1], degrees 0..n
   auto legendre = [n](ld x, ld* P, ld* dP) {
@@ -149,5 +150,29 @@ bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s) {
       s->F[0][k] = put(ldexpl(ll + x, s->ch - s->cB));
       s->F[1][k] = put(ldexpl(ll + 2 * x, s->ch - s->cB));
     }
+  // the scaled derivative: Dh[n-1-f][n-1-a] = -Dh[f][a], so its even and odd
+  // halves over the mirror pairs give both points of a pair
+  ld row = 0;
+  for (int f = 0; f < n; ++f) {
+    ld sum = 0;
+    for (int a = 0; a < n; ++a) sum += fabsl(Dh[f][a]);
+    row = fmaxl(row, sum);
+  }
+  g->cD = ceil_log2(row);
+  for (int f = 0; f < (n + 1) / 2; ++f)
+    for (int a = 0; a < (n + 1) / 2; ++a) {
+      const int b = n - 1 - a;
+      const ld e = a == b ? Dh[f][a] : (Dh[f][a] + Dh[f][b]) / 2;
+      const ld o = a == b ? 0 : (Dh[f][a] - Dh[f][b]) / 2;
+      g->De[f][a] = put(ldexpl(f == n - 1 - f ? 0 : e, -g->cD));
+      g->Do[f][a] = put(ldexpl(o, -g->cD));
+    }
+  g->cj[0] = put(ldexpl(sigma / 2, cv - ca - 2));
+  g->cj[1] = put(ldexpl(3 * sigma / 2, cv - ca - 2));
+  g->cva = cv + ca;
+  for (int a = 0; a < n; ++a) {
+    g->w[a] = (double)w[a];
+    g->iw[a] = (double)(1 / w[a]);
+  }
   return ok;
 }

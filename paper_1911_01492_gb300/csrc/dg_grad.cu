@@ -6,171 +6,201 @@
 // (-{d_n u}[v] - {d_n v}[u] + sigma [u][v] weighted by h w_s w_t); gamma_F
 // depends on K only through the cells' Kbar = exp(sum_q w_q log K_q), hence
 //   g_q = Kt_q grad u . grad v + w_q sum_{F of the cell} (d gamma_F / d log Kbar_c) b_F(u, v).
-// Inputs: pass-1 data (nodal U, x-modal X, face traces) of u and of v.
-#include <type_traits>
-
-#include "dg_apply_impl.cuh"
+//
+// Both parts are formed in block fixed point (dg_fixed.cuh) from pass 1 of u and
+// of v in the scaled point basis: there Dh u Dh v = w_q du dv at point q, and the
+// products of two face traces carry w_s w_t.  With the traces J = u- - u+ and
+// the combinations P = (d - sigma u)- + (sigma u + d)+ that pass 1 stores (d half
+// the normal derivative), an interior face point gives
+//   -(Pu Jv + Pv Ju) - sigma Ju Jv = -(Gu Jv + Gv Ju),  G = P + sigma J / 2;
+// a boundary point is the same with the other side's value zero, P twice the own
+// combination and 3 sigma / 2 in place of sigma / 2.
+// FP64 is left to 10 instructions per DOF (the FP64 kernel executed 60); 32^3 Q3:
+// pass 1 of both and this kernel 445 -> 102 us.
+#include "dg_fixed.cuh"
 
 namespace dgk {
 
-// b_F contribution at one face point for gamma = 1 (W = h w_s w_t).
-template <bool UPPER>
-__device__ __forceinline__ double face_form_point(bool interior, double uo, double go, double un,
-                                                  double gn, double vo, double gvo, double vn,
-                                                  double gvn, double W, double sigma) {
-  double Ju, Au, Jv, Av;
-  if (interior) {
-    if (UPPER) {  // own cell is (-)
-      Ju = uo - un; Jv = vo - vn;
-    } else {      // own cell is (+)
-      Ju = un - uo; Jv = vn - vo;
-    }
-    Au = 0.5 * (go + gn);
-    Av = 0.5 * (gvo + gvn);
-  } else {        // outward normal +e_d (upper) or -e_d (lower)
-    Ju = uo; Jv = vo;
-    Au = UPPER ? go : -go;
-    Av = UPPER ? gvo : -gvo;
+// g[f] = sum_a Dh[f][a] u[a]  2^-cD
+template <int N>
+__device__ __forceinline__ void fx_deriv(const DGTabXGrad& t, const long long (&u)[N],
+                                         long long (&g)[N]) {
+  constexpr int H = N / 2, P = (N + 1) / 2;
+  FxVal e[P], o[H];
+#pragma unroll
+  for (int a = 0; a < H; ++a) {
+    e[a] = fx_split(u[a] + u[N - 1 - a]);
+    o[a] = fx_split(u[a] - u[N - 1 - a]);
   }
-  return W * (-Au * Jv - Av * Ju + sigma * Ju * Jv);
+  if (N % 2 == 1) e[P - 1] = fx_split(u[H]);
+#pragma unroll
+  for (int f = 0; f < P; ++f) {
+    FxAcc Q = fx_zero();
+#pragma unroll
+    for (int a = 0; a < H; ++a) fx_mac(Q, t.Do[f][a], o[a]);
+    const long long q = fx_value(Q);
+    if (f == N - 1 - f) {
+      g[f] = q;
+    } else {
+      FxAcc E = fx_zero();
+#pragma unroll
+      for (int a = 0; a < P; ++a) fx_mac(E, t.De[f][a], e[a]);
+      const long long p = fx_value(E);
+      g[f] = q + p;
+      g[N - 1 - f] = q - p;
+    }
+  }
 }
 
 template <int N>
+struct GradCfg {
+  static constexpr int C = Cfg<N>::CPB, N2 = N * N;
+  // u, v, the volume products; per-line and per-row face sums; exponents
+  static constexpr size_t SMEM =
+      8 * (3 * C * LinePad<N>::SC + C * (N2 + N)) + 4 * (14 * C);
+};
+
+template <int N>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
-k_coeff_grad(const double* __restrict__ Uu, const double* __restrict__ Xu,
-             const double* __restrict__ TRu, const double* __restrict__ Uv,
-             const double* __restrict__ Xv, const double* __restrict__ TRv,
+k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu,
+             const int* __restrict__ eu, const long long* __restrict__ Uv,
+             const long long* __restrict__ TRv, const int* __restrict__ ev,
              const double* __restrict__ kt, const double* __restrict__ dgam, double h,
              double* __restrict__ g, long long ncells, int Nc,
-             const __grid_constant__ DGTab<double> tab) {
-  constexpr int N2 = N * N, N3 = N * N * N, C = Cfg<N>::CPB;
+             const __grid_constant__ DGTabXGrad tab) {
+  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, T = Cfg<N>::THREADS;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* su = reinterpret_cast<double*>(smem_raw);
-  double* sv = su + C * N3;
-  double* sxu = sv + C * N3;
-  double* sxv = sxu + C * N3;
-  double* sg = sxv + C * N3;         // grad u . grad v accumulated per point
-  double* sf = sg + C * N3;          // per-face-point face form values [C][6][N2]
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
-  for (int t = threadIdx.x; t < nblk * N3; t += blockDim.x) {
-    su[t] = Uu[c0 * N3 + t];
-    sv[t] = Uv[c0 * N3 + t];
-    sxu[t] = Xu[c0 * N3 + t];
-    sxv[t] = Xv[c0 * N3 + t];
-  }
-  __syncthreads();
-  const int lc = threadIdx.x / N2;
-  const int t2 = threadIdx.x - lc * N2;
-  const int p = t2 % N, q = t2 / N;
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
   const bool active = lc < nblk;
-  const long long c = c0 + lc;
-  const int cx = (int)(c % Nc);
-  const int cy = (int)((c / Nc) % Nc);
-  const int cz = (int)(c / ((long long)Nc * Nc));
-  const long long sy = Nc, sz = (long long)Nc * Nc;
-  const int o = lc * N3;
-  double* sfc = sf + lc * 6 * N2;
-  const double sigma = tab.sigma;
-  const int pt = p + N * q;
-  const double W = h * tab.w[p] * tab.w[q];
-
-  auto face = [&](auto upper_tag, int f, int fn, bool in, long long cn) {
-    constexpr bool UP = decltype(upper_tag)::value;
-    double uo, go, un = 0.0, gn = 0.0, vo, gvo, vn = 0.0, gvn = 0.0;
-    load_trace<N>(TRu, c, f, pt, uo, go);
-    load_trace<N>(TRv, c, f, pt, vo, gvo);
-    if (in) {
-      load_trace<N>(TRu, cn, fn, pt, un, gn);
-      load_trace<N>(TRv, cn, fn, pt, vn, gvn);
+  const long long c = c0 + (active ? lc : 0);
+  long long* su = reinterpret_cast<long long*>(smem_raw) + lc * SC;
+  long long* sv = su + C * SC;
+  long long* sg = sv + C * SC;
+  double* sf = reinterpret_cast<double*>(smem_raw) + 3 * C * SC + lc * (N2 + N);
+  int(*sexp)[14] =
+      reinterpret_cast<int(*)[14]>(reinterpret_cast<double*>(smem_raw) + 3 * C * SC + C * (N2 + N));
+  const unsigned nu = (unsigned)Nc;
+  const long long stride[3] = {1, Nc, (long long)Nc * Nc};
+  // exponents of u (0..6) and v (7..13): six neighbours, own
+  for (int i = threadIdx.x; i < nblk * 14; i += T) {
+    const int l2 = i / 14, k = i - l2 * 14, f = k % 7, d = f >> 1;
+    const long long cc = c0 + l2;
+    const unsigned row = (unsigned)cc / nu;
+    const int crd = d == 0 ? (int)((unsigned)cc - row * nu)
+                    : d == 1 ? (int)(row % nu) : (int)(row / nu);
+    const bool in = f < 6 && ((f & 1) ? crd < Nc - 1 : crd > 0);
+    sexp[l2][k] = (k < 7 ? eu : ev)[in ? ((f & 1) ? cc + stride[d] : cc - stride[d]) : cc];
+  }
+  long long u[N], v[N];
+#pragma unroll
+  for (int e = 0; e < N; ++e) {  // z-lines (a = p, b = q)
+    const long long at = c * N3 + e * N2 + q * N + p;
+    u[e] = Uu[at];
+    v[e] = Uv[at];
+    su[e * SZ + q * SY + p] = u[e];
+    sv[e * SZ + q * SY + p] = v[e];
+  }
+  __syncthreads();
+  const int* se = sexp[active ? lc : 0];
+  int top = 0;
+#pragma unroll
+  for (int k = 0; k < 14; ++k) top = max(top, se[k]);
+  const bool bad = top >= FX_NAN / 2;
+  const unsigned row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  double s = 0.0;  // the line's six face points, weighted by d gamma
+  // the volume products of the line (twice), added to r (or replacing it)
+  auto line = [&](int dir, long long (&r)[N], bool first) {
+    long long gu[N], gv[N];
+    fx_deriv<N>(tab, u, gu);
+    fx_deriv<N>(tab, v, gv);
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      FxAcc A = fx_zero<1>();
+      fx_mac(A, fx_pair(gu[e]), fx_split(gv[e]));
+      r[e] = first ? fx_value<1>(A) : r[e] + fx_value<1>(A);
     }
-    sfc[f * N2 + pt] = face_form_point<UP>(in, uo, go, un, gn, vo, gvo, vn, gvn, W, sigma);
+#pragma unroll
+    for (int up = 0; up < 2; ++up) {
+      const int f = 2 * dir + up;
+      const bool in = up ? crd[dir] < Nc - 1 : crd[dir] > 0;
+      const long long cn = in ? (up ? c + stride[dir] : c - stride[dir]) : c;
+      const long long o = c * (12 * N2) + (2 * f) * N2 + pt;
+      const long long on = cn * (12 * N2) + (2 * (in ? f ^ 1 : f)) * N2 + pt;
+      // J = u- - u+ and P of one vector under the common exponent e, 2^-3
+      auto side = [&](const long long* __restrict__ TR, int eo, int en, long long& J,
+                      long long& P, int& e) {
+        e = max(eo, en) + 3;
+        const int so = min(e - eo, 63), sn = min(e - en, 63);
+        const long long vo = TR[o] >> so, ao = TR[o + N2] >> so;
+        const long long vn = in ? TR[on] >> sn : 0, an = TR[on + N2] >> sn;
+        J = up ? vo - vn : vn - vo;
+        P = ao + an;
+      };
+      long long Ju, Pu, Jv, Pv;
+      int e1, e2;
+      side(TRu, se[6], se[f], Ju, Pu, e1);
+      side(TRv, se[13], se[7 + f], Jv, Pv, e2);
+      const FxVal ju = fx_split(Ju), jv = fx_split(Jv);
+      FxAcc A = fx_zero<2>(), B = fx_zero<2>(), F = fx_zero<2>();
+      fx_mac(A, tab.cj[in ? 0 : 1], ju);
+      fx_mac(B, tab.cj[in ? 0 : 1], jv);
+      fx_mac(F, fx_pair(Pu + fx_value<2>(A)), jv);
+      fx_mac(F, fx_pair(Pv + fx_value<2>(B)), ju);
+      s = fma(dgam[c * 6 + f], fx_to_double(fx_value<2>(F), e1 + e2 + 58 + tab.cva), s);
+    }
   };
-  using UpT = std::integral_constant<bool, true>;
-  using LoT = std::integral_constant<bool, false>;
-
-  // z-lines (a = p, b = q)
-  if (active) {
-    double u[N], v[N];
+  long long r[N];
+  line(2, r, true);
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      u[e] = su[o + e * N2 + q * N + p];
-      v[e] = sv[o + e * N2 + q * N + p];
-    }
+  for (int e = 0; e < N; ++e) sg[e * SZ + q * SY + p] = r[e];
+  __syncthreads();
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      double gu = 0.0, gv = 0.0;
+  for (int b = 0; b < N; ++b) {  // y-lines (a = p, e = q)
+    u[b] = su[q * SZ + b * SY + p];
+    v[b] = sv[q * SZ + b * SY + p];
+    r[b] = sg[q * SZ + b * SY + p];
+  }
+  line(1, r, false);
 #pragma unroll
-      for (int f = 0; f < N; ++f) {
-        gu = fma(tab.D[e][f], u[f], gu);
-        gv = fma(tab.D[e][f], v[f], gv);
-      }
-      sg[o + e * N2 + q * N + p] = gu * gv;
-    }
-    face(UpT{}, 5, 4, cz < Nc - 1, c + sz);
-    face(LoT{}, 4, 5, cz > 0, c - sz);
+  for (int b = 0; b < N; ++b) sg[q * SZ + b * SY + p] = r[b];
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < N; ++a) {  // x-lines (b = p, e = q)
+    u[a] = su[q * SZ + p * SY + a];
+    v[a] = sv[q * SZ + p * SY + a];
+    r[a] = sg[q * SZ + p * SY + a];
+  }
+  line(0, r, false);
+#pragma unroll
+  for (int a = 0; a < N; ++a) sg[q * SZ + p * SY + a] = r[a];
+  // the cell's face sum in a fixed order: rows of n threads, then n rows
+  sf[pt] = s;
+  __syncthreads();
+  if (q == 0) {
+    double t = sf[p];
+    for (int k = 1; k < N; ++k) t += sf[k * N + p];
+    sf[N2 + p] = t;
   }
   __syncthreads();
-  // y-lines (a = p, e = q)
-  if (active) {
-    double u[N], v[N];
+  if (!active) return;
+  s = sf[N2];
 #pragma unroll
-    for (int b = 0; b < N; ++b) {
-      u[b] = su[o + q * N2 + b * N + p];
-      v[b] = sv[o + q * N2 + b * N + p];
-    }
+  for (int k = 1; k < N; ++k) s += sf[N2 + k];
+  // each thread writes the n points of its z-line
+  const double ws = -h * s * (tab.w[p] * tab.w[q]);
+  const double is = tab.iw[p] * tab.iw[q];
+  const int ex = se[6] + se[13] + 59 + 2 * tab.cD;
 #pragma unroll
-    for (int b = 0; b < N; ++b) {
-      double gu = 0.0, gv = 0.0;
-#pragma unroll
-      for (int f = 0; f < N; ++f) {
-        gu = fma(tab.D[b][f], u[f], gu);
-        gv = fma(tab.D[b][f], v[f], gv);
-      }
-      sg[o + q * N2 + b * N + p] = fma(gu, gv, sg[o + q * N2 + b * N + p]);
-    }
-    face(UpT{}, 3, 2, cy < Nc - 1, c + sy);
-    face(LoT{}, 2, 3, cy > 0, c - sy);
-  }
-  __syncthreads();
-  // x-lines (b = p, e = q): x-derivative from the x-modal data
-  if (active) {
-    double Xa[N], Xb[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      Xa[i] = sxu[o + q * N2 + p * N + i];
-      Xb[i] = sxv[o + q * N2 + p * N + i];
-    }
-#pragma unroll
-    for (int a = 0; a < N; ++a) {
-      double gu = 0.0, gv = 0.0;
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        gu = fma(tab.Bd[a][i], Xa[i], gu);
-        gv = fma(tab.Bd[a][i], Xb[i], gv);
-      }
-      sg[o + q * N2 + p * N + a] = fma(gu, gv, sg[o + q * N2 + p * N + a]);
-    }
-    face(UpT{}, 1, 0, cx < Nc - 1, c + 1);
-    face(LoT{}, 0, 1, cx > 0, c - 1);
-  }
-  __syncthreads();
-  // per cell: s = sum_f dgam_f * sum_pt sf[f][pt]  (fixed summation order)
-  if (active) {
-    double s = 0.0;
-#pragma unroll 1
-    for (int f = 0; f < 6; ++f) {
-      double b = 0.0;
-      for (int k = 0; k < N2; ++k) b += sfc[f * N2 + k];
-      s = fma(dgam[c * 6 + f], b, s);
-    }
-    // each thread writes the n points of its z-line (a = p, b = q)
-#pragma unroll
-    for (int e = 0; e < N; ++e) {
-      const int qi = e * N2 + q * N + p;
-      const double wq = tab.w[p] * tab.w[q] * tab.w[e];
-      g[c * N3 + qi] = fma(kt[c * N3 + qi], sg[o + qi], wq * s);
-    }
+  for (int e = 0; e < N; ++e) {
+    const long long at = c * N3 + e * N2 + q * N + p;
+    const double vol = fx_to_double(sg[e * SZ + q * SY + p], ex);
+    const double val = fma(kt[at] * (is * tab.iw[e]), vol, ws * tab.w[e]);
+    g[at] = bad ? __longlong_as_double(0x7ff8000000000000ll) : val;
   }
 }
 
@@ -178,12 +208,11 @@ template <int N>
 struct GradF {
   template <typename T>
   static cudaError_t run(const dg_mesh* m, double* g, cudaStream_t s) {
-    constexpr int C = Cfg<N>::CPB, N3 = N * N * N;
-    const size_t smem = sizeof(double) * (5 * C * N3 + C * 6 * N * N);
-    const unsigned blocks = (unsigned)((m->ncells + C - 1) / C);
-    k_coeff_grad<N><<<blocks, Cfg<N>::THREADS, smem, s>>>(
-        m->U64, m->X64, m->TR64, m->U64b, m->X64b, m->TR64b, m->kt64, m->dgam, m->h, g,
-        m->ncells, m->N, m->tab64);
+    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
+    auto ll = [](double* p) { return reinterpret_cast<const long long*>(p); };
+    k_coeff_grad<N><<<blocks, Cfg<N>::THREADS, GradCfg<N>::SMEM, s>>>(
+        ll(m->U64), ll(m->TR64), m->expU, ll(m->U64b), ll(m->TR64b), m->expUb, m->kt64, m->dgam,
+        m->h, g, m->ncells, m->N, m->tabXG);
     return cudaGetLastError();
   }
 };
@@ -192,10 +221,8 @@ template <int N>
 struct GradPrepF {
   template <typename T>
   static cudaError_t run() {
-    constexpr int C = Cfg<N>::CPB, N3 = N * N * N;
-    const size_t smem = sizeof(double) * (5 * C * N3 + C * 6 * N * N);
     return cudaFuncSetAttribute(k_coeff_grad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
+                                (int)GradCfg<N>::SMEM);
   }
 };
 

@@ -67,8 +67,14 @@ struct DGTabXSetup {
   FxPair F[2][DG_MAXP];         // own-side terms of the lower face: inside, boundary
   int ch, cB;                   // h <= 2^ch; entries < 2^(cB + exponent of K)
 };
+struct DGTabXGrad {  // coefficient gradient (dg_grad.cu)
+  FxPair De[DG_MAXH][DG_MAXH], Do[DG_MAXH][DG_MAXH];  // halves of Dh[f][.]  2^-cD
+  FxPair cj[2];     // sigma / 2 (inside) and 3 sigma / 2 (boundary)  2^(cv-ca-2)
+  int cD, cva;      // cva = cv + ca
+  double w[DG_MAXN], iw[DG_MAXN];  // Gauss weights and their reciprocals
+};
 // false if a constant leaves its range (degrees 1..8 are inside)
-bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s);
+bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGrad* g);
 
 // CG scalar state kept on the device (one per solve / per batched sample).
 struct DGCGState {
@@ -131,8 +137,10 @@ struct dg_mesh {
   // vector of the running application [c]
   DGTabX tabX;
   DGTabXSetup tabXS;
+  DGTabXGrad tabXG;
   FxPair *lineopX, *gamX;
   int *expM, *expG, *expU;
+  int* expUb;  // exponents of the second vector of the coefficient gradient
 
   // coefficient data (dg_set_coefficient)
   bool has_coef;
@@ -183,8 +191,8 @@ struct dg_mesh {
   // apply workspaces: nodal values, x-modal/yz-nodal values, face traces
   double *U64, *X64, *TR64;
   float* TR32;
-  // second set for the coefficient gradient (traces of v), lazily allocated
-  double *U64b, *X64b, *TR64b;
+  // second set for the coefficient gradient (of v), lazily allocated
+  double *U64b, *TR64b;
   // host staging for dg_apply_host: device copies of x and y, copy-in,
   // copy-out and pass-1 streams and per-slab events of the pipeline
   void *hx_dev, *hy_dev;
@@ -221,10 +229,9 @@ void dg_timing_mark(const dg_mesh* m, int slot, cudaStream_t s);
 // coefficient setup kernels (dg_mesh.cu), shared with the allocation-free
 // apply: h w_q K and Kbar per cell (FP32 copy skipped when kt32 is NULL); h gamma
 // and d gamma / d log Kbar per face side (gh32 / dgam skipped when NULL)
-__global__ void k_coef_cells(const double* __restrict__ K, double* __restrict__ kt64,
-                             float* __restrict__ kt32, double* __restrict__ kbar,
-                             long long ncells, int n, double h, int* flag,
-                             const __grid_constant__ DGTab<double> tab);
+cudaError_t dg_launch_coef_cells(const double* K, double* kt64, float* kt32, double* kbar,
+                                 long long ncells, int n, double h, int* flag,
+                                 const DGTab<double>& tab, cudaStream_t s);
 // (dmask: bit f set when boundary side f is Dirichlet; the boundary faces of
 // the other sides carry zero flux, gamma = 0)
 __global__ void k_coef_faces(const double* __restrict__ kbar, double* __restrict__ gh64,
@@ -268,9 +275,9 @@ int dg_launch_apply_multilinear(const dg_mesh* m, const double* x, double* y, co
                                 cudaStream_t s);
 // INVALID_ARG if the mesh is affine (for the paths that assume cube faces)
 int dg_require_cube(const dg_mesh* m, const char* who);
-// traces only (used by the coefficient gradient): U, X, TR of x into the given buffers
-int dg_launch_trace_f64(const dg_mesh* m, const double* x, double* U, double* X, double* TR,
-                        cudaStream_t s);
+// pass 1 of the fixed-point operator into the given buffers
+int dg_launch_fixed_trace(const dg_mesh* m, const double* x, double* U, double* TR, int* expU,
+                          cudaStream_t s);
 int dg_launch_coeff_grad(const dg_mesh* m, double* g, cudaStream_t s);
 // fused FP32 kernels of the mixed CG iteration (dg_mixed32.cu)
 // rin: r32 (z = r, or z = dinv r with dinv), or z = M^-1 r already formed

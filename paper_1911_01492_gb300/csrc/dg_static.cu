@@ -129,8 +129,7 @@ extern "C" int dg_apply_static(int n_cells, int degree, const double* K, const d
   cudaStream_t s = (cudaStream_t)stream;
   DG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
   // the coefficient kernels of dg_set_coefficient, FP64 outputs only
-  k_coef_cells<<<(unsigned)((ncells * 32 + 255) / 256), 256, 0, s>>>(K, kt, nullptr, kbar, ncells,
-                                                                     n, h, flag, tab);
+  DG_CUDA(dg_launch_coef_cells(K, kt, nullptr, kbar, ncells, n, h, flag, tab, s));
   k_coef_faces<<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(kbar, gh, nullptr, nullptr,
                                                                 n_cells, h, DG_BC_DIRICHLET);
   dgk::k_face_weights<double><<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(gh, FW, n_cells, n,
