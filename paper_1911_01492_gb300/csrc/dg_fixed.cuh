@@ -199,6 +199,37 @@ __device__ __forceinline__ void fx_bwd(const DGTabX& t, const long long (&r)[N],
   }
 }
 
+// g[f] = sum_a Dh[f][a] u[a]  2^-cD
+template <int N>
+__device__ __forceinline__ void fx_deriv(const DGTabXGrad& t, const long long (&u)[N],
+                                         long long (&g)[N]) {
+  constexpr int H = N / 2, P = (N + 1) / 2;
+  FxVal e[P], o[H];
+#pragma unroll
+  for (int a = 0; a < H; ++a) {
+    e[a] = fx_split(u[a] + u[N - 1 - a]);
+    o[a] = fx_split(u[a] - u[N - 1 - a]);
+  }
+  if (N % 2 == 1) e[P - 1] = fx_split(u[H]);
+#pragma unroll
+  for (int f = 0; f < P; ++f) {
+    FxAcc Q = fx_zero();
+#pragma unroll
+    for (int a = 0; a < H; ++a) fx_mac(Q, t.Do[f][a], o[a]);
+    const long long q = fx_value(Q);
+    if (f == N - 1 - f) {
+      g[f] = q;
+    } else {
+      FxAcc E = fx_zero();
+#pragma unroll
+      for (int a = 0; a < P; ++a) fx_mac(E, t.De[f][a], e[a]);
+      const long long p = fx_value(E);
+      g[f] = q + p;
+      g[N - 1 - f] = q - p;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // The two passes (dg_fixed.cu), as functions of a block over a group of cells.
 // ---------------------------------------------------------------------------

@@ -157,6 +157,9 @@ bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGra
     ld sum = 0;
     for (int a = 0; a < n; ++a) sum += fabsl(Dh[f][a]);
     row = fmaxl(row, sum);
+    sum = 0;  // and of the transpose
+    for (int a = 0; a < n; ++a) sum += fabsl(Dh[a][f]);
+    row = fmaxl(row, sum);
   }
   g->cD = ceil_log2(row);
   for (int f = 0; f < (n + 1) / 2; ++f)
@@ -170,6 +173,8 @@ bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGra
   g->cj[0] = put(ldexpl(sigma / 2, cv - ca - 2));
   g->cj[1] = put(ldexpl(3 * sigma / 2, cv - ca - 2));
   g->cva = cv + ca;
+  g->cv = cv;
+  g->cl = cl;
   for (int a = 0; a < n; ++a) {
     g->w[a] = (double)w[a];
     g->iw[a] = (double)(1 / w[a]);

@@ -70,7 +70,7 @@ struct DGTabXSetup {
 struct DGTabXGrad {  // coefficient gradient (dg_grad.cu)
   FxPair De[DG_MAXH][DG_MAXH], Do[DG_MAXH][DG_MAXH];  // halves of Dh[f][.]  2^-cD
   FxPair cj[2];     // sigma / 2 (inside) and 3 sigma / 2 (boundary)  2^(cv-ca-2)
-  int cD, cva;      // cva = cv + ca
+  int cD, cva, cv, cl;  // cva = cv + ca
   double w[DG_MAXN], iw[DG_MAXN];  // Gauss weights and their reciprocals
 };
 // false if a constant leaves its range (degrees 1..8 are inside)
@@ -126,6 +126,9 @@ struct dg_mesh {
   // and the own-side vector J^-1 n [c][6][4][n^2]; per cell face sigma / h_F [c][6]
   bool multilinear;
   double *geo_vol, *geo_det, *geo_face, *geo_pen;
+  // its fixed-point products with the coefficient (dg_multilinear.cu)
+  FxPair *mlV, *mlF;
+  int *mlExpV, *mlExpM, *mlExpF;
   int device;
   int sm_count;
   DGTab<double> tab64;
@@ -271,6 +274,7 @@ int dg_launch_apply_f32(const dg_mesh* m, const float* x, float* y, const int* s
 int dg_launch_apply_affine(const dg_mesh* m, const double* x, double* y, const int* skip,
                            cudaStream_t s);
 int dg_prepare_affine(int n);
+int dg_setup_multilinear(dg_mesh* m, cudaStream_t s);  // after the coefficient
 int dg_launch_apply_multilinear(const dg_mesh* m, const double* x, double* y, const int* skip,
                                 cudaStream_t s);
 // INVALID_ARG if the mesh is affine (for the paths that assume cube faces)

@@ -13,16 +13,29 @@
 //     the boundary (|T| cell volume, |F| face area).
 // Affine vertices give the affine operator exactly.
 //
-// dg_set_vertices forms the per-point data once (k_geo_points, k_geo_penalty).
-// The pass-2 kernel k_cell_ml is the affine kernel with those per-point
-// values; since the two sides of a face have different Jacobians, each side's
-// normal flux m . grad u needs the tangential derivatives of that side's own
-// trace, so the face step exchanges both traces (and the test side's
-// tangential multipliers) on the face grid.  FP64 only.
+// dg_set_vertices forms the per-point geometry once (k_geo_points,
+// k_geo_penalty), dg_set_coefficient the products with the coefficient
+// (k_ml_setup).  The operator runs in block fixed point (dg_fixed.cuh) in the
+// scaled point basis: with g_d = Dh u along direction d (sqrt(w_q) times the
+// reference derivative),
+//   volume:  r += sum_d Dh^T F_d,  F_d = sum_e (h K G)_de g_e  per point;
+//   faces:   a trace of a point field is its contraction with the scaled end
+//            values l along the normal line, for u and for each g_j, so a
+//            side's normal derivative is m . (traces of g).  With the weight
+//            Ws = h gamma A / (h w_s w_t), J = u- - u+ and D = m . grad u summed
+//            over the sides (halved inside),
+//              r += +- l (Ws pen J - Ws D),   F_j += -l m_j Ws J  (halved inside);
+//            the second line is the derivative of the test function, which
+//            joins the volume flux before Dh^T.
+// Pass 1 (k_trace_ml) leaves v and m . grad u on every face, each side with its
+// own m; pass 2 (k_cell_ml) reads the neighbours'.  Every array has its own
+// exponent (per cell, or per face for the face coefficients) and the sums take
+// the largest.  The FP64 kernels executed 196 FP64 flops per DOF at one
+// instruction per 64 cycles: 40^3 Q3 1003 us, now 256 us.
 #include <cmath>
 #include <vector>
 
-#include "dg_apply_impl.cuh"
+#include "dg_fixed.cuh"
 
 namespace {
 
@@ -163,273 +176,497 @@ __global__ void k_geo_penalty(const double* __restrict__ cellvol,
   }
 }
 
-template <int N>
-struct MlCfg {
-  static constexpr int CPB = dgk::Cfg<N>::CPB;
-  static constexpr int THREADS = CPB * N * N;
-  static constexpr int N2 = N * N, N3 = N * N * N;
-  // per cell: U, X, gx, gy, gz, r, kt (n^3 each), face buffers 2 faces x 4 x n^2
-  static constexpr int PER_CELL = 7 * N3 + 8 * N2;
-  static size_t smem() { return sizeof(double) * (size_t)CPB * PER_CELL; }
-};
+}  // namespace
 
-// One direction's face step (both faces of the thread's line) on a
-// multilinear mesh: per side the normal flux m . grad u with that side's own
-// tangential trace derivatives.  mo/mn: J^-1 n of the own and the neighbour
-// side; Ah: area element / h; pen: sigma / h_F; gh: h gamma.
+namespace dgk {
+
+// F[e] = sum_f Dh[f][e] G[f]  2^-cD
 template <int N>
-__device__ __forceinline__ void face_pair_ml(const DGTab<double>& tab, int d, int t1, int t2,
-                                             int s1, int s2, const double (&uo)[2],
-                                             const double (&go)[2], const double (&un)[2],
-                                             const double (&gn)[2], const bool (&in)[2],
-                                             const double (&mo)[2][3], const double (&mn)[2][3],
-                                             const double (&W)[2], const double (&pen)[2],
-                                             double* fb, bool active, double (&cv)[2],
-                                             double (&cd)[2]) {
-  constexpr int N2 = N * N;
-  const int pt = s1 + N * s2;
-  double J[2];
-  if (active) {
+__device__ __forceinline__ void fx_deriv_t(const DGTabXGrad& t, const long long (&G)[N],
+                                           long long (&r)[N]) {
+  constexpr int H = N / 2, P = (N + 1) / 2;
+  FxVal e[P], o[H];
 #pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      J[f] = f == 1 ? uo[f] - (in[f] ? un[f] : 0.0) : (in[f] ? un[f] : 0.0) - uo[f];
-      fb[(4 * f + 0) * N2 + pt] = uo[f];
-      fb[(4 * f + 1) * N2 + pt] = in[f] ? un[f] : 0.0;
-    }
+  for (int f = 0; f < H; ++f) {
+    e[f] = fx_split(G[f] + G[N - 1 - f]);
+    o[f] = fx_split(G[f] - G[N - 1 - f]);
   }
-  __syncthreads();
-  if (active) {
+  if (N % 2 == 1) e[P - 1] = fx_split(G[H]);
 #pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      double o1 = 0.0, o2 = 0.0, n1 = 0.0, n2v = 0.0;  // tangential derivatives of each trace
+  for (int a = 0; a < P; ++a) {
+    FxAcc E = fx_zero();
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        o1 = fma(tab.D[s1][k], fb[(4 * f) * N2 + k + N * s2], o1);
-        o2 = fma(tab.D[s2][k], fb[(4 * f) * N2 + s1 + N * k], o2);
-        n1 = fma(tab.D[s1][k], fb[(4 * f + 1) * N2 + k + N * s2], n1);
-        n2v = fma(tab.D[s2][k], fb[(4 * f + 1) * N2 + s1 + N * k], n2v);
-      }
-      const double Fo = fma(mo[f][d], go[f], fma(mo[f][t1], o1, mo[f][t2] * o2));
-      double F = Fo;
-      if (in[f]) F = 0.5 * (Fo + fma(mn[f][d], gn[f], fma(mn[f][t1], n1, mn[f][t2] * n2v)));
-      const double s = f == 1 ? 1.0 : -1.0;
-      cv[f] = W[f] * s * fma(pen[f], J[f], -F);
-      const double cD = -(in[f] ? 0.5 : 1.0) * W[f] * J[f];
-      cd[f] = mo[f][d] * cD;
-      fb[(4 * f + 2) * N2 + pt] = mo[f][t1] * cD;
-      fb[(4 * f + 3) * N2 + pt] = mo[f][t2] * cD;
-    }
-  }
-  __syncthreads();
-  if (active) {
+    for (int f = 0; f < H; ++f) fx_mac(E, t.De[f][a], o[f]);
+    const long long p = fx_value(E);
+    if (a == N - 1 - a) {
+      r[a] = p;
+    } else {
+      FxAcc Q = fx_zero();
 #pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      double e = cv[f];
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        e = fma(tab.D[k][s1], fb[(4 * f + 2) * N2 + k + N * s2], e);
-        e = fma(tab.D[k][s2], fb[(4 * f + 3) * N2 + s1 + N * k], e);
-      }
-      cv[f] = e;
+      for (int f = 0; f < P; ++f) fx_mac(Q, t.Do[f][a], e[f]);
+      const long long q = fx_value(Q);
+      r[a] = p + q;
+      r[N - 1 - a] = p - q;
     }
   }
 }
 
+// the field's values at both ends of the line, 2^-cv
 template <int N>
-__global__ void __launch_bounds__(MlCfg<N>::THREADS)
-k_cell_ml(const double* __restrict__ U, const double* __restrict__ Xm,
-          const double* __restrict__ TR, const double* __restrict__ kt,
-          const double* __restrict__ gh, const double* __restrict__ gvol,
-          const double* __restrict__ gface, const double* __restrict__ gpen,
-          double* __restrict__ y, long long ncells, int Nc, const int* __restrict__ skip,
-          const __grid_constant__ DGTab<double> tab) {
-  using Cf = MlCfg<N>;
-  constexpr int C = Cf::CPB, N2 = N * N, N3 = N * N * N;
-  if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) double sm[];
+__device__ __forceinline__ void fx_ends(const DGTabX& t, const long long (&u)[N], long long& lo,
+                                        long long& up) {
+  constexpr int H = N / 2;
+  FxAcc E = fx_zero(), O = fx_zero();
+#pragma unroll
+  for (int a = 0; a < H; ++a) {
+    fx_mac(E, t.ve[a], fx_split(u[a] + u[N - 1 - a]));
+    fx_mac(O, t.vo[a], fx_split(u[a] - u[N - 1 - a]));
+  }
+  if (N % 2 == 1) fx_mac(E, t.ve[H], fx_split(u[H]));
+  const long long e = fx_value(E), o = fx_value(O);
+  lo = e + o;
+  up = e - o;
+}
+
+// u[a] += l[a] lo + l[n-1-a] up, l 2^-cl
+template <int N>
+__device__ __forceinline__ void fx_lift(const DGTabX& t, long long lo, long long up,
+                                        long long (&u)[N]) {
+  const FxVal s = fx_split(lo + up), d = fx_split(lo - up);
+#pragma unroll
+  for (int a = 0; a < (N + 1) / 2; ++a) {
+    FxAcc E = fx_zero();
+    fx_mac(E, t.le[a], s);
+    const long long e = fx_value(E);
+    if (a == N - 1 - a) {
+      u[a] += e;
+    } else {
+      FxAcc O = fx_zero();
+      fx_mac(O, t.lo[a], d);
+      const long long o = fx_value(O);
+      u[a] += e + o;
+      u[N - 1 - a] += e - o;
+    }
+  }
+}
+
+// Per-mesh data of the fixed-point operator on curved cells.  V: h K G [c][xx, yy,
+// zz, xy, xz, yz][n^3], exponent eV; per face point [c][6][8][n^2]: m (3),
+// exponent em per cell, then -m Ws (halved inside; 3), Ws (halved inside) and
+// Ws pen, exponents ef[c][6][3].
+struct MlData {
+  FxPair *V, *F;
+  int *eV, *em, *ef;
+};
+
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::THREADS)
+k_ml_setup(const double* __restrict__ kt, const double* __restrict__ gh,
+           const double* __restrict__ gvol, const double* __restrict__ gface,
+           const double* __restrict__ gpen, MlData md, long long ncells, int Nc,
+           const __grid_constant__ DGTabXGrad tab) {
+  constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
+  constexpr int NS = FxSmem<N, T>::NS;
+  __shared__ unsigned slots[20][NS];
+  for (int i = threadIdx.x; i < 20 * NS; i += T) slots[i / NS][i % NS] = 0;
+  __syncthreads();
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
-  const int lc = threadIdx.x / N2;
-  const int t2 = threadIdx.x - lc * N2;
-  const int p = t2 % N, q = t2 / N;
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
   const bool active = lc < nblk;
-  double* base = sm + lc * Cf::PER_CELL;
-  double* su = base;
-  double* sx = su + N3;
-  double* sg[3] = {sx + N3, sx + 2 * N3, sx + 3 * N3};
-  double* sr = sx + 4 * N3;
-  double* sk = sx + 5 * N3;
-  double* fb = sx + 6 * N3;
-  {
-    const double* ub = U + c0 * N3;
-    const double* xb = Xm + c0 * N3;
-    const double* kb = kt + c0 * N3;
-    for (int t = threadIdx.x; t < nblk * N3; t += blockDim.x) {
-      const int cl = t / N3, o = t - cl * N3;
-      sm[cl * Cf::PER_CELL + o] = ub[t];
-      sm[cl * Cf::PER_CELL + N3 + o] = xb[t];
-      sm[cl * Cf::PER_CELL + 6 * N3 + o] = kb[t];
-    }
+  const long long c = c0 + (active ? lc : 0);
+  const double is = tab.iw[p] * tab.iw[q];
+  double M[6];
+  auto metric = [&](int e) {  // h K G at point e of the thread's z-line
+    const int o = e * N2 + pt;
+    const double k = kt[c * N3 + o] * (is * tab.iw[e]);
+#pragma unroll
+    for (int t = 0; t < 6; ++t) M[t] = k * gvol[(c * 6 + t) * N3 + o];
+  };
+  unsigned big = 0;
+  for (int e = 0; e < N; ++e) {
+    metric(e);
+    const double x = fabs(M[3]), y = fabs(M[4]), z = fabs(M[5]);
+    big = max(big, fx_abs_hi(fmax(M[0] + x + y, fmax(M[1] + x + z, M[2] + y + z))));
   }
-  __syncthreads();
-  const long long c = c0 + lc;
-  int crd[3] = {0, 0, 0};
+  const int EV = fx_exponent(fx_cell_max<N, T>(big, lc, slots[0]));
   if (active) {
-    crd[0] = (int)(c % Nc);
-    crd[1] = (int)((c / Nc) % Nc);
-    crd[2] = (int)(c / ((long long)Nc * Nc));
+    for (int e = 0; e < N; ++e) {
+      metric(e);
+#pragma unroll
+      for (int t = 0; t < 6; ++t)
+        md.V[(c * 6 + t) * N3 + e * N2 + pt] = fx_pair(fx_from_double(M[t], 60 - EV, EV));
+    }
+    if (pt == 0) md.eV[c] = EV;
   }
+  const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  auto geo = [&](int f, int k) { return gface[((c * 6 + f) * 4 + k) * N2 + pt]; };
+  big = 0;
+  for (int f = 0; f < 6; ++f)
+    big = max(big, fx_abs_hi(fabs(geo(f, 1)) + fabs(geo(f, 2)) + fabs(geo(f, 3))));
+  const int Em = fx_exponent(fx_cell_max<N, T>(big, lc, slots[1]));
+  if (active && pt == 0) md.em[c] = Em;
+  for (int f = 0; f < 6; ++f) {
+    const int d = f >> 1;
+    const bool in = f & 1 ? crd[d] < Nc - 1 : crd[d] > 0;
+    const double W = gh[c * 6 + f] * geo(f, 0) * is, Wh = in ? 0.5 * W : W;
+    const double v[8] = {geo(f, 1),       geo(f, 2),       geo(f, 3), -Wh * geo(f, 1),
+                         -Wh * geo(f, 2), -Wh * geo(f, 3), Wh,        W * gpen[c * 6 + f]};
+    unsigned b[3] = {max(fx_abs_hi(v[3]), max(fx_abs_hi(v[4]), fx_abs_hi(v[5]))),
+                     fx_abs_hi(v[6]), fx_abs_hi(v[7])};
+    int E[4] = {Em, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      E[k + 1] = fx_exponent(fx_cell_max<N, T>(b[k], lc, slots[2 + 3 * f + k]));
+      if (active && pt == 0) md.ef[(c * 6 + f) * 3 + k] = E[k + 1];
+    }
+    if (active) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int e = E[k < 3 ? 0 : k < 6 ? 1 : k - 4];
+        md.F[((c * 6 + f) * 8 + k) * N2 + pt] = fx_pair(fx_from_double(v[k], 60 - e, e));
+      }
+    }
+  }
+}
+
+// Pass 1: the point values U under one exponent, and per face v and m . grad u
+// (exponents expU + cv, and expU + em + cD + cv).
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::THREADS)
+k_trace_ml(const double* __restrict__ x, long long* __restrict__ U, long long* __restrict__ TR,
+           int* __restrict__ expU, const FxPair* __restrict__ F, long long ncells,
+           const int* __restrict__ skip, const __grid_constant__ DGTabX tab,
+           const __grid_constant__ DGTabXGrad tg) {
+  constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
+  constexpr int S0 = FxScale<N>::S0, NS = FxSmem<N, T>::NS;
+  if (skip != nullptr && *skip) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned slots[2 * NS];
+  const long long c0 = (long long)blockIdx.x * C;
+  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
+  const bool active = lc < nblk;
+  const long long c = c0 + (active ? lc : 0);
+  // u, then its derivatives along x, y, z
+  long long* su = reinterpret_cast<long long*>(smem_raw) + lc * 4 * SC;
+  long long* sd[3] = {su + SC, su + 2 * SC, su + 3 * SC};
+  if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
+  __syncthreads();
+  double xv[N];
+  unsigned big = 0;
+#pragma unroll
+  for (int l = 0; l < N; ++l) {
+    xv[l] = active ? x[c * N3 + l * N2 + q * N + p] : 0.0;
+    big = max(big, fx_abs_hi(xv[l]));
+  }
+  const int E = fx_exponent(fx_cell_max<N, T>(big, lc, slots));
+  const int zl = q * SY + p, yl = q * SZ + p, xl = q * SZ + p * SY;
+  long long v[N], u[N];
+#pragma unroll
+  for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], S0 - E, E);
+  fx_fwd<N>(tab, v, u);
+#pragma unroll
+  for (int e = 0; e < N; ++e) su[zl + e * SZ] = u[e];
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j] = su[yl + j * SY];
+  fx_fwd<N>(tab, v, u);
+#pragma unroll
+  for (int b = 0; b < N; ++b) su[yl + b * SY] = u[b];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = su[xl + i];
+  fx_fwd<N>(tab, v, u);
+  big = 0;
+#pragma unroll
+  for (int a = 0; a < N; ++a) big = max(big, fx_mag_hi(u[a]));
+  const int up = 60 - fx_bits(fx_cell_max<N, T>(big, lc, slots + NS));
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    u[a] = fx_shift(u[a], up);
+    su[xl + a] = u[a];
+  }
+  fx_deriv<N>(tg, u, v);
+#pragma unroll
+  for (int a = 0; a < N; ++a) sd[0][xl + a] = v[a];
+  if (active && pt == 0) expU[c] = E == FX_NAN ? FX_NAN : E - S0 - up;
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < N; ++b) u[b] = su[yl + b * SY];
+  fx_deriv<N>(tg, u, v);
+#pragma unroll
+  for (int b = 0; b < N; ++b) sd[1][yl + b * SY] = v[b];
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    u[e] = su[zl + e * SZ];
+    if (active) U[c * N3 + e * N2 + pt] = u[e];
+  }
+  fx_deriv<N>(tg, u, v);
+#pragma unroll
+  for (int e = 0; e < N; ++e) sd[2][zl + e * SZ] = v[e];
+  __syncthreads();
+  if (!active) return;  // no barrier follows
+  long long* tr = TR + c * (12 * N2) + pt;
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir) {
+    const int at = dir == 0 ? xl : dir == 1 ? yl : zl, step = dir == 0 ? 1 : dir == 1 ? SY : SZ;
+    FxAcc A[2] = {fx_zero(), fx_zero()};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int e = 0; e < N; ++e) u[e] = su[k * SC + at + e * step];
+      long long end[2];
+      fx_ends<N>(tab, u, end[0], end[1]);
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        if (k == 0)
+          tr[(4 * dir + 2 * f) * N2] = end[f];
+        else
+          fx_mac(A[f], F[((c * 6 + 2 * dir + f) * 8 + k - 1) * N2 + pt], fx_split(end[f]));
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 2; ++f) tr[(4 * dir + 2 * f + 1) * N2] = fx_value(A[f]);
+  }
+}
+
+template <int N>
+struct MlSmem {
+  static constexpr int C = Cfg<N>::CPB;
+  static constexpr size_t trace = 8 * 4 * C * LinePad<N>::SC;
+  // u / r, the flux; per cell: nine shifts per face, then F's and Dh^T F's, ER
+  static constexpr int SH = 6 * 9 + 3;
+  static constexpr size_t cell = 8 * 5 * C * LinePad<N>::SC + 4 * (SH * C);
+};
+
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::THREADS)
+k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
+          const int* __restrict__ expU, MlData md, double* __restrict__ y, long long ncells,
+          int Nc, const int* __restrict__ skip, const __grid_constant__ DGTabX tab,
+          const __grid_constant__ DGTabXGrad tg) {
+  constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
+  constexpr int NS = FxSmem<N, T>::NS, SH = MlSmem<N>::SH;
+  if (skip != nullptr && *skip) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned slots[NS];
+  const long long c0 = (long long)blockIdx.x * C;
+  const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
+  const bool active = lc < nblk;
+  const long long c = c0 + (active ? lc : 0);
+  long long* su = reinterpret_cast<long long*>(smem_raw) + lc * 5 * SC;  // u
+  long long* sF = su + SC;                                              // F_x, F_y, F_z
+  long long* sr = su + 4 * SC;                                          // r
+  int* sh = reinterpret_cast<int*>(reinterpret_cast<long long*>(smem_raw) + 5 * C * SC) +
+            (active ? lc : 0) * SH;
+  const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
-  if (active) {  // gradients at every point (as the affine kernel)
-    double u[N], g[N];
+  if (threadIdx.x < NS) slots[threadIdx.x] = 0;
+  // Exponents and shifts, one thread per cell.  F sums the volume flux, halved
+  // (<= 2^59), and six lifted terms (each below 2^61, five bits down): below
+  // 2^60.  r sums Dh^T F in three directions and six lifted terms three bits
+  // down: below 2^62.5.
+  if (active && pt == 0) {
+    const int Eo = expU[c], em = md.em[c];
+    int EF = md.eV[c] + tg.cD + Eo + 1, ER = -4 * FX_NAN, eJ[6], eD[6];
+    bool nan = Eo >= FX_NAN / 2 || md.eV[c] >= FX_NAN / 2;
 #pragma unroll
-    for (int e = 0; e < N; ++e) u[e] = su[e * N2 + q * N + p];
+    for (int f = 0; f < 6; ++f) {
+      const int d = f >> 1;
+      const bool in = f & 1 ? crd[d] < Nc - 1 : crd[d] > 0;
+      const long long cn = in ? (f & 1 ? c + stride[d] : c - stride[d]) : c;
+      const int En = expU[cn], mn = md.em[cn];
+      nan = nan || En >= FX_NAN / 2 || md.ef[(c * 6 + f) * 3] >= FX_NAN / 2;
+      eJ[f] = max(Eo, En) + 1;
+      eD[f] = max(Eo + em, En + mn) + 1;
+      sh[9 * f + 0] = min(eJ[f] - Eo, 63);
+      sh[9 * f + 1] = min(eJ[f] - En, 63);
+      sh[9 * f + 2] = min(eD[f] - Eo - em, 63);
+      sh[9 * f + 3] = min(eD[f] - En - mn, 63);
+      eJ[f] += tg.cv;
+      eD[f] += tg.cv + tg.cD;
+      EF = max(EF, md.ef[(c * 6 + f) * 3] + eJ[f] + tg.cl + 5);
+      ER = max(ER, max(md.ef[(c * 6 + f) * 3 + 2] + eJ[f], md.ef[(c * 6 + f) * 3 + 1] + eD[f]) +
+                       tg.cl + 3);
+    }
+    ER = max(ER, EF + tg.cD);
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      const int* ef = md.ef + (c * 6 + f) * 3;
+      sh[9 * f + 4] = min(EF - tg.cl - ef[0] - eJ[f], 63);
+      sh[9 * f + 5] = min(ER - tg.cl - ef[2] - eJ[f], 63);
+      sh[9 * f + 6] = min(ER - tg.cl - ef[1] - eD[f], 63);
+    }
+    sh[54] = min(EF - md.eV[c] - tg.cD - Eo, 63);
+    sh[55] = min(ER - EF - tg.cD, 63);
+    sh[56] = nan ? FX_NAN : ER;
+  }
+  const int zl = q * SY + p, yl = q * SZ + p, xl = q * SZ + p * SY;
+  long long u[N], v[N], F[3][N], r[N];
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    u[e] = U[c * N3 + e * N2 + pt];
+    su[zl + e * SZ] = u[e];
+  }
+  fx_deriv<N>(tg, u, F[2]);
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < N; ++b) u[b] = su[yl + b * SY];
+  fx_deriv<N>(tg, u, v);
+#pragma unroll
+  for (int b = 0; b < N; ++b) sF[SC + yl + b * SY] = v[b];
+#pragma unroll
+  for (int a = 0; a < N; ++a) u[a] = su[xl + a];
+  fx_deriv<N>(tg, u, v);
+#pragma unroll
+  for (int a = 0; a < N; ++a) sF[xl + a] = v[a];
+  __syncthreads();
+  // the flux at the points of the z-line
+  {
+    const FxPair* V = md.V + c * 6 * N3 + pt;
+    const int down = sh[54];
 #pragma unroll
     for (int e = 0; e < N; ++e) {
-      double a = 0.0;
-#pragma unroll
-      for (int f = 0; f < N; ++f) a = fma(tab.D[e][f], u[f], a);
-      sg[2][e * N2 + q * N + p] = a;
-    }
-#pragma unroll
-    for (int b = 0; b < N; ++b) u[b] = su[q * N2 + b * N + p];
-#pragma unroll
-    for (int b = 0; b < N; ++b) {
-      double a = 0.0;
-#pragma unroll
-      for (int f = 0; f < N; ++f) a = fma(tab.D[b][f], u[f], a);
-      sg[1][q * N2 + b * N + p] = a;
-    }
-    double X[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) X[i] = sx[q * N2 + p * N + i];
-    dgk::bd_fwd<N>(tab, X, g);
-#pragma unroll
-    for (int a = 0; a < N; ++a) sg[0][q * N2 + p * N + a] = g[a];
-  }
-  __syncthreads();
-  if (active) {  // flux h w K G_q grad u at the points of the thread's z-line
-    const double* Gc = gvol + c * 6 * N3;
-#pragma unroll
-    for (int e = 0; e < N; ++e) {
-      const int idx = e * N2 + q * N + p;
-      const double gx = sg[0][idx], gy = sg[1][idx], gz = sg[2][idx], k = sk[idx];
-      const double xx = Gc[idx], yy = Gc[N3 + idx], zz = Gc[2 * N3 + idx];
-      const double xy = Gc[3 * N3 + idx], xz = Gc[4 * N3 + idx], yz = Gc[5 * N3 + idx];
-      sg[0][idx] = k * fma(xx, gx, fma(xy, gy, xz * gz));
-      sg[1][idx] = k * fma(xy, gx, fma(yy, gy, yz * gz));
-      sg[2][idx] = k * fma(xz, gx, fma(yz, gy, zz * gz));
+      const FxVal gx = fx_split(sF[zl + e * SZ]), gy = fx_split(sF[SC + zl + e * SZ]),
+                  gz = fx_split(F[2][e]);
+      const FxPair xx = V[e * N2], yy = V[N3 + e * N2], zz = V[2 * N3 + e * N2],
+                   xy = V[3 * N3 + e * N2], xz = V[4 * N3 + e * N2], yz = V[5 * N3 + e * N2];
+      FxAcc A = fx_zero(), B = fx_zero(), D = fx_zero();
+      fx_mac(A, xx, gx);
+      fx_mac(A, xy, gy);
+      fx_mac(A, xz, gz);
+      fx_mac(B, xy, gx);
+      fx_mac(B, yy, gy);
+      fx_mac(B, yz, gz);
+      fx_mac(D, xz, gx);
+      fx_mac(D, yz, gy);
+      fx_mac(D, zz, gz);
+      F[0][e] = fx_value(A) >> down;
+      F[1][e] = fx_value(B) >> down;
+      F[2][e] = fx_value(D) >> down;
     }
   }
-  __syncthreads();
-  // face data of face f at the thread's face point pt
-  auto load_face = [&](int face, int pt, int f, double (&uo)[2], double (&go)[2],
-                       double (&un)[2], double (&gn)[2], bool (&in)[2], double (&mo)[2][3],
-                       double (&mn)[2][3], double (&W)[2], double (&pen)[2]) {
-    const int d = face >> 1;
-    in[f] = f == 1 ? crd[d] < Nc - 1 : crd[d] > 0;
-    dgk::load_trace<N>(TR, c, face, pt, uo[f], go[f]);
-    const double* gf = gface + (c * 6 + face) * 4 * N2;
-    W[f] = gh[c * 6 + face] * gf[pt];
-    for (int i = 0; i < 3; ++i) mo[f][i] = gf[(1 + i) * N2 + pt];
-    pen[f] = gpen[c * 6 + face];
-    un[f] = gn[f] = 0.0;
-    for (int i = 0; i < 3; ++i) mn[f][i] = 0.0;
-    if (in[f]) {
-      const long long cn = f == 1 ? c + stride[d] : c - stride[d];
-      dgk::load_trace<N>(TR, cn, face ^ 1, pt, un[f], gn[f]);
-      const double* gn_ = gface + (cn * 6 + (face ^ 1)) * 4 * N2;
-      for (int i = 0; i < 3; ++i) mn[f][i] = gn_[(1 + i) * N2 + pt];
+  // both faces of the thread's line: their terms into F and r of the line
+  auto faces = [&](int dir) {
+    long long t[2][3], w[2];
+#pragma unroll
+    for (int up = 0; up < 2; ++up) {
+      const int f = 2 * dir + up;
+      const bool in = up ? crd[dir] < Nc - 1 : crd[dir] > 0;
+      const long long cn = in ? (up ? c + stride[dir] : c - stride[dir]) : c;
+      const long long* to = TR + c * (12 * N2) + (2 * f) * N2 + pt;
+      const long long* tn = TR + cn * (12 * N2) + (2 * (in ? f ^ 1 : f)) * N2 + pt;
+      const FxPair* W = md.F + (c * 6 + f) * 8 * N2 + pt;
+      const int* s = sh + 9 * f;
+      const long long vo = to[0] >> s[0], vn = in ? tn[0] >> s[1] : 0;
+      const long long D = (to[N2] >> s[2]) + (in ? tn[N2] >> s[3] : 0);
+      const FxVal J = fx_split(up ? vo - vn : vn - vo);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        FxAcc A = fx_zero();
+        fx_mac(A, W[(3 + j) * N2], J);
+        t[up][j] = fx_value(A) >> s[4];
+      }
+      FxAcc A = fx_zero(), B = fx_zero();
+      fx_mac(A, W[7 * N2], J);
+      fx_mac(B, W[6 * N2], fx_split(D));
+      const long long cv = (fx_value(A) >> s[5]) - (fx_value(B) >> s[6]);
+      w[up] = up ? cv : -cv;
     }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) fx_lift<N>(tab, t[0][j], t[1][j], F[j]);
+    fx_lift<N>(tab, w[0], w[1], r);
   };
 #pragma unroll
-  for (int dir = 0; dir < 2; ++dir) {
-    const int d = dir == 0 ? 2 : 1;
-    const int lbase = (dir == 0) ? (q * N + p) : (q * N2 + p);
-    const int step = (dir == 0) ? N2 : N;
-    double r[N];
-    bool in[2] = {false, false};
-    double uo[2] = {0, 0}, go[2] = {0, 0}, un[2] = {0, 0}, gn[2] = {0, 0}, W[2] = {0, 0},
-           pen[2] = {0, 0}, mo[2][3] = {}, mn[2][3] = {};
-    const int pt = p + N * q;
-    if (active) {
-      double fl[N];
+  for (int e = 0; e < N; ++e) r[e] = 0;
+  faces(2);
 #pragma unroll
-      for (int e = 0; e < N; ++e) fl[e] = sg[d][lbase + e * step];
+  for (int e = 0; e < N; ++e) {
+    sr[zl + e * SZ] = r[e];
 #pragma unroll
-      for (int e = 0; e < N; ++e) {
-        double a = (dir == 0) ? 0.0 : sr[lbase + e * step];
-#pragma unroll
-        for (int f = 0; f < N; ++f) a = fma(tab.D[f][e], fl[f], a);
-        r[e] = a;
-      }
-      load_face(2 * d, pt, 0, uo, go, un, gn, in, mo, mn, W, pen);
-      load_face(2 * d + 1, pt, 1, uo, go, un, gn, in, mo, mn, W, pen);
-    }
-    double cv[2] = {0, 0}, cd[2] = {0, 0};
-    face_pair_ml<N>(tab, d, 0, dir == 0 ? 1 : 2, p, q, uo, go, un, gn, in, mo, mn, W, pen, fb,
-                    active, cv, cd);
-    if (active) {
-#pragma unroll
-      for (int e = 0; e < N; ++e) {
-        double a = fma(tab.l1[e], cv[1], r[e]);
-        a = fma(tab.dl1[e], cd[1], a);
-        a = fma(tab.l0[e], cv[0], a);
-        r[e] = fma(tab.dl0[e], cd[0], a);
-      }
-#pragma unroll
-      for (int e = 0; e < N; ++e) sr[lbase + e * step] = r[e];
-    }
-    __syncthreads();
-  }
-  {  // x-lines (b = p, e = q)
-    double R[N];
-    bool in[2] = {false, false};
-    double uo[2] = {0, 0}, go[2] = {0, 0}, un[2] = {0, 0}, gn[2] = {0, 0}, W[2] = {0, 0},
-           pen[2] = {0, 0}, mo[2][3] = {}, mn[2][3] = {};
-    const int pt = p + N * q;
-    if (active) {
-      double rr[N], fx[N];
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        rr[i] = sr[q * N2 + p * N + i];
-        fx[i] = sg[0][q * N2 + p * N + i];
-      }
-      dgk::bt_bdt<N>(tab, rr, fx, R);
-      load_face(0, pt, 0, uo, go, un, gn, in, mo, mn, W, pen);
-      load_face(1, pt, 1, uo, go, un, gn, in, mo, mn, W, pen);
-    }
-    double cv[2] = {0, 0}, cd[2] = {0, 0};
-    face_pair_ml<N>(tab, 0, 1, 2, p, q, uo, go, un, gn, in, mo, mn, W, pen, fb, active, cv, cd);
-    if (active) {
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        double a = fma(tab.a1[i], cv[1], R[i]);
-        a = fma(tab.d1[i], cd[1], a);
-        a = fma(tab.a0[i], cv[0], a);
-        R[i] = fma(tab.d0[i], cd[0], a);
-      }
-#pragma unroll
-      for (int i = 0; i < N; ++i) sx[q * N2 + p * N + i] = R[i];
-    }
+    for (int j = 0; j < 3; ++j) sF[j * SC + zl + e * SZ] = F[j][e];
   }
   __syncthreads();
-  if (active) {
-    double v[N], R[N];
 #pragma unroll
-    for (int b = 0; b < N; ++b) v[b] = sx[q * N2 + b * N + p];
-    dgk::b_bwd<N>(tab, v, R);
+  for (int b = 0; b < N; ++b) {
+    r[b] = sr[yl + b * SY];
 #pragma unroll
-    for (int j = 0; j < N; ++j) sx[q * N2 + j * N + p] = R[j];
+    for (int j = 0; j < 3; ++j) F[j][b] = sF[j * SC + yl + b * SY];
+  }
+  faces(1);
+#pragma unroll
+  for (int b = 0; b < N; ++b) {
+    sr[yl + b * SY] = r[b];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) sF[j * SC + yl + b * SY] = F[j][b];
   }
   __syncthreads();
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    r[a] = sr[xl + a];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) F[j][a] = sF[j * SC + xl + a];
+  }
+  faces(0);
+  const int down = sh[55];
+  fx_deriv_t<N>(tg, F[0], v);
+#pragma unroll
+  for (int a = 0; a < N; ++a) {
+    sr[xl + a] = r[a] + (v[a] >> down);
+    sF[SC + xl + a] = F[1][a];
+    sF[2 * SC + xl + a] = F[2][a];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < N; ++b) u[b] = sF[SC + yl + b * SY];
+  fx_deriv_t<N>(tg, u, v);
+#pragma unroll
+  for (int b = 0; b < N; ++b) sr[yl + b * SY] += v[b] >> down;
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < N; ++e) u[e] = sF[2 * SC + zl + e * SZ];
+  fx_deriv_t<N>(tg, u, v);
+  unsigned big = 0;
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    r[e] = sr[zl + e * SZ] + (v[e] >> down);
+    big = max(big, fx_mag_hi(r[e]));
+  }
+  // Q^T along z, y, x, then out through the z-lines
+  const int up = FxScale<N>::S0 - fx_bits(fx_cell_max<N, T>(big, lc, slots));
+#pragma unroll
+  for (int e = 0; e < N; ++e) r[e] = fx_shift(r[e], up);
+  fx_bwd<N>(tab, r, u);
+#pragma unroll
+  for (int l = 0; l < N; ++l) su[zl + l * SZ] = u[l];
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < N; ++b) r[b] = su[yl + b * SY];
+  fx_bwd<N>(tab, r, u);
+#pragma unroll
+  for (int j = 0; j < N; ++j) su[yl + j * SY] = u[j];
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < N; ++a) r[a] = su[xl + a];
+  fx_bwd<N>(tab, r, u);
+#pragma unroll
+  for (int i = 0; i < N; ++i) su[xl + i] = u[i];
+  __syncthreads();
   if (active) {
-    double v[N], R[N];
+    const int ER = sh[56];
 #pragma unroll
-    for (int e = 0; e < N; ++e) v[e] = sx[e * N2 + q * N + p];
-    dgk::b_bwd<N>(tab, v, R);
-#pragma unroll
-    for (int l = 0; l < N; ++l) y[c * N3 + l * N2 + q * N + p] = R[l];
+    for (int l = 0; l < N; ++l)
+      y[c * N3 + l * N2 + pt] = ER == FX_NAN ? __longlong_as_double(0x7ff8000000000000ll)
+                                             : fx_to_double(su[zl + l * SZ], ER - up);
   }
 }
 
@@ -438,17 +675,29 @@ struct MlApplyF {
   template <typename T>
   static cudaError_t run(const dg_mesh* m, const double* x, double* yv, const int* skip,
                          cudaStream_t s) {
-    using Cf = MlCfg<N>;
-    const unsigned blocks = (unsigned)((m->ncells + Cf::CPB - 1) / Cf::CPB);
+    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
+    long long* U = reinterpret_cast<long long*>(m->U64);
+    long long* TR = reinterpret_cast<long long*>(m->TR64);
+    const MlData md{m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF};
     dg_timing_mark(m, 0, s);
-    dgk::k_trace<N, double><<<blocks, dgk::Cfg<N>::THREADS, dgk::trace_smem<N, double>(), s>>>(
-        x, m->U64, m->X64, m->TR64, 0, m->ncells, skip, m->tab64);
+    k_trace_ml<N><<<blocks, Cfg<N>::THREADS, MlSmem<N>::trace, s>>>(
+        x, U, TR, m->expU, m->mlF, m->ncells, skip, m->tabX, m->tabXG);
     dg_timing_mark(m, 1, s);
-    k_cell_ml<N><<<blocks, Cf::THREADS, Cf::smem(), s>>>(m->U64, m->X64, m->TR64, m->kt64,
-                                                         m->gh64, m->geo_vol, m->geo_face,
-                                                         m->geo_pen, yv, m->ncells, m->N, skip,
-                                                         m->tab64);
+    k_cell_ml<N><<<blocks, Cfg<N>::THREADS, MlSmem<N>::cell, s>>>(
+        U, TR, m->expU, md, yv, m->ncells, m->N, skip, m->tabX, m->tabXG);
     dg_timing_mark(m, 2, s);
+    return cudaGetLastError();
+  }
+};
+
+template <int N>
+struct MlSetupF {
+  template <typename T>
+  static cudaError_t run(const dg_mesh* m, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
+    k_ml_setup<N><<<blocks, Cfg<N>::THREADS, 0, s>>>(
+        m->kt64, m->gh64, m->geo_vol, m->geo_face, m->geo_pen,
+        MlData{m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF}, m->ncells, m->N, m->tabXG);
     return cudaGetLastError();
   }
 };
@@ -457,16 +706,33 @@ template <int N>
 struct MlPrepareF {
   template <typename T>
   static cudaError_t run() {
-    return cudaFuncSetAttribute(k_cell_ml<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)MlCfg<N>::smem());
+    cudaError_t e = cudaFuncSetAttribute(
+        k_trace_ml<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MlSmem<N>::trace);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_cell_ml<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)MlSmem<N>::cell);
+    return e;
   }
 };
 
-}  // namespace
+}  // namespace dgk
+
+int dg_setup_multilinear(dg_mesh* m, cudaStream_t s) {
+  const size_t n3 = (size_t)m->n * m->n * m->n, n2 = (size_t)m->n * m->n;
+  const size_t nc = (size_t)m->ncells;
+  if (m->mlV == nullptr) DG_CUDA(cudaMalloc((void**)&m->mlV, sizeof(FxPair) * 6 * n3 * nc));
+  if (m->mlF == nullptr) DG_CUDA(cudaMalloc((void**)&m->mlF, sizeof(FxPair) * 48 * n2 * nc));
+  if (m->mlExpV == nullptr) DG_CUDA(cudaMalloc((void**)&m->mlExpV, sizeof(int) * nc));
+  if (m->mlExpM == nullptr) DG_CUDA(cudaMalloc((void**)&m->mlExpM, sizeof(int) * nc));
+  if (m->mlExpF == nullptr) DG_CUDA(cudaMalloc((void**)&m->mlExpF, sizeof(int) * 18 * nc));
+  cudaError_t e = dgk::dispatch_n<double, dgk::MlSetupF>(m->n, (const dg_mesh*)m, s);
+  if (e != cudaSuccess) return dg_cuda_fail(e, "multilinear coefficient data: launch");
+  return DG_OK;
+}
 
 int dg_launch_apply_multilinear(const dg_mesh* m, const double* x, double* y, const int* skip,
                                 cudaStream_t s) {
-  cudaError_t e = dgk::dispatch_n<double, MlApplyF>(m->n, m, x, y, skip, s);
+  cudaError_t e = dgk::dispatch_n<double, dgk::MlApplyF>(m->n, m, x, y, skip, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "multilinear apply: launch");
   return DG_OK;
 }
@@ -514,7 +780,7 @@ extern "C" int dg_set_vertices(dg_mesh* m, const double* X) {
                    "dg_set_vertices: a cell's Jacobian determinant is not positive (inverted "
                    "or degenerate cell)");
   }
-  cudaError_t ea = dgk::dispatch_n<double, MlPrepareF>(m->n);
+  cudaError_t ea = dgk::dispatch_n<double, dgk::MlPrepareF>(m->n);
   if (ea != cudaSuccess) return dg_cuda_fail(ea, "multilinear apply: kernel attributes");
   m->multilinear = true;
   m->affine = false;
