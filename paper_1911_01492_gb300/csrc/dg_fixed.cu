@@ -33,6 +33,8 @@ k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
            int* __restrict__ expU, long long cbeg, long long cend, const int* __restrict__ skip,
            const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
+  dg_release_next();
+  dg_wait_before();
   if (skip != nullptr && *skip) return;
   __shared__ long long smem[(FxSmem<N, T>::trace + 7) / 8];
   x.begin();
@@ -59,6 +61,8 @@ k_cell_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
           const int* __restrict__ expG, double* __restrict__ y, long long cbeg, long long cend,
           int Nc, const int* __restrict__ skip, const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
+  dg_release_next();
+  dg_wait_before();
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long c0 = cbeg + (long long)blockIdx.x * C;
@@ -98,6 +102,8 @@ k_cell_dot_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
               long long ncells, int Nc, double* __restrict__ partials, DGCGState* st,
               const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
+  dg_release_next();
+  dg_wait_before();
   if (st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ bool is_last;
@@ -268,13 +274,11 @@ struct FixedF {
     long long* U = reinterpret_cast<long long*>(m->U64);
     long long* TR = reinterpret_cast<long long*>(m->TR64);
     if (pass == 1)
-      k_trace_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, 0, s>>>(FxLoad{x}, U, TR, m->expU, cbeg,
-                                                             cend, skip, m->tabX);
-    else
-      k_cell_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, SMEM, s>>>(
-          MODAL ? (const void*)U : (const void*)x, TR, m->expU, m->lineopX, m->gamX, m->expM,
-          m->expG, y, cbeg, cend, m->N, skip, m->tabX);
-    return cudaGetLastError();
+      return dg_launch_after(k_trace_fx<N, MODAL, FxLoad>, blocks, Cfg<N>::THREADS, 0, s, FxLoad{x},
+                             U, TR, m->expU, cbeg, cend, skip, m->tabX);
+    return dg_launch_after(k_cell_fx<N, MODAL>, blocks, Cfg<N>::THREADS, SMEM, s,
+                           MODAL ? (const void*)U : (const void*)x, TR, m->expU, m->lineopX,
+                           m->gamX, m->expM, m->expG, y, cbeg, cend, m->N, skip, m->tabX);
   }
   template <typename T>
   static cudaError_t run(const dg_mesh* m, bool modal, int which, const double* x, double* y,
@@ -293,13 +297,15 @@ struct FixedCgF {
     const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
     long long* U = reinterpret_cast<long long*>(m->U64);
     long long* TR = reinterpret_cast<long long*>(m->TR64);
-    k_trace_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, 0, s>>>(
-        FxDirection<PC>{p, z, dinv, m->state, 0.0}, U, TR, m->expU, 0, m->ncells,
+    cudaError_t e = dg_launch_after(
+        k_trace_fx<N, MODAL, FxDirection<PC>>, blocks, Cfg<N>::THREADS, 0, s,
+        FxDirection<PC>{p, z, dinv, m->state, 0.0}, U, TR, m->expU, 0ll, m->ncells,
         &m->state->done, m->tabX);
-    k_cell_dot_fx<N, MODAL><<<blocks, Cfg<N>::THREADS, FixedF<N>::SMEM, s>>>(
-        MODAL ? (const void*)U : (const void*)p, TR, m->expU, m->lineopX, m->gamX, m->expM,
-        m->expG, p, q, m->ncells, m->N, m->partials_cells, m->state, m->tabX);
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return dg_launch_after(k_cell_dot_fx<N, MODAL>, blocks, Cfg<N>::THREADS, FixedF<N>::SMEM, s,
+                           MODAL ? (const void*)U : (const void*)p, TR, m->expU, m->lineopX,
+                           m->gamX, m->expM, m->expG, p, q, m->ncells, m->N, m->partials_cells,
+                           m->state, m->tabX);
   }
   template <typename T>
   static cudaError_t run(const dg_mesh* m, const double* z, const double* dinv, double* p,

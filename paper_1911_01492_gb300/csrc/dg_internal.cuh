@@ -250,6 +250,35 @@ int dg_cuda_fail(cudaError_t e, const char* what);
     if (e__ != cudaSuccess) return dg_cuda_fail(e__, #call); \
   } while (0)
 
+// Dependent launches.  A kernel launched with dg_launch_after may be set up
+// while its predecessor in the stream still runs; it calls dg_wait_before
+// before it reads or writes anything, in every block and on every path, so that
+// it - and what follows it - sees the predecessor complete.  dg_release_next
+// lets the successor's blocks take the room that this grid's tail leaves.
+// 8^3 Q2 apply in a loop: 16.4 -> 12.3 us together with the raw stream handle in
+// the binding; large kernels gain about 1 %.
+__device__ __forceinline__ void dg_wait_before() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void dg_release_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... K, typename... A>
+cudaError_t dg_launch_after(void (*kernel)(K...), unsigned blocks, unsigned threads, size_t smem,
+                            cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
 // launchers (dg_apply_f64.cu, dg_mixed32.cu)
 // the FP64 operator in fixed point (dg_fixed.cu), for vectors of Legendre
 // coefficients (modal) or scaled point values: its coefficient data, one pass
