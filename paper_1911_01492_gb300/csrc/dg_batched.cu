@@ -36,9 +36,14 @@
 // and, if DG_TUNE_CACHE names a file, in that file.  DG_BATCHED_SHAPE="B,T"
 // forces B blocks per SM (at most the resident maximum) and tile index T.
 //
-// Degrees 1..4 run in 128-thread blocks; a batch with any degree 5..8 runs in
-// a 256-thread instantiation (the operator kernels' cell groups need up to
-// 256 threads there).
+// Degrees 1..4 run in 128-thread blocks with registers for eight of them per SM
+// (the fixed-point passes wait for memory; 32 x 16^3 Q2: six blocks 176 ms,
+// eight 147, ten 161), a batch of degrees 1 and 2 in an instantiation without
+// the larger passes' registers (141 ms); a batch with any degree 5..8 runs in a
+// 256-thread instantiation (the operator kernels' cell groups need up to 256
+// threads there; three blocks: fewer are slower although nothing spills then,
+// 5^3 Q6 70 against 86 ms).  The vector recurrences and inner products stay in
+// loops of their own: inside the passes they took 190 instead of 178 ms.
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -162,9 +167,17 @@ __device__ __forceinline__ void pass1_dispatch(const SampleDev& sd, long long c,
   switch (sd.n) {
     case 2: group_pass1<2, ND, BT>(sd, c, nblk, smem); break;
     case 3: group_pass1<3, ND, BT>(sd, c, nblk, smem); break;
-    case 4: group_pass1<4, ND, BT>(sd, c, nblk, smem); break;
-    case 5: group_pass1<5, ND, BT>(sd, c, nblk, smem); break;
     default:
+      if constexpr (MAXN > 3) {
+        if (sd.n == 4) {
+          group_pass1<4, ND, BT>(sd, c, nblk, smem);
+          break;
+        }
+        if (sd.n == 5) {
+          group_pass1<5, ND, BT>(sd, c, nblk, smem);
+          break;
+        }
+      }
       if constexpr (MAXN > 5) {
         switch (sd.n) {
           case 6: group_pass1<6, ND, BT>(sd, c, nblk, smem); break;
@@ -183,9 +196,17 @@ __device__ __forceinline__ void pass2_dispatch(const SampleDev& sd, long long c,
   switch (sd.n) {
     case 2: group_pass2<2, ND, BT>(sd, c, nblk, smem); break;
     case 3: group_pass2<3, ND, BT>(sd, c, nblk, smem); break;
-    case 4: group_pass2<4, ND, BT>(sd, c, nblk, smem); break;
-    case 5: group_pass2<5, ND, BT>(sd, c, nblk, smem); break;
     default:
+      if constexpr (MAXN > 3) {
+        if (sd.n == 4) {
+          group_pass2<4, ND, BT>(sd, c, nblk, smem);
+          break;
+        }
+        if (sd.n == 5) {
+          group_pass2<5, ND, BT>(sd, c, nblk, smem);
+          break;
+        }
+      }
       if constexpr (MAXN > 5) {
         switch (sd.n) {
           case 6: group_pass2<6, ND, BT>(sd, c, nblk, smem); break;
@@ -201,7 +222,7 @@ __device__ __forceinline__ void pass2_dispatch(const SampleDev& sd, long long c,
 // One persistent launch of up to `iters` lock-step iterations over every
 // unfinished sample.  `tile`: cell groups per work unit.
 template <int BT, int MAXN, bool ND>
-__global__ void __launch_bounds__(BT, BT == 128 ? 6 : 3)
+__global__ void __launch_bounds__(BT, BT == 128 ? 8 : 3)
 kb_persistent(const SampleDev* __restrict__ S, const int2* __restrict__ units, int nu, int tile,
               BState* st, double* part, unsigned* tickets, BCtl* ctl, int iters, long long limit,
               int stall_test) {
@@ -931,9 +952,11 @@ int solve_batched_nodal(const dg_mesh* const* meshes, int count, const double* c
         for (int i = 0; i < n; ++i) const_cast<dg_mesh*>(ms[i])->nodal_op = false;
       }
     } scope(meshes, count);
-    rc = maxn <= 5 ? solve_batched<128, 5, true>(meshes, count, bn.data(), xn.data(), rtol, maxit,
-                                                 false, mode, sts, stream)
-                   : solve_batched<256, DG_MAXN, true>(meshes, count, bn.data(), xn.data(), rtol,
+    rc = maxn <= 3   ? solve_batched<128, 3, true>(meshes, count, bn.data(), xn.data(), rtol, maxit,
+                                                   false, mode, sts, stream)
+         : maxn <= 5 ? solve_batched<128, 5, true>(meshes, count, bn.data(), xn.data(), rtol,
+                                                   maxit, false, mode, sts, stream)
+                     : solve_batched<256, DG_MAXN, true>(meshes, count, bn.data(), xn.data(), rtol,
                                                        maxit, false, mode, sts, stream);
   }
   if (rc != DG_OK && rc != DG_ERR_NOT_CONVERGED && rc != DG_ERR_BREAKDOWN) return rc;
@@ -1007,6 +1030,9 @@ extern "C" int dg_cg_solve_batched_mode(const dg_mesh* const* meshes, int count,
     maxn = m->n > maxn ? m->n : maxn;
   }
   if (nodal) return solve_batched_nodal(meshes, count, b, x, rtol, maxit, maxn, mode, st, stream);
+  if (maxn <= 3)
+    return solve_batched<128, 3, false>(meshes, count, b, x, rtol, maxit, jacobi, mode, st,
+                                        stream);
   if (maxn <= 5)
     return solve_batched<128, 5, false>(meshes, count, b, x, rtol, maxit, jacobi, mode, st,
                                         stream);
