@@ -40,28 +40,26 @@
 namespace dgk {
 
 // Sum of partials[0 .. count) in the last block of a grid reduction, by all
-// NT threads of the block in a fixed order: each thread keeps sixteen
-// independent chains of L2 loads (ld.global.cg: the other blocks' partials,
-// published before their ticket increment) - one SM reads them alone, so with
-// four chains 22,000 partials took 35 dependent round trips - then warp 0
-// adds the threads' sums with a fixed tree.  Valid in warp 0; every thread of
-// the block calls it.
+// NT threads of the block in a fixed order: each thread has eight independent
+// L2 loads in flight (ld.global.cg: the other blocks' partials, published
+// before their ticket increment), since one SM reads them alone: with four,
+// 22,000 partials took 35 dependent round trips; sixteen cost the FP32 kernels
+// resident blocks for their registers.  Then warp 0 adds the threads' sums
+// with a fixed tree.  Valid in warp 0; every thread of the block calls it.
 template <int NT>
 __device__ __forceinline__ double last_block_total(const double* __restrict__ partials,
                                                    int count, double* scratch) {
-  constexpr int CH = 16;
-  double a[CH];
-#pragma unroll
-  for (int k = 0; k < CH; ++k) a[k] = 0.0;
+  constexpr int CH = 8;
+  double a[CH / 2] = {};
   for (int b = threadIdx.x; b < count; b += CH * NT) {
     double v[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k) v[k] = b + k * NT < count ? __ldcg(partials + b + k * NT) : 0.0;
 #pragma unroll
-    for (int k = 0; k < CH; ++k) a[k] += v[k];
+    for (int k = 0; k < CH; ++k) a[k / 2] += v[k];
   }
 #pragma unroll
-  for (int w = CH / 2; w > 0; w /= 2)
+  for (int w = CH / 4; w > 0; w /= 2)
 #pragma unroll
     for (int k = 0; k < w; ++k) a[k] += a[k + w];
   scratch[threadIdx.x] = a[0];

@@ -619,7 +619,8 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
   std::vector<SampleDev> hs(count);
   std::vector<int2> hu[3];
   std::vector<SampleDev> hst3;
-  std::string sig = "bt" + std::to_string(BT) + "_mode" + std::to_string(mode);
+  std::string sig = "fx" + std::to_string(BT) + "n" + std::to_string(MAXN) + "_mode" +
+                    std::to_string(mode);
   long long total_dofs = 0;
   for (int s = 0; s < count; ++s) {
     dg_mesh* m = const_cast<dg_mesh*>(meshes[s]);
