@@ -75,7 +75,7 @@ k_cell_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
 // With FP64 passes that was slower than separate kernels (they shared the FP64
 // pipe); the fixed-point passes leave that pipe idle, and the two vector kernels,
 // their traffic (40 B per DOF) and their launches go.  32^3 Q3 with Jacobi:
-// 236 -> 213 ms per solve (with the shorter pass 2).
+// 236 -> 190 ms per solve, together with the shorter pass 2 and reductions.
 // Pass 1 of p = z + beta p, z = r, dinv r (PC) or M^-1 r already formed.
 template <bool PC>
 struct FxDirection {
@@ -91,15 +91,17 @@ struct FxDirection {
   }
 };
 
-// Pass 2 with <p, q> and alpha = rho / <p, q>: one partial per block, added by
-// the last block in a fixed order.
+// Pass 2 with <p, q> and alpha = rho / <p, q>: the products of point values are
+// integers already there (from p and q in FP64 they were 8 bytes of traffic and an
+// FP64 instruction per DOF: 201 -> 190 ms per solve); one partial per block, added
+// by the last block in a fixed order.
 template <int N, bool MODAL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, FxCellBlocks<N>::value)
 k_cell_dot_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
               const int* __restrict__ expU, const FxPair* __restrict__ lineop,
               const FxPair* __restrict__ gam, const int* __restrict__ expM,
-              const int* __restrict__ expG, const double* __restrict__ p, double* __restrict__ q,
-              long long ncells, int Nc, double* __restrict__ partials, DGCGState* st,
+              const int* __restrict__ expG, double* __restrict__ q, long long ncells, int Nc,
+              double* __restrict__ partials, DGCGState* st,
               const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
@@ -109,14 +111,9 @@ k_cell_dot_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
   __shared__ bool is_last;
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
-  double acc = 0.0;
-  fx_cell_cells<N, MODAL, T>(
-      xU, TR, expU, lineop, gam, expM, expG,
-      [&](long long i, double v) {
-        q[i] = v;
-        acc = fma(p[i], v, acc);
-      },
-      c0, nblk, Nc, tab, reinterpret_cast<long long*>(smem_raw));
+  const double acc = fx_cell_cells<N, MODAL, T, true>(
+      xU, TR, expU, lineop, gam, expM, expG, FxStore{q}, c0, nblk, Nc, tab,
+      reinterpret_cast<long long*>(smem_raw));
   __syncthreads();
   double* rd = reinterpret_cast<double*>(smem_raw);
   static_assert(FxSmem<N, T>::cell >= sizeof(double) * T, "reduction scratch");
@@ -304,7 +301,7 @@ struct FixedCgF {
     if (e != cudaSuccess) return e;
     return dg_launch_after(k_cell_dot_fx<N, MODAL>, blocks, Cfg<N>::THREADS, FixedF<N>::SMEM, s,
                            MODAL ? (const void*)U : (const void*)p, TR, m->expU, m->lineopX,
-                           m->gamX, m->expM, m->expG, p, q, m->ncells, m->N, m->partials_cells,
+                           m->gamX, m->expM, m->expG, q, m->ncells, m->N, m->partials_cells,
                            m->state, m->tabX);
   }
   template <typename T>

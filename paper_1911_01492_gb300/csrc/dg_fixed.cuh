@@ -377,9 +377,10 @@ __device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
 
 // Pass 2 over the cells c0 .. c0+nblk-1, called like pass 1; smem:
 // FxSmem<N, BT>::cell bytes.  xU: MODAL: the point values of pass 1 (integers);
-// otherwise the vector itself.
-template <int N, bool MODAL, int BT, typename YS>
-__device__ __forceinline__ void fx_cell_cells(
+// otherwise the vector itself.  DOT: returns the thread's part of <x, A x>,
+// formed from the point values and the sum r before Q^T (Q is orthogonal).
+template <int N, bool MODAL, int BT, bool DOT = false, typename YS>
+__device__ __forceinline__ double fx_cell_cells(
     const void* __restrict__ xU, const long long* __restrict__ TR, const int* __restrict__ expU,
     const FxPair* __restrict__ lineop, const FxPair* __restrict__ gam,
     const int* __restrict__ expM, const int* __restrict__ expG, YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
@@ -548,6 +549,17 @@ __device__ __forceinline__ void fx_cell_cells(
     r[a] = sr[q * SZ + p * SY + a];
   }
   line(0, false);
+  // u r / 2^60 in units 2^(eout - expM) 2^(eout - 1); r, below 2^62.3, three
+  // bits down
+  double dot = 0.0;
+  if constexpr (DOT) {
+    if (active) {
+      FxAcc A = {0, 0};
+#pragma unroll
+      for (int a = 0; a < N; ++a) fx_mac(A, fx_pair(r[a] >> 3), fx_split(u[a]));
+      dot = fx_scale(fma((double)A.m, 0x1p-30, (double)A.h), 2 * eout - expM[c] + 62);
+    }
+  }
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
   if (!MODAL) {
 #pragma unroll
@@ -561,7 +573,7 @@ __device__ __forceinline__ void fx_cell_cells(
       for (int e = 0; e < N; ++e)
         y(c * N3 + e * N2 + q * N + p, __longlong_as_double(sr[e * SZ + q * SY + p]));
     }
-    return;
+    return DOT && bad ? qnan : dot;
   }
   // the sum to a cell 2-norm of at most 2^60, then Q^T
   unsigned big = 0;
@@ -595,6 +607,7 @@ __device__ __forceinline__ void fx_cell_cells(
     for (int l = 0; l < N; ++l)
       y(c * N3 + l * N2 + q * N + p, bad ? qnan : fx_to_double(u[l], eout - 1 - up));
   }
+  return DOT && bad ? qnan : dot;
 }
 
 }  // namespace dgk
