@@ -54,36 +54,43 @@ CONFIG4 = {"n_cells": 32, "degree": 3, "K_seed": 5, "x_seed": 6, "K_ref_seed": 4
 BATCH_LEVELS = [(128, 16, 2), (96, 24, 3), (32, 32, 4)]   # (samples, n_cells, degree)
 METRIC = "SIPG-DG apply GDOF/s (FP64)"
 NOMINAL_FP64_TFLOPS = 1.25   # GB300 FP64 rate: 152 SMs x 2 DFMA/clk x 2 flop x ~2.06 GHz
-# Executed FP64 operations of the apply kernels at Q3 (DFMA counted 2, DADD and
-# DMUL 1), from ncu's sm__sass_thread_inst_executed_op_{dfma,dadd,dmul} counters
-# on 32^3 and 40^3 launches, which fit (per cell, per interior face side)
-# exactly (profiles/apply_fp64_q3_executed_flops.md).  Set an entry to None
-# when its kernel changes until it is counted again.
-EXEC_FP64_Q3 = {"k_trace": (1792.0, 0.0), "k_cell_lo": (3440.0, 64.0),
-                "k_trace_nd": (1344.0, 0.0), "k_cell_nd": (3008.0, 64.0)}
-# The same counters as FP64 instructions (DFMA, DADD and DMUL one each: every
-# one takes an issue slot of the FP64 pipe, whatever its flops), per cell and
-# per interior face side, exact at both sizes
-EXEC_FP64_INSTR_Q3 = {"k_trace": (1136.0, 0.0), "k_cell_lo": (1984.0, 48.0),
-                      "k_trace_nd": (768.0, 0.0), "k_cell_nd": (1536.0, 48.0)}
+HBM_FALLBACK_GBS = 6800.0    # one measurement on a GB300, if MEASURED_PEAKS.json is absent
 
 
-def executed_fp64_per_dof(kernel: str, N: int, n: int, table=None):
-    """Executed FP64 operations (or, with table=EXEC_FP64_INSTR_Q3, FP64
-    instructions) per DOF of one launch on an N^3 mesh (Q3 only)."""
-    e = (table or EXEC_FP64_Q3).get(kernel) if n == 4 else None
-    if e is None:
+def hbm_gbs():
+    """Measured copy bandwidth of this GPU model in GB/s, and where it is from."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["hbm_gbs"]), "measured copy bandwidth"
+    except (OSError, ValueError, KeyError):
+        return HBM_FALLBACK_GBS, "fallback copy bandwidth"
+
+
+def pass_bytes_per_dof(kernel: str, n: int):
+    """Bytes per DOF that one launch of a fixed-point kernel reads and writes,
+    every array once (csrc/dg_fixed.cuh, dg_multilinear.cu), in 8-byte words:
+    k_trace_fx   x, the point values (Legendre basis only), 12 n^2 trace words per cell;
+    k_cell_fx    the point values, the line operators 3 n^2 n(n+1)/2, one trace pair
+                 per neighbour face point, six face coefficients, y;
+    k_cell_ml    the point values, 6 metric words, 5 coefficients per face point,
+                 own and neighbour trace pairs, y."""
+    words = {"k_trace_fx": 2 + 12 / n, "k_trace_fx_nd": 1 + 12 / n,
+             "k_cell_fx": 2 + 1.5 * (n + 1) + 12 / n + 10 / n ** 3,
+             "k_cell_ml": 8 + 30 / n + 24 / n}
+    return 8.0 * words[kernel]
+
+
+def memory_roofline(kernel, n, nd, ms):
+    """Achieved bandwidth of one launch against the measured copy bandwidth."""
+    if ms <= 0:
         return None
-    per_cell, per_face_side = e
-    face_sides = 6 * N * N * (N - 1)       # interior faces, seen from both cells
-    return (per_cell * N ** 3 + per_face_side * face_sides) / (N ** 3 * n ** 3)
-
-
-# DRAM bytes (read + write) per DOF of one pass-2 launch (k_cell_lo<4,double>),
-# from an ncu capture of the 40^3 Q3 case (462.4 MB read + 27.6 MB written for
-# 4,096,000 DOFs), scaled by DOFs to the benchmark's launch; set to None when
-# the kernel changes until it is captured again.
-K_CELL_TRAFFIC_PER_DOF = (462.4e6 + 27.6e6) / 4096000
+    peak, source = hbm_gbs()
+    b = pass_bytes_per_dof(kernel, n)
+    a = b * nd / (ms * 1e-3) / 1e9
+    return {"bound": "memory", "kernel": kernel, "unit": "GB/s", "achieved": a, "peak": peak,
+            "frac": a / peak, "bytes_per_dof": b, "traffic": b * nd, "peak_source": source,
+            "traffic_source": "every array of the kernel once; ncu on 40^3 Q3 counts 99 B per "
+                              "DOF for k_cell_fx"}
 
 
 def flops_per_dof(n: int):
@@ -705,11 +712,10 @@ def run_fp32_apply(m, xd, world, steps=8):
             "pass_ms": {"pass1": ms1 / max(napp, 1), "pass2": ms2 / max(napp, 1)}}
 
 
-def run_nodal_apply(m, xd, world, peak_fp64=None, steps=8):
+def run_nodal_apply(m, xd, world, steps=8):
     """The operator of the benchmark workload in the scaled Gauss-point basis
     (dg_apply_nodal, the apply inside DG_CG_NODAL solves), timed like `value`,
-    with per-pass times, executed FP64 rates from the ncu counts and its
-    one-time setup (the basis's line operators)."""
+    with per-pass times and bandwidths."""
     import torch
     xh = m.to_nodal(xd)
     yh = torch.empty_like(xh)
@@ -719,18 +725,9 @@ def run_nodal_apply(m, xd, world, peak_fp64=None, steps=8):
     t1, t2 = ms1 / max(napp, 1), ms2 / max(napp, 1)
     out = {"workload": "the benchmark workload, x mapped to the scaled Gauss-point basis",
            "apply_gdof_s": world * nd * steps * APPLIES_PER_STEP / (ms * 1e-3) / 1e9,
-           "pass_ms": {"k_trace_nd": t1, "k_cell_nd": t2}}
-    if peak_fp64:
-        for name, t in (("k_trace_nd", t1), ("k_cell_nd", t2)):
-            epd = executed_fp64_per_dof(name, WORKLOAD["n_cells"], n)
-            ipd = executed_fp64_per_dof(name, WORKLOAD["n_cells"], n, EXEC_FP64_INSTR_Q3)
-            if epd is not None and t > 0:
-                a = epd * nd / (t * 1e-3) / 1e12
-                rate = ipd * nd / (t * 1e-3) / 1e12
-                out.setdefault("roofline", {})[name] = {
-                    "executed_flops_per_dof": epd, "achieved_tflops": a, "peak": peak_fp64,
-                    "frac": a / peak_fp64, "fp64_instructions_per_dof": ipd,
-                    "issue_frac": rate / (peak_fp64 / 2)}
+           "pass_ms": {"k_trace_fx": t1, "k_cell_fx": t2},
+           "roofline": {"k_trace_fx": memory_roofline("k_trace_fx_nd", n, nd, t1),
+                        "k_cell_fx": memory_roofline("k_cell_fx", n, nd, t2)}}
     return out
 
 
@@ -774,12 +771,11 @@ def run_geometry_probe(n_cells: int, applies: int = 4):
         m.close()
 
 
-# Executed FP64 operations per DOF of the geometry pass-2 kernels at Q3 (ncu
-# instruction counters, DFMA x2 + DADD + DMUL): k_cell_aff 11,056 per cell at
-# 32^3 and 40^3 alike, k_cell_ml 12,571 per cell at 32^3
-EXEC_FP64_GEOMETRY_Q3 = {"k_cell_aff": 11056 / 64, "k_cell_ml": 12571 / 64}
-# and as FP64 instructions (DFMA + DADD + DMUL) per DOF: 6,528 and 7,281 per cell
-EXEC_FP64_INSTR_GEOMETRY_Q3 = {"k_cell_aff": 6528 / 64, "k_cell_ml": 7281 / 64}
+# Executed FP64 operations per DOF of the affine pass-2 kernel at Q3 (ncu
+# instruction counters, DFMA x2 + DADD + DMUL): 11,056 per cell at 32^3 and 40^3
+# alike, and as FP64 instructions (DFMA + DADD + DMUL) 6,528 per cell
+EXEC_FP64_GEOMETRY_Q3 = {"k_cell_aff": 11056 / 64}
+EXEC_FP64_INSTR_GEOMETRY_Q3 = {"k_cell_aff": 6528 / 64}
 
 
 def _geometry_roofline(kernel, n, nd, ms, peak_fp64):
@@ -824,10 +820,10 @@ def run_affine(world, K64, peak_fp64=None):
     ms, napp, ms1, ms2 = time_applies(m, x, y, steps, 2, world)
     out["multilinear"] = {"perturbation": "interior vertices moved by up to 0.2 h (seed 7)",
                           "apply_gdof_s": world * nd * steps * APPLIES_PER_STEP / (ms * 1e-3) / 1e9,
-                          "pass_ms": {"k_trace": ms1 / max(napp, 1),
+                          "pass_ms": {"k_trace_ml": ms1 / max(napp, 1),
                                       "k_cell_ml": ms2 / max(napp, 1)},
-                          "roofline": _geometry_roofline("k_cell_ml", k + 1, nd,
-                                                         ms2 / max(napp, 1), peak_fp64)}
+                          "roofline": memory_roofline("k_cell_ml", k + 1, nd,
+                                                      ms2 / max(napp, 1))}
     m.close()
     del x, y
     N2, k2 = 32, 3
@@ -1017,59 +1013,21 @@ def run_nodal_probe(n_cells: int, applies: int = 4):
 
 
 def roofline_entry(N, n, nd, napp, ms1, ms2, ms_step, peak_fp64):
-    """Roofline of the dominant apply kernel against the FP64 pipe: executed
-    FP64 operations (ncu counts per DOF) per launch over its CUDA-event
-    duration, divided by the FP64 rate measured in this run."""
+    """Roofline of the dominant apply kernel: its bytes per launch over its
+    CUDA-event duration against the measured copy bandwidth.  The operator's
+    contractions run on the integer pipe, so the FP64 rate measured in this run
+    is context: the algorithmic flops (FMA = 2) per second exceed it."""
     f1, f2 = flops_per_dof(n)
     t1, t2 = ms1 / max(napp, 1), ms2 / max(napp, 1)
-    if t2 >= t1:
-        dom_ms, dom_alg, dom_name, slot = t2, f2 * nd, "k_cell_lo", "k_cell_lo"
-    else:
-        dom_ms, dom_alg, dom_name, slot = t1, f1 * nd, "k_trace", "k_trace"
-    exec_per_dof = executed_fp64_per_dof(slot, N, n)
-    other = "k_trace" if slot == "k_cell_lo" else "k_cell_lo"
-    exec_other = executed_fp64_per_dof(other, N, n)
-    alg_tflops = dom_alg / (dom_ms * 1e-3) / 1e12
-    r = {"bound": "alu", "kernel": dom_name, "unit": "TFLOP/s",
-         "pass_ms": {"k_trace": t1, "k_cell_lo": t2},
-         "algorithmic_tflops": alg_tflops,
-         "apply_tflops_algorithmic": (f1 + f2) * nd / (ms_step * 1e-3 / APPLIES_PER_STEP) / 1e12,
-         "peak_nominal": NOMINAL_FP64_TFLOPS,
-         "peak_source": "FP64 DFMA throughput measured in this run by dg_peak_probe "
-                        "(best of 6 launches filling every SM); nominal 1.25"}
-    if exec_per_dof is not None:
-        achieved = exec_per_dof * nd / (dom_ms * 1e-3) / 1e12
-        r.update({"achieved": achieved, "peak": peak_fp64, "frac": achieved / peak_fp64,
-                  "executed_flops_per_dof": exec_per_dof,
-                  "frac_of_nominal": achieved / NOMINAL_FP64_TFLOPS,
-                  "achieved_source": "executed FP64 operations per DOF from ncu instruction "
-                                     "counters (DFMA x2 + DADD + DMUL) x DOFs / live "
-                                     "CUDA-event duration of the kernel"})
-    else:
-        r.update({"achieved": alg_tflops, "peak": peak_fp64, "frac": alg_tflops / peak_fp64,
-                  "achieved_source": "algorithmic flops (no executed-operation count for "
-                                     "this kernel build)"})
-    # the FP64 pipe's issue rate: instructions per launch over the launch time,
-    # against the DFMA instruction rate of the probe (its flops / 2)
-    issue = {}
-    for name, t in (("k_trace", t1), ("k_cell_lo", t2)):
-        ipd = executed_fp64_per_dof(name, N, n, EXEC_FP64_INSTR_Q3)
-        if ipd is not None and t > 0:
-            rate = ipd * nd / (t * 1e-3) / 1e12
-            issue[name] = {"fp64_instructions_per_dof": ipd, "achieved_tinst_s": rate,
-                           "peak_tinst_s": peak_fp64 / 2, "frac": rate / (peak_fp64 / 2)}
-    if issue:
-        r["fp64_issue"] = issue
-    if exec_other is not None:
-        t_other = t1 if other == "k_trace" else t2
-        r["other_kernel"] = {"kernel": other, "executed_flops_per_dof": exec_other,
-                             "achieved": exec_other * nd / (t_other * 1e-3) / 1e12,
-                             "frac": exec_other * nd / (t_other * 1e-3) / 1e12 / peak_fp64}
-    traffic = (K_CELL_TRAFFIC_PER_DOF * nd
-               if (dom_name == "k_cell_lo" and n == 4 and K_CELL_TRAFFIC_PER_DOF) else None)
-    r["traffic"] = traffic
-    r["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the pass-2 "
-                           "kernel on 40^3 Q3, scaled by DOFs")
+    name, t, other, to = (("k_cell_fx", t2, "k_trace_fx", t1) if t2 >= t1
+                          else ("k_trace_fx", t1, "k_cell_fx", t2))
+    r = memory_roofline(name, n, nd, t)
+    r["pass_ms"] = {"k_trace_fx": t1, "k_cell_fx": t2}
+    r["other_kernel"] = memory_roofline(other, n, nd, to)
+    r["apply_tflops_algorithmic"] = \
+        (f1 + f2) * nd / (ms_step * 1e-3 / APPLIES_PER_STEP) / 1e12
+    r["fp64_peak_measured_tflops"] = peak_fp64
+    r["fp64_peak_nominal_tflops"] = NOMINAL_FP64_TFLOPS
     return r
 
 
@@ -1175,7 +1133,7 @@ def main(argv=None):
     fp32 = nodal = None
     if not args.no_extra:
         fp32 = _leg(run_fp32_apply, m, xd, world)
-        nodal = _leg(run_nodal_apply, m, xd, world, peak_fp64)
+        nodal = _leg(run_nodal_apply, m, xd, world)
     cg2 = cg = K48 = None
     if not args.no_cg:
         cg2 = _leg(run_config2_cg, m, world)
