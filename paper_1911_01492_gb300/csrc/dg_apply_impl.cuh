@@ -81,6 +81,20 @@ struct Cfg {
   static constexpr int THREADS = CPB * N * N;
 };
 
+// Barrier between the threads of a cell.  The n^2 threads of a cell exchange
+// lines only among themselves; where they are part of one warp (n = 2, 4) the
+// warp's barrier is enough, and warps of a block run on independently.  Every
+// thread of the block calls it.  64^3 Q3 pass 2: block barriers throughout
+// 331 us, the block's in the prologue and the warp's after it 318, the warp's
+// throughout 337 (the warps drift apart and share fewer lines).
+template <int N>
+__device__ __forceinline__ void cell_sync() {
+  if constexpr (32 % (N * N) == 0)
+    __syncwarp();
+  else
+    __syncthreads();
+}
+
 // Shared-memory strides of a cell's n x n x n values: with an odd row length the
 // x- and y-lines of the lanes of a warp start on different banks.
 template <int N>
@@ -402,7 +416,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
 #pragma unroll
     for (int e = 0; e < N; ++e) sc[e * SZ + q * SY + p] = u[e];
   }
-  __syncthreads();
+  cell_sync<N>();
   // along y: thread owns (i = p, e = q)
   if (active) {
     T v[N], u[N];
@@ -412,7 +426,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
 #pragma unroll
     for (int b = 0; b < N; ++b) sc[q * SZ + b * SY + p] = u[b];
   }
-  __syncthreads();
+  cell_sync<N>();
   // along x: thread owns (b = p, e = q); X is modal in x, nodal in y and z
   T* tr = (MODE == 3) ? nullptr : TR + c * (12 * N2);
   if (active) {
@@ -455,7 +469,7 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
     }
   }
   if (MODE == 3) return;  // the caller synchronises before reading s
-  __syncthreads();
+  cell_sync<N>();
   if (active) {
     // y-faces: thread owns points (a = p, e = q); z-faces: (a = p, b = q)
 #pragma unroll

@@ -291,7 +291,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
   constexpr int NS = FxSmem<N, BT>::NS;
   if (32 % N2 != 0) {
     if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
-    __syncthreads();
+    cell_sync<N>();
   }
   double xv[N];
   unsigned big = 0;
@@ -313,7 +313,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
 #pragma unroll
     for (int e = 0; e < N; ++e)
       if (live) sc[e * SZ + q * SY + p] = u[e];
-    __syncthreads();
+    cell_sync<N>();
     // along y: (i = p, e = q)
 #pragma unroll
     for (int j = 0; j < N; ++j) v[j] = sc[q * SZ + j * SY + p];
@@ -321,7 +321,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
 #pragma unroll
     for (int b = 0; b < N; ++b)
       if (live) sc[q * SZ + b * SY + p] = u[b];
-    __syncthreads();
+    cell_sync<N>();
     // along x: (b = p, e = q)
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = sc[q * SZ + p * SY + i];
@@ -351,7 +351,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
   }
   if (E == FX_NAN) eu = FX_NAN;
   if (active && pt == 0) expU[c] = eu;
-  __syncthreads();
+  cell_sync<N>();
   if (!active) return;  // no barrier follows
   long long* tr = TR + c * (12 * N2);
   if (MODAL) {
@@ -404,20 +404,22 @@ __device__ __forceinline__ double fx_cell_cells(
   const unsigned nu = (unsigned)Nc;
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
   // exponents of the seven contributions to a cell
-  for (int i = threadIdx.x; i < nblk * 7; i += BT) {
-    const int l2 = i / 7, f = i - l2 * 7, d = f >> 1;
-    const long long cc = c0 + l2;
-    const unsigned row = (unsigned)cc / nu;
-    const int crd = d == 0 ? (int)((unsigned)cc - row * nu) : d == 1 ? (int)(row % nu) : (int)(row / nu);
-    int e;
-    if (f == 6) {
-      e = expU[cc] + expM[cc];
-    } else {
-      const long long st = f & 1 ? stride[d] : -stride[d];
-      e = (f & 1 ? crd < Nc - 1 : crd > 0) ? expU[cc + st] + expG[cc * 6 + f] : -4 * FX_NAN;
+  const unsigned row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  if (active) {
+    for (int f = pt; f < 7; f += N2) {
+      int e;
+      if (f == 6) {
+        e = expU[c] + expM[c];
+      } else {
+        const int d = f >> 1, cd = d == 0 ? crd[0] : d == 1 ? crd[1] : crd[2];
+        const long long st = d == 0 ? stride[0] : d == 1 ? stride[1] : stride[2];
+        e = (f & 1 ? cd < Nc - 1 : cd > 0) ? expU[f & 1 ? c + st : c - st] + expG[c * 6 + f]
+                                           : -4 * FX_NAN;
+        sg[lc][f] = gam[c * 6 + f];
+      }
+      sexp[lc][f] = e;
     }
-    sexp[l2][f] = e;
-    if (f < 6) sg[l2][f] = gam[cc * 6 + f];
   }
   if (MODAL && 32 % N2 != 0 && threadIdx.x < FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
   long long u[N], r[N];
@@ -436,7 +438,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
     for (int k = 0; k < NP; ++k) Mz[k] = lineop[((c * 3 + 2) * NP + k) * N2 + pt];
   }
-  __syncthreads();
+  __syncthreads();  // the block's: its warps start on neighbouring cells together
   const int eown = sexp[active ? lc : 0][6];
   int eout = eown;
 #pragma unroll
@@ -464,8 +466,6 @@ __device__ __forceinline__ double fx_cell_cells(
     }
   }
   __syncthreads();
-  const unsigned row = (unsigned)c / nu;
-  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   // r (= or +=) the line's terms: |r| < 2^62.3 in the end
   auto line = [&](int dir, bool first) {
     const FxPair* Mp = lineop + ((c * 3 + dir) * NP) * N2 + pt;
@@ -530,7 +530,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
   for (int e = 0; e < N; ++e)
     if (live) sr[e * SZ + q * SY + p] = r[e];
-  __syncthreads();
+  cell_sync<N>();
   // y-lines (a = p, e = q)
 #pragma unroll
   for (int b = 0; b < N; ++b) {
@@ -541,7 +541,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
   for (int b = 0; b < N; ++b)
     if (live) sr[q * SZ + b * SY + p] = r[b];
-  __syncthreads();
+  cell_sync<N>();
   // x-lines (b = p, e = q): the sum of all three directions
 #pragma unroll
   for (int a = 0; a < N; ++a) {
@@ -567,7 +567,7 @@ __device__ __forceinline__ double fx_cell_cells(
       if (live)
         sr[q * SZ + p * SY + a] =
             __double_as_longlong(bad ? qnan : fx_to_double(r[a], eout - 1));
-    __syncthreads();
+    cell_sync<N>();
     if (active) {  // written from the z-lines: consecutive lanes, consecutive words
 #pragma unroll
       for (int e = 0; e < N; ++e)
@@ -589,7 +589,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
   for (int i = 0; i < N; ++i)
     if (live) su[q * SZ + p * SY + i] = u[i];
-  __syncthreads();
+  cell_sync<N>();
   // y: (i = p, e = q)
 #pragma unroll
   for (int b = 0; b < N; ++b) r[b] = su[q * SZ + b * SY + p];
@@ -597,7 +597,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
   for (int j = 0; j < N; ++j)
     if (live) su[q * SZ + j * SY + p] = u[j];
-  __syncthreads();
+  cell_sync<N>();
   // z: (i = p, j = q)
 #pragma unroll
   for (int e = 0; e < N; ++e) r[e] = su[e * SZ + q * SY + p];

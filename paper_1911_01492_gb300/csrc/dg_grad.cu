@@ -37,7 +37,7 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
              const double* __restrict__ kt, const double* __restrict__ dgam, double h,
              double* __restrict__ g, long long ncells, int Nc,
              const __grid_constant__ DGTabXGrad tab) {
-  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, T = Cfg<N>::THREADS;
+  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long c0 = (long long)blockIdx.x * C;
@@ -54,15 +54,16 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
       reinterpret_cast<int(*)[14]>(reinterpret_cast<double*>(smem_raw) + 3 * C * SC + C * (N2 + N));
   const unsigned nu = (unsigned)Nc;
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
+  const unsigned row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   // exponents of u (0..6) and v (7..13): six neighbours, own
-  for (int i = threadIdx.x; i < nblk * 14; i += T) {
-    const int l2 = i / 14, k = i - l2 * 14, f = k % 7, d = f >> 1;
-    const long long cc = c0 + l2;
-    const unsigned row = (unsigned)cc / nu;
-    const int crd = d == 0 ? (int)((unsigned)cc - row * nu)
-                    : d == 1 ? (int)(row % nu) : (int)(row / nu);
-    const bool in = f < 6 && ((f & 1) ? crd < Nc - 1 : crd > 0);
-    sexp[l2][k] = (k < 7 ? eu : ev)[in ? ((f & 1) ? cc + stride[d] : cc - stride[d]) : cc];
+  if (active) {
+    for (int k = pt; k < 14; k += N2) {
+      const int f = k % 7, d = f >> 1, cd = d == 0 ? crd[0] : d == 1 ? crd[1] : crd[2];
+      const long long st = d == 0 ? stride[0] : d == 1 ? stride[1] : stride[2];
+      const bool in = f < 6 && ((f & 1) ? cd < Nc - 1 : cd > 0);
+      sexp[lc][k] = (k < 7 ? eu : ev)[in ? ((f & 1) ? c + st : c - st) : c];
+    }
   }
   long long u[N], v[N];
 #pragma unroll
@@ -79,8 +80,6 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
 #pragma unroll
   for (int k = 0; k < 14; ++k) top = max(top, se[k]);
   const bool bad = top >= FX_NAN / 2;
-  const unsigned row = (unsigned)c / nu;
-  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   double s = 0.0;  // the line's six face points, weighted by d gamma
   // the volume products of the line (twice), added to r (or replacing it)
   auto line = [&](int dir, long long (&r)[N], bool first) {

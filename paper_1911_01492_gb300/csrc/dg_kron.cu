@@ -373,7 +373,7 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
   auto put = [&](int at, int step) {
 #pragma unroll
     for (int i = 0; i < N; ++i) sc[at + i * step] = u[i];
-    __syncthreads();
+    cell_sync<N>();
   };
   auto get = [&](int at, int step) {
 #pragma unroll

@@ -343,7 +343,6 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   F2* sk = sr + C * SC;
   __shared__ float rh[DOT ? NT : 1], rl[DOT ? NT : 1];
   __shared__ bool is_last;
-  __shared__ int sbase[3];
   const long long c0 = cbeg + (long long)blockIdx.x * (2 * C);
   const int lc = threadIdx.x / N2;
   const int t2 = threadIdx.x - lc * N2;
@@ -351,21 +350,13 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   const long long ca = c0 + 2 * lc, cb = ca + 1;
   const bool va = ca < ncells, vb = cb < ncells;
   const int o = lc * SC;
-  if (threadIdx.x == 0) {
-    const unsigned cu = (unsigned)c0, n = (unsigned)Nc;
-    sbase[0] = (int)(cu % n);
-    sbase[1] = (int)((cu / n) % n);
-    sbase[2] = (int)(cu / n / n);
-  }
   // h w K of the block's cell pairs into registers (stored to shared memory
   // after pass 1), in flight together with the z-line loads of p
   F2 kreg[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const int t = threadIdx.x + k * NT;  // < C N3 = N NT
-    const int pr = t / N3, pos = t - pr * N3;
-    const long long c = c0 + 2 * pr;
-    kreg[k] = F2(c < ncells ? kt[c * N3 + pos] : 0.0f, c + 1 < ncells ? kt[(c + 1) * N3 + pos] : 0.0f);
+    const int pos = k * N2 + t2;
+    kreg[k] = F2(va ? kt[ca * N3 + pos] : 0.0f, vb ? kt[cb * N3 + pos] : 0.0f);
   }
   // pass 1 in shared memory.  z-lines: thread owns (i = p, j = q); it loads its
   // z-line of p (both cells) and keeps it for <p, q>
@@ -381,7 +372,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
 #pragma unroll
     for (int e = 0; e < N; ++e) su[o + e * SZ + q * SY + p] = u[e];
   }
-  __syncthreads();
+  cell_sync<N>();
   {  // y-lines: (i = p, e = q)
     F2 v[N], u[N];
 #pragma unroll
@@ -390,7 +381,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
 #pragma unroll
     for (int b = 0; b < N; ++b) su[o + q * SZ + b * SY + p] = u[b];
   }
-  __syncthreads();
+  cell_sync<N>();
   {  // x-lines: (b = p, e = q); X (x-modal) kept in sx, nodal values in su
     F2 X[N], u[N];
 #pragma unroll
@@ -402,20 +393,11 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
     for (int a = 0; a < N; ++a) su[o + q * SZ + p * SY + a] = u[a];
   }
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const int t = threadIdx.x + k * NT;  // cell, then e, b, a
-    sk[t / N3 * SC + t % N3 / N2 * SZ + t % N2 / N * SY + t % N] = kreg[k];
-  }
+  for (int k = 0; k < N; ++k) sk[o + k * SZ + q * SY + p] = kreg[k];
   // cell coordinates of both lanes; interior flags as bits (face f: bit f for
   // lane a, bit 8 + f for lane b)
-  int cxa = sbase[0] + 2 * lc, cya = sbase[1], cza = sbase[2];
-  while (cxa >= Nc) {
-    cxa -= Nc;
-    if (++cya == Nc) {
-      cya = 0;
-      ++cza;
-    }
-  }
+  const unsigned nu = (unsigned)Nc, rowa = (unsigned)ca / nu;
+  const int cxa = (int)((unsigned)ca - rowa * nu), cya = (int)(rowa % nu), cza = (int)(rowa / nu);
   int cxb = cxa + 1, cyb = cya, czb = cza;
   if (cxb == Nc) {
     cxb = 0;
@@ -447,7 +429,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   face(5, va && cza < Nc - 1, vb && czb < Nc - 1, ca + sz, cb + sz, un[1], gn[1], wh[1], ee[1]);
   face(2, va && cya > 0, vb && cyb > 0, ca - sy, cb - sy, un[2], gn[2], wh[2], ee[2]);
   face(3, va && cya < Nc - 1, vb && cyb < Nc - 1, ca + sy, cb + sy, un[3], gn[3], wh[3], ee[3]);
-  __syncthreads();
+  cell_sync<N>();
   // flux of one face point from the own trace (uo, go) and the face data:
   // cv multiplies the test value, -cd the test derivative
   auto flux = [&](bool upper, F2 uo, F2 go, F2 unf, F2 gnf, F2 whf, F2 ef, F2& cv, F2& cd) {
@@ -510,7 +492,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
       face(1, va && cxa < Nc - 1, vb && cxb < Nc - 1, ca + 1, cb + 1, un[1], gn[1], wh[1],
            ee[1], !pairrow, true);
     }
-    __syncthreads();
+    cell_sync<N>();
   }
   {  // x-lines: (b = p, e = q); result x-modal, yz-nodal
     const int base = q * SZ + p * SY;
@@ -559,7 +541,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
 #pragma unroll
     for (int i = 0; i < N; ++i) sx[o + base + i] = R[i];
   }
-  __syncthreads();
+  cell_sync<N>();
   {  // back along y: (i = p, e = q)
     F2 v[N], R[N];
 #pragma unroll
@@ -568,7 +550,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
 #pragma unroll
     for (int j = 0; j < N; ++j) sx[o + q * SZ + j * SY + p] = R[j];
   }
-  __syncthreads();
+  cell_sync<N>();
   // back along z: (i = p, j = q), the thread's z-line of q: store it and fold
   // <p, q> over it (exact products, compensated float-float sums per lane)
   F2 hi = F2(0.0f), lo = F2(0.0f);
