@@ -319,8 +319,8 @@ def time_e2e(m, xh, yh, steps, warmup, world, per_step=APPLIES_PER_STEP):
 
 
 def time_setup(m, Kd, reps=3):
-    """Wall time of dg_set_coefficient (coefficient kernels, line operators,
-    face weights and its blocking validity check), best of reps."""
+    """Wall time of dg_set_coefficient (coefficient kernels, line operators
+    and its blocking validity check), best of reps."""
     import torch
     best = 1e300
     for _ in range(reps):

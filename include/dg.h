@@ -159,7 +159,7 @@ int dg_apply_adjoint(const dg_mesh* mesh, const void* ybar, void* xbar, int prec
 /* Same as dg_apply but x and y are HOST buffers (pinned or pageable): the
  * Section 3.3 operator application with the host<->device copies inside the
  * call (the paper has no counterpart; it runs on host memory throughout).  The
- * mesh is cut into at most 16 slabs of z-layers: x is copied in slab by slab
+ * mesh is cut into slabs of z-layers, one per 3 MB and at most 16: x is copied in slab by slab
  * on a copy stream, pass 1 of each slab runs on an internal stream as soon as
  * its x has arrived, pass 2 of slab s runs on `stream` once pass 1 has covered
  * slab s+1, and y is copied back slab by slab on a second copy stream, so that
@@ -224,10 +224,8 @@ int dg_coeff_grad(const dg_mesh* mesh, const double* u, const double* v, double*
  *   the Legendre basis, and if the mapping's rounding left it above rtol, the
  *   same solver (precision and preconditioner) continues from x in the
  *   Legendre basis (its iterations counted in iterations, one more outer
- *   iteration).  Formed on the first such solve after dg_set_coefficient: the
- *   line operators of Q A Q^T (as many values as dg_set_coefficient's, ~7.5
- *   doubles per DOF at degree 3), two solve vectors, for the mixed mode h K at
- *   the points in FP32, for the Kronecker blocks the rotated factors.  Cube
+ *   iteration).  Formed on the first such solve after dg_set_coefficient:
+ *   two solve vectors, for the mixed mode h K at the points in FP32, for the Kronecker blocks the rotated factors.  Cube
  *   meshes only.
  * Stops when ||b - A x|| <= rtol ||b|| recomputed in FP64.  Blocking.
  * Returns NOT_CONVERGED at maxit (x holds the last iterate), BREAKDOWN on
@@ -390,8 +388,7 @@ int dg_peak_probe(int kind, double* tflops, void* stream);
  * `stream`; INVALID_ARG on NULL, aliased vectors or an affine or multilinear
  * mesh.  dg_apply_nodal: y_hat = (Q A(K) Q^T) x_hat in FP64 (two kernels:
  * face traces by Lagrange end values, then per-line operators and neighbour
- * face terms); its first call after dg_set_coefficient forms the line
- * operators of Q A Q^T (allocated once per mesh). */
+ * face terms), with the line operators that dg_set_coefficient formed. */
 int dg_to_nodal(const dg_mesh* mesh, const double* x, double* xhat, void* stream);
 int dg_to_modal(const dg_mesh* mesh, const double* xhat, double* x, void* stream);
 int dg_apply_nodal(const dg_mesh* mesh, const double* xhat, double* yhat, void* stream);

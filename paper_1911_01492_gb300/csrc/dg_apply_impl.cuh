@@ -1,5 +1,7 @@
 // Sum-factorised SIPG operator application y = A(K) x (Section 3.3 applied to
-// the Section 4.1 form), in two passes over the cells.
+// the Section 4.1 form), in two passes over the cells, in floating point: the
+// affine geometry's pass 1, the allocation-free apply, and the building blocks
+// of the FP32 kernels.  The FP64 cube operator is in dg_fixed.cuh.
 //
 // Pass 1 (trace kernel), per cell: modal -> nodal values by three 1D
 // contractions with B[a][i] = L_i(xi_a) (along z, then y, then x).  It keeps
@@ -291,63 +293,16 @@ template <typename T>
 struct FaceGlobal {
   const T* TR;
   const T* FW;
-  static constexpr bool OWN_IN_THREAD = false;  // own traces come from TR
   struct Pre {};  // nothing prefetched: the FP64 kernels hide load latency behind the FP64 pipe
   template <int N>
   __device__ __forceinline__ void prefetch(Pre&, long long, int, const bool (&)[6],
                                            const long long (&)[6]) const {}
   template <int N, bool UPPER>
   __device__ __forceinline__ void get(const Pre&, long long c, int lc, int f, bool in,
-                                      long long cn, int fn, int pt, T, T, T& cv,
+                                      long long cn, int fn, int pt, T& cv,
                                       T& cdm) const {
     (void)lc;
     face_point<N, UPPER>(TR, FW, c, f, in, cn, fn, pt, cv, cdm);
-  }
-};
-
-// FaceLocal: own traces formed by the calling line-thread from its own line's
-// values (passed in as uo, go), neighbour traces from the pass-1 buffer,
-// weights from h*gamma per face (W/2 = h gamma w_s w_t / 2; the derivative
-// weight doubles on the boundary).
-// The global loads (neighbour traces, h*gamma) of all six faces are issued
-// together by prefetch() when the cell phase starts, so their latency overlaps
-// the volume work instead of stalling each direction's face step.
-template <typename T>
-struct FaceLocal {
-  const T* TR;
-  const T* gh;
-  const DGTab<T>* tab;
-  static constexpr bool OWN_IN_THREAD = true;
-  struct Pre {
-    T un[6], gn[6], wh[6];  // neighbour trace; W/2 = h gamma w_s w_t / 2 per face
-  };
-  // in[f], cn[f]: whether face f is interior and its neighbour cell; the
-  // neighbour's face is f ^ 1 (x- <-> x+, ...).
-  template <int N>
-  __device__ __forceinline__ void prefetch(Pre& pre, long long c, int pt, const bool (&in)[6],
-                                           const long long (&cn)[6]) const {
-    // the line's face point has the same Gauss weights on all six faces
-    const T hw2 = T(0.5) * tab->w[pt % N] * tab->w[pt / N];
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      pre.un[f] = T(0);
-      pre.gn[f] = T(0);
-      if (in[f]) load_trace<N>(TR, cn[f], f ^ 1, pt, pre.un[f], pre.gn[f]);
-      pre.wh[f] = hw2 * gh[c * 6 + f];
-    }
-  }
-  template <int N, bool UPPER>
-  __device__ __forceinline__ void get(const Pre& pre, long long c, int lc, int f, bool in,
-                                      long long cn, int fn, int pt, T uo, T go, T& cv,
-                                      T& cdm) const {
-    (void)c;
-    (void)lc;
-    (void)cn;
-    (void)fn;
-    (void)pt;
-    const T un = pre.un[f], gn = in ? pre.gn[f] : go;
-    const T wh = pre.wh[f];
-    flux<N, UPPER>(uo, go, un, gn, wh, in ? wh : wh + wh, cv, cdm);
   }
 };
 
@@ -362,9 +317,7 @@ struct FaceLocal {
 // in the loads and barriers.
 // trace_core: s already holds the cells' modal coefficients.
 //   MODE 0 (pass 1): writes U, X and the face traces to global memory;
-//   MODE 2: writes only the face traces to global memory;
-//   MODE 3: leaves U in s and copies X to sx, no traces (the cell phase forms
-//           each line's own traces itself, FaceLocal).
+//   MODE 2: writes only the face traces to global memory.
 // Default z-line input of trace_core: the line's modal values already in s.
 struct ZFromShared {
   template <int N, typename T>
@@ -397,7 +350,7 @@ struct ZFromGlobal {
 template <int N, typename T, int MODE, typename ZL = ZFromShared, int SY = N, int SZ = N * N>
 __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm,
                                            T* __restrict__ TR, long long c0, int nblk,
-                                           const DGTab<T>& tab, T* s, T* sx,
+                                           const DGTab<T>& tab, T* s,
                                            const ZL& zload = ZL()) {
   constexpr int N2 = N * N, N3 = N * N * N, H = N / 2;
 
@@ -428,19 +381,19 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
   }
   cell_sync<N>();
   // along x: thread owns (b = p, e = q); X is modal in x, nodal in y and z
-  T* tr = (MODE == 3) ? nullptr : TR + c * (12 * N2);
+  T* tr = TR + c * (12 * N2);
   if (active) {
     T X[N], u[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) X[i] = sc[q * SZ + p * SY + i];
     if (MODE != 2) {
-      T* xm = (MODE == 0) ? Xm + c * N3 + q * N2 + p * N : sx + lc * N3 + q * N2 + p * N;
+      T* xm = Xm + c * N3 + q * N2 + p * N;
 #pragma unroll
       for (int i = 0; i < N; ++i) xm[i] = X[i];
     }
     // x-face traces from the modes: L_i(1) = a_i, L_i(0) = (-1)^i a_i,
     // L_i'(1) = d_i, L_i'(0) = (-1)^(i+1) d_i, a_0 = 1, d_0 = 0
-    if (MODE != 3) {
+    {
       T Se = X[0], So = tab.a1[1] * X[1];
 #pragma unroll
       for (int i = 2; i < N; i += 2) Se = fma(tab.a1[i], X[i], Se);
@@ -468,7 +421,6 @@ __device__ __forceinline__ void trace_core(T* __restrict__ U, T* __restrict__ Xm
       if (MODE == 0) U[c * N3 + q * N2 + p * N + a] = u[a];
     }
   }
-  if (MODE == 3) return;  // the caller synchronises before reading s
   cell_sync<N>();
   if (active) {
     // y-faces: thread owns points (a = p, e = q); z-faces: (a = p, b = q)
@@ -513,7 +465,7 @@ __device__ __forceinline__ void trace_cells(const T* __restrict__ x, T* __restri
   constexpr int N3 = N * N * N;
   // each z-line thread loads its own line of x: no staging barrier
   const ZFromGlobal<T> zl{x + c0 * N3};
-  trace_core<N, T, 0>(U, Xm, TR, c0, nblk, tab, s, nullptr, zl);
+  trace_core<N, T, 0>(U, Xm, TR, c0, nblk, tab, s, zl);
 }
 
 template <int N, typename T>
@@ -617,24 +569,8 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       const bool inl = (dir == 0) ? (cz > 0) : (cy > 0);
       const long long st = (dir == 0) ? sz : sy;
       T cv1, cd1, cv0, cd0;
-      // own traces of the line's end points (FaceLocal only): Lagrange end
-      // values and derivatives of the line's nodal values
-      T vm = T(0), vp = T(0), gm = T(0), gp = T(0);
-      if constexpr (FS::OWN_IN_THREAD) {
-        vm = tab.l0[0] * u[0];
-        vp = tab.l1[0] * u[0];
-        gm = tab.dl0[0] * u[0];
-        gp = tab.dl1[0] * u[0];
-#pragma unroll
-        for (int e = 1; e < N; ++e) {
-          vm = fma(tab.l0[e], u[e], vm);
-          vp = fma(tab.l1[e], u[e], vp);
-          gm = fma(tab.dl0[e], u[e], gm);
-          gp = fma(tab.dl1[e], u[e], gp);
-        }
-      }
-      fs.template get<N, true>(pre, c, lc, fu, inu, c + st, fl, pt, vp, gp, cv1, cd1);
-      fs.template get<N, false>(pre, c, lc, fl, inl, c - st, fu, pt, vm, gm, cv0, cd0);
+      fs.template get<N, true>(pre, c, lc, fu, inu, c + st, fl, pt, cv1, cd1);
+      fs.template get<N, false>(pre, c, lc, fl, inl, c - st, fu, pt, cv0, cd0);
 #pragma unroll
       for (int e = 0; e < N; ++e) {
         T acc = fma(tab.l1[e], cv1, r[e]);
@@ -664,29 +600,8 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       bt_bdt<N>(tab, rr, kg, R);
     }
     T cv1, cd1, cv0, cd0;
-    // own x-face traces from the modes (FaceLocal only): L_i(1) = a_i,
-    // L_i(0) = (-1)^i a_i, L_i'(1) = d_i, L_i'(0) = (-1)^(i+1) d_i
-    T xm = T(0), xp = T(0), dxm = T(0), dxp = T(0);
-    if constexpr (FS::OWN_IN_THREAD) {
-      T Se = X[0], So = tab.a1[1] * X[1], Do = tab.d1[1] * X[1], De = T(0);
-#pragma unroll
-      for (int i = 2; i < N; i += 2) Se = fma(tab.a1[i], X[i], Se);
-#pragma unroll
-      for (int i = 3; i < N; i += 2) So = fma(tab.a1[i], X[i], So);
-#pragma unroll
-      for (int i = 3; i < N; i += 2) Do = fma(tab.d1[i], X[i], Do);
-      if (N > 2) {
-        De = tab.d1[2] * X[2];
-#pragma unroll
-        for (int i = 4; i < N; i += 2) De = fma(tab.d1[i], X[i], De);
-      }
-      xm = Se - So;
-      xp = Se + So;
-      dxm = Do - De;
-      dxp = Do + De;
-    }
-    fs.template get<N, true>(pre, c, lc, 1, cx < Nc - 1, c + 1, 0, pt, xp, dxp, cv1, cd1);
-    fs.template get<N, false>(pre, c, lc, 0, cx > 0, c - 1, 1, pt, xm, dxm, cv0, cd0);
+    fs.template get<N, true>(pre, c, lc, 1, cx < Nc - 1, c + 1, 0, pt, cv1, cd1);
+    fs.template get<N, false>(pre, c, lc, 0, cx > 0, c - 1, 1, pt, cv0, cd0);
     // modal test functions: value a_i at 1, (-1)^i a_i at 0; derivative -d_i cd
     // at 1, -(-1)^(i+1) d_i cd at 0 (a_0 = 1, d_0 = 0)
     const T sp = cv1 + cv0, sm = cv1 - cv0;

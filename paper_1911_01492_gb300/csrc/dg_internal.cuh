@@ -171,8 +171,8 @@ struct dg_mesh {
   double* kronW;
   bool has_kron_x, has_kron_nx;
   // scaled Gauss-point basis (DG_CG_NODAL, dg_nodal.cu): its 1D tables, the
-  // line operators and Jacobi diagonal of Q A Q^T (formed on first use after
-  // the coefficient is set) and the solve's b and x in that basis
+  // Jacobi diagonal of Q A Q^T (formed on first use after the coefficient is
+  // set) and the solve's b and x in that basis
   DGTabN<double> tabN64;
   DGTabN<float> tabN32;
   bool has_nodal_diag;
@@ -325,7 +325,7 @@ int dg_prepare_apply_f32(int n);
 int dg_prepare_grad(int n);
 
 // scaled Gauss-point basis (dg_nodal.cu): tables (at mesh creation), the
-// line operators of Q A Q^T and solve vectors (formed if needed), its Jacobi
+// solve vectors (formed if needed), its Jacobi
 // diagonal, the FP64 apply of Q A Q^T, and x_hat = Q x / x = Q^T x_hat
 void dg_build_nodal_tables(const DGTab<double>& t, int n, DGTabN<double>* d, DGTabN<float>* f);
 int dg_ensure_nodal(dg_mesh* m, cudaStream_t s);

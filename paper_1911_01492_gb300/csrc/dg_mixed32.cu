@@ -284,7 +284,7 @@ k_dir32_bulk(const float* __restrict__ r, float* __restrict__ p, float* __restri
       if constexpr (ND)
         trace_core_nd<N, float>(TR, cg0, nblk, tn, bp(b), zl);
       else
-        trace_core<N, float, 2>(nullptr, nullptr, TR, cg0, nblk, tab, bp(b), nullptr, zl);
+        trace_core<N, float, 2>(nullptr, nullptr, TR, cg0, nblk, tab, bp(b), zl);
       __syncthreads();
     }
   }
@@ -961,7 +961,7 @@ struct PrepareMixed32F {
 // dg_apply in FP32.  Pass 1 writes the face traces only; pass 2 (k_cell32x2)
 // transforms x again in shared memory, which costs less than the nodal and
 // x-modal workspaces' 16 bytes per DOF of traffic, two cells per instruction.
-// 64^3 Q3: 220 us with the generic passes, 129 us now; 48^3 Q4 183 and 115 us.
+// 64^3 Q3: 220 us with the generic passes, 127 us now; 48^3 Q4 183 and 115 us.
 // ---------------------------------------------------------------------------
 template <int N>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
@@ -975,7 +975,7 @@ k_trace32(const float* __restrict__ x, float* __restrict__ TR, long long cbeg, l
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
   const ZFromGlobal<float> zl{x + c0 * N3};
   trace_core<N, float, 2, ZFromGlobal<float>, LP::SY, LP::SZ>(nullptr, nullptr, TR, c0, nblk, tab,
-                                                              s, nullptr, zl);
+                                                              s, zl);
 }
 
 // pass 1 or 2 of the FP32 operator over the cells [cbeg, cend)

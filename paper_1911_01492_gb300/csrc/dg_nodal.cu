@@ -10,17 +10,15 @@
 // (Q A Q^T) x_hat = Q b produces exactly Q times the iterates of CG on
 // A x = b, since Q preserves every inner product.
 //
-// Why: in the Legendre basis every application of A spends its FP64
-// instructions on six 1D basis transforms per cell (three forward, three
-// back), about a quarter of the FP64 work at Q3.  In the scaled point basis
+// Why: in the Legendre basis every application of A spends six 1D basis
+// transforms per cell (three forward, three back).  In the scaled point basis
 // those transforms vanish: pass 1 only forms face traces (Lagrange end values
 // of each line), pass 2 only applies the per-line operators (the volume term
 // and the own-side face terms) and the neighbours' face terms.  A solve maps b
 // and x into the basis once and x back once.
 //
 // In that basis the scaling is folded into the data: the line operators of
-// Q A Q^T are those of A_pt times isw_i isw_j / (w_s w_t) (k_line_ops<N,
-// true>); the Lagrange end values carry isw_a = 1/sqrt(w_a); the face weight
+// Q A Q^T are those of A_pt times isw_i isw_j / (w_s w_t) (k_lines_fx, dg_fixed.cu); the Lagrange end values carry isw_a = 1/sqrt(w_a); the face weight
 // h gamma w_s w_t / 2 of a face point loses its tangential weights against
 // the two isw factors of the traces, so every point of a face has the weight
 // h gamma / 2 and no per-point face-weight array is read.
