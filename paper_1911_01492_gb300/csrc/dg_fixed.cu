@@ -214,13 +214,14 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
       const int E = eK + t.ch + 1;
       g[m] = fx_split(fx_from_double(w, 60 - E, E));
       if (pt == 0) {
-        // normalised to [2^60, 2^61), taking up the table scales 2^cg
+        // normalised to [2^59, 2^60), taking up the table scales 2^cg (an octave
+        // higher the largest mantissas would round to 2^61, past what a pair holds)
         const double w2 = fx_abs_hi(w) < 0x00100000u ? w * 0x1p64 : w;
         const int e = (int)(fx_abs_hi(w2) >> 20);
         const long long mant = (__double_as_longlong(w2) & 0xfffffffffffffll) | 0x10000000000000ll;
-        gam[c * 6 + 2 * dir + m] = w > 0.0 ? fx_pair(mant << 8) : FxPair{0, 0};
+        gam[c * 6 + 2 * dir + m] = w > 0.0 ? fx_pair(mant << 7) : FxPair{0, 0};
         expG[c * 6 + 2 * dir + m] =
-            w > 0.0 ? e - 1022 - (fx_abs_hi(w) < 0x00100000u ? 64 : 0) + cg : -2 * FX_NAN;
+            w > 0.0 ? e - 1021 - (fx_abs_hi(w) < 0x00100000u ? 64 : 0) + cg : -2 * FX_NAN;
       }
     }
     unsigned long long rs[N];
@@ -251,7 +252,9 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   }
   __syncthreads();
   if (!active) return;
-  // largest row sum over the three directions to (2^60, 2^61]
+  // the sum of the directions' largest row sums to (2^60, 2^61]: each direction
+  // holds the cell's largest K against table rows of similar size (within 2^6 for
+  // every n), so an entry stays clear of a pair's upper end
   const int bits = 68 - __clzll((long long)(rmax[lc][0] + rmax[lc][1] + rmax[lc][2]));
   const int up = 61 - bits;
   if (t2 == 0) expM[c] = sbad[lc] ? FX_NAN : eK + t.cB - up + 1;

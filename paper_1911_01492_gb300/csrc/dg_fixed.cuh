@@ -10,8 +10,8 @@
 // 1204 with FP64 multiply-adds.
 //
 // Number format.  A value v stands for v 2^E with E per cell.  A constant or
-// coefficient T in (-2, 2) is stored as T 2^60 = h 2^30 + l with |l| <= 2^29
-// (FxPair).  A value splits as v = h 2^30 + l with 0 <= l < 2^30.  Their product
+// coefficient T is stored as T 2^60 = h 2^30 + l with |l| <= 2^29 (FxPair); h is a
+// 32-bit integer, so T < 2 - 2^-31.  A value splits as v = h 2^30 + l with 0 <= l < 2^30.  Their product
 // over 2^60 is h h' + (h l' + l h') / 2^30, where the l l' term (below 2^-1 of
 // the last place) is left out: an absolute error of about one unit, 2^-59 of the
 // cell's largest value, against 2^-53 of each partial sum in FP64.
@@ -77,6 +77,10 @@ __device__ __forceinline__ long long fx_value(const FxAcc& a) {
   return (a.h << SH) + (a.m >> (30 - SH));
 }
 
+// -2^61 - 2^29 <= t < 2^61 - 2^29.  Who calls it: values below 2^60 (face
+// coefficients, metric terms, derivatives and traces, eigenbases), sums brought
+// down to that, and line operator entries, whose row sums are at most 2^61 in
+// three directions together.
 __device__ __forceinline__ FxPair fx_pair(long long t) {
   const int h = (int)((t + (1ll << 29)) >> 30);
   return {h, (int)(t - ((long long)h << 30))};

@@ -100,15 +100,16 @@ bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGra
   }
   const int cv = ceil_log2(V), ca = ceil_log2(A), cl = ceil_log2(lm) - 1;
   t->cg = ca + cl;
-  // one face adds at most gamma (lm A + dm V) max|u|; six of them, each
-  // 2^bump below the common exponent, stay within 1.45 of the own terms' bound
+  // one face adds at most gamma (lm A + dm V) max|u| with gamma below half of its
+  // exponent's unit; six of them, each 2^bump below the common exponent, stay
+  // within 1.45 of the own terms' bound
   const ld kappa = (lm * A + dm * V) / ldexpl(1, ca + cl);
-  t->bump = ceil_log2(6 * kappa / 1.45L);
+  t->bump = ceil_log2(3 * kappa / 1.45L);
   for (int a = 0; a < n; ++a)
     for (int i = 0; i < n; ++i) t->q[a][i] = pair_of(q[a][i]);
   bool ok = true;
   auto put = [&ok](ld v) {
-    ok = ok && fabsl(v) < 2;
+    ok = ok && fabsl(v) < 2 - 0x1p-30L;  // a pair ends just below 2
     return pair_of(v);
   };
   for (int a = 0; a < (n + 1) / 2; ++a) {
