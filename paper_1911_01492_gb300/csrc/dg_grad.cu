@@ -15,6 +15,12 @@
 //   -(Pu Jv + Pv Ju) - sigma Ju Jv = -(Gu Jv + Gv Ju),  G = P + sigma J / 2;
 // a boundary point is the same with the other side's value zero, P twice the own
 // combination and 3 sigma / 2 in place of sigma / 2.
+// Precision.  The gradient of a smooth field is small against the field, so a
+// product of two gradients, rounded to the last place of the cell's largest
+// value, would lose twice the digits that each factor has lost.  Every factor is
+// therefore brought up to the full range by itself before it is multiplied
+// (fx_top) and a point's sum carries its own exponent: what the products add is
+// below 2^-59 of each of them.
 // FP64 is left to 10 instructions per DOF (the FP64 kernel executed 60); 32^3 Q3:
 // pass 1 of both and this kernel 445 -> 102 us.
 #include "dg_fixed.cuh"
@@ -24,10 +30,33 @@ namespace dgk {
 template <int N>
 struct GradCfg {
   static constexpr int C = Cfg<N>::CPB, N2 = N * N;
-  // u, v, the volume products; per-line and per-row face sums; exponents
+  // u, v, the volume products; per-line and per-row face sums; exponents of the
+  // neighbours and of the points' products
   static constexpr size_t SMEM =
-      8 * (3 * C * LinePad<N>::SC + C * (N2 + N)) + 4 * (14 * C);
+      8 * (3 * C * LinePad<N>::SC + C * (N2 + N)) + 4 * (14 * C + C * LinePad<N>::SC);
 };
+
+// v 2^s with |v| 2^s in [2^59, 2^60) (s <= 28 when the upper half is zero); e -= s
+__device__ __forceinline__ long long fx_top(long long v, int& e) {
+  const int s = 60 - fx_bits(fx_mag_hi(v));
+  e -= s;
+  return fx_shift(v, s);
+}
+
+// a b / 2^60 with both factors at the top of the range
+__device__ __forceinline__ long long fx_product(long long a, long long b) {
+  FxAcc A = fx_zero();
+  fx_mac(A, fx_pair(a), fx_split(b));
+  return fx_value(A);
+}
+
+// r 2^er + v 2^ev under the larger exponent, left in er
+__device__ __forceinline__ long long fx_sum(long long r, int& er, long long v, int ev) {
+  const int e = max(er, ev);
+  const long long t = (r >> min(e - er, 63)) + (v >> min(e - ev, 63));
+  er = e;
+  return t;
+}
 
 template <int N>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
@@ -52,6 +81,7 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
   double* sf = reinterpret_cast<double*>(smem_raw) + 3 * C * SC + lc * (N2 + N);
   int(*sexp)[14] =
       reinterpret_cast<int(*)[14]>(reinterpret_cast<double*>(smem_raw) + 3 * C * SC + C * (N2 + N));
+  int* se2 = reinterpret_cast<int*>(sexp + C) + lc * SC;  // exponents of sg
   const unsigned nu = (unsigned)Nc;
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
   const unsigned row = (unsigned)c / nu;
@@ -81,16 +111,22 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
   for (int k = 0; k < 14; ++k) top = max(top, se[k]);
   const bool bad = top >= FX_NAN / 2;
   double s = 0.0;  // the line's six face points, weighted by d gamma
-  // the volume products of the line (twice), added to r (or replacing it)
-  auto line = [&](int dir, long long (&r)[N], bool first) {
+  // the volume products of the line, added to r 2^er (or replacing it)
+  auto line = [&](int dir, long long (&r)[N], int (&er)[N], bool first) {
     long long gu[N], gv[N];
     fx_deriv<N>(tab, u, gu);
     fx_deriv<N>(tab, v, gv);
 #pragma unroll
     for (int e = 0; e < N; ++e) {
-      FxAcc A = fx_zero<1>();
-      fx_mac(A, fx_pair(gu[e]), fx_split(gv[e]));
-      r[e] = first ? fx_value<1>(A) : r[e] + fx_value<1>(A);
+      int ep = 0;
+      const long long a = fx_top(gu[e], ep), b = fx_top(gv[e], ep);
+      const long long pr = fx_product(a, b);
+      if (first) {
+        r[e] = pr;
+        er[e] = ep;
+      } else {
+        r[e] = fx_sum(r[e], er[e], pr, ep);
+      }
     }
 #pragma unroll
     for (int up = 0; up < 2; ++up) {
@@ -113,39 +149,52 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
       int e1, e2;
       side(TRu, se[6], se[f], Ju, Pu, e1);
       side(TRv, se[13], se[7 + f], Jv, Pv, e2);
-      const FxVal ju = fx_split(Ju), jv = fx_split(Jv);
-      FxAcc A = fx_zero<2>(), B = fx_zero<2>(), F = fx_zero<2>();
-      fx_mac(A, tab.cj[in ? 0 : 1], ju);
-      fx_mac(B, tab.cj[in ? 0 : 1], jv);
-      fx_mac(F, fx_pair(Pu + fx_value<2>(A)), jv);
-      fx_mac(F, fx_pair(Pv + fx_value<2>(B)), ju);
-      s = fma(dgam[c * 6 + f], fx_to_double(fx_value<2>(F), e1 + e2 + 58 + tab.cva), s);
+      FxAcc A = fx_zero<2>(), B = fx_zero<2>();
+      fx_mac(A, tab.cj[in ? 0 : 1], fx_split(Ju));
+      fx_mac(B, tab.cj[in ? 0 : 1], fx_split(Jv));
+      int e3 = 0, e4 = 0;
+      const long long Gu = fx_top(Pu + fx_value<2>(A), e3), ju = fx_top(Ju, e4);
+      const long long Gv = fx_top(Pv + fx_value<2>(B), e4), jv = fx_top(Jv, e3);
+      const long long F = fx_sum(fx_product(Gu, jv), e3, fx_product(Gv, ju), e4);
+      s = fma(dgam[c * 6 + f], fx_to_double(F, e1 + e2 + e3 + 60 + tab.cva), s);
     }
   };
   long long r[N];
-  line(2, r, true);
+  int er[N];
+  line(2, r, er, true);
 #pragma unroll
-  for (int e = 0; e < N; ++e) sg[e * SZ + q * SY + p] = r[e];
+  for (int e = 0; e < N; ++e) {
+    sg[e * SZ + q * SY + p] = r[e];
+    se2[e * SZ + q * SY + p] = er[e];
+  }
   __syncthreads();
 #pragma unroll
   for (int b = 0; b < N; ++b) {  // y-lines (a = p, e = q)
     u[b] = su[q * SZ + b * SY + p];
     v[b] = sv[q * SZ + b * SY + p];
     r[b] = sg[q * SZ + b * SY + p];
+    er[b] = se2[q * SZ + b * SY + p];
   }
-  line(1, r, false);
+  line(1, r, er, false);
 #pragma unroll
-  for (int b = 0; b < N; ++b) sg[q * SZ + b * SY + p] = r[b];
+  for (int b = 0; b < N; ++b) {
+    sg[q * SZ + b * SY + p] = r[b];
+    se2[q * SZ + b * SY + p] = er[b];
+  }
   __syncthreads();
 #pragma unroll
   for (int a = 0; a < N; ++a) {  // x-lines (b = p, e = q)
     u[a] = su[q * SZ + p * SY + a];
     v[a] = sv[q * SZ + p * SY + a];
     r[a] = sg[q * SZ + p * SY + a];
+    er[a] = se2[q * SZ + p * SY + a];
   }
-  line(0, r, false);
+  line(0, r, er, false);
 #pragma unroll
-  for (int a = 0; a < N; ++a) sg[q * SZ + p * SY + a] = r[a];
+  for (int a = 0; a < N; ++a) {
+    sg[q * SZ + p * SY + a] = r[a];
+    se2[q * SZ + p * SY + a] = er[a];
+  }
   // the cell's face sum in a fixed order: rows of n threads, then n rows
   sf[pt] = s;
   __syncthreads();
@@ -162,11 +211,12 @@ k_coeff_grad(const long long* __restrict__ Uu, const long long* __restrict__ TRu
   // each thread writes the n points of its z-line
   const double ws = -h * s * (tab.w[p] * tab.w[q]);
   const double is = tab.iw[p] * tab.iw[q];
-  const int ex = se[6] + se[13] + 59 + 2 * tab.cD;
+  const int ex = se[6] + se[13] + 60 + 2 * tab.cD;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     const long long at = c * N3 + e * N2 + q * N + p;
-    const double vol = fx_to_double(sg[e * SZ + q * SY + p], ex);
+    const int o = e * SZ + q * SY + p;
+    const double vol = fx_to_double(sg[o], ex + se2[o]);
     const double val = fma(kt[at] * (is * tab.iw[e]), vol, ws * tab.w[e]);
     g[at] = bad ? __longlong_as_double(0x7ff8000000000000ll) : val;
   }
