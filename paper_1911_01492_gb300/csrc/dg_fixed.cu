@@ -30,7 +30,7 @@ namespace dgk {
 template <int N, bool MODAL, typename XL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
 k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
-           int* __restrict__ expU, long long cbeg, long long cend, const int* __restrict__ skip,
+           int* __restrict__ expU, long long cbeg, long long cend, const int* skip,
            const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
@@ -55,11 +55,11 @@ struct FxCellBlocks {
 
 template <int N, bool MODAL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, FxCellBlocks<N>::value)
-k_cell_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
-          const int* __restrict__ expU, const FxPair* __restrict__ lineop,
+k_cell_fx(const void* xU, const long long* TR, const int* expU,
+          const FxPair* __restrict__ lineop,
           const FxPair* __restrict__ gam, const int* __restrict__ expM,
           const int* __restrict__ expG, double* __restrict__ y, long long cbeg, long long cend,
-          int Nc, const int* __restrict__ skip, const __grid_constant__ DGTabX tab) {
+          int Nc, const int* skip, const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
   dg_wait_before();
@@ -97,8 +97,8 @@ struct FxDirection {
 // by the last block in a fixed order.
 template <int N, bool MODAL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, FxCellBlocks<N>::value)
-k_cell_dot_fx(const void* __restrict__ xU, const long long* __restrict__ TR,
-              const int* __restrict__ expU, const FxPair* __restrict__ lineop,
+k_cell_dot_fx(const void* xU, const long long* TR, const int* expU,
+              const FxPair* __restrict__ lineop,
               const FxPair* __restrict__ gam, const int* __restrict__ expM,
               const int* __restrict__ expG, double* __restrict__ q, long long ncells, int Nc,
               double* __restrict__ partials, DGCGState* st,

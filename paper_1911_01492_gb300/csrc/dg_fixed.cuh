@@ -385,9 +385,9 @@ __device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
 // formed from the point values and the sum r before Q^T (Q is orthogonal).
 template <int N, bool MODAL, int BT, bool DOT = false, typename YS>
 __device__ __forceinline__ double fx_cell_cells(
-    const void* __restrict__ xU, const long long* __restrict__ TR, const int* __restrict__ expU,
-    const FxPair* __restrict__ lineop, const FxPair* __restrict__ gam,
-    const int* __restrict__ expM, const int* __restrict__ expG, YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
+    const void* xU, const long long* TR, const int* expU, const FxPair* __restrict__ lineop,
+    const FxPair* __restrict__ gam, const int* __restrict__ expM, const int* __restrict__ expG,
+    YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;

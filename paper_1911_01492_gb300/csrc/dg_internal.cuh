@@ -253,7 +253,12 @@ int dg_cuda_fail(cudaError_t e, const char* what);
 // Dependent launches.  A kernel launched with dg_launch_after may be set up
 // while its predecessor in the stream still runs; it calls dg_wait_before
 // before it reads or writes anything, in every block and on every path, so that
-// it - and what follows it - sees the predecessor complete.  dg_release_next
+// it - and what follows it - sees the predecessor complete.  What an earlier
+// kernel of the stream writes (vectors, traces, exponents, the solver's state)
+// must not reach it as `const ... __restrict__`: such data may be read through
+// the non-coherent path, or ahead of the wait, as it has to be read-only for the
+// kernel's whole lifetime, which begins before its predecessor's ends.
+// dg_release_next
 // lets the successor's blocks take the room that this grid's tail leaves.
 // 8^3 Q2 apply in a loop: 16.4 -> 12.3 us together with the raw stream handle in
 // the binding; large kernels gain about 1 %.
