@@ -263,6 +263,16 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   for (int k2 = 0; k2 < NP; ++k2) out[k2 * N2] = fx_pair(fx_shift(M[k2], up));
 }
 
+// K from the kept h w_q K.
+__global__ void k_point_coefficient(const double* __restrict__ kt, double* __restrict__ K,
+                                    long long ndofs, int n, double h,
+                                    const __grid_constant__ DGTab<double> tab) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= ndofs) return;
+  const int q = (int)(t % ((long long)n * n * n));
+  K[t] = kt[t] / (h * (tab.w[q % n] * tab.w[(q / n) % n] * tab.w[q / (n * n)]));
+}
+
 template <int N>
 struct FixedF {
   static constexpr size_t SMEM = FxSmem<N, Cfg<N>::THREADS>::cell;
@@ -372,6 +382,14 @@ int dg_setup_fixed(dg_mesh* m, const double* K, cudaStream_t s) {
   cudaError_t e = dgk::dispatch_n<double, dgk::FixedSetupF>(m->n, (const dg_mesh*)m, K, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "line operators launch");
   return DG_OK;
+}
+
+int dg_restore_fixed(dg_mesh* m, cudaStream_t s) {
+  double* K = m->U64;  // the point values of an application: free between calls
+  dgk::k_point_coefficient<<<(unsigned)((m->ndofs + 255) / 256), 256, 0, s>>>(
+      m->kt64, K, m->ndofs, m->n, m->h, m->tab64);
+  DG_CUDA(cudaGetLastError());
+  return dg_setup_fixed(m, K, s);
 }
 
 int dg_launch_fixed_pass(const dg_mesh* m, bool modal, int pass, const double* x, double* y,

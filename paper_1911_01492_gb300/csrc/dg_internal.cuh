@@ -290,6 +290,7 @@ cudaError_t dg_launch_after(void (*kernel)(K...), unsigned blocks, unsigned thre
 // (1: traces, 2: cell terms) over the cells [cbeg, cend), both passes
 int dg_prepare_fixed(int n);
 int dg_setup_fixed(dg_mesh* m, const double* K, cudaStream_t s);
+int dg_restore_fixed(dg_mesh* m, cudaStream_t s);  // the same from the coefficient in place
 int dg_launch_fixed_pass(const dg_mesh* m, bool modal, int pass, const double* x, double* y,
                          long long cbeg, long long cend, const int* skip, cudaStream_t s);
 int dg_launch_fixed_apply(const dg_mesh* m, bool modal, const double* x, double* y,

@@ -775,6 +775,14 @@ extern "C" int dg_set_vertices(dg_mesh* m, const double* X) {
   cudaFree(darea);
   if (e != cudaSuccess) return dg_cuda_fail(e, "dg_set_vertices");
   if (flag) {
+    // the mesh is the cube again, under the coefficient that it has: a curved mesh
+    // has not formed the cube's operators from it
+    if (m->multilinear && m->has_coef) {
+      m->has_coef = false;
+      if (int rc = dg_restore_fixed(m, nullptr)) return rc;
+      DG_CUDA(cudaDeviceSynchronize());
+      m->has_coef = true;
+    }
     m->multilinear = false;
     return dg_fail(DG_ERR_INVALID_ARG,
                    "dg_set_vertices: a cell's Jacobian determinant is not positive (inverted "
