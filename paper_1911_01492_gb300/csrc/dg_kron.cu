@@ -438,10 +438,13 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
 }
 
 // Factors of the FP64 application from the FP64 ones: the eigenbases as
-// fixed-point pairs, one reciprocal per DOF.  One thread per DOF.
+// fixed-point pairs, one reciprocal per DOF.  One thread per DOF.  A cell whose
+// three factors share a zero eigenvalue (every face coefficient zero) has no
+// inverse: its reciprocal raises *flag, since the application reads mantissas
+// and would take an infinity for a number.
 template <int N>
 __global__ void k_kron_fix(const double* __restrict__ K64, FxPair* __restrict__ KX,
-                           double* __restrict__ winv, long long ncells) {
+                           double* __restrict__ winv, long long ncells, int* flag) {
   constexpr int N2 = N * N, N3 = N * N * N, KS = 3 * N2 + 3 * N;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ncells * N3) return;
@@ -449,7 +452,9 @@ __global__ void k_kron_fix(const double* __restrict__ K64, FxPair* __restrict__ 
   const int k = (int)(t - c * N3);
   const double* L = K64 + c * KS + 3 * N2;
   const int i = k / N2, j = k % N, l = (k / N) % N;
-  winv[t] = 1.0 / (L[i] + L[N + j] + L[2 * N + l]);
+  const double w = 1.0 / (L[i] + L[N + j] + L[2 * N + l]);
+  winv[t] = w;
+  if (!(w > 0.0) || !isfinite(w)) atomicOr(flag, 1);
   for (int e = k; e < 3 * N2; e += N3)
     KX[c * 3 * N2 + e] = fx_pair(__double2ll_rn(K64[c * KS + e] * 0x1p60));
 }
@@ -458,9 +463,9 @@ template <int N>
 struct KronFixF {
   template <typename T>
   static cudaError_t run(const double* K64, FxPair* KX, double* winv, long long ncells,
-                         cudaStream_t s) {
+                         int* flag, cudaStream_t s) {
     const long long n = ncells * N * N * N;
-    k_kron_fix<N><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(K64, KX, winv, ncells);
+    k_kron_fix<N><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(K64, KX, winv, ncells, flag);
     return cudaGetLastError();
   }
 };
@@ -601,9 +606,16 @@ static int ensure_kron_fx(dg_mesh* m, cudaStream_t s) {
   if (X == nullptr) DG_CUDA(cudaMalloc((void**)&X, sizeof(FxPair) * nq));
   if (m->kronW == nullptr)
     DG_CUDA(cudaMalloc((void**)&m->kronW, sizeof(double) * (size_t)m->ndofs));
+  DG_CUDA(cudaMemsetAsync(m->dflag, 0, sizeof(int), s));
   cudaError_t e = dgk::dispatch_n<double, dgk::KronFixF>(
-      m->n, (const double*)(m->nodal_op ? m->kronN64 : m->kron64), X, m->kronW, m->ncells, s);
+      m->n, (const double*)(m->nodal_op ? m->kronN64 : m->kron64), X, m->kronW, m->ncells,
+      m->dflag, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "Kronecker cell blocks: fixed-point factors");
+  int flag = 0;
+  DG_CUDA(cudaMemcpyAsync(&flag, m->dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaStreamSynchronize(s));
+  if (flag)
+    return dg_fail(DG_ERR_BREAKDOWN, "Kronecker cell blocks: a cell's block is singular");
   has = true;
   return DG_OK;
 }
