@@ -19,3 +19,6 @@ def test_singular_cell_block_breaks_down(cuda_device, k, nodal):
         _, st = m.cg_solve(b, rtol=1e-8, maxit=20, precond="kron", nodal=nodal,
                            raise_on_error=False)
         assert st["status"] == dg.DG_ERR_BREAKDOWN
+        # reported where the reciprocals are formed, before an iteration uses them
+        with pytest.raises(dg.DGError, match="singular"):
+            m.cg_solve(b, rtol=1e-8, maxit=20, precond="kron", nodal=nodal)
