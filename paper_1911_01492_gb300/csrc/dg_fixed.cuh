@@ -31,20 +31,24 @@ namespace dgk {
 // cells whose data holds a NaN or an infinity carry this exponent
 constexpr int FX_NAN = 1 << 24;
 
-// Largest power of two S0 with n^{3/2} 2^S0 <= 2^60: values of magnitude below
-// 2^S0 have a cell 2-norm of at most 2^60.
-template <int N>
-struct FxScale {
-  static constexpr int S0 = N == 2 ? 58 : N == 3 ? 57 : N == 4 ? 57 : N <= 6 ? 56 : 55;
-};
+// A transform preserves the 2-norm of a cell and no value of its stages exceeds it,
+// so a cell is scaled until its norm, not its largest value times n^{3/2}, reaches
+// 2^60: for a vector that one mode per cell dominates (any smooth one) that is up to
+// 4.7 bits more.  Without them the noise in A x of such a vector was 17 times FP64's
+// at degree 8 and twice at degree 4, and mixed solves of 48^3 Q4 to 1e-10 could
+// stall above it; with them it is below FP64's at every degree.  They cost 3 % of an
+// application (64^3 Q3 448 -> 462 us).  The norm comes from 11-bit magnitudes m
+// (rounded up) under the exponent E of the cell's largest value: norm < 2^(E - 11)
+// sqrt(sum of m^2).  fx_norm_bits: the bits that it takes above 2^(E - 11).
+__device__ __forceinline__ int fx_norm_bits(unsigned sum) { return (33 - __clz((int)sum)) >> 1; }
 
 // Shared memory of the two passes in a block of BT threads.
 template <int N, int BT>
 struct FxSmem {
   static constexpr int C = Cfg<N>::CPB;
   static constexpr int NS = (BT + N * N - 1) / (N * N);  // n^2 thread groups of the block
-  static constexpr size_t trace = 8 * C * LinePad<N>::SC + 4 * 2 * NS;
-  static constexpr size_t cell = 8 * 2 * C * LinePad<N>::SC + 8 * 6 * C + 4 * (7 * C + NS);
+  static constexpr size_t trace = 8 * C * LinePad<N>::SC + 4 * 3 * NS;
+  static constexpr size_t cell = 8 * 2 * C * LinePad<N>::SC + 8 * 6 * C + 4 * (7 * C + 2 * NS);
 };
 
 struct FxVal { int h, l; };  // a value v = h 2^30 + l
@@ -132,11 +136,11 @@ __device__ __forceinline__ unsigned fx_mag_hi(long long v) {
 // smallest b >= 32 with every magnitude below 2^b
 __device__ __forceinline__ int fx_bits(unsigned mag_hi) { return 64 - __clz((int)mag_hi); }
 
-// Largest v over the threads of the calling thread's cell.  Cells that lie
-// inside one warp need no barrier; otherwise slots (zeroed before an
-// earlier barrier) collects the warps' maxima.  Every thread of the block calls it.
-template <int N, int BT>
-__device__ __forceinline__ unsigned fx_cell_max(unsigned v, int lc, unsigned* slots) {
+// Largest v, or the sum of v, over the threads of the calling thread's cell.
+// Cells that lie inside one warp need no barrier; otherwise slots (zeroed before an
+// earlier barrier) collects the warps' results.  Every thread of the block calls it.
+template <int N, int BT, bool SUM>
+__device__ __forceinline__ unsigned fx_cell_reduce(unsigned v, int lc, unsigned* slots) {
   constexpr int N2 = N * N;
   const int lane = threadIdx.x & 31, base = (int)threadIdx.x - lane;
   const int lo = lc * N2 > base ? lc * N2 - base : 0;
@@ -144,11 +148,53 @@ __device__ __forceinline__ unsigned fx_cell_max(unsigned v, int lc, unsigned* sl
   const int lanes = BT - base < 32 ? BT - base : 32;
   if (hi > lanes) hi = lanes;
   const unsigned mask = (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
-  v = __reduce_max_sync(mask, v);
+  v = SUM ? __reduce_add_sync(mask, v) : __reduce_max_sync(mask, v);
   if constexpr (32 % N2 == 0) return v;
-  if (lane == lo) atomicMax(slots + lc, v);
+  if (lane == lo) {
+    if (SUM)
+      atomicAdd(slots + lc, v);
+    else
+      atomicMax(slots + lc, v);
+  }
   __syncthreads();
   return slots[lc];
+}
+template <int N, int BT>
+__device__ __forceinline__ unsigned fx_cell_max(unsigned v, int lc, unsigned* slots) {
+  return fx_cell_reduce<N, BT, false>(v, lc, slots);
+}
+
+// k with cell 2-norm of x 2^k below 2^60, for |x| < 2^E.  The upper halves, with
+// their exponents moved, are FP32 numbers in [0, 2^11] that are at most 2^-20
+// below x 2^(11 - E); a thread's squares are added in FP32, with a margin for that
+// and for its roundings, and the cell's in integers (at most 2^31.6).
+template <int N, int BT>
+__device__ __forceinline__ int fx_norm_scale(const double (&x)[N], int E, int lc,
+                                             unsigned* slots) {
+  float sum = 0.0f;
+#pragma unroll
+  for (int l = 0; l < N; ++l) {
+    // subnormal numbers count as 2^11
+    const int t = min((int)(fx_abs_hi(x[l]) - ((unsigned)(E + 885) << 20)), 138 << 20);
+    const float f = __int_as_float(max(t, 0) << 3);
+    sum = fmaf(f, f, sum);
+  }
+  const unsigned m = __float2uint_ru(sum * (1.0f + 0x1p-16f)) + 1u;
+  return 71 - E - fx_norm_bits(fx_cell_reduce<N, BT, true>(m, lc, slots));
+}
+// The same for integers below 2^b: the shift that brings the cell's norm below
+// 2^60, from the upper halves (b >= 32; those below 2^43 are taken as they are).
+template <int N, int BT>
+__device__ __forceinline__ int fx_norm_shift(const long long (&r)[N], int b, int lc,
+                                             unsigned* slots) {
+  b = max(b, 43);
+  unsigned sum = 0;
+#pragma unroll
+  for (int l = 0; l < N; ++l) {
+    const unsigned m = (fx_mag_hi(r[l]) >> (b - 43)) + 1u;
+    sum += m * m;
+  }
+  return 71 - b - fx_norm_bits(fx_cell_reduce<N, BT, true>(sum, lc, slots));
 }
 
 // u[a] = sum_i q[a][i] x[i], parity split (q[N-1-a][i] = (-1)^i q[a][i])
@@ -294,7 +340,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
   unsigned* slots = reinterpret_cast<unsigned*>(smem + C * SC);
   constexpr int NS = FxSmem<N, BT>::NS;
   if (32 % N2 != 0) {
-    if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
+    if (threadIdx.x < 3 * NS) slots[threadIdx.x] = 0;
     cell_sync<N>();
   }
   double xv[N];
@@ -309,9 +355,9 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
   long long v[N], u[N];
   int eu;  // u[] 2^eu
   if (MODAL) {
-    constexpr int S0 = FxScale<N>::S0;
+    const int k = fx_norm_scale<N, BT>(xv, E, lc, slots + 2 * NS);
 #pragma unroll
-    for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], S0 - E, E);
+    for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], k, E);
     // along z: thread owns (i = p, j = q)
     fx_fwd<N>(tab, v, u);
 #pragma unroll
@@ -343,7 +389,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
       u[a] = fx_shift(u[a], up);
       if (live) sc[q * SZ + p * SY + a] = u[a];
     }
-    eu = E - S0 - up;
+    eu = -k - up;
     if (active) fx_store_traces<N>(tab, u, TR + c * (12 * N2), 0, pt);
   } else {
 #pragma unroll
@@ -425,7 +471,7 @@ __device__ __forceinline__ double fx_cell_cells(
       sexp[lc][f] = e;
     }
   }
-  if (MODAL && 32 % N2 != 0 && threadIdx.x < FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
+  if (MODAL && 32 % N2 != 0 && threadIdx.x < 2 * FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
   long long u[N], r[N];
   // z-lines (a = p, b = q)
 #pragma unroll
@@ -586,7 +632,8 @@ __device__ __forceinline__ double fx_cell_cells(
     const unsigned m = fx_mag_hi(r[a]);
     big = m > big ? m : big;
   }
-  const int up = FxScale<N>::S0 - fx_bits(fx_cell_max<N, BT>(big, lc, slots));
+  const int up = fx_norm_shift<N, BT>(r, fx_bits(fx_cell_max<N, BT>(big, lc, slots)), lc,
+                                      slots + FxSmem<N, BT>::NS);
 #pragma unroll
   for (int a = 0; a < N; ++a) r[a] = fx_shift(r[a], up);
   fx_bwd<N>(tab, r, u);

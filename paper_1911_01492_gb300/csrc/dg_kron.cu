@@ -320,20 +320,20 @@ k_kron_apply(const T* __restrict__ KD, const T* __restrict__ r, T* __restrict__ 
 // products of 12 issue cycles each and the divisions are done once,
 // in k_kron_fix.  KX: the 1D factors [c][x,y,z][i][j] 2^60; winv: 1 / (lx + ly
 // + lz) [c][i][j + n l].  The transformed residual t is scaled to w t with the
-// largest magnitude of the cell again below 2^S0, whatever the spread of the
-// eigenvalues; <z, r> = sum w t^2 accumulates in 64-bit integers per thread.
+// cell's 2-norm again below 2^60, whatever the spread of the eigenvalues; <z, r> =
+// sum w t^2 accumulates in 64-bit integers per thread.
 template <int N, int MODE>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
 k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
                 const double* __restrict__ r, double* __restrict__ z, double* __restrict__ p,
                 long long ncells, double* __restrict__ partials, DGCGState* st) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
-  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC, S0 = FxScale<N>::S0;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC, NS = FxSmem<N, T>::NS;
   if (MODE != 1 && st->done) return;
   __shared__ long long s[C * SC];
   __shared__ FxPair sq[C * 3 * N2];
   __shared__ double rd[T];
-  __shared__ unsigned slots[2][FxSmem<N, T>::NS];
+  __shared__ unsigned slots[4 * NS];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -348,15 +348,16 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
 #pragma unroll
   for (int i = 0; i < N; ++i) w[i] = winv[c * N3 + i * N2 + pt];
   for (int i = threadIdx.x; i < nblk * 3 * N2; i += T) sq[i] = KX[c0 * 3 * N2 + i];
-  if (threadIdx.x < FxSmem<N, T>::NS) slots[0][threadIdx.x] = slots[1][threadIdx.x] = 0;
+  for (int i = threadIdx.x; i < 4 * NS; i += T) slots[i] = 0;
   unsigned big = 0;
 #pragma unroll
   for (int l = 0; l < N; ++l) big = max(big, fx_abs_hi(rv[l]));
   __syncthreads();
-  const int E = fx_exponent(fx_cell_max<N, T>(big, lc, slots[0]));
+  const int E = fx_exponent(fx_cell_max<N, T>(big, lc, slots));
+  const int k0 = fx_norm_scale<N, T>(rv, E, lc, slots + 2 * NS);
   long long v[N], u[N];
 #pragma unroll
-  for (int l = 0; l < N; ++l) v[l] = fx_from_double(rv[l], S0 - E, E);
+  for (int l = 0; l < N; ++l) v[l] = fx_from_double(rv[l], k0, E);
   // u[k] = sum_i Q[i][k] v[i] (tr) or sum_i Q[k][i] v[i]
   auto line = [&](int d, bool tr) {
     FxVal e[N];
@@ -399,25 +400,29 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
     // biased to stay positive
     top = max(top, (unsigned)(fx_bits(fx_mag_hi(u[i])) + ew[i] + 4096));
   }
-  const int B = (int)fx_cell_max<N, T>(top, lc, slots[1]) - 4096;
-  FxAcc dot = {0, 0};
+  const int B = (int)fx_cell_max<N, T>(top, lc, slots + NS) - 4096;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     FxAcc A = fx_zero();
-    const FxPair t = fx_pair(u[i]);
-    fx_mac(A, t, m[i]);
-    const int sh = ew[i] + S0 - B;
+    fx_mac(A, fx_pair(u[i]), m[i]);
+    const int sh = ew[i] + 60 - B;
     v[i] = fx_shift(fx_value(A), sh < -63 ? -63 : sh);
-    fx_mac(dot, t, fx_split(v[i]));
   }
-  // v stands for v 2^(E - S0 + B - S0); <z, r> sums t v
+  const int up = fx_norm_shift<N, T>(v, 60, lc, slots + 3 * NS);
+  FxAcc dot = {0, 0};
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    v[i] = fx_shift(v[i], up);
+    fx_mac(dot, fx_pair(u[i]), fx_split(v[i]));
+  }
+  // v stands for v 2^(B - 60 - up - k0); <z, r> sums t v, t 2^-k0
   const bool bad = E >= FX_NAN;
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-  const int ez = E - 2 * S0 + B;
+  const int ez = B - 60 - up - k0;
   const double acc = !active ? 0.0
                      : bad   ? qnan
                              : fx_scale(fma((double)dot.m, 0x1p-30, (double)dot.h),
-                                        ez + E - S0 + 60);
+                                        ez - k0 + 60);
   line(0, false);
   put(xl, 1);
   get(yl, SY);

@@ -342,10 +342,10 @@ k_trace_ml(const double* __restrict__ x, long long* __restrict__ U, long long* _
            const __grid_constant__ DGTabXGrad tg) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
-  constexpr int S0 = FxScale<N>::S0, NS = FxSmem<N, T>::NS;
+  constexpr int NS = FxSmem<N, T>::NS;
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned slots[2 * NS];
+  __shared__ unsigned slots[3 * NS];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -355,7 +355,7 @@ k_trace_ml(const double* __restrict__ x, long long* __restrict__ U, long long* _
   // u, then its derivatives along x, y, z
   long long* su = reinterpret_cast<long long*>(smem_raw) + lc * 4 * SC;
   long long* sd[3] = {su + SC, su + 2 * SC, su + 3 * SC};
-  if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
+  for (int i = threadIdx.x; i < 3 * NS; i += T) slots[i] = 0;
   __syncthreads();
   double xv[N];
   unsigned big = 0;
@@ -365,10 +365,11 @@ k_trace_ml(const double* __restrict__ x, long long* __restrict__ U, long long* _
     big = max(big, fx_abs_hi(xv[l]));
   }
   const int E = fx_exponent(fx_cell_max<N, T>(big, lc, slots));
+  const int k = fx_norm_scale<N, T>(xv, E, lc, slots + 2 * NS);
   const int zl = q * SY + p, yl = q * SZ + p, xl = q * SZ + p * SY;
   long long v[N], u[N];
 #pragma unroll
-  for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], S0 - E, E);
+  for (int l = 0; l < N; ++l) v[l] = fx_from_double(xv[l], k, E);
   fx_fwd<N>(tab, v, u);
 #pragma unroll
   for (int e = 0; e < N; ++e) su[zl + e * SZ] = u[e];
@@ -394,7 +395,7 @@ k_trace_ml(const double* __restrict__ x, long long* __restrict__ U, long long* _
   fx_deriv<N>(tg, u, v);
 #pragma unroll
   for (int a = 0; a < N; ++a) sd[0][xl + a] = v[a];
-  if (active && pt == 0) expU[c] = E == FX_NAN ? FX_NAN : E - S0 - up;
+  if (active && pt == 0) expU[c] = E == FX_NAN ? FX_NAN : -k - up;
   __syncthreads();
 #pragma unroll
   for (int b = 0; b < N; ++b) u[b] = su[yl + b * SY];
@@ -455,7 +456,7 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
   constexpr int NS = FxSmem<N, T>::NS, SH = MlSmem<N>::SH;
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned slots[NS];
+  __shared__ unsigned slots[2 * NS];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -470,7 +471,7 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
   const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
   const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
-  if (threadIdx.x < NS) slots[threadIdx.x] = 0;
+  if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
   // Exponents and shifts, one thread per cell.  F sums the volume flux, halved
   // (<= 2^59), and six lifted terms (each below 2^61, five bits down): below
   // 2^60.  r sums Dh^T F in three directions and six lifted terms three bits
@@ -642,7 +643,8 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
     big = max(big, fx_mag_hi(r[e]));
   }
   // Q^T along z, y, x, then out through the z-lines
-  const int up = FxScale<N>::S0 - fx_bits(fx_cell_max<N, T>(big, lc, slots));
+  const int up = fx_norm_shift<N, T>(r, fx_bits(fx_cell_max<N, T>(big, lc, slots)), lc,
+                                     slots + NS);
 #pragma unroll
   for (int e = 0; e < N; ++e) r[e] = fx_shift(r[e], up);
   fx_bwd<N>(tab, r, u);
