@@ -148,9 +148,12 @@ k_cell_dot_fx(const void* xU, const long long* TR, const int* expU,
 }
 
 // Line operators, face coefficients and their exponents from K and h gamma: one
-// thread per cell, direction and line.  Integer arithmetic throughout: K in
-// units of the cell's largest, h gamma < 2^(1 + exponents of h and K), both to
-// 2^-59; products of the 1D tables are constants.
+// thread per cell, direction and line.  Integer arithmetic throughout: the volume
+// part with K in units of the cell's largest, the faces' part with the 53 bits of
+// h gamma, each a product with constants of the 1D tables under a scale of its own,
+// rounded to the larger one.  (Under one scale the faces' bound, sigma times
+// the volume part's, took up to 7 bits from an operator whose K is large at few
+// points, and then a smooth vector, whose terms cancel, lost more than in FP64.)
 template <int N>
 struct FxSetup {
   static constexpr int L = 3 * N * N;                    // lines of a cell
@@ -158,8 +161,9 @@ struct FxSetup {
   static constexpr int THREADS = C * L;
 };
 
+// Registers for six (n = 3) and five (n = 4) blocks per SM, which cost no spill.
 template <int N>
-__global__ void __launch_bounds__(FxSetup<N>::THREADS)
+__global__ void __launch_bounds__(FxSetup<N>::THREADS, N == 3 ? 6 : N == 4 ? 5 : 0)
 k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
            FxPair* __restrict__ lineop, FxPair* __restrict__ gam, int* __restrict__ expM,
            int* __restrict__ expG, long long ncells, int Nc, int cg,
@@ -169,12 +173,13 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   __shared__ long long sk[C * N3];
   __shared__ unsigned kmax[C];
   __shared__ unsigned long long rmax[C][3];
-  __shared__ int sbad[C];
+  __shared__ int sbad[C], stop[C];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   if (threadIdx.x < C) {
     kmax[threadIdx.x] = 0;
     sbad[threadIdx.x] = 0;
+    stop[threadIdx.x] = -FX_NAN;
     for (int d = 0; d < 3; ++d) rmax[threadIdx.x][d] = 0;
   }
   __syncthreads();
@@ -197,33 +202,44 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   const int eK = active ? fx_exponent(kmax[lc]) : 0;
   long long M[NP];
   bool bad = eK == FX_NAN;
+  bool edge[2] = {false, false};
+  long long mant[2] = {0, 0};                // h gamma 2^(60 - eg), in [2^59, 2^60)
+  int eg[2] = {-(1 << 20), -(1 << 20)};
   if (active) {
-    const int step = dir == 0 ? 1 : dir == 1 ? N : N2;
-    const int at = lc * N3 + (dir == 0 ? N * (p + N * q) : dir == 1 ? p + N2 * q : p + N * q);
     const unsigned cu = (unsigned)c, nu = (unsigned)Nc;
     const int crd = (int)(dir == 0 ? cu % nu : dir == 1 ? (cu / nu) % nu : cu / nu / nu);
-    FxVal k[N];
-#pragma unroll
-    for (int f = 0; f < N; ++f) k[f] = fx_split(sk[at + f * step]);
-    FxVal g[2];
-    bool edge[2] = {crd == 0, crd == Nc - 1};
+    edge[0] = crd == 0;
+    edge[1] = crd == Nc - 1;
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
       const double w = gh[c * 6 + 2 * dir + m];
       bad = bad || fx_abs_hi(w) >= 0x7ff00000u;
-      const int E = eK + t.ch + 1;
-      g[m] = fx_split(fx_from_double(w, 60 - E, E));
-      if (pt == 0) {
-        // normalised to [2^59, 2^60), taking up the table scales 2^cg (an octave
-        // higher the largest mantissas would round to 2^61, past what a pair holds)
-        const double w2 = fx_abs_hi(w) < 0x00100000u ? w * 0x1p64 : w;
-        const int e = (int)(fx_abs_hi(w2) >> 20);
-        const long long mant = (__double_as_longlong(w2) & 0xfffffffffffffll) | 0x10000000000000ll;
-        gam[c * 6 + 2 * dir + m] = w > 0.0 ? fx_pair(mant << 7) : FxPair{0, 0};
-        expG[c * 6 + 2 * dir + m] =
-            w > 0.0 ? e - 1021 - (fx_abs_hi(w) < 0x00100000u ? 64 : 0) + cg : -2 * FX_NAN;
+      const bool sub = fx_abs_hi(w) < 0x00100000u;
+      const double w2 = sub ? w * 0x1p64 : w;
+      if (w > 0.0) {
+        mant[m] = ((__double_as_longlong(w2) & 0xfffffffffffffll) | 0x10000000000000ll) << 7;
+        eg[m] = (int)(fx_abs_hi(w2) >> 20) - 1022 - (sub ? 64 : 0);
+      }
+      if (pt == 0) {  // an octave higher a mantissa could round to 2^61, past a pair's end
+        gam[c * 6 + 2 * dir + m] = fx_pair(mant[m]);
+        expG[c * 6 + 2 * dir + m] = w > 0.0 ? eg[m] + 1 + cg : -2 * FX_NAN;
       }
     }
+    if (pt == 0) atomicMax(&stop[lc], max(eg[0], eg[1]) + t.cF);
+  }
+  __syncthreads();
+  // the common exponent: volume part and two faces, each at most 2^60
+  const int E0 = active ? max(eK + t.cV, stop[lc]) : 0;
+  if (active) {
+    const int step = dir == 0 ? 1 : dir == 1 ? N : N2;
+    const int at = lc * N3 + (dir == 0 ? N * (p + N * q) : dir == 1 ? p + N2 * q : p + N * q);
+    FxVal k[N];
+#pragma unroll
+    for (int f = 0; f < N; ++f) k[f] = fx_split(sk[at + f * step]);
+    const int egm = max(eg[0], eg[1]);  // both faces under the larger exponent
+    const FxVal g[2] = {fx_split(mant[0] >> min(egm - eg[0], 63)),
+                        fx_split(mant[1] >> min(egm - eg[1], 63))};
+    const int sV = min(E0 - eK - t.cV, 62), sF = min(E0 - egm - t.cF, 62);
     unsigned long long rs[N];
 #pragma unroll
     for (int e = 0; e < N; ++e) rs[e] = 0;
@@ -232,12 +248,12 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
 #pragma unroll
       for (int j = i; j < N; ++j) {
         const int ij = packed<N>(i, j), ji = packed<N>(N - 1 - i, N - 1 - j);
-        FxAcc A = fx_zero<1>();
+        FxAcc A = fx_zero<1>(), B = fx_zero();
 #pragma unroll
         for (int f = 0; f < N; ++f) fx_mac(A, t.DD[f][ij], k[f]);
-        fx_mac(A, edge[0] ? t.F[1][ij] : t.F[0][ij], g[0]);
-        fx_mac(A, edge[1] ? t.F[1][ji] : t.F[0][ji], g[1]);
-        const long long v = fx_value<1>(A);
+        fx_mac(B, edge[0] ? t.F[1][ij] : t.F[0][ij], g[0]);
+        fx_mac(B, edge[1] ? t.F[1][ji] : t.F[0][ji], g[1]);
+        const long long v = fx_round(fx_value<1>(A), sV) + fx_round(fx_value(B), sF);
         M[ij] = v;
         const unsigned long long mag = (unsigned long long)(v < 0 ? -v : v) >> 4;
         rs[i] += mag;
@@ -257,10 +273,11 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   // every n), so an entry stays clear of a pair's upper end
   const int bits = 68 - __clzll((long long)(rmax[lc][0] + rmax[lc][1] + rmax[lc][2]));
   const int up = 61 - bits;
-  if (t2 == 0) expM[c] = sbad[lc] ? FX_NAN : eK + t.cB - up + 1;
+  if (t2 == 0) expM[c] = sbad[lc] ? FX_NAN : E0 - up + 1;
   FxPair* out = lineop + ((c * 3 + dir) * NP) * N2 + pt;
 #pragma unroll
-  for (int k2 = 0; k2 < NP; ++k2) out[k2 * N2] = fx_pair(fx_shift(M[k2], up));
+  for (int k2 = 0; k2 < NP; ++k2)
+    out[k2 * N2] = fx_pair(up < 0 ? fx_round(M[k2], -up) : M[k2] << up);
 }
 
 // K from the kept h w_q K.

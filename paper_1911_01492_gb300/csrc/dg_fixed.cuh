@@ -94,6 +94,11 @@ __device__ __forceinline__ long long fx_shift(long long v, int s) {  // v 2^s, |
   return s >= 0 ? v << s : v >> -s;
 }
 
+// v 2^-s to nearest, 0 <= s < 63
+__device__ __forceinline__ long long fx_round(long long v, int s) {
+  return (v + ((1ll << s) >> 1)) >> s;
+}
+
 // exponent E with |x| < 2^E for every x whose high word without sign is at most
 // hi; FX_NAN for NaN or infinity
 __device__ __forceinline__ int fx_exponent(unsigned hi) {

@@ -127,29 +127,26 @@ bool dg_build_fixed_tables(int n, double h, DGTabX* t, DGTabXSetup* s, DGTabXGra
   }
   // line operators: h sum_f K_f Dh[f][i] Dh[f][j] + h gamma F[i][j] per face,
   // F = sigma l l^T + c (l d^T + d l^T) on the lower face (c = 1 inside, 2 on
-  // the boundary), mirrored on the upper one; K < 2^eK and gamma < 2^(eK + 1)
-  ld big = 0;
-  for (int i = 0; i < n; ++i)
-    for (int j = i; j < n; ++j) {
-      ld sum = 0;
-      for (int f = 0; f < n; ++f) sum += fabsl(Dh[f][i] * Dh[f][j]);
-      for (int m = 0; m < 2; ++m) {
-        const int ii = m ? n - 1 - i : i, jj = m ? n - 1 - j : j;
-        sum += 2 * (sigma * fabsl(l[ii] * l[jj]) +
-                    2 * (fabsl(l[ii] * d[jj]) + fabsl(d[ii] * l[jj])));
-      }
-      big = fmaxl(big, sum);
-    }
+  // the boundary), mirrored on the upper one; each of the two under its own scale
   const ld hl = (ld)h;
-  s->ch = ceil_log2(hl);
-  s->cB = ceil_log2(hl * big);
+  ld big[2] = {0, 0}, Ff[2][DG_MAXP];
+  for (int i = 0, k = 0; i < n; ++i)
+    for (int j = i; j < n; ++j, ++k) {
+      ld sum = 0;
+      for (int f = 0; f < n; ++f) sum += fabsl(hl * Dh[f][i] * Dh[f][j]);
+      big[0] = fmaxl(big[0], sum);
+      for (int m = 0; m < 2; ++m) {
+        Ff[m][k] = sigma * l[i] * l[j] + (m + 1) * (l[i] * d[j] + d[i] * l[j]);
+        big[1] = fmaxl(big[1], fabsl(Ff[m][k]));
+      }
+    }
+  s->cV = ceil_log2(big[0]);
+  s->cF = ceil_log2(big[1]);
   for (int i = 0, k = 0; i < n; ++i)
     for (int j = i; j < n; ++j, ++k) {
       for (int f = 0; f < n; ++f)
-        s->DD[f][k] = put(ldexpl(hl * Dh[f][i] * Dh[f][j], -s->cB));
-      const ld ll = sigma * l[i] * l[j], x = l[i] * d[j] + d[i] * l[j];
-      s->F[0][k] = put(ldexpl(ll + x, s->ch - s->cB));
-      s->F[1][k] = put(ldexpl(ll + 2 * x, s->ch - s->cB));
+        s->DD[f][k] = put(ldexpl(hl * Dh[f][i] * Dh[f][j], -s->cV));
+      for (int m = 0; m < 2; ++m) s->F[m][k] = put(ldexpl(Ff[m][k], -s->cF));
     }
   // the scaled derivative: Dh[n-1-f][n-1-a] = -Dh[f][a], so its even and odd
   // halves over the mirror pairs give both points of a pair

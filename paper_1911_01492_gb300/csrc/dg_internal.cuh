@@ -63,9 +63,9 @@ struct DGTabX {
   int bump;  // face contributions sit 2^bump below the common exponent
 };
 struct DGTabXSetup {
-  FxPair DD[DG_MAXN][DG_MAXP];  // h Dh[f][i] Dh[f][j]  2^-cB
-  FxPair F[2][DG_MAXP];         // own-side terms of the lower face: inside, boundary
-  int ch, cB;                   // h <= 2^ch; entries < 2^(cB + exponent of K)
+  FxPair DD[DG_MAXN][DG_MAXP];  // h Dh[f][i] Dh[f][j]  2^-cV
+  FxPair F[2][DG_MAXP];         // own-side terms of the lower face: inside, boundary  2^-cF
+  int cV, cF;                   // their sums over f and entries are at most one
 };
 struct DGTabXGrad {  // coefficient gradient (dg_grad.cu)
   FxPair De[DG_MAXH][DG_MAXH], Do[DG_MAXH][DG_MAXH];  // halves of Dh[f][.]  2^-cD
