@@ -37,7 +37,7 @@ constexpr int FX_NAN = 1 << 24;
 // 4.7 bits more.  Without them the noise in A x of such a vector was 17 times FP64's
 // at degree 8 and twice at degree 4, and mixed solves of 48^3 Q4 to 1e-10 could
 // stall above it; with them it is below FP64's at every degree.  They cost 3 % of an
-// application (64^3 Q3 448 -> 462 us).  The norm comes from 11-bit magnitudes m
+// application (27^3 Q5 166 -> 171 us).  The norm comes from 11-bit magnitudes m
 // (rounded up) under the exponent E of the cell's largest value: norm < 2^(E - 11)
 // sqrt(sum of m^2).  fx_norm_bits: the bits that it takes above 2^(E - 11).
 __device__ __forceinline__ int fx_norm_bits(unsigned sum) { return (33 - __clz((int)sum)) >> 1; }
@@ -142,11 +142,21 @@ __device__ __forceinline__ unsigned fx_mag_hi(long long v) {
 __device__ __forceinline__ int fx_bits(unsigned mag_hi) { return 64 - __clz((int)mag_hi); }
 
 // Largest v, or the sum of v, over the threads of the calling thread's cell.
-// Cells that lie inside one warp need no barrier; otherwise slots (zeroed before an
-// earlier barrier) collects the warps' results.  Every thread of the block calls it.
+// Cells that lie inside one warp need no barrier and take shuffles (a reduction
+// instruction runs once per cell of the warp: 64^3 Q3 464 against 435 us, 100^3 Q1
+// 368 against 273); otherwise slots (zeroed before an earlier barrier) collects the
+// warps' results.  Every thread of the block calls it.
 template <int N, int BT, bool SUM>
 __device__ __forceinline__ unsigned fx_cell_reduce(unsigned v, int lc, unsigned* slots) {
   constexpr int N2 = N * N;
+  if constexpr (32 % N2 == 0) {
+#pragma unroll
+    for (int off = N2 / 2; off > 0; off >>= 1) {
+      const unsigned o = __shfl_xor_sync(0xffffffffu, v, off);
+      v = SUM ? v + o : max(v, o);
+    }
+    return v;
+  }
   const int lane = threadIdx.x & 31, base = (int)threadIdx.x - lane;
   const int lo = lc * N2 > base ? lc * N2 - base : 0;
   int hi = (lc + 1) * N2 - base;
@@ -154,7 +164,6 @@ __device__ __forceinline__ unsigned fx_cell_reduce(unsigned v, int lc, unsigned*
   if (hi > lanes) hi = lanes;
   const unsigned mask = (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
   v = SUM ? __reduce_add_sync(mask, v) : __reduce_max_sync(mask, v);
-  if constexpr (32 % N2 == 0) return v;
   if (lane == lo) {
     if (SUM)
       atomicAdd(slots + lc, v);
