@@ -64,6 +64,7 @@ constexpr double LAUNCH_SECONDS = 2.0;   // work per production launch (estimate
 constexpr double EST_DOF_RATE = 7.0e9;   // DOF-iterations per second for that estimate
 
 __constant__ DGTabX c_btab[DG_MAXN - 1];  // fixed-point tables for n = 2..9
+__constant__ DGTabN<double> c_btabN[DG_MAXN - 1];  // FP64, scaled Gauss-point basis
 
 struct SampleDev {
   const double* b;
@@ -71,7 +72,8 @@ struct SampleDev {
   double *r, *u, *w, *p, *s;  // u == r when M = I
   // fixed-point operator (dg_fixed.cuh)
   long long *U, *TR;
-  int* expU;
+  int *expU, *mark;
+  const double *kt, *gh;
   const FxPair *lineop, *gam;
   const int *expM, *expG;
   const double* dinv;  // 1 / diag(A) for M = diag(A); nullptr for M = I
@@ -151,14 +153,16 @@ __host__ __device__ constexpr int group_cells(int n) {
 template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass1(const SampleDev& S, long long c0, int nblk,
                                             long long* smem) {
-  dgk::fx_trace_cells<N, !ND, BT>(dgk::FxLoad{S.u}, S.U, S.TR, S.expU, c0, nblk, c_btab[N - 2], smem);
+  dgk::fx_trace_cells<N, !ND, BT>(dgk::FxLoad{S.u}, S.U, S.TR, S.expU, S.mark, c0, nblk,
+                                  c_btab[N - 2], smem);
 }
 template <int N, bool ND, int BT>
 __device__ __forceinline__ void group_pass2(const SampleDev& S, long long c0, int nblk,
                                             long long* smem) {
   dgk::fx_cell_cells<N, !ND, BT>(ND ? (const void*)S.u : (const void*)S.U, S.TR, S.expU,
-                                 S.lineop, S.gam, S.expM, S.expG, dgk::FxStore{S.w}, c0, nblk, S.Nc,
-                                 c_btab[N - 2], smem);
+                                 S.lineop, S.gam, S.expM, S.expG,
+                                 dgk::FxWide{S.kt, S.gh, S.mark, &c_btabN[N - 2]},
+                                 dgk::FxStore{S.w}, c0, nblk, S.Nc, c_btab[N - 2], smem);
 }
 
 template <int MAXN, bool ND, int BT>
@@ -638,9 +642,12 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
     d.U = reinterpret_cast<long long*>(m->U64);
     d.TR = reinterpret_cast<long long*>(m->TR64);
     d.expU = m->expU;
+    d.mark = m->markU;
+    d.kt = m->kt64;
+    d.gh = m->gh64;
     d.lineop = m->lineopX;
     d.gam = m->gamX;
-    d.expM = m->expM;
+    d.expM = ND ? m->expN : m->expM;
     d.expG = m->expG;
     d.dinv = nullptr;
     if (jacobi) {
@@ -698,6 +705,10 @@ int solve_batched(const dg_mesh* const* meshes, int count, const double* const* 
     DG_CUDA(cudaMemcpyToSymbolAsync(c_btab, &m->tabX, sizeof(DGTabX),
                                     sizeof(DGTabX) * (size_t)(m->n - 2), cudaMemcpyHostToDevice,
                                     s));
+    if (ND)
+      DG_CUDA(cudaMemcpyToSymbolAsync(c_btabN, &m->tabN64, sizeof(DGTabN<double>),
+                                      sizeof(DGTabN<double>) * (size_t)(m->n - 2),
+                                      cudaMemcpyHostToDevice, s));
   }
   const size_t smem = persistent_smem<2, MAXN, BT>();
   DG_CUDA(cudaFuncSetAttribute(kb_persistent<BT, MAXN, ND>,

@@ -30,8 +30,8 @@ namespace dgk {
 template <int N, bool MODAL, typename XL>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
 k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
-           int* __restrict__ expU, long long cbeg, long long cend, const int* skip,
-           const __grid_constant__ DGTabX tab) {
+           int* __restrict__ expU, int* __restrict__ mark, long long cbeg, long long cend,
+           const int* skip, const __grid_constant__ DGTabX tab) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
   dg_wait_before();
@@ -40,7 +40,27 @@ k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
   x.begin();
   const long long c0 = cbeg + (long long)blockIdx.x * C;
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
-  fx_trace_cells<N, MODAL, T>(x, U, TR, expU, c0, nblk, tab, smem);
+  fx_trace_cells<N, MODAL, T>(x, U, TR, expU, mark, c0, nblk, tab, smem);
+}
+
+// Kernel parameter with the data of fx_cell_wide: in the point basis only.
+template <bool MODAL>
+struct FxWideArg {
+  __device__ __forceinline__ FxWide get() const { return {}; }
+};
+template <>
+struct FxWideArg<false> {
+  const double *kt, *gh;
+  const int* mark;
+  DGTabN<double> tn;
+  __device__ __forceinline__ FxWide get() const { return {kt, gh, mark, &tn}; }
+};
+template <bool MODAL>
+FxWideArg<MODAL> wide_arg(const dg_mesh* m) {
+  if constexpr (MODAL)
+    return {};
+  else
+    return {m->kt64, m->gh64, m->markU, m->tabN64};
 }
 
 // Resident blocks per SM that the register allocation of pass 2 aims at.  It
@@ -59,7 +79,8 @@ k_cell_fx(const void* xU, const long long* TR, const int* expU,
           const FxPair* __restrict__ lineop,
           const FxPair* __restrict__ gam, const int* __restrict__ expM,
           const int* __restrict__ expG, double* __restrict__ y, long long cbeg, long long cend,
-          int Nc, const int* skip, const __grid_constant__ DGTabX tab) {
+          int Nc, const int* skip, const __grid_constant__ DGTabX tab,
+          const __grid_constant__ FxWideArg<MODAL> wd) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
   dg_wait_before();
@@ -67,8 +88,8 @@ k_cell_fx(const void* xU, const long long* TR, const int* expU,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long c0 = cbeg + (long long)blockIdx.x * C;
   const int nblk = (int)((cend - c0) < C ? (cend - c0) : C);
-  fx_cell_cells<N, MODAL, T>(xU, TR, expU, lineop, gam, expM, expG, FxStore{y}, c0, nblk, Nc,
-                             tab, reinterpret_cast<long long*>(smem_raw));
+  fx_cell_cells<N, MODAL, T>(xU, TR, expU, lineop, gam, expM, expG, wd.get(), FxStore{y}, c0,
+                             nblk, Nc, tab, reinterpret_cast<long long*>(smem_raw));
 }
 
 // Inside a CG iteration (Section 2.4) the passes take the vector work along.
@@ -101,8 +122,8 @@ k_cell_dot_fx(const void* xU, const long long* TR, const int* expU,
               const FxPair* __restrict__ lineop,
               const FxPair* __restrict__ gam, const int* __restrict__ expM,
               const int* __restrict__ expG, double* __restrict__ q, long long ncells, int Nc,
-              double* __restrict__ partials, DGCGState* st,
-              const __grid_constant__ DGTabX tab) {
+              double* __restrict__ partials, DGCGState* st, const __grid_constant__ DGTabX tab,
+              const __grid_constant__ FxWideArg<MODAL> wd) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS;
   dg_release_next();
   dg_wait_before();
@@ -112,7 +133,7 @@ k_cell_dot_fx(const void* xU, const long long* TR, const int* expU,
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   const double acc = fx_cell_cells<N, MODAL, T, true>(
-      xU, TR, expU, lineop, gam, expM, expG, FxStore{q}, c0, nblk, Nc, tab,
+      xU, TR, expU, lineop, gam, expM, expG, wd.get(), FxStore{q}, c0, nblk, Nc, tab,
       reinterpret_cast<long long*>(smem_raw));
   __syncthreads();
   double* rd = reinterpret_cast<double*>(smem_raw);
@@ -166,19 +187,20 @@ template <int N>
 __global__ void __launch_bounds__(FxSetup<N>::THREADS, N == 3 ? 6 : N == 4 ? 5 : 0)
 k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
            FxPair* __restrict__ lineop, FxPair* __restrict__ gam, int* __restrict__ expM,
-           int* __restrict__ expG, long long ncells, int Nc, int cg,
+           int* __restrict__ expN, int* __restrict__ expG, long long ncells, int Nc, int cg,
            const __grid_constant__ DGTabXSetup t) {
   constexpr int C = FxSetup<N>::C, L = FxSetup<N>::L, T = FxSetup<N>::THREADS;
   constexpr int N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
   __shared__ long long sk[C * N3];
   __shared__ unsigned kmax[C];
   __shared__ unsigned long long rmax[C][3];
-  __shared__ int sbad[C], stop[C];
+  __shared__ int sbad[C], stop[C], smark[C];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   if (threadIdx.x < C) {
     kmax[threadIdx.x] = 0;
     sbad[threadIdx.x] = 0;
+    smark[threadIdx.x] = 0;
     stop[threadIdx.x] = -FX_NAN;
     for (int d = 0; d < 3; ++d) rmax[threadIdx.x][d] = 0;
   }
@@ -230,6 +252,7 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   __syncthreads();
   // the common exponent: volume part and two faces, each at most 2^60
   const int E0 = active ? max(eK + t.cV, stop[lc]) : 0;
+  unsigned long long R = 0;  // the line's largest row sum
   if (active) {
     const int step = dir == 0 ? 1 : dir == 1 ? N : N2;
     const int at = lc * N3 + (dir == 0 ? N * (p + N * q) : dir == 1 ? p + N2 * q : p + N * q);
@@ -260,12 +283,14 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
         if (i != j) rs[j] += mag;
       }
     }
-    unsigned long long R = 0;
 #pragma unroll
     for (int e = 0; e < N; ++e) R = rs[e] > R ? rs[e] : R;
     atomicMax(&rmax[lc][dir], R + N);
     if (bad) sbad[lc] = 1;
   }
+  __syncthreads();
+  if (active && R < max(rmax[lc][0], max(rmax[lc][1], rmax[lc][2])) >> 4)
+    atomicOr(&smark[lc], 1 << dir);
   __syncthreads();
   if (!active) return;
   // the sum of the directions' largest row sums to (2^60, 2^61]: each direction
@@ -273,7 +298,11 @@ k_lines_fx(const double* __restrict__ K, const double* __restrict__ gh,
   // every n), so an entry stays clear of a pair's upper end
   const int bits = 68 - __clzll((long long)(rmax[lc][0] + rmax[lc][1] + rmax[lc][2]));
   const int up = 61 - bits;
-  if (t2 == 0) expM[c] = sbad[lc] ? FX_NAN : E0 - up + 1;
+  if (t2 == 0) {
+    const int e = sbad[lc] ? FX_NAN : E0 - up + 1;
+    expM[c] = e;
+    expN[c] = e + (smark[lc] == FX_MARKS ? FX_WIDE : 0);
+  }
   FxPair* out = lineop + ((c * 3 + dir) * NP) * N2 + pt;
 #pragma unroll
   for (int k2 = 0; k2 < NP; ++k2)
@@ -302,10 +331,11 @@ struct FixedF {
     long long* TR = reinterpret_cast<long long*>(m->TR64);
     if (pass == 1)
       return dg_launch_after(k_trace_fx<N, MODAL, FxLoad>, blocks, Cfg<N>::THREADS, 0, s, FxLoad{x},
-                             U, TR, m->expU, cbeg, cend, skip, m->tabX);
+                             U, TR, m->expU, m->markU, cbeg, cend, skip, m->tabX);
     return dg_launch_after(k_cell_fx<N, MODAL>, blocks, Cfg<N>::THREADS, SMEM, s,
                            MODAL ? (const void*)U : (const void*)x, TR, m->expU, m->lineopX,
-                           m->gamX, m->expM, m->expG, y, cbeg, cend, m->N, skip, m->tabX);
+                           m->gamX, MODAL ? m->expM : m->expN, m->expG, y, cbeg, cend, m->N, skip,
+                           m->tabX, wide_arg<MODAL>(m));
   }
   template <typename T>
   static cudaError_t run(const dg_mesh* m, bool modal, int which, const double* x, double* y,
@@ -326,13 +356,13 @@ struct FixedCgF {
     long long* TR = reinterpret_cast<long long*>(m->TR64);
     cudaError_t e = dg_launch_after(
         k_trace_fx<N, MODAL, FxDirection<PC>>, blocks, Cfg<N>::THREADS, 0, s,
-        FxDirection<PC>{p, z, dinv, m->state, 0.0}, U, TR, m->expU, 0ll, m->ncells,
+        FxDirection<PC>{p, z, dinv, m->state, 0.0}, U, TR, m->expU, m->markU, 0ll, m->ncells,
         &m->state->done, m->tabX);
     if (e != cudaSuccess) return e;
     return dg_launch_after(k_cell_dot_fx<N, MODAL>, blocks, Cfg<N>::THREADS, FixedF<N>::SMEM, s,
                            MODAL ? (const void*)U : (const void*)p, TR, m->expU, m->lineopX,
-                           m->gamX, m->expM, m->expG, q, m->ncells, m->N, m->partials_cells,
-                           m->state, m->tabX);
+                           m->gamX, MODAL ? m->expM : m->expN, m->expG, q, m->ncells, m->N,
+                           m->partials_cells, m->state, m->tabX, wide_arg<MODAL>(m));
   }
   template <typename T>
   static cudaError_t run(const dg_mesh* m, const double* z, const double* dinv, double* p,
@@ -349,8 +379,8 @@ struct FixedTraceF {
   static cudaError_t run(const dg_mesh* m, const double* x, long long* U, long long* TR,
                          int* expU, cudaStream_t s) {
     const unsigned blocks = (unsigned)((m->ncells + Cfg<N>::CPB - 1) / Cfg<N>::CPB);
-    k_trace_fx<N, true><<<blocks, Cfg<N>::THREADS, 0, s>>>(FxLoad{x}, U, TR, expU, 0, m->ncells,
-                                                          nullptr, m->tabX);
+    k_trace_fx<N, true><<<blocks, Cfg<N>::THREADS, 0, s>>>(FxLoad{x}, U, TR, expU, nullptr, 0,
+                                                          m->ncells, nullptr, m->tabX);
     return cudaGetLastError();
   }
 };
@@ -381,7 +411,7 @@ struct FixedSetupF {
   static cudaError_t run(const dg_mesh* m, const double* K, cudaStream_t s) {
     using S = FxSetup<N>;
     k_lines_fx<N><<<(unsigned)((m->ncells + S::C - 1) / S::C), S::THREADS, 0, s>>>(
-        K, m->gh64, m->lineopX, m->gamX, m->expM, m->expG, m->ncells, m->N, m->tabX.cg,
+        K, m->gh64, m->lineopX, m->gamX, m->expM, m->expN, m->expG, m->ncells, m->N, m->tabX.cg,
         m->tabXS);
     return cudaGetLastError();
   }

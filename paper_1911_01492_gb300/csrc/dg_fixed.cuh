@@ -22,6 +22,18 @@
 //     same bound (the bases are orthonormal: the transforms preserve the
 //     2-norm of a cell, which starts at <= 2^60);
 //   * low-order sums: at most 9 terms of 2^30 2^30 and 2^29 2^31 stay below 2^63.
+//
+// Ranges inside a cell.  One exponent per cell keeps 60 bits of its largest values
+// and 60 - b of those 2^b below.  In the Legendre basis every result mixes the
+// whole cell and FP64 rounds relative to it too.  In the point basis a point only
+// sees its three lines, and FP64 keeps 53 bits of each: there a cell that may hold
+// points whose lines are all small against the cell's largest one, in the vector
+// (2^7) or in the operator (2^4), or that is outweighed by 2^9 by a neighbour with
+// small lines towards it, is applied in FP64 (fx_cell_wide), as exact
+// as FP64 throughout.  Lognormal fields of unit variance have no such cells (line
+// operators of a cell within 2^3.2) and pay 3 % for the marks (64^3 Q3 345 -> 356
+// us); a field of which every cell is marked takes 2.7 ms there, the FP64 kernels
+// took 1.25.
 #pragma once
 
 #include "dg_apply_impl.cuh"
@@ -30,6 +42,11 @@ namespace dgk {
 
 // cells whose data holds a NaN or an infinity carry this exponent
 constexpr int FX_NAN = 1 << 24;
+// added to the own exponent of a cell of the point basis that is applied in FP64
+constexpr int FX_WIDE = 1 << 20;
+// bit d of a cell's mark: it has a line along direction d below 2^-7 (vector) or
+// 2^-4 (operator) of its largest; a point small in all three needs all bits
+constexpr int FX_MARKS = 7;
 
 // A transform preserves the 2-norm of a cell and no value of its stages exceeds it,
 // so a cell is scaled until its norm, not its largest value times n^{3/2}, reaches
@@ -48,7 +65,8 @@ struct FxSmem {
   static constexpr int C = Cfg<N>::CPB;
   static constexpr int NS = (BT + N * N - 1) / (N * N);  // n^2 thread groups of the block
   static constexpr size_t trace = 8 * C * LinePad<N>::SC + 4 * 3 * NS;
-  static constexpr size_t cell = 8 * 2 * C * LinePad<N>::SC + 8 * 6 * C + 4 * (7 * C + 2 * NS);
+  static constexpr size_t cell =
+      8 * 2 * C * LinePad<N>::SC + 8 * 6 * C + 4 * (13 * C + 2 * NS);
 };
 
 struct FxVal { int h, l; };  // a value v = h 2^30 + l
@@ -338,10 +356,12 @@ struct FxStore {
 // BT threads (at least CPB n^2; the others only take part in the barriers).
 // smem: FxSmem<N, BT>::trace bytes.  Every thread of the block calls it; a
 // barrier must follow before smem is used again.
+// mark: the cells' marks of the vector (point basis).
 template <int N, bool MODAL, int BT, typename XL>
 __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restrict__ U,
                                                long long* __restrict__ TR,
-                                               int* __restrict__ expU, long long c0, int nblk,
+                                               int* __restrict__ expU, int* __restrict__ mark,
+                                               long long c0, int nblk,
                                                const DGTabX& tab, long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
@@ -366,6 +386,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
     big = m > big ? m : big;
   }
   const int E = fx_exponent(fx_cell_max<N, BT>(big, lc, slots));
+  const bool zsmall = (int)(big >> 20) < E + 1016;  // the z-line is below 2^(E - 7)
   long long v[N], u[N];
   int eu;  // u[] 2^eu
   if (MODAL) {
@@ -414,10 +435,21 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
     eu = E - 60;
   }
   if (E == FX_NAN) eu = FX_NAN;
-  if (active && pt == 0) expU[c] = eu;
+  if (active && pt == 0) {
+    expU[c] = eu;
+    if (!MODAL) mark[c] = 0;
+  }
   cell_sync<N>();
   if (!active) return;  // no barrier follows
   long long* tr = TR + c * (12 * N2);
+  // whether a line's largest value is below 2^53, the cell's at least 2^59
+  auto small = [](const long long (&w)[N]) {
+    int m = 0;
+#pragma unroll
+    for (int e = 0; e < N; ++e) m |= (int)(w[e] >> 32) ^ (int)(w[e] >> 63);
+    return m < 1 << 21;
+  };
+  int marks = 0;
   if (MODAL) {
 #pragma unroll
     for (int e = 0; e < N; ++e) {
@@ -428,11 +460,126 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
 #pragma unroll
     for (int a = 0; a < N; ++a) v[a] = sc[q * SZ + p * SY + a];
     fx_store_traces<N>(tab, v, tr, 0, pt);
+    marks = (small(v) ? 1 : 0) | (zsmall ? 4 : 0);
   }
   fx_store_traces<N>(tab, u, tr, 2, pt);
 #pragma unroll
   for (int b = 0; b < N; ++b) v[b] = sc[q * SZ + b * SY + p];
   fx_store_traces<N>(tab, v, tr, 1, pt);
+  if (!MODAL) {
+    if (small(v)) marks |= 2;
+    if (marks != 0 && E > -1042) atomicOr(mark + c, marks);  // E: the cell is not zero
+  }
+}
+
+// What fx_cell_wide reads: h w_q K, h gamma [c][6], the marks of the vector, the
+// FP64 tables of the scaled point basis.
+struct FxWide {
+  const double *kt, *gh;
+  const int* mark;
+  const DGTabN<double>* tn;
+};
+
+// Pass 2 in FP64 for the cells of a block whose threads call it with `mine`
+// (fx_cell_cells; the others only help with the barriers): y = sum over the
+// directions of Dh^T (h K . Dh x) and the face terms, from x itself.  Returns the
+// thread's part of <x, A x>.  Kept out of line, so that the fixed-point path keeps
+// its registers.
+template <int N, int BT>
+__device__ __noinline__ double fx_cell_wide(const double* x, const double* kt, const double* gh,
+                                            const DGTabN<double>* tn, double* y, long long c0,
+                                            int nblk, int Nc, bool mine, double* smem) {
+  constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
+  constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
+  constexpr double sigma = 2.0 * N * N;
+  const DGTabN<double>& t = *tn;
+  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int p = pt % N, q = pt / N;
+  mine = mine && lc < nblk;
+  const long long c = c0 + (mine ? lc : 0);
+  double* su = smem + (mine ? lc : 0) * SC;
+  double* sr = su + C * SC;
+  const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
+  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  const double iw = t.isw[p] * t.isw[p] * (t.isw[q] * t.isw[q]);
+  if (mine) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) su[e * SZ + q * SY + p] = x[c * N3 + e * N2 + pt];
+  }
+#pragma unroll 1
+  for (int dir = 2; dir >= 0; --dir) {
+    // the thread's line: points at + f step of the cell, at2 + f step2 in smem
+    const int at = dir == 2 ? pt : dir == 1 ? q * N2 + p : q * N2 + p * N;
+    const int step = dir == 2 ? N2 : dir == 1 ? N : 1;
+    const int at2 = dir == 2 ? q * SY + p : dir == 1 ? q * SZ + p : q * SZ + p * SY;
+    const int step2 = dir == 2 ? SZ : dir == 1 ? SY : 1;
+    __syncthreads();
+    if (!mine) continue;
+    double F[N], cv[2], cd[2];
+    {
+      double u[N], v0 = 0.0, v1 = 0.0, q0 = 0.0, q1 = 0.0;
+#pragma unroll
+      for (int f = 0; f < N; ++f) {
+        u[f] = su[at2 + f * step2];
+        // end values and outward half derivatives
+        v0 = fma(t.l0[f], u[f], v0);
+        v1 = fma(t.l1[f], u[f], v1);
+        q0 = fma(-t.hdl0[f], u[f], q0);
+        q1 = fma(t.hdl1[f], u[f], q1);
+      }
+#pragma unroll
+      for (int f = 0; f < N; ++f) {
+        double g = 0.0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) g = fma(t.Dh[f][j], u[j], g);
+        F[f] = kt[c * N3 + at + f * step] * (iw * (t.isw[f] * t.isw[f])) * g;
+      }
+      const long long stride = dir == 0 ? 1 : dir == 1 ? Nc : (long long)Nc * Nc;
+      const int cdir = dir == 0 ? crd[0] : dir == 1 ? crd[1] : crd[2];
+#pragma unroll
+      for (int up = 0; up < 2; ++up) {
+        double J = up ? v1 : v0, S = 2.0 * (up ? q1 : q0), once = 2.0;
+        if (up ? cdir < Nc - 1 : cdir > 0) {
+          const double* xn = x + (up ? c + stride : c - stride) * N3 + at;
+          double vn = 0.0, qn = 0.0;  // its outward direction is the opposite one
+#pragma unroll
+          for (int f = 0; f < N; ++f) {
+            const double w = xn[f * step];
+            vn = fma(up ? t.l0[f] : t.l1[f], w, vn);
+            qn = fma(up ? t.hdl0[f] : -t.hdl1[f], w, qn);
+          }
+          J -= vn;
+          S = (up ? q1 : q0) + qn;
+          once = 1.0;
+        }
+        const double g = gh[c * 6 + 2 * dir + up];
+        cv[up] = g * (sigma * J - S);
+        cd[up] = g * once * J;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      double r = dir == 2 ? 0.0 : sr[at2 + i * step2];
+      r = fma(t.l0[i], cv[0], r);
+      r = fma(t.hdl0[i], cd[0], r);
+      r = fma(t.l1[i], cv[1], r);
+      r = fma(-t.hdl1[i], cd[1], r);
+#pragma unroll
+      for (int f = 0; f < N; ++f) r = fma(t.Dh[f][i], F[f], r);
+      sr[at2 + i * step2] = r;
+    }
+  }
+  __syncthreads();
+  double dot = 0.0;
+  if (mine) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int o = e * SZ + q * SY + p;
+      y[c * N3 + e * N2 + pt] = sr[o];
+      dot = fma(su[o], sr[o], dot);
+    }
+  }
+  return dot;
 }
 
 __device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
@@ -441,13 +588,15 @@ __device__ __forceinline__ void fx_prefetch_l2(const void* p, unsigned bytes) {
 
 // Pass 2 over the cells c0 .. c0+nblk-1, called like pass 1; smem:
 // FxSmem<N, BT>::cell bytes.  xU: MODAL: the point values of pass 1 (integers);
-// otherwise the vector itself.  DOT: returns the thread's part of <x, A x>,
-// formed from the point values and the sum r before Q^T (Q is orthogonal).
-template <int N, bool MODAL, int BT, bool DOT = false, typename YS>
+// otherwise the vector itself, with FX_WIDE added to expM in the marked cells, and
+// wd.  DOT: returns the thread's part of <x, A x>, formed from the point values and
+// the sum r before Q^T (Q is orthogonal).
+template <int N, bool MODAL, int BT, bool DOT = false>
 __device__ __forceinline__ double fx_cell_cells(
     const void* xU, const long long* TR, const int* expU, const FxPair* __restrict__ lineop,
     const FxPair* __restrict__ gam, const int* __restrict__ expM, const int* __restrict__ expG,
-    YS&& y, long long c0, int nblk, int Nc, const DGTabX& tab, long long* smem) {
+    const FxWide wd, const FxStore y, long long c0, int nblk, int Nc, const DGTabX& tab,
+    long long* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -458,7 +607,8 @@ __device__ __forceinline__ double fx_cell_cells(
   long long* su = smem + (live ? lc : 0) * SC;
   long long* sr = su + C * SC;
   FxPair(*sg)[6] = reinterpret_cast<FxPair(*)[6]>(smem + 2 * C * SC);  // face coefficients
-  int(*sexp)[7] = reinterpret_cast<int(*)[7]>(sg + C);  // exponents: six faces, own terms
+  // exponents: six faces, own terms, the faces of neighbours with small lines
+  int(*sexp)[13] = reinterpret_cast<int(*)[13]>(sg + C);
   unsigned* slots = reinterpret_cast<unsigned*>(sexp + C);
   // the block's operators to L2, while exponents and vectors arrive (odd sizes
   // would leave the 16-byte grid)
@@ -475,17 +625,24 @@ __device__ __forceinline__ double fx_cell_cells(
       int e;
       if (f == 6) {
         e = expU[c] + expM[c];
+        if (!MODAL && wd.mark[c] == FX_MARKS) e += FX_WIDE;
       } else {
         const int d = f >> 1, cd = d == 0 ? crd[0] : d == 1 ? crd[1] : crd[2];
         const long long st = d == 0 ? stride[0] : d == 1 ? stride[1] : stride[2];
         e = (f & 1 ? cd < Nc - 1 : cd > 0) ? expU[f & 1 ? c + st : c - st] + expG[c * 6 + f]
                                            : -4 * FX_NAN;
         sg[lc][f] = gam[c * 6 + f];
+        if (!MODAL)  // an absent neighbour's own mark: the coefficient is zero
+          sexp[lc][7 + f] = wd.mark[f & 1 ? (cd < Nc - 1 ? c + st : c) : (cd > 0 ? c - st : c)] &
+                                    (1 << d)
+                                ? e
+                                : -4 * FX_NAN;
       }
       sexp[lc][f] = e;
     }
   }
   if (MODAL && 32 % N2 != 0 && threadIdx.x < 2 * FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
+  if (!MODAL && threadIdx.x == 0) slots[0] = 0;  // set if a cell of the block is applied in FP64
   long long u[N], r[N];
   // z-lines (a = p, b = q)
 #pragma unroll
@@ -508,6 +665,14 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
   for (int f = 0; f < 6; ++f) eout = max(eout, sexp[active ? lc : 0][f] + tab.bump);
   const bool bad = eout >= FX_NAN / 2;
+  bool wide = false;
+  if (!MODAL) {
+    int enb = eown;
+#pragma unroll
+    for (int f = 7; f < 13; ++f) enb = max(enb, sexp[active ? lc : 0][f] + tab.bump);
+    wide = active && !bad && (eown >= FX_WIDE / 2 || enb - eown > 9);
+    if (wide) slots[0] = 1;
+  }
   for (int f = pt; f < 6; f += N2) {
     if (!active) break;
     const int down = min(eout - sexp[lc][f], 63);
@@ -632,10 +797,17 @@ __device__ __forceinline__ double fx_cell_cells(
         sr[q * SZ + p * SY + a] =
             __double_as_longlong(bad ? qnan : fx_to_double(r[a], eout - 1));
     cell_sync<N>();
-    if (active) {  // written from the z-lines: consecutive lanes, consecutive words
+    if (active && !wide) {  // written from the z-lines: consecutive lanes, consecutive words
 #pragma unroll
       for (int e = 0; e < N; ++e)
         y(c * N3 + e * N2 + q * N + p, __longlong_as_double(sr[e * SZ + q * SY + p]));
+    }
+    if (slots[0] != 0) {
+      __syncthreads();
+      const double d =
+          fx_cell_wide<N, BT>(static_cast<const double*>(xU), wd.kt, wd.gh, wd.tn, y.y, c0, nblk,
+                              Nc, wide, reinterpret_cast<double*>(smem));
+      if (wide) dot = d;
     }
     return DOT && bad ? qnan : dot;
   }

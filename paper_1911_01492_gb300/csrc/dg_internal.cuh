@@ -143,6 +143,8 @@ struct dg_mesh {
   DGTabXGrad tabXG;
   FxPair *lineopX, *gamX;
   int *expM, *expG, *expU;
+  // point basis: expM with the mark of the operator, the marks of the vector
+  int *expN, *markU;
   int* expUb;  // exponents of the second vector of the coefficient gradient
 
   // coefficient data (dg_set_coefficient)

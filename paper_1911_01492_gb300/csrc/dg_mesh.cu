@@ -157,7 +157,7 @@ static cudaError_t dmalloc(P** p, size_t count) {
 }
 
 static void free_all(dg_mesh* m) {
-  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->expUb, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen, m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF,
+  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->expN, m->markU, m->expUb, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen, m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF,
                   m->U64,  m->X64,  m->TR64, m->TR32, m->U64b,
                   m->TR64b, m->hx_dev, m->hy_dev, m->r64, m->p64, m->q64,
                   m->t64,  m->s64, m->d32,  m->r32, m->p32, m->q32, m->partials, m->state,
@@ -223,6 +223,8 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->expM, nc);
   if (e == cudaSuccess) e = dmalloc(&m->expG, 6 * nc);
   if (e == cudaSuccess) e = dmalloc(&m->expU, nc);
+  if (e == cudaSuccess) e = dmalloc(&m->expN, nc);
+  if (e == cudaSuccess) e = dmalloc(&m->markU, nc);
   if (e == cudaSuccess) e = dmalloc(&m->kbar, nc);
   if (e == cudaSuccess) e = dmalloc(&m->dflag, 1);
   if (e == cudaSuccess) e = dmalloc(&m->U64, nd);

@@ -22,7 +22,7 @@
 // h gamma w_s w_t / 2 of a face point loses its tangential weights against
 // the two isw factors of the traces, so every point of a face has the weight
 // h gamma / 2 and no per-point face-weight array is read.
-#include "dg_apply_impl.cuh"
+#include "dg_fixed.cuh"
 
 namespace dgk {
 
@@ -112,26 +112,48 @@ k_collocation(const double* __restrict__ in, double* __restrict__ out, long long
 // 1 / diag(Q A Q^T): at point (a, b, e) the sum of the diagonal entries of the
 // x-, y- and z-line operators through it (the neighbour terms couple other
 // cells only).  The operators are integers with one exponent per cell
-// (dg_fixed.cu): the sum is one too.  One thread per DOF.
+// (dg_fixed.cu): the sum is one too.  In the marked cells, whose small entries do
+// not hold FP64's bits, it is formed from h w K and h gamma.  One thread per DOF.
 template <int N>
-__global__ void k_diag_nd(const FxPair* __restrict__ lineop, const int* __restrict__ expM,
+__global__ void k_diag_nd(const FxPair* __restrict__ lineop, const int* __restrict__ expN,
+                          const double* __restrict__ kt, const double* __restrict__ gh,
                           double* __restrict__ dinv64, float* __restrict__ dinv32,
-                          long long ndofs) {
+                          long long ndofs, int Nc, const __grid_constant__ DGTabN<double> tn) {
   constexpr int N2 = N * N, N3 = N * N * N, NP = N * (N + 1) / 2;
+  constexpr double sigma = 2.0 * N2;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ndofs) return;
   const long long c = t / N3;
   const int qi = (int)(t - c * N3);
   const int a = qi % N, b = (qi / N) % N, e = qi / N2;
-  const FxPair* L = lineop + c * 3 * NP * N2;
-  auto entry = [L](int dir, int line, int k) {
-    const FxPair v = L[(dir * NP + k) * N2 + line];
-    return ((long long)v.h << 30) + v.l;
-  };
-  const long long sum = entry(0, b + N * e, packed<N>(a, a)) +
-                        entry(1, a + N * e, packed<N>(b, b)) +
-                        entry(2, a + N * b, packed<N>(e, e));
-  const double di = 1.0 / scalbn((double)sum, expM[c] - 61);
+  double di;
+  if (expN[c] < FX_WIDE / 2) {
+    const FxPair* L = lineop + c * 3 * NP * N2;
+    auto entry = [L](int dir, int line, int k) {
+      const FxPair v = L[(dir * NP + k) * N2 + line];
+      return ((long long)v.h << 30) + v.l;
+    };
+    const long long sum = entry(0, b + N * e, packed<N>(a, a)) +
+                          entry(1, a + N * e, packed<N>(b, b)) +
+                          entry(2, a + N * b, packed<N>(e, e));
+    di = 1.0 / scalbn((double)sum, expN[c] - 61);
+  } else {
+    const int at[3] = {a, b, e}, step[3] = {1, N, N2};
+    const int crd[3] = {(int)(c % Nc), (int)((c / Nc) % Nc), (int)(c / ((long long)Nc * Nc))};
+    const double iw[3] = {tn.isw[a] * tn.isw[a], tn.isw[b] * tn.isw[b], tn.isw[e] * tn.isw[e]};
+    double sum = 0.0;
+    for (int d = 0; d < 3; ++d) {
+      const int i = at[d];
+      const double w = iw[(d + 1) % 3] * iw[(d + 2) % 3];
+      const double* k = kt + c * N3 + (qi - i * step[d]);
+      for (int f = 0; f < N; ++f)
+        sum = fma(k[f * step[d]] * (w * (tn.isw[f] * tn.isw[f])), tn.Dh[f][i] * tn.Dh[f][i], sum);
+      const double lo = crd[d] > 0 ? 2.0 : 4.0, up = crd[d] < Nc - 1 ? 2.0 : 4.0;
+      sum = fma(gh[c * 6 + 2 * d], tn.l0[i] * (sigma * tn.l0[i] + lo * tn.hdl0[i]), sum);
+      sum = fma(gh[c * 6 + 2 * d + 1], tn.l1[i] * (sigma * tn.l1[i] - up * tn.hdl1[i]), sum);
+    }
+    di = 1.0 / sum;
+  }
   dinv64[t] = di;
   dinv32[t] = (float)di;
 }
@@ -165,7 +187,8 @@ struct NodalF {
         return cudaGetLastError();
       case 3:
         k_diag_nd<N><<<(unsigned)((m->ndofs + 255) / 256), 256, 0, s>>>(
-            m->lineopX, m->expM, m->dinvN64, m->dinvN32, m->ndofs);
+            m->lineopX, m->expN, m->kt64, m->gh64, m->dinvN64, m->dinvN32, m->ndofs, m->N,
+            m->tabN64);
         return cudaGetLastError();
       default: return cudaErrorInvalidValue;
     }
