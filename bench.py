@@ -69,12 +69,13 @@ def hbm_gbs():
 def pass_bytes_per_dof(kernel: str, n: int):
     """Bytes per DOF that one launch of a fixed-point kernel reads and writes,
     every array once (csrc/dg_fixed.cuh, dg_multilinear.cu), in 8-byte words:
-    k_trace_fx   x, the point values (Legendre basis only), 12 n^2 trace words per cell;
+    k_trace_fx   x, the point values (Legendre basis only: the other one is
+                 k_trace_fx<n, false>), 12 n^2 trace words per cell;
     k_cell_fx    the point values, the line operators 3 n^2 n(n+1)/2, one trace pair
                  per neighbour face point, six face coefficients, y;
     k_cell_ml    the point values, 6 metric words, 5 coefficients per face point,
                  own and neighbour trace pairs, y."""
-    words = {"k_trace_fx": 2 + 12 / n, "k_trace_fx_nd": 1 + 12 / n,
+    words = {"k_trace_fx": 2 + 12 / n, "k_trace_fx<n, false>": 1 + 12 / n,
              "k_cell_fx": 2 + 1.5 * (n + 1) + 12 / n + 10 / n ** 3,
              "k_cell_ml": 8 + 30 / n + 24 / n}
     return 8.0 * words[kernel]
@@ -726,7 +727,7 @@ def run_nodal_apply(m, xd, world, steps=8):
     out = {"workload": "the benchmark workload, x mapped to the scaled Gauss-point basis",
            "apply_gdof_s": world * nd * steps * APPLIES_PER_STEP / (ms * 1e-3) / 1e9,
            "pass_ms": {"k_trace_fx": t1, "k_cell_fx": t2},
-           "roofline": {"k_trace_fx": memory_roofline("k_trace_fx_nd", n, nd, t1),
+           "roofline": {"k_trace_fx": memory_roofline("k_trace_fx<n, false>", n, nd, t1),
                         "k_cell_fx": memory_roofline("k_cell_fx", n, nd, t2)}}
     return out
 

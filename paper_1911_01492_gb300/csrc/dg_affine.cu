@@ -368,6 +368,8 @@ extern "C" int dg_set_geometry(dg_mesh* m, const double* A) {
   bool identity = true;
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) identity = identity && A[3 * i + j] == (i == j ? 1.0 : 0.0);
+  if (!identity && m->X64 == nullptr)
+    DG_CUDA(cudaMalloc((void**)&m->X64, sizeof(double) * (size_t)m->ndofs));
   for (int i = 0; i < 3; ++i) {
     for (int j = 0; j < 3; ++j) {
       double s = 0.0;

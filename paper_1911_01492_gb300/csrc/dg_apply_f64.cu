@@ -1,5 +1,4 @@
-// FP64 operator application by geometry and basis; the FP64 passes that remain
-// (traces for the curved geometries and the coefficient gradient).
+// FP64 operator application by geometry and basis.
 #include "dg_apply_impl.cuh"
 
 int dg_launch_apply_f64(const dg_mesh* m, const double* x, double* y, const int* skip,

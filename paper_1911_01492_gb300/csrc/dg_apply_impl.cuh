@@ -26,9 +26,9 @@
 //     remove further terms;
 //   * x-face traces and x-face test functions use the same parity split;
 //   * face-point weights W/2 = h gamma_F w_s w_t / 2 and the derivative weight
-//     (W/2 inside, W on the boundary) are precomputed when K is set, and
-//     2 sigma = 4 n^2 is a compile-time constant, so a face point costs five
-//     operations.
+//     (W/2 inside, W on the boundary) are read per point (dg_apply_static forms
+//     them from its K), and 2 sigma = 4 n^2 is a compile-time constant, so a face
+//     point costs five operations.
 // The only duplicated arithmetic is the pointwise flux of an interior face,
 // which both of its cells evaluate.
 //
@@ -293,15 +293,9 @@ template <typename T>
 struct FaceGlobal {
   const T* TR;
   const T* FW;
-  struct Pre {};  // nothing prefetched: the FP64 kernels hide load latency behind the FP64 pipe
-  template <int N>
-  __device__ __forceinline__ void prefetch(Pre&, long long, int, const bool (&)[6],
-                                           const long long (&)[6]) const {}
   template <int N, bool UPPER>
-  __device__ __forceinline__ void get(const Pre&, long long c, int lc, int f, bool in,
-                                      long long cn, int fn, int pt, T& cv,
-                                      T& cdm) const {
-    (void)lc;
+  __device__ __forceinline__ void get(long long c, int f, bool in, long long cn, int fn, int pt,
+                                      T& cv, T& cdm) const {
     face_point<N, UPPER>(TR, FW, c, f, in, cn, fn, pt, cv, cdm);
   }
 };
@@ -530,11 +524,6 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
   const long long sy = Nc, sz = (long long)Nc * Nc;
   const int o = lc * N3;
   const int pt = p + N * q;
-  // face f = x-, x+, y-, y+, z-, z+: interior?  neighbour cell
-  const bool in6[6] = {cx > 0, cx < Nc - 1, cy > 0, cy < Nc - 1, cz > 0, cz < Nc - 1};
-  const long long cn6[6] = {c - 1, c + 1, c - sy, c + sy, c - sz, c + sz};
-  typename FS::Pre pre;
-  if (active) fs.template prefetch<N>(pre, c, pt, in6, cn6);
 
   // z-lines then y-lines: collocation derivative, Kt, transpose, face terms
 #pragma unroll
@@ -569,8 +558,8 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       const bool inl = (dir == 0) ? (cz > 0) : (cy > 0);
       const long long st = (dir == 0) ? sz : sy;
       T cv1, cd1, cv0, cd0;
-      fs.template get<N, true>(pre, c, lc, fu, inu, c + st, fl, pt, cv1, cd1);
-      fs.template get<N, false>(pre, c, lc, fl, inl, c - st, fu, pt, cv0, cd0);
+      fs.template get<N, true>(c, fu, inu, c + st, fl, pt, cv1, cd1);
+      fs.template get<N, false>(c, fl, inl, c - st, fu, pt, cv0, cd0);
 #pragma unroll
       for (int e = 0; e < N; ++e) {
         T acc = fma(tab.l1[e], cv1, r[e]);
@@ -600,8 +589,8 @@ __device__ __forceinline__ void cell_core(const FS& fs, T* __restrict__ y, long 
       bt_bdt<N>(tab, rr, kg, R);
     }
     T cv1, cd1, cv0, cd0;
-    fs.template get<N, true>(pre, c, lc, 1, cx < Nc - 1, c + 1, 0, pt, cv1, cd1);
-    fs.template get<N, false>(pre, c, lc, 0, cx > 0, c - 1, 1, pt, cv0, cd0);
+    fs.template get<N, true>(c, 1, cx < Nc - 1, c + 1, 0, pt, cv1, cd1);
+    fs.template get<N, false>(c, 0, cx > 0, c - 1, 1, pt, cv0, cd0);
     // modal test functions: value a_i at 1, (-1)^i a_i at 0; derivative -d_i cd
     // at 1, -(-1)^(i+1) d_i cd at 0 (a_0 = 1, d_0 = 0)
     const T sp = cv1 + cv0, sm = cv1 - cv0;

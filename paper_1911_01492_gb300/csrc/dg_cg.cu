@@ -619,7 +619,7 @@ int launch_iteration_blocks(dg_mesh* m, double* x, bool kron, cudaStream_t s) {
                                                                    nullptr, n, m->partials,
                                                                    m->state);
   DG_CUDA(cudaGetLastError());
-  return kron ? dg_launch_kron_apply(m, m->r64, m->t64, nullptr, DG_KRON_FP64, s)
+  return kron ? dg_launch_kron_apply(m, m->r64, m->t64, DG_KRON_FP64, s)
               : dg_launch_block_apply(m, m->r64, m->t64, nullptr, false, s);
 }
 
@@ -638,7 +638,7 @@ int launch_iteration_mixed(dg_mesh* m, const float* dinv, cudaStream_t s, bool k
                                                                 nullptr, n, m->partials,
                                                                 m->state);
     DG_CUDA(cudaGetLastError());
-    return dg_launch_kron_apply(m, m->r32, m->q32, nullptr, DG_KRON_FP32, s);
+    return dg_launch_kron_apply(m, m->r32, m->q32, DG_KRON_FP32, s);
   }
   // all operands are the mesh's own allocations (256-byte aligned)
   if (dinv)
@@ -663,7 +663,7 @@ int refine_mixed(dg_mesh* m, const double* b, double* x, const double* dinv, cud
   else
     k_refine_r<false><<<RED_LAUNCH>>>(b, m->q64, m->r64, m->r32, dinv, n, m->partials, m->state);
   DG_CUDA(cudaGetLastError());
-  if (kron) return dg_launch_kron_apply(m, m->r32, m->q32, nullptr, DG_KRON_FP32, s);
+  if (kron) return dg_launch_kron_apply(m, m->r32, m->q32, DG_KRON_FP32, s);
   return DG_OK;
 }
 
@@ -758,7 +758,7 @@ int cg_fp64(dg_mesh* m, const double* b, double* x, double rtol, int maxit, dg_c
       if (rc) return rc;
     }
     if (kron) {
-      rc = dg_launch_kron_apply(m, m->r64, m->t64, m->p64, DG_KRON_FP64_INIT, s);
+      rc = dg_launch_kron_apply(m, m->r64, m->t64, DG_KRON_FP64_INIT, s);
       if (rc) return rc;
     }
     rc = run_graph(m, s, chunk_for(m), [&] {
@@ -835,7 +835,7 @@ int cg_mixed(dg_mesh* m, const double* b, double* x, double rtol, int maxit, dg_
                             s));
   }
   if (kron) {  // z = M^-1 r into q32, rho_new = <z, r>, beta = 0 (restart)
-    rc = dg_launch_kron_apply(m, m->r32, m->q32, nullptr, DG_KRON_FP32, s);
+    rc = dg_launch_kron_apply(m, m->r32, m->q32, DG_KRON_FP32, s);
     if (rc) return rc;
   }
   // replay a graph of FP32 iterations; refine in FP64 whenever one asked for it

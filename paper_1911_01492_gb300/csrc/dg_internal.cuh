@@ -193,8 +193,9 @@ struct dg_mesh {
   double* kbar;     // Kbar_c                          [c]
   int* dflag;       // device-side error flag of the setup kernels
 
-  // apply workspaces: nodal values, x-modal/yz-nodal values, face traces
-  double *U64, *X64, *TR64;
+  // apply workspaces: nodal values, face traces; x-modal/yz-nodal values (affine
+  // geometry, allocated by dg_set_geometry)
+  double *U64, *TR64, *X64;
   float* TR32;
   // second set for the coefficient gradient (of v), lazily allocated
   double *U64b, *TR64b;
@@ -349,12 +350,11 @@ int dg_ensure_diagonal(dg_mesh* m, cudaStream_t s);
 int dg_ensure_block(dg_mesh* m, cudaStream_t s);
 // Kronecker cell-block preconditioner (dg_kron.cu): factors formed once per
 // coefficient; z = M^-1 r with <z, r> into the CG state (mode: FP64 iteration,
-// FP64 initialisation with p = z, FP32 mixed iteration)
+// FP64 initialisation, FP32 mixed iteration)
 enum { DG_KRON_FP64 = 0, DG_KRON_FP64_INIT = 1, DG_KRON_FP32 = 2 };
 int dg_ensure_kron(dg_mesh* m, cudaStream_t s);
 int dg_ensure_kron_nodal(dg_mesh* m, cudaStream_t s);  // the same in the point basis
-int dg_launch_kron_apply(const dg_mesh* m, const void* r, void* z, void* p, int mode,
-                         cudaStream_t s);
+int dg_launch_kron_apply(const dg_mesh* m, const void* r, void* z, int mode, cudaStream_t s);
 int dg_launch_block_apply(const dg_mesh* m, const double* r, double* z, double* p, bool init,
                           cudaStream_t s);
 // workspace helpers (dg_mesh.cu)

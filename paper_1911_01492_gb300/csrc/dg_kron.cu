@@ -133,10 +133,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& t) {
 // cell, ~128 threads), shared memory for the work array and the factors
 // within 40 KB (48 KB with the reduction arrays); at least Cfg<N>::CPB so the
 // block count fits the mesh's per-block partials.
-template <int N, typename T>
+template <int N>
 struct KronCfg {
   static constexpr int KS = 3 * N * N + 3 * N;
-  static constexpr int PER_CELL = (N * N * N + KS) * (int)sizeof(T);
+  static constexpr int PER_CELL = (N * N * N + KS) * (int)sizeof(float);
   static constexpr int BY_THREADS = 128 / N, BY_SMEM = 40960 / PER_CELL;
   static constexpr int C = BY_THREADS < BY_SMEM ? BY_THREADS : BY_SMEM;  // cells per block
   static constexpr int THREADS = C * N;
@@ -144,7 +144,10 @@ struct KronCfg {
 };
 
 // The grid reduction of <z, r>: each block publishes its partial, the last
-// block sums them in a fixed order and sets the CG scalars by MODE.
+// block sums them in a fixed order and sets the CG scalars by MODE: 0 FP64
+// iteration (beta = <z,r> / rho, rho = <z,r>); 1 FP64 initialisation (rho = <z,r>,
+// runs even when done; the first direction update takes z with beta = 0); 2 FP32
+// mixed iteration (rho_new = <z,r>, beta = 0 on a restart, else <z,r> / rho).
 template <int NT, int MODE>
 __device__ __forceinline__ void kron_finish(double part, double* __restrict__ partials,
                                             DGCGState* st, double* rd) {
@@ -186,61 +189,61 @@ __device__ __forceinline__ void kron_finish(double part, double* __restrict__ pa
 // uses a fast reciprocal (two ulps: the preconditioner only needs to be a
 // fixed symmetric positive definite operator).  Every thread of the block
 // calls it; it synchronises before returning.
-template <int N, typename T>
-__device__ __forceinline__ T kron_solve_cells(T* sw, const T* sq, int nblk) {
+template <int N>
+__device__ __forceinline__ float kron_solve_cells(float* sw, const float* sq, int nblk) {
   constexpr int N2 = N * N, N3 = N * N * N, KS = 3 * N2 + 3 * N;
   const int lc = threadIdx.x / N;
   const int t = threadIdx.x - lc * N;
   const bool active = lc < nblk;
-  T* w = sw + lc * N3;
-  const T* Qx = sq + lc * KS;
-  const T* Qy = Qx + N2;
-  const T* Qz = Qy + N2;
-  const T* lam = Qx + 3 * N2;
-  T q[N][N];
-  auto load_q = [&](const T* Q) {
+  float* w = sw + lc * N3;
+  const float* Qx = sq + lc * KS;
+  const float* Qy = Qx + N2;
+  const float* Qz = Qy + N2;
+  const float* lam = Qx + 3 * N2;
+  float q[N][N];
+  auto load_q = [&](const float* Q) {
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
       for (int k = 0; k < N; ++k) q[i][k] = Q[i * N + k];
   };
-  // one line of w (first element f, stride sd): w <- Q^T w (TR) or Q w
+  // one line of w (first element f, stride sd): w <- Q^float w (TR) or Q w
   auto line = [&](int f, int sd, bool tr) {
-    T v[N];
+    float v[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = w[f + i * sd];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      T a = (tr ? q[0][k] : q[k][0]) * v[0];
+      float a = (tr ? q[0][k] : q[k][0]) * v[0];
 #pragma unroll
       for (int i = 1; i < N; ++i) a = fma(tr ? q[i][k] : q[k][i], v[i], a);
       w[f + k * sd] = a;
     }
   };
-  if (active) {  // (Q_x)^T along the x-lines (j, l = t)
+  if (active) {  // (Q_x)^float along the x-lines (j, l = t)
     load_q(Qx);
 #pragma unroll
     for (int j = 0; j < N; ++j) line(t * N2 + j * N, 1, true);
   }
   __syncthreads();
-  if (active) {  // (Q_y)^T along the y-lines (i, l = t)
+  if (active) {  // (Q_y)^float along the y-lines (i, l = t)
     load_q(Qy);
 #pragma unroll
     for (int i = 0; i < N; ++i) line(t * N2 + i, N, true);
   }
   __syncthreads();
-  T acc = T(0);
+  float acc = 0.0f;
   if (active) {  // z-lines (i, j = t): (Q_z)^T, the scaling, Q_z
     load_q(Qz);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      T v[N], u[N];
+      float v[N], u[N];
 #pragma unroll
       for (int l = 0; l < N; ++l) v[l] = w[l * N2 + t * N + i];
-      const T lxy = lam[i] + lam[N + t];
+      const float lxy = lam[i] + lam[N + t];
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        T a = q[0][k] * v[0];
+        float a = q[0][k] * v[0];
 #pragma unroll
         for (int l = 1; l < N; ++l) a = fma(q[l][k], v[l], a);
         u[k] = a * __fdividef(1.0f, lxy + lam[2 * N + k]);
@@ -248,7 +251,7 @@ __device__ __forceinline__ T kron_solve_cells(T* sw, const T* sq, int nblk) {
       }
 #pragma unroll
       for (int l = 0; l < N; ++l) {
-        T a = q[l][0] * u[0];
+        float a = q[l][0] * u[0];
 #pragma unroll
         for (int k = 1; k < N; ++k) a = fma(q[l][k], u[k], a);
         w[l * N2 + t * N + i] = a;
@@ -286,32 +289,25 @@ __device__ __forceinline__ double block_total(double v, double* rd) {
   return s;
 }
 
-// MODE: 0 FP64 PCG iteration (beta = <z,r> / rho, rho = <z,r>); 1 FP64
-// initialisation (rho = <z,r>, p = z, runs even when done); 2 FP32 mixed
-// iteration (rho_new = <z,r>, beta = 0 on a restart, else <z,r> / rho).
-template <int N, typename T, int MODE>
-__global__ void __launch_bounds__(KronCfg<N, T>::THREADS)
-k_kron_apply(const T* __restrict__ KD, const T* __restrict__ r, T* __restrict__ z,
-             T* __restrict__ p, long long ncells, double* __restrict__ partials, DGCGState* st) {
-  using KC = KronCfg<N, T>;
+// The FP32 form, of the mixed iteration (kron_finish MODE 2).
+template <int N>
+__global__ void __launch_bounds__(KronCfg<N>::THREADS)
+k_kron_apply(const float* __restrict__ KD, const float* __restrict__ r, float* __restrict__ z,
+             long long ncells, double* __restrict__ partials, DGCGState* st) {
+  using KC = KronCfg<N>;
   constexpr int C = KC::C, N3 = N * N * N, NT = KC::THREADS, KS = KC::KS;
-  if (MODE != 1 && st->done) return;
-  if (MODE == 2 && st->ru_skip == 0) return;  // an FP64 refinement is pending
-  __shared__ T sw[C * N3], sq[C * KS];
+  if (st->done || st->ru_skip == 0) return;  // ru_skip = 0: an FP64 refinement is pending
+  __shared__ float sw[C * N3], sq[C * KS];
   __shared__ double rd[NT];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   for (int i = threadIdx.x; i < nblk * N3; i += NT) sw[i] = r[c0 * N3 + i];
   for (int i = threadIdx.x; i < nblk * KS; i += NT) sq[i] = KD[c0 * KS + i];
   __syncthreads();
-  const T acc = kron_solve_cells<N, T>(sw, sq, nblk);
-  for (int i = threadIdx.x; i < nblk * N3; i += NT) {
-    const T zv = sw[i];
-    z[c0 * N3 + i] = zv;
-    if (MODE == 1) p[c0 * N3 + i] = zv;
-  }
+  const float acc = kron_solve_cells<N>(sw, sq, nblk);
+  for (int i = threadIdx.x; i < nblk * N3; i += NT) z[c0 * N3 + i] = sw[i];
   const double part = block_total<NT>((double)acc, rd);
-  kron_finish<NT, MODE>(part, partials, st, rd);
+  kron_finish<NT, 2>(part, partials, st, rd);
 }
 
 // z = M^-1 r in FP64 vectors, contractions in block fixed point: in FP64 the
@@ -325,8 +321,8 @@ k_kron_apply(const T* __restrict__ KD, const T* __restrict__ r, T* __restrict__ 
 template <int N, int MODE>
 __global__ void __launch_bounds__(Cfg<N>::THREADS)
 k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
-                const double* __restrict__ r, double* __restrict__ z, double* __restrict__ p,
-                long long ncells, double* __restrict__ partials, DGCGState* st) {
+                const double* __restrict__ r, double* __restrict__ z, long long ncells,
+                double* __restrict__ partials, DGCGState* st) {
   constexpr int C = Cfg<N>::CPB, T = Cfg<N>::THREADS, N2 = N * N, N3 = N * N * N;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC, NS = FxSmem<N, T>::NS;
   if (MODE != 1 && st->done) return;
@@ -435,7 +431,6 @@ k_kron_apply_fx(const FxPair* __restrict__ KX, const double* __restrict__ winv,
     for (int l = 0; l < N; ++l) {
       const double zv = bad ? qnan : fx_to_double(u[l], ez);
       z[c * N3 + l * N2 + pt] = zv;
-      if (MODE == 1) p[c * N3 + l * N2 + pt] = zv;
     }
   }
   const double part = block_total<T>(acc, rd);
@@ -532,9 +527,8 @@ struct KronSetupF {
 template <int N>
 struct KronApplyF {
   template <typename T>
-  static cudaError_t run(const dg_mesh* m, const void* r, void* z, void* p, int mode,
-                         cudaStream_t s) {
-    using K32 = KronCfg<N, float>;
+  static cudaError_t run(const dg_mesh* m, const void* r, void* z, int mode, cudaStream_t s) {
+    using K32 = KronCfg<N>;
     // inside a solve in the scaled Gauss-point basis: the rotated factors
     const FxPair* fx = m->nodal_op ? m->kronNX : m->kronX;
     const float* f32 = m->nodal_op ? m->kronN32 : m->kron32;
@@ -543,18 +537,15 @@ struct KronApplyF {
     switch (mode) {
       case DG_KRON_FP64:
         k_kron_apply_fx<N, 0><<<bx, Cfg<N>::THREADS, 0, s>>>(
-            fx, m->kronW, (const double*)r, (double*)z, nullptr, m->ncells, m->partials_cells,
-            m->state);
+            fx, m->kronW, (const double*)r, (double*)z, m->ncells, m->partials_cells, m->state);
         break;
       case DG_KRON_FP64_INIT:
         k_kron_apply_fx<N, 1><<<bx, Cfg<N>::THREADS, 0, s>>>(
-            fx, m->kronW, (const double*)r, (double*)z, (double*)p, m->ncells,
-            m->partials_cells, m->state);
+            fx, m->kronW, (const double*)r, (double*)z, m->ncells, m->partials_cells, m->state);
         break;
       default:
-        k_kron_apply<N, float, 2><<<b32, K32::THREADS, 0, s>>>(
-            f32, (const float*)r, (float*)z, nullptr, m->ncells, m->partials_cells,
-            m->state);
+        k_kron_apply<N><<<b32, K32::THREADS, 0, s>>>(f32, (const float*)r, (float*)z, m->ncells,
+                                                     m->partials_cells, m->state);
         break;
     }
     return cudaGetLastError();
@@ -625,11 +616,10 @@ static int ensure_kron_fx(dg_mesh* m, cudaStream_t s) {
   return DG_OK;
 }
 
-int dg_launch_kron_apply(const dg_mesh* m, const void* r, void* z, void* p, int mode,
-                         cudaStream_t s) {
+int dg_launch_kron_apply(const dg_mesh* m, const void* r, void* z, int mode, cudaStream_t s) {
   if (mode == DG_KRON_FP64_INIT)  // runs before the iterations are captured
     if (int rc = ensure_kron_fx(const_cast<dg_mesh*>(m), s)) return rc;
-  cudaError_t e = dgk::dispatch_n<double, dgk::KronApplyF>(m->n, m, r, z, p, mode, s);
+  cudaError_t e = dgk::dispatch_n<double, dgk::KronApplyF>(m->n, m, r, z, mode, s);
   if (e != cudaSuccess) return dg_cuda_fail(e, "Kronecker cell blocks: apply");
   return DG_OK;
 }

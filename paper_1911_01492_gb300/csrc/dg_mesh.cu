@@ -228,7 +228,6 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->kbar, nc);
   if (e == cudaSuccess) e = dmalloc(&m->dflag, 1);
   if (e == cudaSuccess) e = dmalloc(&m->U64, nd);
-  if (e == cudaSuccess) e = dmalloc(&m->X64, nd);
   if (e == cudaSuccess) e = dmalloc(&m->TR64, ntr);
   if (e == cudaSuccess) e = dmalloc(&m->TR32, ntr);
   if (e != cudaSuccess) {
