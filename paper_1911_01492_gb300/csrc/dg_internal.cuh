@@ -19,6 +19,7 @@ struct DGTab {
   T Bd[DG_MAXN][DG_MAXN];  // Bd[a][i] = L_i'(xi_a)     modal -> nodal derivative
   T D[DG_MAXN][DG_MAXN];   // D[a][b]  = l_b'(xi_a)     nodal collocation derivative
   T w[DG_MAXN];            // Gauss weights on [0,1] (sum 1)
+  T wl[DG_MAXN];           // what rounding to T left of them (FP32)
   T a0[DG_MAXN], a1[DG_MAXN];    // L_i(0), L_i(1)
   T d0[DG_MAXN], d1[DG_MAXN];    // L_i'(0), L_i'(1)
   T l0[DG_MAXN], l1[DG_MAXN];    // l_a(0), l_a(1)     (Lagrange basis on the Gauss points)
@@ -153,6 +154,7 @@ struct dg_mesh {
   float* kt32;
   double* gh64;     // h gamma_F per face side        [c][6] (x-, x+, y-, y+, z-, z+)
   float* gh32;
+  float2* gh32s;    // the same as a sum of two numbers (dg_apply in FP32)
   double* dgam;     // d gamma_F / d log Kbar_c       [c][6]
   // Jacobi preconditioner: 1 / diag(A), formed on the first preconditioned solve
   double* diag64;
@@ -234,15 +236,15 @@ void dg_timing_mark(const dg_mesh* m, int slot, cudaStream_t s);
 
 // coefficient setup kernels (dg_mesh.cu), shared with the allocation-free
 // apply: h w_q K and Kbar per cell (FP32 copy skipped when kt32 is NULL); h gamma
-// and d gamma / d log Kbar per face side (gh32 / dgam skipped when NULL)
+// and d gamma / d log Kbar per face side (gh32 with gh32s / dgam skipped when NULL)
 cudaError_t dg_launch_coef_cells(const double* K, double* kt64, float* kt32, double* kbar,
                                  long long ncells, int n, double h, int* flag,
                                  const DGTab<double>& tab, cudaStream_t s);
 // (dmask: bit f set when boundary side f is Dirichlet; the boundary faces of
 // the other sides carry zero flux, gamma = 0)
 __global__ void k_coef_faces(const double* __restrict__ kbar, double* __restrict__ gh64,
-                             float* __restrict__ gh32, double* __restrict__ dgam, int Nc,
-                             double h, int dmask);
+                             float* __restrict__ gh32, float2* __restrict__ gh32s,
+                             double* __restrict__ dgam, int Nc, double h, int dmask);
 
 // error reporting (dg_mesh.cu)
 int dg_fail(int code, const char* fmt, ...);

@@ -118,8 +118,8 @@ cudaError_t dg_launch_coef_cells(const double* K, double* kt64, float* kt32, dou
 // side whose bit is clear in dmask carries zero flux (homogeneous Neumann): no
 // face term at all, i.e. gamma = 0 there.
 __global__ void k_coef_faces(const double* __restrict__ kbar, double* __restrict__ gh64,
-                             float* __restrict__ gh32, double* __restrict__ dgam, int Nc,
-                             double h, int dmask) {
+                             float* __restrict__ gh32, float2* __restrict__ gh32s,
+                             double* __restrict__ dgam, int Nc, double h, int dmask) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nc = (long long)Nc * Nc * Nc;
   if (c >= nc) return;
@@ -143,7 +143,11 @@ __global__ void k_coef_faces(const double* __restrict__ kbar, double* __restrict
       dg = 0.0;
     }
     gh64[c * 6 + f] = h * g;
-    if (gh32 != nullptr) gh32[c * 6 + f] = (float)(h * g);
+    if (gh32 != nullptr) {
+      const float hi = (float)(h * g);
+      gh32[c * 6 + f] = hi;
+      gh32s[c * 6 + f] = make_float2(hi, isfinite(hi) ? (float)(h * g - (double)hi) : 0.0f);
+    }
     if (dgam != nullptr) dgam[c * 6 + f] = dg;
   }
 }
@@ -157,7 +161,7 @@ static cudaError_t dmalloc(P** p, size_t count) {
 }
 
 static void free_all(dg_mesh* m) {
-  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->dgam, m->kbar, m->dflag, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->expN, m->markU, m->expUb, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen, m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF,
+  void* ptrs[] = {m->kt64, m->kt32, m->gh64, m->gh32, m->gh32s, m->dgam, m->kbar, m->dflag, m->lineopX, m->gamX, m->expM, m->expG, m->expU, m->expN, m->markU, m->expUb, m->diag64, m->dinv64, m->dinv32, m->binv64, m->kron64, m->kron32, m->kronX, m->kronNX, m->kronW, m->dinvN64, m->dinvN32, m->bN64, m->xN64, m->hk32, m->kronN64, m->kronN32, m->geo_vol, m->geo_det, m->geo_face, m->geo_pen, m->mlV, m->mlF, m->mlExpV, m->mlExpM, m->mlExpF,
                   m->U64,  m->X64,  m->TR64, m->TR32, m->U64b,
                   m->TR64b, m->hx_dev, m->hy_dev, m->r64, m->p64, m->q64,
                   m->t64,  m->s64, m->d32,  m->r32, m->p32, m->q32, m->partials, m->state,
@@ -216,6 +220,7 @@ extern "C" int dg_create_mesh(int n_cells, int degree, dg_mesh** out) {
   if (e == cudaSuccess) e = dmalloc(&m->kt32, nd);
   if (e == cudaSuccess) e = dmalloc(&m->gh64, 6 * nc);
   if (e == cudaSuccess) e = dmalloc(&m->gh32, 6 * nc);
+  if (e == cudaSuccess) e = dmalloc(&m->gh32s, 6 * nc);
   if (e == cudaSuccess) e = dmalloc(&m->dgam, 6 * nc);
   if (e == cudaSuccess)
     e = dmalloc(&m->lineopX, (size_t)3 * n2 * (size_t)(m->n * (m->n + 1) / 2) * nc);
@@ -351,7 +356,7 @@ extern "C" int dg_set_coefficient(dg_mesh* m, const double* K, void* stream) {
                                m->tab64, s));
   {
     const unsigned blocks = (unsigned)((m->ncells + 255) / 256);
-    k_coef_faces<<<blocks, 256, 0, s>>>(m->kbar, m->gh64, m->gh32, m->dgam, m->N, m->h,
+    k_coef_faces<<<blocks, 256, 0, s>>>(m->kbar, m->gh64, m->gh32, m->gh32s, m->dgam, m->N, m->h,
                                         m->dirichlet_mask);
     DG_CUDA(cudaGetLastError());
     if (!m->affine)

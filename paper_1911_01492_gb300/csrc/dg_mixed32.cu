@@ -326,7 +326,7 @@ k_dir32_bulk(const float* __restrict__ r, float* __restrict__ p, float* __restri
 template <int N, bool DOT>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, N <= 5 ? 8 : 1)
 k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
-           const float* __restrict__ kt, const float* __restrict__ gh, float* __restrict__ qg,
+           const float* __restrict__ kt, const void* __restrict__ gh, float* __restrict__ qg,
            long long cbeg, long long ncells, int Nc, const int* __restrict__ skip,
            double* __restrict__ partials, DGCGState* st,
            const __grid_constant__ DGTab<float> tab) {
@@ -409,7 +409,19 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
   const bool pairrow = vb && cxb != 0;  // both cells of the pair in one x-row
   const long long sy = Nc, sz = (long long)Nc * Nc;
   const int pt = p + N * q;
-  const float hw2 = 0.5f * tab.w[pt % N] * tab.w[pt / N];
+  // Half the face weight of the thread's point.  The operator alone takes it and h
+  // gamma as sums of two numbers, so that W/2 carries one rounding, as the stored
+  // weights of the generic passes did: with five the error of an application of
+  // degree 2 was a third larger.
+  const float w0 = 0.5f * tab.w[pt % N], w1 = tab.w[pt / N], hw2 = w0 * w1;
+  const float hwl = DOT ? 0.0f
+                        : fmaf(w0, w1, -hw2) +
+                              fmaf(w0, tab.wl[pt / N], 0.5f * tab.wl[pt % N] * w1);
+  auto weight = [&](long long c, int f) {
+    if constexpr (DOT) return hw2 * static_cast<const float*>(gh)[c * 6 + f];
+    const float2 g = static_cast<const float2*>(gh)[c * 6 + f];
+    return fmaf(g.x, hw2, fmaf(g.x, hwl, g.y * hw2));
+  };
   // face f's neighbour trace (value, derivative) and weight W/2 for both lanes;
   // zero trace on a boundary lane
   auto face = [&](int f, bool ina, bool inb, long long cna, long long cnb, F2& un, F2& gn,
@@ -419,7 +431,7 @@ k_cell32x2(const float* __restrict__ pg, const float* __restrict__ TR,
     if (inb && ldb) load_trace<N>(TR, cnb, f ^ 1, pt, ub, gb);
     un = F2(ua, ub);
     gn = F2(ga, gb);
-    wh = F2(va ? hw2 * gh[ca * 6 + f] : 0.0f, vb ? hw2 * gh[cb * 6 + f] : 0.0f);
+    wh = F2(va ? weight(ca, f) : 0.0f, vb ? weight(cb, f) : 0.0f);
     e = F2(ina ? 1.0f : 2.0f, inb ? 1.0f : 2.0f);
   };
   F2 un[4], gn[4], wh[4], ee[4];  // faces z-, z+, y-, y+ (then x-, x+ in slots 0, 1)
@@ -991,7 +1003,7 @@ struct Pass32F {
           x, m->TR32, cbeg, cend, skip, m->tab32);
     else
       k_cell32x2<N, false><<<(unsigned)((cend - cbeg + 2 * C - 1) / (2 * C)), Cfg<N>::THREADS,
-                             sizeof(F2) * 4 * C * LinePad<N>::SC, s>>>(x, m->TR32, m->kt32, m->gh32, y, cbeg,
+                             sizeof(F2) * 4 * C * LinePad<N>::SC, s>>>(x, m->TR32, m->kt32, m->gh32s, y, cbeg,
                                                           cend, m->N, skip, nullptr, nullptr,
                                                           m->tab32);
     return cudaGetLastError();

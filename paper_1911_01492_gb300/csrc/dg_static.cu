@@ -130,7 +130,7 @@ extern "C" int dg_apply_static(int n_cells, int degree, const double* K, const d
   DG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
   // the coefficient kernels of dg_set_coefficient, FP64 outputs only
   DG_CUDA(dg_launch_coef_cells(K, kt, nullptr, kbar, ncells, n, h, flag, tab, s));
-  k_coef_faces<<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(kbar, gh, nullptr, nullptr,
+  k_coef_faces<<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(kbar, gh, nullptr, nullptr, nullptr,
                                                                 n_cells, h, DG_BC_DIRICHLET);
   dgk::k_face_weights<double><<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(gh, FW, n_cells, n,
                                                                               tab);

@@ -100,6 +100,7 @@ void copy_round(const DGTab<S>& s, DGTab<D>* d) {
       d->D[a][b] = (D)s.D[a][b];
     }
     d->w[a] = (D)s.w[a];
+    d->wl[a] = (D)(s.w[a] - (S)d->w[a]);
     d->a0[a] = (D)s.a0[a];
     d->a1[a] = (D)s.a1[a];
     d->d0[a] = (D)s.d0[a];
