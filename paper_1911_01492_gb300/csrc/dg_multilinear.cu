@@ -440,13 +440,15 @@ template <int N>
 struct MlSmem {
   static constexpr int C = Cfg<N>::CPB;
   static constexpr size_t trace = 8 * 4 * C * LinePad<N>::SC;
-  // u / r, the flux; per cell: nine shifts per face, then F's and Dh^T F's, ER
+  // u / r, the flux; per cell: nine shifts and exponents per face, then those of
+  // the volume flux and the largest of F's and of r's lifted terms
   static constexpr int SH = 6 * 9 + 3;
   static constexpr size_t cell = 8 * 5 * C * LinePad<N>::SC + 4 * (SH * C);
 };
 
+// Registers for one block per SM more than they would allow by themselves (n = 6-8).
 template <int N>
-__global__ void __launch_bounds__(Cfg<N>::THREADS)
+__global__ void __launch_bounds__(Cfg<N>::THREADS, N == 8 ? 4 : N == 6 || N == 7 ? 3 : 0)
 k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
           const int* __restrict__ expU, MlData md, double* __restrict__ y, long long ncells,
           int Nc, const int* __restrict__ skip, const __grid_constant__ DGTabX tab,
@@ -456,7 +458,7 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
   constexpr int NS = FxSmem<N, T>::NS, SH = MlSmem<N>::SH;
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned slots[2 * NS];
+  __shared__ unsigned slots[3 * NS];
   const long long c0 = (long long)blockIdx.x * C;
   const int nblk = (int)((ncells - c0) < C ? (ncells - c0) : C);
   const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
@@ -471,14 +473,15 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
   const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
   const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
   const long long stride[3] = {1, Nc, (long long)Nc * Nc};
-  if (threadIdx.x < 2 * NS) slots[threadIdx.x] = 0;
-  // Exponents and shifts, one thread per cell.  F sums the volume flux, halved
+  for (int i = threadIdx.x; i < 3 * NS; i += T) slots[i] = 0;
+  // Exponents and shifts, one thread per cell; EF and ER, those of F and r, follow
+  // once the cell's largest derivative is known.  F sums the volume flux, halved
   // (<= 2^59), and six lifted terms (each below 2^61, five bits down): below
   // 2^60.  r sums Dh^T F in three directions and six lifted terms three bits
   // down: below 2^62.5.
   if (active && pt == 0) {
     const int Eo = expU[c], em = md.em[c];
-    int EF = md.eV[c] + tg.cD + Eo + 1, ER = -4 * FX_NAN, eJ[6], eD[6];
+    int EF = -4 * FX_NAN, ER = -4 * FX_NAN, eJ, eD;
     bool nan = Eo >= FX_NAN / 2 || md.eV[c] >= FX_NAN / 2;
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
@@ -487,29 +490,26 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
       const long long cn = in ? (f & 1 ? c + stride[d] : c - stride[d]) : c;
       const int En = expU[cn], mn = md.em[cn];
       nan = nan || En >= FX_NAN / 2 || md.ef[(c * 6 + f) * 3] >= FX_NAN / 2;
-      eJ[f] = max(Eo, En) + 1;
-      eD[f] = max(Eo + em, En + mn) + 1;
-      sh[9 * f + 0] = min(eJ[f] - Eo, 63);
-      sh[9 * f + 1] = min(eJ[f] - En, 63);
-      sh[9 * f + 2] = min(eD[f] - Eo - em, 63);
-      sh[9 * f + 3] = min(eD[f] - En - mn, 63);
-      eJ[f] += tg.cv;
-      eD[f] += tg.cv + tg.cD;
-      EF = max(EF, md.ef[(c * 6 + f) * 3] + eJ[f] + tg.cl + 5);
-      ER = max(ER, max(md.ef[(c * 6 + f) * 3 + 2] + eJ[f], md.ef[(c * 6 + f) * 3 + 1] + eD[f]) +
-                       tg.cl + 3);
-    }
-    ER = max(ER, EF + tg.cD);
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
+      eJ = max(Eo, En) + 1;
+      eD = max(Eo + em, En + mn) + 1;
+      sh[9 * f + 0] = min(eJ - Eo, 63);
+      sh[9 * f + 1] = min(eJ - En, 63);
+      sh[9 * f + 2] = min(eD - Eo - em, 63);
+      sh[9 * f + 3] = min(eD - En - mn, 63);
+      eJ += tg.cv;
+      eD += tg.cv + tg.cD;
+      // exponents of the lifted terms of F, and of the two of r
       const int* ef = md.ef + (c * 6 + f) * 3;
-      sh[9 * f + 4] = min(EF - tg.cl - ef[0] - eJ[f], 63);
-      sh[9 * f + 5] = min(ER - tg.cl - ef[2] - eJ[f], 63);
-      sh[9 * f + 6] = min(ER - tg.cl - ef[1] - eD[f], 63);
+      sh[9 * f + 4] = ef[0] + eJ + tg.cl;
+      sh[9 * f + 5] = ef[2] + eJ + tg.cl;
+      sh[9 * f + 6] = ef[1] + eD + tg.cl;
+      EF = max(EF, sh[9 * f + 4] + 5);
+      ER = max(ER, max(sh[9 * f + 5], sh[9 * f + 6]) + 3);
     }
-    sh[54] = min(EF - md.eV[c] - tg.cD - Eo, 63);
-    sh[55] = min(ER - EF - tg.cD, 63);
-    sh[56] = nan ? FX_NAN : ER;
+    sh[54] = md.eV[c] + tg.cD + Eo;
+    sh[55] = EF;
+    sh[56] = ER;
+    sh[7] = nan;
   }
   const int zl = q * SY + p, yl = q * SZ + p, xl = q * SZ + p * SY;
   long long u[N], v[N], F[3][N], r[N];
@@ -518,42 +518,56 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
     u[e] = U[c * N3 + e * N2 + pt];
     su[zl + e * SZ] = u[e];
   }
+  unsigned top = 0;
+  auto largest = [&](const long long (&w)[N]) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) top = max(top, fx_mag_hi(w[e]));
+  };
   fx_deriv<N>(tg, u, F[2]);
+  largest(F[2]);
   __syncthreads();
 #pragma unroll
   for (int b = 0; b < N; ++b) u[b] = su[yl + b * SY];
   fx_deriv<N>(tg, u, v);
+  largest(v);
 #pragma unroll
   for (int b = 0; b < N; ++b) sF[SC + yl + b * SY] = v[b];
 #pragma unroll
   for (int a = 0; a < N; ++a) u[a] = su[xl + a];
   fx_deriv<N>(tg, u, v);
+  largest(v);
 #pragma unroll
   for (int a = 0; a < N; ++a) sF[xl + a] = v[a];
-  __syncthreads();
+  // The derivatives of a smooth field are small against their bound: the flux is
+  // kept `spare` bits finer, the low halves' products included, so that points of
+  // small K do not take the rounding of the cell's largest one.
+  const int spare =
+      min(max(60 - fx_bits(fx_cell_max<N, T>(top, lc, slots + 2 * NS)), 0), 28);
+  if (32 % N2 == 0) __syncthreads();
+  const int EF = max(sh[54] + 1 - spare, sh[55]), ER = max(sh[56], EF + tg.cD);
   // the flux at the points of the z-line
   {
     const FxPair* V = md.V + c * 6 * N3 + pt;
-    const int down = sh[54];
+    const int down = min(EF - sh[54], 63), finer = max(-down, 0), coarser = max(down, 0);
+    auto flux = [&](const FxPair& a, const FxVal& x, const FxPair& b, const FxVal& y,
+                    const FxPair& d, const FxVal& z) {
+      FxAcc A = {0, 1ll << (29 - finer)};
+      fx_mac(A, a, x);
+      fx_mac(A, b, y);
+      fx_mac(A, d, z);
+      const long long low = fx_madw(a.l, x.l, fx_madw(b.l, y.l, fx_madw(d.l, z.l, 0)));
+      const long long m = A.m + (low >> 30);
+      return ((A.h << finer) + (m >> (30 - finer))) >> coarser;
+    };
 #pragma unroll
     for (int e = 0; e < N; ++e) {
       const FxVal gx = fx_split(sF[zl + e * SZ]), gy = fx_split(sF[SC + zl + e * SZ]),
                   gz = fx_split(F[2][e]);
       const FxPair xx = V[e * N2], yy = V[N3 + e * N2], zz = V[2 * N3 + e * N2],
                    xy = V[3 * N3 + e * N2], xz = V[4 * N3 + e * N2], yz = V[5 * N3 + e * N2];
-      FxAcc A = fx_zero(), B = fx_zero(), D = fx_zero();
-      fx_mac(A, xx, gx);
-      fx_mac(A, xy, gy);
-      fx_mac(A, xz, gz);
-      fx_mac(B, xy, gx);
-      fx_mac(B, yy, gy);
-      fx_mac(B, yz, gz);
-      fx_mac(D, xz, gx);
-      fx_mac(D, yz, gy);
-      fx_mac(D, zz, gz);
-      F[0][e] = fx_value(A) >> down;
-      F[1][e] = fx_value(B) >> down;
-      F[2][e] = fx_value(D) >> down;
+      F[0][e] = flux(xx, gx, xy, gy, xz, gz);
+      F[1][e] = flux(xy, gx, yy, gy, yz, gz);
+      F[2][e] = flux(xz, gx, yz, gy, zz, gz);
     }
   }
   // both faces of the thread's line: their terms into F and r of the line
@@ -575,12 +589,13 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
       for (int j = 0; j < 3; ++j) {
         FxAcc A = fx_zero();
         fx_mac(A, W[(3 + j) * N2], J);
-        t[up][j] = fx_value(A) >> s[4];
+        t[up][j] = fx_value(A) >> min(EF - s[4], 63);
       }
       FxAcc A = fx_zero(), B = fx_zero();
       fx_mac(A, W[7 * N2], J);
       fx_mac(B, W[6 * N2], fx_split(D));
-      const long long cv = (fx_value(A) >> s[5]) - (fx_value(B) >> s[6]);
+      const long long cv =
+          (fx_value(A) >> min(ER - s[5], 63)) - (fx_value(B) >> min(ER - s[6], 63));
       w[up] = up ? cv : -cv;
     }
 #pragma unroll
@@ -618,7 +633,7 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
     for (int j = 0; j < 3; ++j) F[j][a] = sF[j * SC + xl + a];
   }
   faces(0);
-  const int down = sh[55];
+  const int down = min(ER - EF - tg.cD, 63);
   fx_deriv_t<N>(tg, F[0], v);
 #pragma unroll
   for (int a = 0; a < N; ++a) {
@@ -664,11 +679,11 @@ k_cell_ml(const long long* __restrict__ U, const long long* __restrict__ TR,
   for (int i = 0; i < N; ++i) su[xl + i] = u[i];
   __syncthreads();
   if (active) {
-    const int ER = sh[56];
+    const bool nan = sh[7] != 0;
 #pragma unroll
     for (int l = 0; l < N; ++l)
-      y[c * N3 + l * N2 + pt] = ER == FX_NAN ? __longlong_as_double(0x7ff8000000000000ll)
-                                             : fx_to_double(su[zl + l * SZ], ER - up);
+      y[c * N3 + l * N2 + pt] = nan ? __longlong_as_double(0x7ff8000000000000ll)
+                                    : fx_to_double(su[zl + l * SZ], ER - up);
   }
 }
 

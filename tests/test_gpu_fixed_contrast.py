@@ -127,3 +127,24 @@ def test_solves_from_a_point_source(dg, k):
               m.cg_solve(b, rtol=1e-12, nodal=True, precond="jacobi")[0],
               m.cg_solve(b, rtol=1e-12, nodal=True, precond="kron")[0], xb[0]):
         assert ((x - ref).norm() / ref.norm()).item() < 1e-6
+
+
+@pytest.mark.parametrize("k", range(1, 9))
+@pytest.mark.parametrize("spread", [0.5, 1.0, 2.0, 4.0])
+def test_smooth_vector_rough_coefficient_on_a_vertex_mesh(dg, k, spread):
+    """test_smooth_vector_rough_coefficient on the multilinear kernels, whose mesh is
+    here the unit cube's own lattice."""
+    N, n3 = 2 if k > 5 else 3, (k + 1) ** 3
+    rng = np.random.default_rng(200 + k)
+    K = np.exp(spread * rng.standard_normal(N ** 3 * n3))
+    t = rng.uniform(-1, 1, (N ** 3, n3))
+    x = 1e-4 * t
+    x[:, 0] = 1.0
+    R = ExtendedReference(N, k, K)
+    unit = norm(R.apply(t * 2.0 ** -53))
+    s = np.linspace(0.0, 1.0, N + 1)
+    m = dg.Mesh(N, k)
+    m.set_vertices(np.stack(np.meshgrid(s, s, s, indexing="ij"), axis=-1))
+    m.set_coefficient(torch.from_numpy(K).cuda())
+    y = m.apply(torch.from_numpy(x.reshape(-1)).cuda()).cpu().numpy()
+    assert norm(y - R.apply(x)) < unit
