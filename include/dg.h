@@ -146,7 +146,13 @@ int dg_set_coefficient(dg_mesh* mesh, const double* K, void* stream);
  * x, y: device pointers to n_dofs values of type double (prec = DG_FP64) or
  * float (prec = DG_FP32); y is overwritten; x == y returns INVALID_ARG
  * (overlapping ranges are not detected).  The FP32 operator computes and
- * accumulates in FP32 from FP32-rounded tables and coefficients. */
+ * accumulates in FP32 from FP32-rounded tables and coefficients.
+ * FP64 on the cube and on multilinear geometries computes in 64-bit fixed point
+ * with one exponent per cell.  What it rounds away in a cell is relative to the
+ * largest values of the cell and its face neighbours, and below what rounding
+ * those to FP64 changes (FP64 arithmetic in this basis, whose results mix the
+ * whole cell, has an error of the same kind).  A NaN or an infinity in a cell
+ * gives NaN in that cell and its face neighbours. */
 int dg_apply(const dg_mesh* mesh, const void* x, void* y, int prec, void* stream);
 
 /* xbar = A(K)^T ybar.  The paper has no counterpart: this is the adjoint that
@@ -159,8 +165,8 @@ int dg_apply_adjoint(const dg_mesh* mesh, const void* ybar, void* xbar, int prec
 /* Same as dg_apply but x and y are HOST buffers (pinned or pageable): the
  * Section 3.3 operator application with the host<->device copies inside the
  * call (the paper has no counterpart; it runs on host memory throughout).  The
- * mesh is cut into slabs of z-layers, one per 3 MB and at most 16: x is copied in slab by slab
- * on a copy stream, pass 1 of each slab runs on an internal stream as soon as
+ * mesh is cut into slabs of z-layers, one per 3 MB and at most 16: x is copied in
+ * slab by slab on a copy stream, pass 1 of each slab runs on an internal stream as soon as
  * its x has arrived, pass 2 of slab s runs on `stream` once pass 1 has covered
  * slab s+1, and y is copied back slab by slab on a second copy stream, so that
  * with pinned buffers both copies overlap the kernels.  Blocks until y is
@@ -225,8 +231,8 @@ int dg_coeff_grad(const dg_mesh* mesh, const double* u, const double* v, double*
  *   same solver (precision and preconditioner) continues from x in the
  *   Legendre basis (its iterations counted in iterations, one more outer
  *   iteration).  Formed on the first such solve after dg_set_coefficient:
- *   two solve vectors, for the mixed mode h K at the points in FP32, for the Kronecker blocks the rotated factors.  Cube
- *   meshes only.
+ *   two solve vectors, for the mixed mode h K at the points in FP32, for the
+ *   Kronecker blocks the rotated factors.  Cube meshes only.
  * Stops when ||b - A x|| <= rtol ||b|| recomputed in FP64.  Blocking.
  * Returns NOT_CONVERGED at maxit (x holds the last iterate), BREAKDOWN on
  * <p, Ap> <= 0 or non-finite scalars, TIMEOUT if a bounded wait of the mixed
@@ -388,7 +394,11 @@ int dg_peak_probe(int kind, double* tflops, void* stream);
  * `stream`; INVALID_ARG on NULL, aliased vectors or an affine or multilinear
  * mesh.  dg_apply_nodal: y_hat = (Q A(K) Q^T) x_hat in FP64 (two kernels:
  * face traces by Lagrange end values, then per-line operators and neighbour
- * face terms), with the line operators that dg_set_coefficient formed. */
+ * face terms), with the line operators that dg_set_coefficient formed.  A point of
+ * this basis is coupled to its three lines only and keeps FP64's precision
+ * relative to them, whatever else the cell holds: cells whose values differ by
+ * more than fixed point allows for (2^7 in x, 2^4 in the line operators) are
+ * computed in FP64 arithmetic, at its speed. */
 int dg_to_nodal(const dg_mesh* mesh, const double* x, double* xhat, void* stream);
 int dg_to_modal(const dg_mesh* mesh, const double* xhat, double* x, void* stream);
 int dg_apply_nodal(const dg_mesh* mesh, const double* xhat, double* yhat, void* stream);

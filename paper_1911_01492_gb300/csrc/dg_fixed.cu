@@ -43,7 +43,7 @@ k_trace_fx(XL x, long long* __restrict__ U, long long* __restrict__ TR,
   fx_trace_cells<N, MODAL, T>(x, U, TR, expU, mark, c0, nblk, tab, smem);
 }
 
-// Kernel parameter with the data of fx_cell_wide: in the point basis only.
+// Kernel parameter with the data of fx_cells_wide: in the point basis only.
 template <bool MODAL>
 struct FxWideArg {
   __device__ __forceinline__ FxWide get() const { return {}; }

@@ -29,10 +29,10 @@
 // sees its three lines, and FP64 keeps 53 bits of each: there a cell that may hold
 // points whose lines are all small against the cell's largest one, in the vector
 // (2^7) or in the operator (2^4), or that is outweighed by 2^9 by a neighbour with
-// small lines towards it, is applied in FP64 (fx_cell_wide), as exact
+// small lines towards it, is applied in FP64 (fx_cells_wide), as exact
 // as FP64 throughout.  Lognormal fields of unit variance have no such cells (line
 // operators of a cell within 2^3.2) and pay 3 % for the marks (64^3 Q3 345 -> 356
-// us); a field of which every cell is marked takes 2.7 ms there, the FP64 kernels
+// us); a field of which every cell is marked takes 2.8 ms there, the FP64 kernels
 // took 1.25.
 #pragma once
 
@@ -472,7 +472,7 @@ __device__ __forceinline__ void fx_trace_cells(const XL& x, long long* __restric
   }
 }
 
-// What fx_cell_wide reads: h w_q K, h gamma [c][6], the marks of the vector, the
+// What fx_cells_wide reads: h w_q K, h gamma [c][6], the marks of the vector, the
 // FP64 tables of the scaled point basis.
 struct FxWide {
   const double *kt, *gh;
@@ -480,103 +480,117 @@ struct FxWide {
   const DGTabN<double>* tn;
 };
 
-// Pass 2 in FP64 for the cells of a block whose threads call it with `mine`
-// (fx_cell_cells; the others only help with the barriers): y = sum over the
-// directions of Dh^T (h K . Dh x) and the face terms, from x itself.  Returns the
-// thread's part of <x, A x>.  Kept out of line, so that the fixed-point path keeps
-// its registers.
+// Pass 2 in FP64 for the marked cells of a block (bit k of cells: c0 + k): y = sum
+// over the directions of Dh^T (h K . Dh x) and the face terms, from x itself.
+// Returns the thread's part of <x, A x> over these cells.  Every thread of the block
+// calls it.  A chain of FP64 instructions is what a block with one marked cell waits
+// for, so the n^2-thread groups of the block take a cell's three directions side by
+// side (Kronecker solves in this basis, whose directions mark a few cells in most
+// iterations, 12^3 Q4: 40.3 ms, one direction after the other 44.0, no cell marked
+// 37.4).  Kept out of line, so that the fixed-point path keeps its registers.
 template <int N, int BT>
-__device__ __noinline__ double fx_cell_wide(const double* x, const double* kt, const double* gh,
-                                            const DGTabN<double>* tn, double* y, long long c0,
-                                            int nblk, int Nc, bool mine, double* smem) {
+__device__ __noinline__ double fx_cells_wide(const double* x, const double* kt, const double* gh,
+                                             const DGTabN<double>* tn, double* y, long long c0,
+                                             unsigned cells, int Nc, double* smem) {
   constexpr int C = Cfg<N>::CPB, N2 = N * N, N3 = N * N * N;
   constexpr int SY = LinePad<N>::SY, SZ = LinePad<N>::SZ, SC = LinePad<N>::SC;
+  constexpr int ROOM = C / 2;  // cells at a time: x and the three directions' sums
   constexpr double sigma = 2.0 * N * N;
   const DGTabN<double>& t = *tn;
-  const int lc = threadIdx.x / N2, pt = threadIdx.x - lc * N2;
+  const int group = threadIdx.x / N2, pt = threadIdx.x - group * N2;
   const int p = pt % N, q = pt / N;
-  mine = mine && lc < nblk;
-  const long long c = c0 + (mine ? lc : 0);
-  double* su = smem + (mine ? lc : 0) * SC;
-  double* sr = su + C * SC;
-  const unsigned nu = (unsigned)Nc, row = (unsigned)c / nu;
-  const int crd[3] = {(int)((unsigned)c - row * nu), (int)(row % nu), (int)(row / nu)};
+  const unsigned nu = (unsigned)Nc;
   const double iw = t.isw[p] * t.isw[p] * (t.isw[q] * t.isw[q]);
-  if (mine) {
-#pragma unroll
-    for (int e = 0; e < N; ++e) su[e * SZ + q * SY + p] = x[c * N3 + e * N2 + pt];
-  }
-#pragma unroll 1
-  for (int dir = 2; dir >= 0; --dir) {
-    // the thread's line: points at + f step of the cell, at2 + f step2 in smem
-    const int at = dir == 2 ? pt : dir == 1 ? q * N2 + p : q * N2 + p * N;
-    const int step = dir == 2 ? N2 : dir == 1 ? N : 1;
-    const int at2 = dir == 2 ? q * SY + p : dir == 1 ? q * SZ + p : q * SZ + p * SY;
-    const int step2 = dir == 2 ? SZ : dir == 1 ? SY : 1;
-    __syncthreads();
-    if (!mine) continue;
-    double F[N], cv[2], cd[2];
-    {
-      double u[N], v0 = 0.0, v1 = 0.0, q0 = 0.0, q1 = 0.0;
-#pragma unroll
-      for (int f = 0; f < N; ++f) {
-        u[f] = su[at2 + f * step2];
-        // end values and outward half derivatives
-        v0 = fma(t.l0[f], u[f], v0);
-        v1 = fma(t.l1[f], u[f], v1);
-        q0 = fma(-t.hdl0[f], u[f], q0);
-        q1 = fma(t.hdl1[f], u[f], q1);
-      }
-#pragma unroll
-      for (int f = 0; f < N; ++f) {
-        double g = 0.0;
-#pragma unroll
-        for (int j = 0; j < N; ++j) g = fma(t.Dh[f][j], u[j], g);
-        F[f] = kt[c * N3 + at + f * step] * (iw * (t.isw[f] * t.isw[f])) * g;
-      }
-      const long long stride = dir == 0 ? 1 : dir == 1 ? Nc : (long long)Nc * Nc;
-      const int cdir = dir == 0 ? crd[0] : dir == 1 ? crd[1] : crd[2];
-#pragma unroll
-      for (int up = 0; up < 2; ++up) {
-        double J = up ? v1 : v0, S = 2.0 * (up ? q1 : q0), once = 2.0;
-        if (up ? cdir < Nc - 1 : cdir > 0) {
-          const double* xn = x + (up ? c + stride : c - stride) * N3 + at;
-          double vn = 0.0, qn = 0.0;  // its outward direction is the opposite one
-#pragma unroll
-          for (int f = 0; f < N; ++f) {
-            const double w = xn[f * step];
-            vn = fma(up ? t.l0[f] : t.l1[f], w, vn);
-            qn = fma(up ? t.hdl0[f] : -t.hdl1[f], w, qn);
-          }
-          J -= vn;
-          S = (up ? q1 : q0) + qn;
-          once = 1.0;
-        }
-        const double g = gh[c * 6 + 2 * dir + up];
-        cv[up] = g * (sigma * J - S);
-        cd[up] = g * once * J;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      double r = dir == 2 ? 0.0 : sr[at2 + i * step2];
-      r = fma(t.l0[i], cv[0], r);
-      r = fma(t.hdl0[i], cd[0], r);
-      r = fma(t.l1[i], cv[1], r);
-      r = fma(-t.hdl1[i], cd[1], r);
-#pragma unroll
-      for (int f = 0; f < N; ++f) r = fma(t.Dh[f][i], F[f], r);
-      sr[at2 + i * step2] = r;
-    }
-  }
-  __syncthreads();
+  const int count = __popc(cells);
+  auto cell = [&](int k) {  // the k-th marked one
+    unsigned m = cells;
+    for (; k > 0; --k) m &= m - 1;
+    return c0 + (__ffs((int)m) - 1);
+  };
   double dot = 0.0;
-  if (mine) {
+  for (int first = 0; first < count; first += ROOM) {
+    const int here = min(count - first, ROOM);
+    __syncthreads();
+    for (int i = threadIdx.x; i < here * N3; i += BT) {
+      const int k = i / N3, o = i - k * N3, e = o / N2, r = o - e * N2;
+      const long long c = cell(first + k);
+      smem[4 * k * SC + e * SZ + (r / N) * SY + r % N] = x[c * N3 + o];
+    }
+    __syncthreads();
+    for (int task = group < C ? group : 3 * here; task < 3 * here; task += C) {
+      const int k = task / 3, dir = task - 3 * k;
+      const long long c = cell(first + k);
+      const double* su = smem + 4 * k * SC;
+      double* sr = smem + (4 * k + 1 + dir) * SC;
+      // the thread's line: points at + f step of the cell, at2 + f step2 in smem
+      const int at = dir == 2 ? pt : dir == 1 ? q * N2 + p : q * N2 + p * N;
+      const int step = dir == 2 ? N2 : dir == 1 ? N : 1;
+      const int at2 = dir == 2 ? q * SY + p : dir == 1 ? q * SZ + p : q * SZ + p * SY;
+      const int step2 = dir == 2 ? SZ : dir == 1 ? SY : 1;
+      const unsigned row = (unsigned)c / nu;
+      const int at_dir = dir == 0   ? (int)((unsigned)c - row * nu)
+                         : dir == 1 ? (int)(row % nu)
+                                    : (int)(row / nu);
+      const long long stride = dir == 0 ? 1 : dir == 1 ? Nc : (long long)Nc * Nc;
+      double F[N], cv[2], cd[2];
+      {
+        double u[N], v0 = 0.0, v1 = 0.0, q0 = 0.0, q1 = 0.0;
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      const int o = e * SZ + q * SY + p;
-      y[c * N3 + e * N2 + pt] = sr[o];
-      dot = fma(su[o], sr[o], dot);
+        for (int f = 0; f < N; ++f) {
+          u[f] = su[at2 + f * step2];
+          // end values and outward half derivatives
+          v0 = fma(t.l0[f], u[f], v0);
+          v1 = fma(t.l1[f], u[f], v1);
+          q0 = fma(-t.hdl0[f], u[f], q0);
+          q1 = fma(t.hdl1[f], u[f], q1);
+        }
+#pragma unroll
+        for (int f = 0; f < N; ++f) {
+          double g = 0.0;
+#pragma unroll
+          for (int j = 0; j < N; ++j) g = fma(t.Dh[f][j], u[j], g);
+          F[f] = kt[c * N3 + at + f * step] * (iw * (t.isw[f] * t.isw[f])) * g;
+        }
+#pragma unroll
+        for (int up = 0; up < 2; ++up) {
+          double J = up ? v1 : v0, S = 2.0 * (up ? q1 : q0), once = 2.0;
+          if (up ? at_dir < Nc - 1 : at_dir > 0) {
+            const double* xn = x + (up ? c + stride : c - stride) * N3 + at;
+            double vn = 0.0, qn = 0.0;  // its outward direction is the opposite one
+#pragma unroll
+            for (int f = 0; f < N; ++f) {
+              const double w = xn[f * step];
+              vn = fma(up ? t.l0[f] : t.l1[f], w, vn);
+              qn = fma(up ? t.hdl0[f] : -t.hdl1[f], w, qn);
+            }
+            J -= vn;
+            S = (up ? q1 : q0) + qn;
+            once = 1.0;
+          }
+          const double g = gh[c * 6 + 2 * dir + up];
+          cv[up] = g * (sigma * J - S);
+          cd[up] = g * once * J;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        double r = t.l0[i] * cv[0];
+        r = fma(t.hdl0[i], cd[0], r);
+        r = fma(t.l1[i], cv[1], r);
+        r = fma(-t.hdl1[i], cd[1], r);
+#pragma unroll
+        for (int f = 0; f < N; ++f) r = fma(t.Dh[f][i], F[f], r);
+        sr[at2 + i * step2] = r;
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < here * N3; i += BT) {
+      const int k = i / N3, o = i - k * N3, e = o / N2, r = o - e * N2;
+      const long long c = cell(first + k);
+      const double* sx = smem + 4 * k * SC + e * SZ + (r / N) * SY + r % N;
+      const double v = (sx[3 * SC] + sx[2 * SC]) + sx[SC];
+      y[c * N3 + o] = v;
+      dot = fma(sx[0], v, dot);
     }
   }
   return dot;
@@ -642,7 +656,7 @@ __device__ __forceinline__ double fx_cell_cells(
     }
   }
   if (MODAL && 32 % N2 != 0 && threadIdx.x < 2 * FxSmem<N, BT>::NS) slots[threadIdx.x] = 0;
-  if (!MODAL && threadIdx.x == 0) slots[0] = 0;  // set if a cell of the block is applied in FP64
+  if (!MODAL && threadIdx.x == 0) slots[0] = 0;  // the cells of the block applied in FP64
   long long u[N], r[N];
   // z-lines (a = p, b = q)
 #pragma unroll
@@ -671,7 +685,7 @@ __device__ __forceinline__ double fx_cell_cells(
 #pragma unroll
     for (int f = 7; f < 13; ++f) enb = max(enb, sexp[active ? lc : 0][f] + tab.bump);
     wide = active && !bad && (eown >= FX_WIDE / 2 || enb - eown > 9);
-    if (wide) slots[0] = 1;
+    if (wide && pt == 0) atomicOr(slots, 1u << lc);
   }
   for (int f = pt; f < 6; f += N2) {
     if (!active) break;
@@ -803,11 +817,9 @@ __device__ __forceinline__ double fx_cell_cells(
         y(c * N3 + e * N2 + q * N + p, __longlong_as_double(sr[e * SZ + q * SY + p]));
     }
     if (slots[0] != 0) {
-      __syncthreads();
-      const double d =
-          fx_cell_wide<N, BT>(static_cast<const double*>(xU), wd.kt, wd.gh, wd.tn, y.y, c0, nblk,
-                              Nc, wide, reinterpret_cast<double*>(smem));
-      if (wide) dot = d;
+      if (wide) dot = 0.0;
+      dot += fx_cells_wide<N, BT>(static_cast<const double*>(xU), wd.kt, wd.gh, wd.tn, y.y, c0,
+                                  slots[0], Nc, reinterpret_cast<double*>(smem));
     }
     return DOT && bad ? qnan : dot;
   }

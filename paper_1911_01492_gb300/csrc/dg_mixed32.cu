@@ -996,7 +996,7 @@ struct Pass32F {
   template <typename T>
   static cudaError_t run(const dg_mesh* m, int pass, const float* x, float* y, long long cbeg,
                          long long cend, const int* skip, cudaStream_t s) {
-    constexpr int C = Cfg<N>::CPB, N3 = N * N * N;
+    constexpr int C = Cfg<N>::CPB;
     if (cend <= cbeg) return cudaSuccess;
     if (pass == 1)
       k_trace32<N><<<(unsigned)((cend - cbeg + C - 1) / C), Cfg<N>::THREADS, 0, s>>>(

@@ -18,7 +18,8 @@
 // and x into the basis once and x back once.
 //
 // In that basis the scaling is folded into the data: the line operators of
-// Q A Q^T are those of A_pt times isw_i isw_j / (w_s w_t) (k_lines_fx, dg_fixed.cu); the Lagrange end values carry isw_a = 1/sqrt(w_a); the face weight
+// Q A Q^T are those of A_pt times isw_i isw_j / (w_s w_t) (k_lines_fx,
+// dg_fixed.cu); the Lagrange end values carry isw_a = 1/sqrt(w_a); the face weight
 // h gamma w_s w_t / 2 of a face point loses its tangential weights against
 // the two isw factors of the traces, so every point of a face has the weight
 // h gamma / 2 and no per-point face-weight array is read.
