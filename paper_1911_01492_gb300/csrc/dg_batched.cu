@@ -39,11 +39,13 @@
 // Degrees 1..4 run in 128-thread blocks with registers for eight of them per SM
 // (the fixed-point passes wait for memory; 32 x 16^3 Q2: six blocks 176 ms,
 // eight 147, ten 161), a batch of degrees 1 and 2 in an instantiation without
-// the larger passes' registers (141 ms); a batch with any degree 5..8 runs in a
-// 256-thread instantiation (the operator kernels' cell groups need up to 256
-// threads there; three blocks: fewer are slower although nothing spills then,
-// 5^3 Q6 70 against 86 ms).  The vector recurrences and inner products stay in
-// loops of their own: inside the passes they took 190 instead of 178 ms.
+// the larger passes' registers (140 ms; 142 in the larger one; 64 x 8^3 Q1 10.9
+// and 10.9, 16 x 24^3 Q1 66.9 and 68.0, 8 x 24^3 Q2 192.7 and 195.9).  A batch
+// with any degree 5..8 runs in a 256-thread instantiation (the operator kernels'
+// cell groups need up to 256 threads there; three blocks: fewer are slower
+// although nothing spills then, 5^3 Q6 70 against 86 ms).  The vector recurrences
+// and inner products stay in loops of their own: inside the passes they took 190
+// instead of 178 ms.
 #include <chrono>
 #include <cmath>
 #include <cstdio>

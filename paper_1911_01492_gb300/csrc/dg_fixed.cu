@@ -67,7 +67,9 @@ FxWideArg<MODAL> wide_arg(const dg_mesh* m) {
 // waits for memory most of the time, so more warps help until values spill.
 // Measured (us; no aim / chosen / one more): 64^3 Q3 370 / 340 / 354,
 // 27^3 Q5 144 / 127 / 128, 24^3 Q6 201 / 156 / 161, 22^3 Q7 201 / 170 / 190,
-// 20^3 Q8 231 / 227 / 227.
+// 20^3 Q8 231 / 227 / 227; with ten in place of one more (Legendre, point basis):
+// 100^3 Q1 181 / 201 / 186, 214 / 198 / 185, 64^3 Q2 166 / 167 / 162,
+// 168 / 151 / 146, 40^3 Q4 193 / 185 / 226, 193 / 169 / 218.
 template <int N>
 struct FxCellBlocks {
   static constexpr int value = N <= 5 ? 8 : N == 6 ? 5 : N == 7 ? 4 : N == 8 ? 5 : 3;

@@ -442,8 +442,9 @@ extern "C" int dg_apply_host(const dg_mesh* mc, const void* x_host, void* y_host
   const long long layer = (long long)m->N * m->N;  // cells per z-layer
   // A slab costs about 10 us of launches and events, hidden only while the copies
   // take longer: one slab per 3 MB of a vector.  Measured (us; 1 / this rule /
-  // always 16): 10^3 Q4 50 / 50 / 134, 18^3 Q3 74 / 74 / 124, 26^3 Q3
-  // 163 / 137 / 208, 40^3 Q3 485 / 324 / 330; 64^3 Q3 16 slabs 1065, 32 1138.
+  // always 16): 10^3 Q4 49 / 51 / 134, 18^3 Q3 71 / 72 / 120, 26^3 Q3
+  // 153 / 146 / 202, 40^3 Q3 477 / 329 / 340; 64^3 Q3 one slab 1796, 16 1070,
+  // 32 1138.
   const long long by_size = (long long)(m->ndofs * (long long)esz) / (3ll << 20);
   int nslab_max = by_size < 1 ? 1 : by_size > DG_HOST_SLABS ? DG_HOST_SLABS : (int)by_size;
   if (nslab_max > m->N) nslab_max = m->N;

@@ -31,7 +31,7 @@
 // own m; pass 2 (k_cell_ml) reads the neighbours'.  Every array has its own
 // exponent (per cell, or per face for the face coefficients) and the sums take
 // the largest.  The FP64 kernels executed 196 FP64 flops per DOF at one
-// instruction per 64 cycles: 40^3 Q3 1003 us, now 256 us.
+// instruction per 64 cycles: 40^3 Q3 1003 us, now 266 us.
 #include <cmath>
 #include <vector>
 
